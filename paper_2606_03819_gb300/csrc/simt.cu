@@ -1,185 +1,351 @@
 // CUDA-core (fp32 FMA) kernels of the TF_F32 path: the same LM-head pass and SwiGLU of Eq. 1
 // as the tensor-core path, for fp32 inputs whose 1e-4 accuracy target rules out TF32 / bf16
 // tensor-core arithmetic. Same partial format, same merge.
+//
+// Both contractions share one main loop: a CTA of 128 threads multiplies kTileW rows of W by RT
+// rows of X (K contiguous in both). What bounds it is the fp32 FMA rate once there are more than
+// about eight rows (W is read once per row group), and HBM below that, so
+//  - each thread keeps 8 x RT/8 outputs in registers (a plain one-column-per-thread layout is
+//    bound by shared-memory loads) and each output as two sums, over even and odd k, so that one
+//    packed fma.rn.f32x2 takes two neighbouring k of both operands as they lie in shared memory;
+//  - stages of 32 k arrive by cp.async into a ring of kStages, rows padded to 36 floats so that
+//    the 16-byte loads of eight neighbouring rows hit all banks once;
+//  - the approximator's GEMMs, which have few output tiles, split K over the CTAs of a cluster:
+//    each leaves its partial tile in shared memory and the cluster's CTAs add the tiles in K
+//    order through distributed shared memory (no workspace, the same bits on every run).
 #include <math.h>
 
 #include "common.cuh"
+#include "tc_ptx.cuh"
 
 namespace tf {
 namespace {
 
-constexpr int kRowsPerCta = 32;
-constexpr int kKChunk = 32;
+constexpr int kTileW = 128;         // rows of W per CTA tile: half a vocabulary block, 64 gate + 64 up, or 128 outputs
+constexpr int kKC = 32;             // k per stage
+constexpr int kLd = kKC + 4;        // padded row of a stage, in floats
+constexpr int kStages = 3;
+constexpr int kThreads = 128;
+constexpr int kZLd = kTileW + 4;    // row of the staged tile: 4 chunks of 33 floats, or 128 and a pad of 4
+static_assert(kZLd == 4 * 33, "the chunk layout of the LM head fills a row");
+constexpr int kMaxClusterK = 8;     // K-ranges of one approximator tile (the portable cluster size)
 
-// One CTA: rows [r0, r0 + 32) x vocabulary block [v0, v0 + 256). Thread t owns vocabulary column
-// v0 + t and accumulates its 32 logits; the block is then staged in shared memory and one warp
-// per row computes, with warp shuffles, the per-chunk three largest logits (ids of the first
-// two) and the per-half max, sum of exp and best entry.
-__global__ void __launch_bounds__(256) lmhead_simt_kernel(const float* __restrict__ W, const float* __restrict__ X,
-                                                          int n_rows, int d, int V, float inv_temp,
-                                                          Partials partials, int n_tiles, int* reset_status) {
-    pdl_trigger();
-    pdl_wait();
-    if (reset_status && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *reset_status = 0;
-    __shared__ float xs[kRowsPerCta][kKChunk + 1];
-    __shared__ float ws[kBlockV][kKChunk + 1];
-    const int vt = blockIdx.x;
-    const int r0 = blockIdx.y * kRowsPerCta;
-    const int t = threadIdx.x;
-    float acc[kRowsPerCta];
-#pragma unroll
-    for (int r = 0; r < kRowsPerCta; ++r) acc[r] = 0.0f;
+template <int RT>
+struct Tile {
+    static constexpr int kStageFloats = (kTileW + RT) * kLd;
+    static constexpr int kSmemBytes = kStages * kStageFloats * 4;
+    static_assert(RT * kZLd <= kStages * kStageFloats, "the staged tile reuses the ring");
+};
 
-    for (int k0 = 0; k0 < d; k0 += kKChunk) {
-        for (int i = t; i < kRowsPerCta * kKChunk; i += 256) {
-            const int r = i / kKChunk, k = i % kKChunk;
-            xs[r][k] = (r0 + r < n_rows && k0 + k < d) ? X[static_cast<size_t>(r0 + r) * d + k0 + k] : 0.0f;
-        }
-        for (int i = t; i < kBlockV * kKChunk; i += 256) {
-            const int v = i / kKChunk, k = i % kKChunk;
-            const int gv = vt * kBlockV + v;
-            ws[v][k] = (gv < V && k0 + k < d) ? W[static_cast<size_t>(gv) * d + k0 + k] : 0.0f;
-        }
-        __syncthreads();
-#pragma unroll 4
-        for (int k = 0; k < kKChunk; ++k) {
-            const float w = ws[t][k];
-#pragma unroll
-            for (int r = 0; r < kRowsPerCta; ++r) acc[r] = fmaf(xs[r][k], w, acc[r]);
-        }
-        __syncthreads();
-    }
-    // stage the logits of the block: zt[r][t]
-    float* zt = &ws[0][0];
-    const bool valid = vt * kBlockV + t < V;
-#pragma unroll
-    for (int r = 0; r < kRowsPerCta; ++r) zt[r * kBlockV + t] = valid ? acc[r] * inv_temp : -INFINITY;
-    __syncthreads();
+// 16 (VEC) or 4 bytes from global to shared memory, zeros where !ok (src then only has to be a
+// valid address, nothing is read).
+template <bool VEC>
+__device__ __forceinline__ void copy_async(float* dst, const float* src, bool ok) {
+    const int n = ok ? (VEC ? 16 : 4) : 0;
+    if constexpr (VEC)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(ptx::smem_u32(dst)), "l"(src), "r"(n) : "memory");
+    else
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(ptx::smem_u32(dst)), "l"(src), "r"(n) : "memory");
+}
+__device__ __forceinline__ void copy_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void copy_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
-    const int warp = t >> 5, lane = t & 31;
-    for (int r = warp; r < kRowsPerCta; r += 8) {
-        if (r0 + r >= n_rows) break;
-        // chunk j = columns [32 j, 32 j + 32) of the block; lane holds column 32 j + lane
-        float z[kChunks];
+// a * b + c on two packed fp32 values, each rounded to nearest.
+__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b, unsigned long long c) {
+    unsigned long long d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ float sum2(unsigned long long v) {
+    return __uint_as_float(static_cast<uint32_t>(v)) + __uint_as_float(static_cast<uint32_t>(v >> 32));
+}
+
+// rows [r0, r0 + n) of a [.., K] matrix (n <= 0: none)
+struct RowsOf {
+    const float* p;   // row r0
+    int n;
+};
+
+// One stage of a tile: rows 0..63 of `lo` and 64..127 of `hi` into the stage's W part (for one
+// matrix hi continues lo), or RT rows of X into its X part; k0 .. k0 + 31, zeros past kend.
+template <bool VEC, int ROWS>
+__device__ __forceinline__ void load_rows(float* dst, const RowsOf& m, int K, int k0, int kend) {
+    constexpr int kPer = VEC ? 4 : 1;                 // floats per copy
+    constexpr int kCols = kKC / kPer;                 // copies per row
+    const int col = (threadIdx.x % kCols) * kPer, row0 = threadIdx.x / kCols;
+    constexpr int kStep = kThreads / kCols;           // rows per pass of the CTA
+    const bool kin = k0 + col < kend;
+    const float* src = m.p + static_cast<size_t>(row0) * K + k0 + col;
 #pragma unroll
-        for (int j = 0; j < kChunks; ++j) z[j] = zt[r * kBlockV + lane + 32 * j];
-        const int row = r0 + r;
-        float hm[2] = {-INFINITY, -INFINITY}, hsum[2] = {0.0f, 0.0f}, hbv[2] = {-INFINITY, -INFINITY};
-        int hbid[2] = {-1, -1};
-#pragma unroll
-        for (int j = 0; j < kChunks; ++j) {
-            const int cbase = vt * kBlockV + 32 * j;
-            // three rounds of a warp-wide (value desc, id asc) arg-max over the chunk
-            float x = z[j];
-            float tv[3];
-            int ti[3];
-#pragma unroll
-            for (int t3 = 0; t3 < 3; ++t3) {
-                float bv = x;
-                int bid = x > -INFINITY ? lane : 64;
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) {
-                    const float ov = __shfl_xor_sync(0xffffffffu, bv, o);
-                    const int oid = __shfl_xor_sync(0xffffffffu, bid, o);
-                    if (ov > bv || (ov == bv && oid < bid)) {
-                        bv = ov;
-                        bid = oid;
-                    }
-                }
-                tv[t3] = bv;
-                ti[t3] = bv > -INFINITY ? bid : 0;
-                if (bv > -INFINITY && lane == bid) x = -INFINITY;
-            }
-            float e = tv[0] > -INFINITY ? expf(z[j] - tv[0]) : 0.0f;
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
-            const int h = j / (kChunks / 2);
-            if (tv[0] > hbv[h]) {
-                hbv[h] = tv[0];
-                hbid[h] = cbase + ti[0];
-            }
-            if (tv[0] > -INFINITY) {
-                const float mn = fmaxf(hm[h], tv[0]);
-                hsum[h] = hsum[h] * expf(hm[h] - mn) + e * expf(tv[0] - mn);
-                hm[h] = mn;
-            }
-            if (lane == 0)
-                partials.chunks[partials.chunk_at(vt, j, row)] =
-                    make_float4(tv[0], tv[1], tv[2], __int_as_float(ti[0] | (ti[1] << 8)));
-        }
-        if (lane == 0)
-            for (int h = 0; h < 2; ++h)
-                partials.halves[partials.half_at(vt, h, row)] = make_float4(hm[h], hsum[h], hbv[h], __int_as_float(hbid[h]));
+    for (int r = row0; r < ROWS; r += kStep, src += static_cast<size_t>(kStep) * K) {
+        const bool ok = kin && r < m.n;
+        copy_async<VEC>(dst + r * kLd + col, ok ? src : m.p, ok);
     }
 }
 
-// C[n_rows, N] = X[n_rows, K] W[N, K]^T on 64 x 64 tiles (16 x 16 threads, 4 x 4 outputs each).
-// GATEUP: out = SiLU(X Wg^T) * (X Wu^T); DOWN: out = hidden[stage-2 row's depth] + X Wd^T.
-template <bool GATEUP>
-__global__ void __launch_bounds__(256) swiglu_simt_kernel(const float* __restrict__ X, const float* __restrict__ W0,
-                                                          const float* __restrict__ W1, int n_rows, int K, int N,
-                                                          float* __restrict__ out, const float* __restrict__ hidden,
-                                                          int R, int M, int gamma) {
-    pdl_trigger();
+// acc[i][j] += W[vt + 16 i] . X[rt + 8 j] over k in [k0, k1): the pipelined main loop. The
+// weights are no kernel's output: the first stages' W is requested before the dependency wait.
+template <int RT, bool VEC>
+__device__ __forceinline__ void mainloop(float* ring, const RowsOf& lo, const RowsOf& hi, const RowsOf& x, int K, int k0,
+                                         int k1, unsigned long long (&acc)[8][RT / 8]) {
+    constexpr int TR = RT / 8;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int vt = (lane & 7) + 8 * (warp & 1), rt = (lane >> 3) + 4 * (warp >> 1);
+    const int n = (k1 - k0 + kKC - 1) / kKC;
+    auto stage = [&](int t) { return ring + (t % kStages) * Tile<RT>::kStageFloats; };
+    auto load_w = [&](int t) {
+        load_rows<VEC, 64>(stage(t), lo, K, k0 + t * kKC, k1);
+        load_rows<VEC, 64>(stage(t) + 64 * kLd, hi, K, k0 + t * kKC, k1);
+    };
+    auto load_x = [&](int t) { load_rows<VEC, RT>(stage(t) + kTileW * kLd, x, K, k0 + t * kKC, k1); };
+#pragma unroll
+    for (int t = 0; t < kStages - 1; ++t)
+        if (t < n) load_w(t);
     pdl_wait();
-    constexpr int T = 64, KC = 16;
-    __shared__ float xs[KC][T + 4];
-    __shared__ float w0s[KC][T + 4];
-    __shared__ float w1s[GATEUP ? KC : 1][T + 4];
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    const int row0 = blockIdx.y * T, col0 = blockIdx.x * T;
-    float a0[4][4] = {}, a1[4][4] = {};
-    for (int k0 = 0; k0 < K; k0 += KC) {
-        for (int i = threadIdx.x; i < T * KC; i += 256) {
-            const int r = i / KC, k = i % KC;
-            const bool kin = k0 + k < K;
-            xs[k][r] = (row0 + r < n_rows && kin) ? X[static_cast<size_t>(row0 + r) * K + k0 + k] : 0.0f;
-            w0s[k][r] = (col0 + r < N && kin) ? W0[static_cast<size_t>(col0 + r) * K + k0 + k] : 0.0f;
-            if (GATEUP) w1s[k][r] = (col0 + r < N && kin) ? W1[static_cast<size_t>(col0 + r) * K + k0 + k] : 0.0f;
-        }
-        __syncthreads();
 #pragma unroll
-        for (int k = 0; k < KC; ++k) {
-            float xv[4], wv0[4], wv1[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                xv[i] = xs[k][ty * 4 + i];
-                wv0[i] = w0s[k][tx * 4 + i];
-                if (GATEUP) wv1[i] = w1s[k][tx * 4 + i];
-            }
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    a0[i][j] = fmaf(xv[i], wv0[j], a0[i][j]);
-                    if (GATEUP) a1[i][j] = fmaf(xv[i], wv1[j], a1[i][j]);
-                }
-        }
-        __syncthreads();
+    for (int t = 0; t < kStages - 1; ++t) {
+        if (t < n) load_x(t);
+        copy_commit();                                // (an empty group keeps the count)
     }
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int r = row0 + ty * 4 + i;
-        if (r >= n_rows) continue;
-        int hid = 0;
-        if (!GATEUP) {
-            const int sq = r / R, rr = r - sq * R;
-            hid = sq * gamma + stage2_hidden_index(rr, M);
-        }
+    for (int i = 0; i < 8; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int c = col0 + tx * 4 + j;
-            if (c >= N) continue;
-            float v;
+        for (int j = 0; j < TR; ++j) acc[i][j] = 0ull;
+    for (int t = 0; t < n; ++t) {
+        copy_wait<kStages - 2>();                     // stage t has landed (this thread's part)
+        __syncthreads();                              // everyone's part, and stage t - 1 is free
+        if (t + kStages - 1 < n) {
+            load_w(t + kStages - 1);
+            load_x(t + kStages - 1);
+        }
+        copy_commit();
+        const float* ws = stage(t) + vt * kLd;
+        const float* xs = stage(t) + (kTileW + rt) * kLd;
+#pragma unroll
+        for (int k = 0; k < kKC; k += 4) {
+            ulonglong2 xv[TR];
+#pragma unroll
+            for (int j = 0; j < TR; ++j) xv[j] = *reinterpret_cast<const ulonglong2*>(xs + 8 * j * kLd + k);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const ulonglong2 wv = *reinterpret_cast<const ulonglong2*>(ws + 16 * i * kLd + k);
+#pragma unroll
+                for (int j = 0; j < TR; ++j) acc[i][j] = fma2(wv.y, xv[j].y, fma2(wv.x, xv[j].x, acc[i][j]));
+            }
+        }
+    }
+    copy_wait<0>();
+    __syncthreads();                                  // the ring may be reused
+}
+
+// ------------------------------------------------------------------------------------------
+// LM head: one CTA per (row group of RT, half vocabulary block of 128). The logits of the tile go
+// through shared memory to one thread per (row, 32-entry chunk), which keeps the chunk's three
+// largest logits, the offsets of the first two (ties to the smaller id) and the sum of
+// exp(z - max); the four threads of a row fold their chunks into the half's summary in id order.
+// Row groups are the fastest grid dimension, so the groups of a half block share its W in L2.
+// ------------------------------------------------------------------------------------------
+template <int RT, bool VEC>
+__global__ void __launch_bounds__(kThreads) lmhead_simt_kernel(const float* __restrict__ W, const float* __restrict__ X,
+                                                               int n_rows, int d, int V, float inv_temp,
+                                                               Partials partials, int* reset_status) {
+    extern __shared__ __align__(16) float ring[];
+    constexpr int TR = RT / 8;
+    pdl_trigger();
+    const int r0 = blockIdx.x * RT, v0 = blockIdx.y * kTileW, t = threadIdx.x;
+    const int rows = min(RT, n_rows - r0), cols = max(0, min(kTileW, V - v0));
+    // (a half block wholly past V has no row of W: nothing is read from row 0 in its place)
+    const float* wbase = W + (cols > 0 ? static_cast<size_t>(v0) * d : 0);
+    const RowsOf lo{wbase, cols}, hi{cols > 64 ? wbase + static_cast<size_t>(64) * d : wbase, cols - 64};
+    const RowsOf x{X + static_cast<size_t>(r0) * d, rows};
+    unsigned long long acc[8][TR];
+    mainloop<RT, VEC>(ring, lo, hi, x, d, 0, d, acc);
+    if (reset_status && blockIdx.x == 0 && blockIdx.y == 0 && t == 0) *reset_status = 0;
+    {
+        const int lane = t & 31, warp = t >> 5;
+        const int vt = (lane & 7) + 8 * (warp & 1), rt = (lane >> 3) + 4 * (warp >> 1);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int v = vt + 16 * i;
+#pragma unroll
+            for (int j = 0; j < TR; ++j)
+                ring[(rt + 8 * j) * kZLd + (v >> 5) * 33 + (v & 31)] = v < cols ? sum2(acc[i][j]) * inv_temp : -INFINITY;
+        }
+    }
+    __syncthreads();
+    const int r = t >> 2, c = t & 3;                  // row of the group, chunk of the half block
+    const bool mine = r < rows;                       // (t < 4 RT; whole groups of four lanes)
+    float a1 = -INFINITY, a2 = -INFINITY, a3 = -INFINITY, s = 0.0f;
+    int i1 = 0, i2 = 0;
+    if (mine) {
+        const float* z = ring + r * kZLd + c * 33;
+        float v[kChunk];
+#pragma unroll
+        for (int i = 0; i < kChunk; ++i) v[i] = z[i];
+#pragma unroll
+        for (int i = 0; i < kChunk; ++i) {
+            // strict comparisons: among equal values the smaller id ranks first
+            const bool g1 = v[i] > a1, g2 = v[i] > a2;
+            a3 = g2 ? a2 : fmaxf(a3, v[i]);
+            i2 = g1 ? i1 : (g2 ? i : i2);
+            a2 = g1 ? a1 : (g2 ? v[i] : a2);
+            i1 = g1 ? i : i1;
+            a1 = g1 ? v[i] : a1;
+        }
+        if (a1 > -INFINITY) {
+#pragma unroll
+            for (int i = 0; i < kChunk; ++i) s += expf(v[i] - a1);
+        }
+        const int tile = blockIdx.y >> 1, chunk = (blockIdx.y & 1) * (kChunks / 2) + c;
+        partials.chunks[partials.chunk_at(tile, chunk, r0 + r)] = make_float4(a1, a2, a3, __int_as_float(i1 | (i2 << 8)));
+    }
+    // the half's summary: chunk pairs, then pairs of pairs; the lower chunk keeps its entry on a tie
+    float m = a1, bv = a1;
+    int bid = a1 > -INFINITY ? v0 + c * kChunk + i1 : -1;
+#pragma unroll
+    for (int o = 1; o < 4; o <<= 1) {
+        const float m2 = __shfl_down_sync(0xffffffffu, m, o), s2 = __shfl_down_sync(0xffffffffu, s, o);
+        const float bv2 = __shfl_down_sync(0xffffffffu, bv, o);
+        const int bid2 = __shfl_down_sync(0xffffffffu, bid, o);
+        const float mn = fmaxf(m, m2);
+        if (mn > -INFINITY) s = s * expf(m - mn) + s2 * expf(m2 - mn);
+        m = mn;
+        if (bv2 > bv) {
+            bv = bv2;
+            bid = bid2;
+        }
+    }
+    if (mine && c == 0)
+        partials.halves[partials.half_at(blockIdx.y >> 1, blockIdx.y & 1, r0 + r)] = make_float4(m, s, bv, __int_as_float(bid));
+}
+
+// ------------------------------------------------------------------------------------------
+// C[n_rows, N] = X[n_rows, K] W[N, K]^T, one cluster per (N tile, row group), its CTAs on
+// consecutive K-ranges.
+// GATEUP (N tile of 64): out = SiLU(X Wg^T) * (X Wu^T); DOWN (N tile of 128): out = hidden of the
+// stage-2 row's depth + X Wd^T.
+// ------------------------------------------------------------------------------------------
+template <bool GATEUP, int RT, bool VEC>
+__global__ void __launch_bounds__(kThreads) swiglu_simt_kernel(const float* __restrict__ X, const float* __restrict__ W0,
+                                                               const float* __restrict__ W1, int n_rows, int K, int N,
+                                                               int n_rg, float* __restrict__ out,
+                                                               const float* __restrict__ hidden, int R, int M, int gamma) {
+    extern __shared__ __align__(16) float ring[];
+    constexpr int TR = RT / 8;
+    constexpr int kOut = GATEUP ? kTileW / 2 : kTileW;    // output columns of a tile
+    pdl_trigger();
+    const int ks = static_cast<int>(ptx::cluster_nctarank()), kr = static_cast<int>(ptx::cluster_ctarank());
+    const int unit = blockIdx.x / ks, rg = unit % n_rg, nt = unit / n_rg;
+    const int r0 = rg * RT, c0 = nt * kOut;
+    const int rows = min(RT, n_rows - r0), cols = min(kOut, N - c0);
+    RowsOf lo{W0 + static_cast<size_t>(c0) * K, cols}, hi;
+    if (GATEUP)
+        hi = RowsOf{W1 + static_cast<size_t>(c0) * K, cols};
+    else
+        hi = RowsOf{cols > 64 ? lo.p + static_cast<size_t>(64) * K : lo.p, cols - 64};
+    const RowsOf x{X + static_cast<size_t>(r0) * K, rows};
+    // K-ranges in whole stages
+    const int nst = (K + kKC - 1) / kKC;
+    const int k0 = static_cast<int>(static_cast<long long>(nst) * kr / ks) * kKC;
+    const int k1 = min(K, static_cast<int>(static_cast<long long>(nst) * (kr + 1) / ks) * kKC);
+    unsigned long long acc[8][TR];
+    mainloop<RT, VEC>(ring, lo, hi, x, K, k0, k1, acc);
+    {
+        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+        const int vt = (lane & 7) + 8 * (warp & 1), rt = (lane >> 3) + 4 * (warp >> 1);
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+#pragma unroll
+            for (int j = 0; j < TR; ++j) ring[(rt + 8 * j) * kZLd + vt + 16 * i] = sum2(acc[i][j]);
+    }
+    ptx::cluster_sync();                              // every partial tile of the cluster is in place
+    // this CTA's share of the tile: four columns of one row per step, summed in K order
+    const bool vec_out = N % 4 == 0;
+    for (int idx = kr * kThreads + static_cast<int>(threadIdx.x); idx < RT * kOut / 4; idx += ks * kThreads) {
+        const int r = idx / (kOut / 4), c = (idx - r * (kOut / 4)) * 4;
+        if (r >= rows || c >= cols) continue;
+        const uint32_t at = ptx::smem_u32(ring + r * kZLd + c);
+        float g[4] = {}, u[4] = {};
+        for (int s = 0; s < ks; ++s) {
+            const float4 a = ptx::ld_cluster_f4(ptx::mapa_shared(at, s));
+            g[0] += a.x; g[1] += a.y; g[2] += a.z; g[3] += a.w;
             if (GATEUP) {
-                const float g = a0[i][j];
-                v = g / (1.0f + expf(-g)) * a1[i][j];
-            } else {
-                v = hidden[static_cast<size_t>(hid) * N + c] + a0[i][j];
+                const float4 b = ptx::ld_cluster_f4(ptx::mapa_shared(at + 64 * 4, s));
+                u[0] += b.x; u[1] += b.y; u[2] += b.z; u[3] += b.w;
             }
-            out[static_cast<size_t>(r) * N + c] = v;
+        }
+        float v[4];
+        if (GATEUP) {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) v[e] = g[e] / (1.0f + expf(-g[e])) * u[e];
+        } else {
+            const int row = r0 + r, sq = row / R, rr = row - sq * R;
+            const float* h = hidden + static_cast<size_t>(sq * gamma + stage2_hidden_index(rr, M)) * N + c0 + c;
+#pragma unroll
+            for (int e = 0; e < 4; ++e) v[e] = c + e < cols ? h[e] + g[e] : 0.0f;
+        }
+        float* dst = out + static_cast<size_t>(r0 + r) * N + c0 + c;
+        if (vec_out) {
+            *reinterpret_cast<float4*>(dst) = make_float4(v[0], v[1], v[2], v[3]);
+        } else {
+            for (int e = 0; e < 4; ++e)
+                if (c + e < cols) dst[e] = v[e];
         }
     }
+    ptx::cluster_sync();                              // no CTA leaves while its tile may still be read
+}
+
+template <int RT, bool VEC>
+cudaError_t run_lmhead(const Ctx& ctx, const float* W, const float* X, int n_rows, int d, int V, float inv_temp,
+                       const Partials& partials, bool reset_status) {
+    auto kern = lmhead_simt_kernel<RT, VEC>;
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Tile<RT>::kSmemBytes);
+    if (e != cudaSuccess) return e;
+    const dim3 grid((n_rows + RT - 1) / RT, 2 * ((V + kBlockV - 1) / kBlockV));
+    return launch_pdl(kern, grid, dim3(kThreads), Tile<RT>::kSmemBytes, ctx.stream, W, X, n_rows, d, V, inv_temp, partials,
+                      reset_status ? ctx.status : static_cast<int*>(nullptr));
+}
+
+template <bool GATEUP, int RT, bool VEC>
+cudaError_t run_swiglu(const Ctx& ctx, const float* X, const float* W0, const float* W1, int n_rows, int K, int N,
+                       float* out, const float* hidden, int R, int M, int gamma, int ks) {
+    auto kern = swiglu_simt_kernel<GATEUP, RT, VEC>;
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Tile<RT>::kSmemBytes);
+    if (e != cudaSuccess) return e;
+    constexpr int kOut = GATEUP ? kTileW / 2 : kTileW;
+    const int n_rg = (n_rows + RT - 1) / RT;
+    const long long ctas = static_cast<long long>((N + kOut - 1) / kOut) * n_rg * ks;
+    if (ctas > 0x7fffffffll) return cudaErrorInvalidConfiguration;
+    return launch_pdl_cluster(kern, dim3(static_cast<unsigned>(ctas)), dim3(kThreads), Tile<RT>::kSmemBytes, ctx.stream,
+                              ks, X, W0, W1, n_rows, K, N, n_rg, out, hidden, R, M, gamma);
+}
+
+// Row group of a contraction with n_rows rows: the smallest that holds them all, at most 32 (the
+// thread tile of 8 x 4 outputs; a larger one saves no shared-memory loads that bound anything).
+int row_group(int n_rows) { return n_rows <= 8 ? 8 : n_rows <= 16 ? 16 : 32; }
+
+template <bool GATEUP>
+cudaError_t swiglu_gemm(const Ctx& ctx, const float* X, const float* W0, const float* W1, int n_rows, int K, int N,
+                        float* out, const float* hidden, int R, int M, int gamma) {
+    constexpr int kOut = GATEUP ? kTileW / 2 : kTileW;
+    // K-ranges per tile: enough CTAs for three on every SM, at least two stages each. Where even
+    // eight ranges of 32-row tiles leave SMs idle, 16-row groups double the tiles.
+    const long long tiles = (N + kOut - 1) / kOut;
+    int rt = row_group(n_rows);
+    if (rt == 32 && tiles * ((n_rows + 31) / 32) * kMaxClusterK < 2ll * ctx.num_sms) rt = 16;
+    const long long base = tiles * ((n_rows + rt - 1) / rt);
+    int ks = 1;
+    while (ks < kMaxClusterK && base * ks * 2 <= 3ll * ctx.num_sms && K >= 2 * kKC * ks * 2) ks *= 2;
+    const bool vec = K % 4 == 0;
+    if (rt == 8)
+        return vec ? run_swiglu<GATEUP, 8, true>(ctx, X, W0, W1, n_rows, K, N, out, hidden, R, M, gamma, ks)
+                   : run_swiglu<GATEUP, 8, false>(ctx, X, W0, W1, n_rows, K, N, out, hidden, R, M, gamma, ks);
+    if (rt == 16)
+        return vec ? run_swiglu<GATEUP, 16, true>(ctx, X, W0, W1, n_rows, K, N, out, hidden, R, M, gamma, ks)
+                   : run_swiglu<GATEUP, 16, false>(ctx, X, W0, W1, n_rows, K, N, out, hidden, R, M, gamma, ks);
+    return vec ? run_swiglu<GATEUP, 32, true>(ctx, X, W0, W1, n_rows, K, N, out, hidden, R, M, gamma, ks)
+               : run_swiglu<GATEUP, 32, false>(ctx, X, W0, W1, n_rows, K, N, out, hidden, R, M, gamma, ks);
 }
 
 }  // namespace
@@ -188,11 +354,20 @@ cudaError_t launch_lmhead_simt(const Ctx& ctx, int dtype, const void* lm_head, c
                                int V, float inv_temp, Partials partials, bool reset_status) {
     if (dtype != TF_F32) return cudaErrorNotSupported;
     if (n_rows <= 0) return cudaSuccess;
-    const int n_tiles = (V + kBlockV - 1) / kBlockV;
-    dim3 grid(n_tiles, (n_rows + kRowsPerCta - 1) / kRowsPerCta);
-    const cudaError_t e = launch_pdl(lmhead_simt_kernel, grid, dim3(256), 0, ctx.stream,
-                                     static_cast<const float*>(lm_head), static_cast<const float*>(x), n_rows, d, V,
-                                     inv_temp, partials, n_tiles, reset_status ? ctx.status : static_cast<int*>(nullptr));
+    const float* W = static_cast<const float*>(lm_head);
+    const float* X = static_cast<const float*>(x);
+    const bool vec = d % 4 == 0;
+    const int rt = row_group(n_rows);
+    cudaError_t e;
+    if (rt == 8)
+        e = vec ? run_lmhead<8, true>(ctx, W, X, n_rows, d, V, inv_temp, partials, reset_status)
+                : run_lmhead<8, false>(ctx, W, X, n_rows, d, V, inv_temp, partials, reset_status);
+    else if (rt == 16)
+        e = vec ? run_lmhead<16, true>(ctx, W, X, n_rows, d, V, inv_temp, partials, reset_status)
+                : run_lmhead<16, false>(ctx, W, X, n_rows, d, V, inv_temp, partials, reset_status);
+    else
+        e = vec ? run_lmhead<32, true>(ctx, W, X, n_rows, d, V, inv_temp, partials, reset_status)
+                : run_lmhead<32, false>(ctx, W, X, n_rows, d, V, inv_temp, partials, reset_status);
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
@@ -200,16 +375,13 @@ cudaError_t launch_swiglu_simt(const Ctx& ctx, const void* X, int k_in, const vo
                                const void* w_down, const void* hidden, int n_rows, int d, int I, int R, int M,
                                int gamma, void* A, void* h_prime) {
     if (n_rows <= 0) return cudaSuccess;
-    dim3 g1((I + 63) / 64, (n_rows + 63) / 64);
-    cudaError_t e = launch_pdl(swiglu_simt_kernel<true>, g1, dim3(256), 0, ctx.stream, static_cast<const float*>(X),
-                               static_cast<const float*>(w_gate), static_cast<const float*>(w_up), n_rows, k_in, I,
-                               static_cast<float*>(A), static_cast<const float*>(nullptr), R, M, gamma);
+    cudaError_t e = swiglu_gemm<true>(ctx, static_cast<const float*>(X), static_cast<const float*>(w_gate),
+                                      static_cast<const float*>(w_up), n_rows, k_in, I, static_cast<float*>(A),
+                                      nullptr, R, M, gamma);
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    dim3 g2((d + 63) / 64, (n_rows + 63) / 64);
-    e = launch_pdl(swiglu_simt_kernel<false>, g2, dim3(256), 0, ctx.stream, static_cast<const float*>(A),
-                   static_cast<const float*>(w_down), static_cast<const float*>(nullptr), n_rows, I, d,
-                   static_cast<float*>(h_prime), static_cast<const float*>(hidden), R, M, gamma);
+    e = swiglu_gemm<false>(ctx, static_cast<const float*>(A), static_cast<const float*>(w_down), nullptr, n_rows, I, d,
+                           static_cast<float*>(h_prime), static_cast<const float*>(hidden), R, M, gamma);
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
@@ -217,11 +389,9 @@ cudaError_t launch_swiglu_simt(const Ctx& ctx, const void* X, int k_in, const vo
 cudaError_t launch_linear_simt(const Ctx& ctx, const void* X, const void* w_lin, const void* hidden, int n_rows, int d,
                                int R, int M, int gamma, void* h_prime) {
     if (n_rows <= 0) return cudaSuccess;
-    dim3 grid((d + 63) / 64, (n_rows + 63) / 64);
-    const cudaError_t e = launch_pdl(swiglu_simt_kernel<false>, grid, dim3(256), 0, ctx.stream,
-                                     static_cast<const float*>(X), static_cast<const float*>(w_lin),
-                                     static_cast<const float*>(nullptr), n_rows, 2 * d, d,
-                                     static_cast<float*>(h_prime), static_cast<const float*>(hidden), R, M, gamma);
+    const cudaError_t e = swiglu_gemm<false>(ctx, static_cast<const float*>(X), static_cast<const float*>(w_lin), nullptr,
+                                             n_rows, 2 * d, d, static_cast<float*>(h_prime),
+                                             static_cast<const float*>(hidden), R, M, gamma);
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 

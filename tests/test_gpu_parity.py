@@ -83,6 +83,24 @@ def test_fp32_brute_force_v16():
     assert parity._paths(gpu["node_tok"][0], gpu["node_parent"][0]) == best
 
 
+# (batch, d, V, I, gamma, M, approx): row groups of 8, 16 and 32 with remainders; half vocabulary
+# blocks empty, one entry or ragged; rows that 16-byte copies cannot read (d or I not a multiple of
+# 4); K split over 2, 4 and 8 CTAs; output tiles with a remainder
+FP32_SIZES = [
+    (1, 128, 129, 66, 3, 2, "swiglu"),           # 3 / 5 rows, one entry in the second half block
+    (2, 100, 1000, 250, 4, 4, "swiglu"),         # 8 / 26 rows
+    (3, 130, 515, 37, 4, 5, "swiglu"),           # 12 / 48 rows, 4-byte copies everywhere
+    (5, 192, 700, 320, 5, 3, "linear"),          # 25 / 65 rows
+    (9, 1024, 2048, 1540, 4, 4, "swiglu"),       # 36 / 117 rows, K split eight ways
+    (2, 260, 640, 100, 4, 3, "swiglu_2prev"),    # 8 / 44 rows, K = 3 d
+]
+
+
+@pytest.mark.parametrize("b,d,V,I,gamma,M,approx", FP32_SIZES)
+def test_fp32_sizes(b, d, V, I, gamma, M, approx):
+    check(synth.get_config("tiny_peaked", batch=b, d=d, V=V, I=I, gamma=gamma, M=M, approx=approx))
+
+
 # ------------------------------------------------------------------ bf16 (tcgen05) path
 
 BF16_SMALL = [
