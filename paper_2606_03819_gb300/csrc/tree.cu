@@ -142,7 +142,7 @@ struct TreeArgs {
     int32_t* node_depth;
     float* node_score;
     int32_t* dev_status;
-    // optional, with B + 1 <= kMaskRows: the builder also writes the verification mask and
+    // optional, with B + 1 <= kFusedMaskMaxNodes: the builder also writes the verification mask and
     // position ids (tf_tree_mask's outputs) from the tree it holds in shared memory
     const int32_t* root_pos;
     uint8_t* mask;
@@ -194,39 +194,30 @@ __device__ __forceinline__ unsigned long long queue_key(float score, int depth, 
            (static_cast<unsigned long long>(127 - depth) << 24) | static_cast<unsigned long long>(0xFFFFFF - parent);
 }
 
-constexpr int kTreeThreads = 256;
-constexpr int kMaskRows = kFusedMaskMaxNodes;    // mask rows per CTA (the fused mask is one block)
 
-// Shared-memory bytes of build_tree_kernel: queue, node arrays, stage-1 top-M, and (when they
-// fit) the sequence's child lists.
+// Shared-memory bytes of the general builder: queue, node arrays, stage-1 top-M, mask bits.
 __host__ __device__ inline size_t tree_mask_words(int n) { return static_cast<size_t>(n) * ((n + 31) / 32); }
 __host__ __device__ inline size_t tree_smem_fixed(int B, int gamma, int M, bool with_mask) {
     return static_cast<size_t>(B + 2) * (8 + 4 * 4) + static_cast<size_t>(B + 1) * 4 * 4 +
            static_cast<size_t>(gamma) * M * 4 + 16 + (with_mask ? tree_mask_words(B + 1) * 4 + 16 : 0);
 }
-// Bytes of the staged list prefixes: the first sw entries of each of the rows child lists.
-__host__ __device__ inline size_t tree_smem_lists(int rows, int sw) { return static_cast<size_t>(rows) * sw * 8; }
 constexpr size_t kTreeSmemLimit = 200 * 1024;
 
-// The child lists of one sequence: the first sw entries of every row staged in shared memory,
-// the rest read from global memory. A list's entry of rank r is reached only after r pops of
-// that list, so sw = min(list length, B + 1) already covers every entry a tree can use.
+// The child lists of one sequence, in global memory.
 struct ListView {
-    const int32_t* s_ids;   // [rows][sw]
-    const float* s_lp;
-    const int32_t* g_ids;   // [rows][stride]
-    const float* g_lp;
-    int sw, stride;
-    __device__ __forceinline__ int tok(int row, int rank) const {
-        return rank < sw ? s_ids[row * sw + rank] : g_ids[static_cast<size_t>(row) * stride + rank];
-    }
-    __device__ __forceinline__ float lp(int row, int rank) const {
-        return rank < sw ? s_lp[row * sw + rank] : g_lp[static_cast<size_t>(row) * stride + rank];
-    }
+    const int32_t* ids;     // [rows][stride]
+    const float* lps;
+    int stride;
+    __device__ __forceinline__ int tok(int row, int rank) const { return ids[static_cast<size_t>(row) * stride + rank]; }
+    __device__ __forceinline__ float lp(int row, int rank) const { return lps[static_cast<size_t>(row) * stride + rank]; }
 };
+__device__ __forceinline__ ListView sequence_lists(const TreeArgs& a, int s) {
+    if (a.mode == TF_MODE_AR)
+        return ListView{a.child_ids + static_cast<size_t>(s) * a.R * a.K2, a.child_logp + static_cast<size_t>(s) * a.R * a.K2, a.K2};
+    return ListView{a.top_ids + static_cast<size_t>(s) * a.gamma * a.K1, a.top_logp + static_cast<size_t>(s) * a.gamma * a.K1, a.K1};
+}
 
-// Shared memory of both builders: queue arrays (used by the general builder only), output nodes,
-// stage-1 top-M and the staged child lists.
+// Shared memory of the general builder: the queue, the output nodes and the stage-1 top-M.
 struct TreeSmem {
     unsigned long long* qkey;
     float* qps;
@@ -235,7 +226,6 @@ struct TreeSmem {
     float* o_score;
     int* topm;        // [gamma, M]
     uint32_t* anc;    // with the fused mask: [B + 1][(B + 32) / 32] ancestor-or-self bits
-    uint8_t* lists;   // staged prefixes: ids [rows][sw] int32, then log-probs [rows][sw] float
 };
 __device__ __forceinline__ TreeSmem tree_smem(uint8_t* base, const TreeArgs& a) {
     TreeSmem t;
@@ -250,93 +240,14 @@ __device__ __forceinline__ TreeSmem tree_smem(uint8_t* base, const TreeArgs& a) 
     t.o_dep = t.o_par + n_out;
     t.o_score = reinterpret_cast<float*>(t.o_dep + n_out);
     t.topm = reinterpret_cast<int*>(t.o_score + n_out);
-    uint8_t* next = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(t.topm + a.gamma * a.M) + 15) &
-                                               ~static_cast<uintptr_t>(15));
-    t.anc = reinterpret_cast<uint32_t*>(next);
-    if (a.mask)
-        next = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(t.anc + tree_mask_words(n_out)) + 15) &
-                                          ~static_cast<uintptr_t>(15));
-    t.lists = next;
+    t.anc = reinterpret_cast<uint32_t*>(t.topm + a.gamma * a.M);
     return t;
-}
-
-// Stage sequence s's stage-1 top-M and the first sw entries of each of its child lists.
-__device__ __forceinline__ ListView stage_sequence(const TreeArgs& a, int s, const TreeSmem& t, int sw) {
-    const int tid = threadIdx.x;
-    const bool ar = a.mode == TF_MODE_AR;
-    const int n_rows_l = ar ? a.R : a.gamma;
-    const int stride = ar ? a.K2 : a.K1;
-    ListView v;
-    v.g_ids = ar ? a.child_ids + static_cast<size_t>(s) * a.R * a.K2 : a.top_ids + static_cast<size_t>(s) * a.gamma * a.K1;
-    v.g_lp = ar ? a.child_logp + static_cast<size_t>(s) * a.R * a.K2 : a.top_logp + static_cast<size_t>(s) * a.gamma * a.K1;
-    v.stride = stride;
-    v.sw = sw;
-    for (int i = tid; i < a.gamma * a.M; i += kTreeThreads)
-        t.topm[i] = a.top_ids[(static_cast<size_t>(s) * a.gamma + i / a.M) * a.K1 + i % a.M];
-    const int n = n_rows_l * sw;
-    int32_t* si = reinterpret_cast<int32_t*>(t.lists);
-    float* sl = reinterpret_cast<float*>(si + n);
-    v.s_ids = si;
-    v.s_lp = sl;
-    const bool vec = sw == stride &&
-                     ((reinterpret_cast<uintptr_t>(v.g_ids) | reinterpret_cast<uintptr_t>(v.g_lp) |
-                       reinterpret_cast<uintptr_t>(si) | reinterpret_cast<uintptr_t>(sl)) & 15) == 0 &&
-                     (n & 3) == 0;
-    constexpr int T = kTreeThreads;
-    if (vec) {
-        // whole lists: 16-byte copies, sixteen per thread in flight before the first store
-        const int4* gi = reinterpret_cast<const int4*>(v.g_ids);
-        const float4* gl = reinterpret_cast<const float4*>(v.g_lp);
-        int4* di = reinterpret_cast<int4*>(si);
-        float4* dl = reinterpret_cast<float4*>(sl);
-        const int n4 = n >> 2;
-        for (int base = tid; base < n4; base += 8 * T) {
-            int4 va[8];
-            float4 vb[8];
-#pragma unroll
-            for (int j = 0; j < 8; ++j)
-                if (base + j * T < n4) {
-                    va[j] = gi[base + j * T];
-                    vb[j] = gl[base + j * T];
-                }
-#pragma unroll
-            for (int j = 0; j < 8; ++j)
-                if (base + j * T < n4) {
-                    di[base + j * T] = va[j];
-                    dl[base + j * T] = vb[j];
-                }
-        }
-    } else {
-        // prefixes of sw entries: element copies, eight per thread in flight
-        for (int base = tid; base < n; base += 8 * T) {
-            int32_t va[8];
-            float vb[8];
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                const int i = base + j * T;
-                if (i < n) {
-                    const size_t g = static_cast<size_t>(i / sw) * stride + i % sw;
-                    va[j] = v.g_ids[g];
-                    vb[j] = v.g_lp[g];
-                }
-            }
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                const int i = base + j * T;
-                if (i < n) {
-                    si[i] = va[j];
-                    sl[i] = vb[j];
-                }
-            }
-        }
-    }
-    return v;
 }
 
 // Nodes from shared memory to the outputs.
 __device__ __forceinline__ void write_nodes(const TreeArgs& a, int s, const TreeSmem& t) {
     const int n_out = a.B + 1;
-    for (int i = threadIdx.x; i < n_out; i += kTreeThreads) {
+    for (int i = threadIdx.x; i < n_out; i += static_cast<int>(blockDim.x)) {
         const size_t o = static_cast<size_t>(s) * n_out + i;
         a.node_tok[o] = t.o_tok[i];
         a.node_parent[o] = t.o_par[i];
@@ -391,12 +302,9 @@ __device__ __forceinline__ void fused_mask(const TreeArgs& a, int s, const TreeS
               a.pos_ids + static_cast<size_t>(s) * n);
 }
 
-// General builder (any B): the queue in shared memory.
-__global__ void __launch_bounds__(kTreeThreads) build_tree_kernel(TreeArgs a, int sw) {
-    pdl_trigger();
-    pdl_wait();
-    extern __shared__ __align__(16) uint8_t smem_raw[];
-    const TreeSmem t = tree_smem(smem_raw, a);
+// General builder (any lists): the queue in shared memory, popped by the CTA's first warp. Every
+// thread of the CTA calls it; on return the nodes are in shared memory and the status is written.
+__device__ void build_tree_queue(const TreeArgs& a, int s, const TreeSmem& t, const ListView& lv) {
     unsigned long long* qkey = t.qkey;
     float* qps = t.qps;
     int* qrow = t.qrow;
@@ -408,11 +316,8 @@ __global__ void __launch_bounds__(kTreeThreads) build_tree_kernel(TreeArgs a, in
     float* o_score = t.o_score;
     int* topm = t.topm;
     const int n_out = a.B + 1;
-    const int s = blockIdx.x;
     const int tid = threadIdx.x;
     const bool ar = a.mode == TF_MODE_AR;
-    const ListView lv = stage_sequence(a, s, t, sw);
-    __syncthreads();
 
     if (tid < 32) {
         const int lane = tid;
@@ -522,151 +427,12 @@ __global__ void __launch_bounds__(kTreeThreads) build_tree_kernel(TreeArgs a, in
         if (lane == 0) a.dev_status[s] = sequence_status(a, flags);
     }
     __syncthreads();
-    write_nodes(a, s, t);
-    fused_mask(a, s, t);
-}
-
-// Builder for B + 1 <= 32 S: the queue in registers, S slots per lane (slot j on lane j % 32,
-// register j / 32). Slots are appended in pop order and an exhausted list leaves an empty slot
-// (key 0, below every real key), so no entry ever moves. Pops, tie rules and results are those
-// of build_tree_kernel.
-template <int S, bool FULL>
-__global__ void __launch_bounds__(kTreeThreads) build_tree_reg_kernel(TreeArgs a, int sw) {
-    pdl_trigger();
-    pdl_wait();
-    extern __shared__ __align__(16) uint8_t smem_raw[];
-    const TreeSmem t = tree_smem(smem_raw, a);
-    const int n_out = a.B + 1;
-    const int s = blockIdx.x;
-    const bool ar = a.mode == TF_MODE_AR;
-    const ListView lv = stage_sequence(a, s, t, sw);
-    // FULL: every rank a pop can reach is staged, so entries are read from shared memory only
-    auto ltok = [&](int row, int rank) { return FULL ? lv.s_ids[row * sw + rank] : lv.tok(row, rank); };
-    auto llp = [&](int row, int rank) { return FULL ? lv.s_lp[row * sw + rank] : lv.lp(row, rank); };
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        const int lane = threadIdx.x;
-        constexpr unsigned kFull = 0xffffffffu;
-        int flags = 0;
-        const int root = a.root_tok[a.two_prev ? 2 * s : s];
-        if (root < 0 || root >= a.V) flags |= TF_DEV_BAD_TOKEN;
-        const int list_len = a.K2;
-        unsigned long long key[S];
-        int srow[S], srank[S], stok[S];
-        float spsc[S];
-#pragma unroll
-        for (int j = 0; j < S; ++j) {
-            key[j] = 0ull;
-            srow[j] = srank[j] = stok[j] = 0;
-            spsc[j] = 0.0f;
-        }
-        if (lane == 0) {
-            key[0] = queue_key(llp(0, 0), 1, 0);
-            stok[0] = ltok(0, 0);
-            t.o_tok[0] = root;
-            t.o_par[0] = -1;
-            t.o_dep[0] = 0;
-            t.o_score[0] = 0.0f;
-        }
-        int n_e = 1;      // slots used so far
-        int count = 1;    // nodes placed
-        while (count < n_out) {
-            // this lane's best slot and its entry
-            unsigned long long lb = key[0];
-            int brow = srow[0], brank = srank[0], btok = stok[0];
-            float bpsc = spsc[0];
-#pragma unroll
-            for (int j = 1; j < S; ++j)
-                if (key[j] > lb) {
-                    lb = key[j];
-                    brow = srow[j];
-                    brank = srank[j];
-                    btok = stok[j];
-                    bpsc = spsc[j];
-                }
-            const uint32_t hi = static_cast<uint32_t>(lb >> 32), lo = static_cast<uint32_t>(lb);
-            const uint32_t mhi = __reduce_max_sync(kFull, hi);
-            if (mhi == 0u) break;                      // queue empty (every real key has hi > 0)
-            unsigned win = __ballot_sync(kFull, hi == mhi);
-            if (__popc(win) > 1) {
-                const uint32_t mlo = __reduce_max_sync(kFull, hi == mhi ? lo : 0u);
-                win = __ballot_sync(kFull, hi == mhi && lo == mlo);
-            }
-            const int wl = __ffs(win) - 1;
-            const uint32_t wlo = __shfl_sync(kFull, lo, wl);
-            const int row = __shfl_sync(kFull, brow, wl);
-            const int rank = __shfl_sync(kFull, brank, wl);
-            const int tok = __shfl_sync(kFull, btok, wl);
-            const float psc = __shfl_sync(kFull, bpsc, wl);
-            const float sc = key_float(mhi);
-            const int dep = 127 - static_cast<int>(wlo >> 24);
-            const int par = 0xFFFFFF - static_cast<int>(wlo & 0xFFFFFFu);
-            const int node = count++;
-            // next sibling of the popped entry (the same shared-memory words for every lane),
-            // read before the expandability test so that both latencies overlap
-            const bool sibling = rank + 1 < list_len;
-            const int sib_tok = sibling ? ltok(row, rank + 1) : 0;
-            const float sib_lp = sibling ? llp(row, rank + 1) : 0.0f;
-            // expandable? (depth cap; M-ary rule)
-            const bool deep_ok = dep < a.gamma;
-            const int m = mary_index(t.topm, dep, a.M, tok, lane, deep_ok && a.mode != TF_MODE_MARGINAL);
-            int crow = !deep_ok ? -1
-                       : a.mode == TF_MODE_MARGINAL ? dep
-                       : m >= 0 ? (ar ? 1 + (dep - 1) * a.M + m : dep) : -1;
-            if (ar && a.two_prev) crow = child_row_2prev(t.topm, t.o_tok, a.M, dep, deep_ok ? m : -1, par, lane);
-            if (tok < 0 || tok >= a.V) flags |= TF_DEV_BAD_TOKEN;
-            if (!isfinite(sc)) flags |= TF_DEV_NONFINITE;
-            const unsigned long long sib_key = sibling ? queue_key(psc + sib_lp, dep, par) : 0ull;
-            if (lane == wl) {
-                // the winner's best slot is the one holding its best key (keys are unique)
-#pragma unroll
-                for (int j = 0; j < S; ++j) {
-                    const bool m = key[j] == lb;
-                    key[j] = m ? sib_key : key[j];
-                    srank[j] = m ? rank + 1 : srank[j];
-                    stok[j] = m ? sib_tok : stok[j];
-                }
-            }
-            if (crow >= 0) {
-                const int ctok = ltok(crow, 0);
-                const unsigned long long ckey = queue_key(sc + llp(crow, 0), dep + 1, node);
-                const bool mine = lane == (n_e & 31);
-#pragma unroll
-                for (int j = 0; j < S; ++j) {
-                    const bool m = mine && j == (n_e >> 5);
-                    key[j] = m ? ckey : key[j];
-                    srow[j] = m ? crow : srow[j];
-                    srank[j] = m ? 0 : srank[j];
-                    stok[j] = m ? ctok : stok[j];
-                    spsc[j] = m ? sc : spsc[j];
-                }
-                ++n_e;
-            }
-            if (lane == 0) {
-                t.o_tok[node] = tok;
-                t.o_par[node] = par;
-                t.o_dep[node] = dep;
-                t.o_score[node] = sc;
-            }
-        }
-        if (count < n_out) flags |= TF_DEV_UNDERFULL;
-        for (int i = count + lane; i < n_out; i += 32) {
-            t.o_tok[i] = -1;
-            t.o_par[i] = -1;
-            t.o_dep[i] = -1;
-            t.o_score[i] = -INFINITY;
-        }
-        if (lane == 0) a.dev_status[s] = sequence_status(a, flags);
-    }
-    __syncthreads();
-    write_nodes(a, s, t);
-    fused_mask(a, s, t);
 }
 
 // ------------------------------------------------------------------------------------------
 // Builder with a sorted queue, for the one-token rule and the marginal modes with B <= 64 and
 // every reachable list entry staged. The same pops, tie rules and results as
-// build_tree_reg_kernel. After t pops only the B - t best live entries can still be popped (each
+// build_tree_queue. After t pops only the B - t best live entries can still be popped (each
 // needs every better entry popped first), and at most t + 1 entries are live (a pop replaces its
 // entry by the next sibling and adds at most the node's first child), so at most
 // min(t + 1, B - t) <= 32 entries matter: lane i of one warp holds the i-th best. A pop takes
@@ -867,9 +633,486 @@ __global__ void __launch_bounds__(kFastThreads) build_tree_fast_kernel(TreeArgs 
 }
 
 // ------------------------------------------------------------------------------------------
+// Builder by levels, for large budgets. A pop sequence is a chain: with the queue in shared memory
+// 512 pops took 343 us on GB300, about 0.65 us each on one warp (46 us this way; 64 pops of the
+// two-token rule 44 us with the queue in registers, 25 us this way). But the B popped nodes are simply
+// the B first of all nodes in the order (score, smaller depth, earlier parent, earlier list entry),
+// as long as no node outscores its parent or its list predecessor (log-probabilities <= 0, lists
+// sorted): then the first B nodes contain every ancestor and predecessor of each of them. So the
+// CTA grows all of them level by level, a warp per (parent, 32 list entries), and keeps only nodes
+// that can still be among the first B: theta, a lower bound of the B-th best score so far, rises
+// with a histogram of the scores after each pass. The survivors (a few more than B) are sorted once.
+//  - Two nodes of equal score and depth under different parents are ordered by their parents' places
+//    in the order, known once shallower levels are: the few such ties are resolved after the sort.
+//  - A list entry above its predecessor or its parent, a score that is not finite, more than
+//    kLvTies ties near the tree, or more nodes at theta than there is room for send the sequence to
+//    the queue (build_tree_queue) instead: the same results, at the old speed.
+// ------------------------------------------------------------------------------------------
+constexpr int kLvThreads = 512;
+constexpr int kLvWarps = kLvThreads / 32;
+constexpr int kLvCap = 4096;       // nodes held at once
+constexpr int kLvBins = 2 * kLvThreads;
+constexpr int kLvSort = 2048;      // nodes that can be sorted
+constexpr int kLvTies = 32;        // ties resolved in place, and the longest run of equal nodes
+
+struct LevelSmem {
+    float* score;          // [kLvCap]; node 0 is the root
+    int* tok;
+    uint16_t *par, *rank;
+    uint16_t* place;       // new index in a compaction; 1 + place in the order at the end
+    uint16_t* act[2];      // parents still to expand (kNoNode: dropped) and the next list chunk of each
+    uint8_t* chunk[2];
+    uint8_t* dep;
+    int8_t* m;             // candidate index of an expandable node (two-token rule), else -1
+    unsigned long long* key;   // [kLvSort]
+    int* hist;             // [kLvBins]
+    int* topm;             // [gamma * M]
+};
+constexpr uint16_t kNoNode = 0xffff;
+constexpr size_t kLvFixedBytes = kLvCap * (4 + 4 + 2 + 2 + 2 + 4 + 2 + 1 + 1) + kLvSort * 8 + kLvBins * 4;
+__host__ __device__ inline size_t level_smem_bytes(int B, int gamma, int M, bool with_mask) {
+    const size_t mine = kLvFixedBytes + static_cast<size_t>(gamma) * M * 4;
+    const size_t queue = tree_smem_fixed(B, gamma, M, with_mask);
+    return mine > queue ? mine : queue;
+}
+__device__ __forceinline__ LevelSmem level_smem(uint8_t* p) {
+    LevelSmem t;
+    auto take = [&](size_t bytes) {
+        uint8_t* q = p;
+        p += bytes;
+        return q;
+    };
+    t.key = reinterpret_cast<unsigned long long*>(take(kLvSort * 8));
+    t.score = reinterpret_cast<float*>(take(kLvCap * 4));
+    t.tok = reinterpret_cast<int*>(take(kLvCap * 4));
+    t.hist = reinterpret_cast<int*>(take(kLvBins * 4));
+    t.par = reinterpret_cast<uint16_t*>(take(kLvCap * 2));
+    t.rank = reinterpret_cast<uint16_t*>(take(kLvCap * 2));
+    t.place = reinterpret_cast<uint16_t*>(take(kLvCap * 2));
+    for (int i = 0; i < 2; ++i) t.act[i] = reinterpret_cast<uint16_t*>(take(kLvCap * 2));
+    for (int i = 0; i < 2; ++i) t.chunk[i] = take(kLvCap);
+    t.dep = take(kLvCap);
+    t.m = reinterpret_cast<int8_t*>(take(kLvCap));
+    t.topm = reinterpret_cast<int*>(p);
+    return t;
+}
+
+// Sort key of node idx: larger score, smaller depth, smaller list rank, then index (unique).
+__device__ __forceinline__ unsigned long long level_key(float score, int dep, int rank, int idx) {
+    return (static_cast<unsigned long long>(float_key(score)) << 32) | (static_cast<unsigned>(127 - dep) << 24) |
+           (static_cast<unsigned>(0xfff - rank) << 12) | static_cast<unsigned>(idx);
+}
+static_assert(kLvCap <= 1 << 12 && kMaxK <= 1 << 12 && kMaxGamma <= 127, "fields of level_key");
+
+__global__ void __launch_bounds__(kLvThreads) build_tree_level_kernel(TreeArgs a) {
+    pdl_trigger();
+    pdl_wait();
+    extern __shared__ __align__(16) uint8_t smem_raw[];
+    __shared__ float theta_s, wmin[kLvWarps];
+    __shared__ int wsum[kLvWarps], count_s, bad_s, n_act_s, n_ties_s, ties[kLvTies], flags_s;
+    constexpr unsigned kFull = 0xffffffffu;
+    const LevelSmem t = level_smem(smem_raw);
+    const int s = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const bool ar = a.mode == TF_MODE_AR, mary = a.mode != TF_MODE_MARGINAL;
+    const ListView lists = sequence_lists(a, s);
+    const int n_chunks = (a.K2 + 31) / 32;
+    const int root = a.root_tok[a.two_prev ? 2 * s : s];
+    if (mary)
+        for (int i = tid; i < a.gamma * a.M; i += kLvThreads)
+            t.topm[i] = a.top_ids[(static_cast<size_t>(s) * a.gamma + i / a.M) * a.K1 + i % a.M];
+    if (tid == 0) {
+        t.score[0] = 0.0f;
+        t.tok[0] = root;
+        t.par[0] = t.rank[0] = 0;
+        t.dep[0] = 0;
+        t.m[0] = -1;
+        t.act[0][0] = 0;
+        t.chunk[0][0] = 0;
+        count_s = 1;
+        bad_s = 0;
+        flags_s = root < 0 || root >= a.V ? TF_DEV_BAD_TOKEN : 0;
+        theta_s = -INFINITY;
+    }
+    __syncthreads();
+
+    // Raises theta to the lower edge of the histogram bin that holds the B-th best score (a little
+    // below it: the bins' arithmetic is rounded). Nothing happens while there are fewer than B.
+    auto raise_theta = [&](int count) {
+        if (count - 1 < a.B) return;
+        float lo = theta_s;
+        if (!(lo > -INFINITY)) {
+            float mn = 0.0f;
+            for (int i = 1 + tid; i < count; i += kLvThreads) mn = fminf(mn, t.score[i]);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) mn = fminf(mn, __shfl_xor_sync(kFull, mn, o));
+            if (lane == 0) wmin[warp] = mn;
+            __syncthreads();
+            lo = wmin[0];
+            for (int w = 1; w < kLvWarps; ++w) lo = fminf(lo, wmin[w]);
+        }
+        if (!(lo < 0.0f) || !(lo > -INFINITY)) return;   // (uniform: every thread holds the same lo)
+        t.hist[2 * tid] = t.hist[2 * tid + 1] = 0;
+        __syncthreads();
+        const float scale = static_cast<float>(kLvBins) / -lo;
+        for (int i = 1 + tid; i < count; i += kLvThreads) {
+            const float x = t.score[i] - lo;
+            if (x >= 0.0f) atomicAdd(&t.hist[min(kLvBins - 1, static_cast<int>(x * scale))], 1);
+        }
+        __syncthreads();
+        const int h0 = t.hist[2 * tid], h1 = t.hist[2 * tid + 1];
+        int incl = h0 + h1;                              // bins 2 tid and above, within the warp
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_down_sync(kFull, incl, o);
+            if (lane + o < 32) incl += v;
+        }
+        if (lane == 0) wsum[warp] = incl;
+        __syncthreads();
+        for (int w = warp + 1; w < kLvWarps; ++w) incl += wsum[w];
+        const int excl = incl - h0 - h1;
+        if (incl >= a.B && excl < a.B) {
+            const int bin = 2 * tid + (excl + h1 >= a.B ? 1 : 0);
+            const float edge = lo + (-lo) * (static_cast<float>(bin) / kLvBins) + lo * 4e-6f;
+            if (edge > theta_s) theta_s = edge;
+        }
+        __syncthreads();
+    };
+
+    // Drops the nodes below theta, keeping the others' order; `first` (the first node of the level)
+    // and the parents still to expand move along. Returns the new count.
+    auto compact = [&](int count, int& first, uint16_t* act, int n_act) {
+        constexpr int kPer = kLvCap / kLvThreads;
+        const float theta = theta_s;
+        float sc[kPer];
+        int tk[kPer];
+        uint16_t pr[kPer], rk[kPer];
+        uint8_t dp[kPer];
+        int8_t mm[kPer];
+        bool keep[kPer];
+        int mine = 0;
+#pragma unroll
+        for (int j = 0; j < kPer; ++j) {
+            const int i = tid * kPer + j;
+            keep[j] = i < count && (i == 0 || t.score[i] >= theta);
+            mine += keep[j] ? 1 : 0;
+            if (keep[j]) {
+                sc[j] = t.score[i];
+                tk[j] = t.tok[i];
+                pr[j] = t.par[i];
+                rk[j] = t.rank[i];
+                dp[j] = t.dep[i];
+                mm[j] = t.m[i];
+            }
+        }
+        int incl = mine;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(kFull, incl, o);
+            if (lane >= o) incl += v;
+        }
+        if (lane == 31) wsum[warp] = incl;
+        __syncthreads();
+        int base = incl - mine, total = 0;
+        for (int w = 0; w < kLvWarps; ++w) {
+            if (w < warp) base += wsum[w];
+            total += wsum[w];
+        }
+#pragma unroll
+        for (int j = 0; j < kPer; ++j) {
+            const int i = tid * kPer + j;
+            t.place[i] = static_cast<uint16_t>(keep[j] ? base : kNoNode);
+            base += keep[j] ? 1 : 0;
+        }
+        __syncthreads();
+        // the level's first kept node: the smallest new index at or after `first`
+        if (tid == 0) {
+            int f = first;
+            while (f < count && t.place[f] == kNoNode) ++f;
+            wsum[0] = f < count ? t.place[f] : total;
+        }
+        for (int i = tid; i < n_act; i += kLvThreads) act[i] = act[i] == kNoNode ? kNoNode : t.place[act[i]];
+        uint16_t to[kPer], np[kPer];
+#pragma unroll
+        for (int j = 0; j < kPer; ++j)
+            if (keep[j]) {
+                to[j] = t.place[tid * kPer + j];
+                np[j] = t.place[pr[j]];                  // a kept node's parent scores no less: kept
+            }
+        __syncthreads();
+        first = wsum[0];
+#pragma unroll
+        for (int j = 0; j < kPer; ++j)
+            if (keep[j]) {
+                t.score[to[j]] = sc[j];
+                t.tok[to[j]] = tk[j];
+                t.par[to[j]] = np[j];
+                t.rank[to[j]] = rk[j];
+                t.dep[to[j]] = dp[j];
+                t.m[to[j]] = mm[j];
+            }
+        if (tid == 0) count_s = total;
+        __syncthreads();
+        return total;
+    };
+
+    int cur = 0, n_act = 1, count = 1, seen = 1;         // seen: the count at the last raise_theta
+    for (int d = 1; d <= a.gamma && n_act > 0; ++d) {
+        // the nodes of depth d: children of the n_act expandable nodes of depth d - 1
+        int first = count;
+        int g = 32 / n_act;                              // list chunks taken of each parent per pass
+        g = g < 1 ? 1 : g > n_chunks ? n_chunks : g;
+        while (n_act > 0) {
+            uint16_t* act = t.act[cur];
+            uint8_t* chunk = t.chunk[cur];
+            uint16_t* nact = t.act[cur ^ 1];
+            uint8_t* nchunk = t.chunk[cur ^ 1];
+            if (kLvCap - count < 32 * kLvWarps) {
+                raise_theta(count);
+                count = seen = compact(count, first, act, n_act);
+            }
+            int nb = (kLvCap - count) / (32 * g);        // parents of this pass: all their entries fit
+            nb = nb < n_act ? nb : n_act;
+            if (nb < 1) {                                // too many nodes at theta
+                if (tid == 0) bad_s = 1;
+                __syncthreads();
+                break;
+            }
+            if (tid == 0) n_act_s = 0;
+            __syncthreads();
+            const float theta = theta_s;
+            for (int item = warp; item < nb * g; item += kLvWarps) {
+                const int pi = item / g, c = chunk[pi] + (item - pi * g);
+                const int p = act[pi];
+                if (p == kNoNode || c >= n_chunks) continue;
+                const float ps = t.score[p];
+                if (ps < theta) continue;
+                int row;
+                if (d == 1) {
+                    row = 0;
+                } else if (!ar) {
+                    row = d - 1;
+                } else {
+                    const int m = t.m[p];
+                    row = !a.two_prev ? 1 + (d - 2) * a.M + m
+                          : d == 2    ? 1 + m
+                                      : 1 + a.M + (d - 3) * a.M * a.M + m * a.M + t.m[t.par[p]];
+                }
+                const int rank = c * 32 + lane;
+                const bool in = rank < a.K2;
+                const float lp = in ? lists.lp(row, rank) : 0.0f;
+                const int tok = in ? lists.tok(row, rank) : 0;
+                const float before = lane == 0 && c > 0 ? lists.lp(row, rank - 1) : 0.0f;
+                const float sc = ps + lp;
+                float prev = __shfl_up_sync(kFull, sc, 1);
+                if (lane == 0) prev = ps + before;       // the parent itself above a list's first entry
+                // (also false for NaN)
+                if (in && !(sc <= prev && sc > -INFINITY)) bad_s = 1;
+                const bool take = in && sc >= theta;
+                const unsigned bal = __ballot_sync(kFull, take);
+                if (bal == 0u) continue;
+                int base = 0;
+                if (lane == 0) {
+                    base = atomicAdd(&count_s, __popc(bal));
+                    // every entry so far counts: the list goes on in the next pass
+                    if (item - pi * g == g - 1 && bal == kFull && c + 1 < n_chunks) {
+                        const int q = atomicAdd(&n_act_s, 1);
+                        nact[q] = static_cast<uint16_t>(p);
+                        nchunk[q] = static_cast<uint8_t>(c + 1);
+                    }
+                }
+                base = __shfl_sync(kFull, base, 0);
+                if (take) {
+                    const int i = base + __popc(bal & ((1u << lane) - 1u));
+                    t.score[i] = sc;
+                    t.tok[i] = tok;
+                    t.par[i] = static_cast<uint16_t>(p);
+                    t.rank[i] = static_cast<uint16_t>(rank);
+                    t.dep[i] = static_cast<uint8_t>(d);
+                    t.m[i] = -1;
+                }
+            }
+            __syncthreads();
+            count = count_s;
+            const int more = n_act_s, rest = n_act - nb;
+            if (bad_s) break;                            // (uniform: written before the barrier)
+            for (int i = tid; i < rest; i += kLvThreads) {
+                nact[more + i] = act[nb + i];
+                nchunk[more + i] = chunk[nb + i];
+            }
+            n_act = more + rest;
+            cur ^= 1;
+            if (count - seen >= (a.B >> 3) || n_act > 0) {
+                __syncthreads();
+                raise_theta(count);
+                seen = count;
+            }
+            __syncthreads();
+        }
+        __syncthreads();
+        if (bad_s) break;
+        n_act = 0;
+        if (d < a.gamma) {
+            // the expandable nodes of depth d
+            if (tid == 0) n_act_s = 0;
+            __syncthreads();
+            const float theta = theta_s;
+            const int* cand = t.topm + (d - 1) * a.M;
+            for (int i = first + tid; i < count; i += kLvThreads) {
+                if (t.score[i] < theta) continue;
+                if (mary) {
+                    const int tok = t.tok[i];
+                    int m = -1;
+                    for (int j = 0; j < a.M; ++j)
+                        if (cand[j] == tok) {
+                            m = j;
+                            break;
+                        }
+                    if (m < 0) continue;
+                    t.m[i] = static_cast<int8_t>(m);
+                }
+                const int q = atomicAdd(&n_act_s, 1);
+                t.act[cur][q] = static_cast<uint16_t>(i);
+                t.chunk[cur][q] = 0;
+            }
+            __syncthreads();
+            n_act = n_act_s;
+        }
+    }
+
+    // ---- the order of the survivors
+    int n = 0;
+    if (!bad_s) {
+        raise_theta(count);
+        __syncthreads();
+        if (tid == 0) {
+            n_act_s = 0;
+            n_ties_s = 0;
+        }
+        __syncthreads();
+        const float theta = theta_s;
+        for (int i = 1 + tid; i < count; i += kLvThreads)
+            if (t.score[i] >= theta) {
+                const int q = atomicAdd(&n_act_s, 1);
+                if (q < kLvSort) t.key[q] = level_key(t.score[i], t.dep[i], t.rank[i], i);
+            }
+        __syncthreads();
+        n = n_act_s;
+        if (n > kLvSort) {
+            if (tid == 0) bad_s = 1;
+        } else {
+            int N = 64;
+            while (N < n) N <<= 1;
+            for (int i = n + tid; i < N; i += kLvThreads) t.key[i] = 0ull;
+            // bitonic sort, largest key first
+            for (int size = 2; size <= N; size <<= 1)
+                for (int step = size >> 1; step > 0; step >>= 1) {
+                    __syncthreads();
+                    for (int q = tid; q < N / 2; q += kLvThreads) {
+                        const int i = 2 * q - (q & (step - 1)), j = i + step;
+                        const unsigned long long x = t.key[i], y = t.key[j];
+                        if ((x < y) == ((i & size) == 0)) {
+                            t.key[i] = y;
+                            t.key[j] = x;
+                        }
+                    }
+                }
+            __syncthreads();
+            for (int i = tid; i < n; i += kLvThreads) {
+                const unsigned long long x = t.key[i];
+                const int xi = static_cast<int>(x & 0xfff);
+                t.place[xi] = static_cast<uint16_t>(i + 1);
+                if (i + 1 < n) {
+                    const unsigned long long y = t.key[i + 1];
+                    if ((x >> 24) == (y >> 24) && t.par[xi] != t.par[y & 0xfff]) {
+                        const int q = atomicAdd(&n_ties_s, 1);
+                        if (q < kLvTies) ties[q] = i;
+                    }
+                }
+            }
+            __syncthreads();
+            if (tid == 0 && n_ties_s > 0) {
+                // equal score and depth, different parents: shallower levels first, each run of
+                // equal nodes by its parents' places, then by list rank
+                const int nt = n_ties_s;
+                bool ok = nt <= kLvTies;
+                for (int dd = 1; ok && dd <= a.gamma; ++dd)
+                    for (int q = 0; ok && q < nt; ++q) {
+                        const unsigned long long x = t.key[ties[q]] >> 24;
+                        if (127 - static_cast<int>(x & 0xff) != dd) continue;
+                        int l = ties[q], r = ties[q] + 1;
+                        while (l > 0 && (t.key[l - 1] >> 24) == x) --l;
+                        while (r + 1 < n && (t.key[r + 1] >> 24) == x) ++r;
+                        ok = r - l < kLvTies;
+                        for (int i = l + 1; ok && i <= r; ++i) {
+                            const unsigned long long v = t.key[i];
+                            const int vp = t.place[t.par[v & 0xfff]], vr = t.rank[v & 0xfff];
+                            int j = i - 1;
+                            for (; j >= l; --j) {
+                                const int u = static_cast<int>(t.key[j] & 0xfff);
+                                const int up = t.place[t.par[u]];
+                                if (up < vp || (up == vp && t.rank[u] < vr)) break;
+                                t.key[j + 1] = t.key[j];
+                            }
+                            t.key[j + 1] = v;
+                        }
+                        for (int i = l; i <= r; ++i) t.place[t.key[i] & 0xfff] = static_cast<uint16_t>(i + 1);
+                    }
+                if (!ok) bad_s = 1;
+            }
+        }
+    }
+    __syncthreads();
+    const int n_out = a.B + 1;
+    if (bad_s) {
+        __syncthreads();
+        const TreeSmem q = tree_smem(smem_raw, a);
+        for (int i = tid; i < a.gamma * a.M; i += kLvThreads)
+            q.topm[i] = a.top_ids[(static_cast<size_t>(s) * a.gamma + i / a.M) * a.K1 + i % a.M];
+        __syncthreads();
+        build_tree_queue(a, s, q, sequence_lists(a, s));
+        write_nodes(a, s, q);
+        fused_mask(a, s, q);
+        return;
+    }
+    const size_t o0 = static_cast<size_t>(s) * n_out;
+    for (int i = tid; i < n_out; i += kLvThreads) {
+        int tok = -1, par = -1, dep = -1;
+        float sc = -INFINITY;
+        if (i == 0) {
+            tok = root;
+            dep = 0;
+            sc = 0.0f;
+        } else if (i <= n) {
+            const int x = static_cast<int>(t.key[i - 1] & 0xfff), p = t.par[x];
+            tok = t.tok[x];
+            par = p == 0 ? 0 : t.place[p];
+            dep = t.dep[x];
+            sc = t.score[x];
+            if (tok < 0 || tok >= a.V) atomicOr(&flags_s, TF_DEV_BAD_TOKEN);
+        } else {
+            atomicOr(&flags_s, TF_DEV_UNDERFULL);
+        }
+        a.node_tok[o0 + i] = tok;
+        a.node_parent[o0 + i] = par;
+        a.node_depth[o0 + i] = dep;
+        a.node_score[o0 + i] = sc;
+        if (a.mask) {                                    // (hist: at most kFusedMaskMaxNodes entries of each)
+            t.hist[i] = par;
+            t.hist[kFusedMaskMaxNodes + i] = dep;
+        }
+    }
+    __syncthreads();
+    if (tid == 0) a.dev_status[s] = sequence_status(a, flags_s);
+    if (a.mask)
+        mask_rows(n_out, t.hist, t.hist + kFusedMaskMaxNodes, a.root_pos[s], 0, n_out, reinterpret_cast<uint32_t*>(t.key),
+                  a.mask + static_cast<size_t>(s) * n_out * n_out, a.pos_ids + o0);
+}
+
+// ------------------------------------------------------------------------------------------
 // The tree-attention mask and position ids (mask_rows) of a drafted tree in global memory: one
 // CTA per sequence and block of kMaskRows rows.
 // ------------------------------------------------------------------------------------------
+constexpr int kMaskRows = 128;
 __global__ void __launch_bounds__(256) tree_mask_kernel(int n, const int32_t* __restrict__ node_parent,
                                                         const int32_t* __restrict__ node_depth,
                                                         const int32_t* __restrict__ root_pos,
@@ -1152,41 +1395,26 @@ cudaError_t launch_build_tree(const Ctx& ctx, int b, int gamma, int M, int K1, i
     TreeArgs a{gamma, M, K1, K2, B, V, mode, R, mode == TF_MODE_AR && two_prev ? 1 : 0, root_tok, top_ids, top_logp,
                child_ids, child_logp, node_tok, node_parent, node_depth, node_score, dev_status, root_pos, mask,
                pos_ids, ws_status};
-    const size_t fixed = tree_smem_fixed(B, gamma, M, mask != nullptr);
     const int rows_l = mode == TF_MODE_AR ? R : gamma;
     const int stride = mode == TF_MODE_AR ? K2 : K1;
-    // stage the entries a tree can reach (rank <= B) when they fit, else a prefix that does
-    const int sw_full = stride < B + 1 ? stride : B + 1;
-    int sw = sw_full;
-    if (fixed + tree_smem_lists(rows_l, sw) > kTreeSmemLimit) {
-        const size_t room = kTreeSmemLimit > fixed ? kTreeSmemLimit - fixed : 0;
-        sw = static_cast<int>(room / (static_cast<size_t>(rows_l) * 8)) & ~3;
-        if (sw > sw_full) sw = sw_full;
+    const int sw = stride < B + 1 ? stride : B + 1;   // list entries that a tree can reach
+    // The sorted-queue builder for the one-token rule and the marginal modes with B <= 64 and every
+    // reachable entry in shared memory: its cost is the pops (0.25 us each), the builder by levels
+    // pays 1 to 1.5 us per level and pass whatever the budget. Measured on GB300 (16 depths, one
+    // sequence): B = 32 13.8 against 16.7 us, B = 64 21.4 against 23.0.
+    const size_t fsm = fast_tree_smem(B, gamma, M, rows_l, sw, mask != nullptr);
+    if (!a.two_prev && B <= 64 && fsm <= kTreeSmemLimit) {
+        cudaError_t e = cudaFuncSetAttribute(build_tree_fast_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             static_cast<int>(fsm));
+        if (e != cudaSuccess) return e;
+        e = launch_pdl(build_tree_fast_kernel, dim3(b), dim3(kFastThreads), fsm, ctx.stream, a, sw);
+        return e != cudaSuccess ? e : cudaGetLastError();
     }
-    // the sorted-queue builder for the one-token rule and the marginal modes with B <= 64 and
-    // every reachable entry staged
-    if (!a.two_prev && B <= 64) {
-        const size_t fsm = fast_tree_smem(B, gamma, M, rows_l, sw_full, mask != nullptr);
-        if (fsm <= kTreeSmemLimit) {
-            cudaError_t e = cudaFuncSetAttribute(build_tree_fast_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 static_cast<int>(fsm));
-            if (e != cudaSuccess) return e;
-            e = launch_pdl(build_tree_fast_kernel, dim3(b), dim3(kFastThreads), fsm, ctx.stream, a, sw_full);
-            return e != cudaSuccess ? e : cudaGetLastError();
-        }
-    }
-    const size_t smem = fixed + tree_smem_lists(rows_l, sw);
-    // otherwise the register-queue builder whenever B + 1 slots fit in four registers per lane
-    const bool full = sw == sw_full;
-    void (*kern)(TreeArgs, int) =
-        B + 1 <= 32    ? (full ? build_tree_reg_kernel<1, true> : build_tree_reg_kernel<1, false>)
-        : B + 1 <= 64  ? (full ? build_tree_reg_kernel<2, true> : build_tree_reg_kernel<2, false>)
-        : B + 1 <= 96  ? (full ? build_tree_reg_kernel<3, true> : build_tree_reg_kernel<3, false>)
-        : B + 1 <= 128 ? (full ? build_tree_reg_kernel<4, true> : build_tree_reg_kernel<4, false>)
-                       : build_tree_kernel;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    const size_t lsm = level_smem_bytes(B, gamma, M, mask != nullptr);
+    cudaError_t e = cudaFuncSetAttribute(build_tree_level_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         static_cast<int>(lsm));
     if (e != cudaSuccess) return e;
-    e = launch_pdl(kern, dim3(b), dim3(kTreeThreads), smem, ctx.stream, a, sw);
+    e = launch_pdl(build_tree_level_kernel, dim3(b), dim3(kLvThreads), lsm, ctx.stream, a);
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 

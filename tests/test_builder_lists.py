@@ -1,9 +1,10 @@
 """Part 2 of Algorithm 1 on hand-made child lists: tf_build_tree against the oracle's lazy queue,
-bit for bit (tokens, parents, depths, scores, status). Log-probabilities are multiples of 1/8 in
-[-6, 0], so every path score is exact in fp32 and fp64 alike and equal scores are frequent (the
-tie rules decide many pops); a random share of every list's tokens are stage-1 candidates of the
+bit for bit (tokens, parents, depths, scores, status). Log-probabilities are multiples of 1/8 (or
+1/4096) in [-6, 0], so every path score is exact in fp32 and fp64 alike and equal scores are frequent
+(or a few per tree: the tie rules decide many pops, or some); a random share of every list's tokens are stage-1 candidates of the
 list's depth, so the M-ary rule expands often and the trees grow deep and wide. Budgets up to 64
-run the sorted-queue builder, larger ones the register and shared-memory builders."""
+run the sorted-queue builder, larger ones and the two-token rule the builder by levels, which hands
+trees with many ties to the queue in shared memory."""
 import numpy as np
 import pytest
 import torch
@@ -15,8 +16,8 @@ pytestmark = pytest.mark.gpu
 BACKGROUND = -1.0e6   # every token outside a list: below every listed value
 
 
-def _sorted_list(rng, ids, V):
-    vals = -rng.integers(0, 49, ids.shape[0]).astype(np.float64) / 8.0 + 0.0   # no -0.0
+def _sorted_list(rng, ids, V, grain):
+    vals = -rng.integers(0, 6 * grain + 1, ids.shape[0]).astype(np.float64) / grain + 0.0   # no -0.0
     order = np.lexsort((ids, -vals))        # larger value first, equal values by smaller id
     return ids[order], vals[order]
 
@@ -30,9 +31,9 @@ def _list_tokens(rng, n, V, cands):
     return np.concatenate([chosen, rng.choice(rest, n - n_c, replace=False)]).astype(np.int64)
 
 
-def _make(rng, mode, b, gamma, M, K2, V):
+def _make(rng, mode, b, gamma, M, K2, V, grain=8, two=False):
     K1 = max(M, K2)
-    R = 1 + M * (gamma - 1)
+    R = 1 + M * (gamma - 1) if not two else 1 + M + M * M * (gamma - 2)
     top_ids = np.zeros((b, gamma, K1), np.int64)
     top_lp = np.zeros((b, gamma, K1))
     child_ids = np.zeros((b, R, K2), np.int64)
@@ -40,11 +41,12 @@ def _make(rng, mode, b, gamma, M, K2, V):
     for s in range(b):
         for i in range(gamma):
             prev = top_ids[s, i - 1, :M] if i > 0 else np.zeros(0, np.int64)
-            top_ids[s, i], top_lp[s, i] = _sorted_list(rng, _list_tokens(rng, K1, V, prev), V)
+            top_ids[s, i], top_lp[s, i] = _sorted_list(rng, _list_tokens(rng, K1, V, prev), V, grain)
         for r in range(R):
-            dep = 1 if r == 0 else (r - 1) // M + 2          # depth of the row's entries (reading R4)
+            # depth of the row's entries (reading R4; R13 for the two-token rule)
+            dep = 1 if r == 0 else (r - 1) // M + 2 if not two else 2 if r <= M else 3 + (r - 1 - M) // (M * M)
             ids = _list_tokens(rng, K2, V, top_ids[s, dep - 1, :M])
-            child_ids[s, r], child_lp[s, r] = _sorted_list(rng, ids, V)
+            child_ids[s, r], child_lp[s, r] = _sorted_list(rng, ids, V, grain)
     root = rng.integers(0, V, b)
     return top_ids, top_lp, child_ids, child_lp, root
 
@@ -68,8 +70,8 @@ CASES = [
     ("ar", 2, 3, 2, 4, 30, 50),            # underfull universe
     ("marginal", 3, 8, 4, 64, 64, 1000),
     ("marginal_mary", 3, 8, 5, 16, 40, 1000),
-    ("ar", 2, 8, 8, 100, 100, 3000),       # register builder
-    ("ar", 1, 8, 8, 64, 200, 3000),        # shared-memory builder, K2 < B
+    ("ar", 2, 8, 8, 100, 100, 3000),       # ties throughout: the queue in shared memory
+    ("ar", 1, 8, 8, 64, 200, 3000),        # K2 < B
 ]
 
 
@@ -107,3 +109,51 @@ def test_builder_equals_the_oracle_on_hand_made_lists(mode, b, gamma, M, K2, B, 
 
 
 O_UNDERFULL = 2   # TF_DEV_UNDERFULL
+
+LEVEL_CASES = [
+    # mode, batch, gamma, M, K2, B, V, two-token rule
+    ("ar", 3, 16, 16, 65, 65, 3000, False),       # the smallest budget of the builder by levels
+    ("ar", 2, 16, 16, 512, 512, 5000, False),     # exact lists, sixteen chunks per list
+    ("ar", 2, 4, 64, 500, 1023, 5000, False),     # the largest budget, wide branching: nodes dropped as theta rises
+    ("ar", 2, 16, 5, 33, 300, 2000, False),       # a list of one chunk and one entry; K2 < B
+    ("ar", 2, 3, 2, 20, 400, 300, False),         # underfull universe
+    ("ar", 2, 1, 4, 100, 100, 500, False),        # one level
+    ("marginal", 2, 6, 4, 256, 256, 1000, False),  # every node expands
+    ("marginal_mary", 2, 12, 20, 130, 127, 2000, False),
+    ("ar", 2, 8, 4, 40, 40, 1000, True),          # two-token rule: small, register-sized and large budgets
+    ("ar", 2, 6, 5, 100, 100, 1000, True),
+    ("ar", 1, 5, 6, 200, 300, 1000, True),
+]
+
+
+@pytest.mark.parametrize("grain", [4096, 64])
+@pytest.mark.parametrize("mode,b,gamma,M,K2,B,V,two", LEVEL_CASES)
+def test_large_budgets_equal_the_oracle(mode, b, gamma, M, K2, B, V, two, grain):
+    # grain 4096: a few equal scores under different parents per tree, resolved in place; grain 64:
+    # too many of them, so the queue takes over
+    from paper_2606_03819_gb300 import Dims
+    from paper_2606_03819_gb300 import binding as Bn
+    dims = Dims(b, 64, V, 64, gamma, M, K2, B, dtype="f32", mode=mode, approx="swiglu_2prev" if two else "swiglu")
+    n = B + 1
+    rng = np.random.default_rng(31 * B + M + grain)
+    top_ids, top_lp, child_ids, child_lp, root = _make(rng, mode, b, gamma, M, K2, V, grain, two)
+    dev = lambda a, t: torch.from_numpy(np.ascontiguousarray(a)).to(device="cuda", dtype=t)  # noqa: E731
+    out = {k: torch.full((b, n), -7, dtype=t, device="cuda") for k, t in
+           (("tok", torch.int32), ("par", torch.int32), ("dep", torch.int32), ("score", torch.float32))}
+    stat = torch.full((b,), -7, dtype=torch.int32, device="cuda")
+    ar = mode == "ar"
+    roots = np.stack([root, root], 1) if two else root
+    Bn.tf_build_tree(dims, dev(roots, torch.int32), dev(top_ids, torch.int32), dev(top_lp, torch.float32),
+                     dev(child_ids, torch.int32) if ar else None, dev(child_lp, torch.float32) if ar else None,
+                     out["tok"], out["par"], out["dep"], out["score"], stat)
+    torch.cuda.synchronize()
+    for s in range(b):
+        s1 = _full_rows(top_ids[s], top_lp[s], V)
+        s2 = _full_rows(child_ids[s], child_lp[s], V) if ar else None
+        src = O.ChildSource(mode, gamma, M, top_ids[s], s1, s2, "swiglu_2prev" if two else "swiglu")
+        t = O.build_tree_lazy(src, int(root[s]), B, keep=K2 if K2 < B else None)
+        np.testing.assert_array_equal(out["tok"][s].cpu().numpy(), t.tok)
+        np.testing.assert_array_equal(out["par"][s].cpu().numpy(), t.parent)
+        np.testing.assert_array_equal(out["dep"][s].cpu().numpy(), t.depth)
+        np.testing.assert_array_equal(out["score"][s].cpu().numpy().astype(np.float64), t.score)
+        assert stat[s].item() == (O_UNDERFULL if t.underfull else 0)
