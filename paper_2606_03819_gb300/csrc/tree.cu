@@ -287,10 +287,35 @@ __device__ __forceinline__ void mask_rows(int n, const int* par, const int* dep,
         pos_s[i] = ok ? root_pos + dep[i] : -1;
     }
     __syncthreads();
-    const int count = (r1 - r0) * n;
-    for (int idx = threadIdx.x; idx < count; idx += blockDim.x) {
-        const int i = idx / n, jcol = idx - (idx / n) * n;
-        mask_s[static_cast<size_t>(r0 + i) * n + jcol] = static_cast<uint8_t>((anc[i * W + (jcol >> 5)] >> (jcol & 31)) & 1u);
+    // The rows are contiguous bytes: aligned words of four entries (a word may run into the next row),
+    // single bytes before the first and after the last.
+    const int total = (r1 - r0) * n;
+    uint8_t* out = mask_s + static_cast<size_t>(r0) * n;
+    const int head = min(total, static_cast<int>(-reinterpret_cast<intptr_t>(out) & 3));
+    const int words = (total - head) / 4;
+    auto entry = [&](int i, int j) { return (anc[i * W + (j >> 5)] >> (j & 31)) & 1u; };
+    for (int w = threadIdx.x; w < words; w += blockDim.x) {
+        const int at = head + 4 * w;
+        int i = at / n, j = at - i * n;
+        uint32_t v = 0u;
+        if ((j & 31) <= 28 && j + 3 < n) {
+            const uint32_t x = anc[i * W + (j >> 5)] >> (j & 31);
+            v = (x & 1u) | ((x & 2u) << 7) | ((x & 4u) << 14) | ((x & 8u) << 21);
+        } else {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                v |= entry(i, j) << (8 * k);
+                if (++j == n) {
+                    j = 0;
+                    ++i;
+                }
+            }
+        }
+        *reinterpret_cast<uint32_t*>(out + at) = v;
+    }
+    for (int k = threadIdx.x; k < total - 4 * words; k += blockDim.x) {
+        const int at = k < head ? k : 4 * words + k, i = at / n;
+        out[at] = static_cast<uint8_t>(entry(i, at - i * n));
     }
 }
 
@@ -1110,9 +1135,11 @@ __global__ void __launch_bounds__(kLvThreads) build_tree_level_kernel(TreeArgs a
 
 // ------------------------------------------------------------------------------------------
 // The tree-attention mask and position ids (mask_rows) of a drafted tree in global memory: one
-// CTA per sequence and block of kMaskRows rows.
+// CTA per sequence and block of kMaskRows rows. Blocks of 16 rows and four-byte stores: 513 nodes take
+// about 5 us on GB300 instead of 23 with blocks of 128 and single bytes (8 or 32 rows: the same
+// within 2 us).
 // ------------------------------------------------------------------------------------------
-constexpr int kMaskRows = 128;
+constexpr int kMaskRows = 16;
 __global__ void __launch_bounds__(256) tree_mask_kernel(int n, const int32_t* __restrict__ node_parent,
                                                         const int32_t* __restrict__ node_depth,
                                                         const int32_t* __restrict__ root_pos,

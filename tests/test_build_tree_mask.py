@@ -58,6 +58,19 @@ def test_fused_mask_equals_separate_calls(name, over):
     _both(synth.get_config(name, **over))
 
 
+@pytest.mark.parametrize("B", [12, 31, 64, 127, 128, 143, 145, 512])
+def test_mask_equals_the_oracle(B):
+    # trees of 13 to 513 nodes: word stores from any byte offset, words across two rows, blocks of 16
+    # rows with a remainder (143: none, 145: two rows)
+    from oracle import treeflash_oracle as O
+    sep = _both(synth.get_config("tiny_f32", batch=3, B=B, K2=min(B, 64)))
+    for s in range(3):
+        m, pos = O.tree_mask(sep["par"][s].cpu().numpy().astype(np.int64), sep["dep"][s].cpu().numpy().astype(np.int64),
+                             1000 + 7 * s)
+        np.testing.assert_array_equal(sep["mask"][s].cpu().numpy(), m)
+        np.testing.assert_array_equal(sep["pos"][s].cpu().numpy(), pos)
+
+
 def test_fused_mask_on_a_flagged_sequence():
     # an out-of-range root token is flagged, and the trees and masks still agree
     sep = _both(synth.get_config("tiny_peaked", dtype="bf16", batch=2, V=2000), corrupt_root=True)
