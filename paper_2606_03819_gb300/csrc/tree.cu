@@ -1235,10 +1235,49 @@ __device__ __forceinline__ __nv_bfloat16 bf16_round_sum(float r, float t) {
     return __ushort_as_bfloat16(static_cast<unsigned short>(bits >> 16));
 }
 
-// bf16 rows with d % 8 == 0: 16-byte loads and stores, 8 elements per thread and step. x is the
-// correctly rounded bf16 value of the definition (an element off by one bf16 ulp would perturb
-// every gate/up output and flip many later roundings), computed in fp32 only (GB300's fp64 is too
-// slow even for the few scalar steps of a row):
+// ---- packed pairs of fp32 values (two independent operations per instruction)
+__device__ __forceinline__ unsigned long long f2_pack(float lo, float hi) {
+    return static_cast<unsigned long long>(__float_as_uint(hi)) << 32 | __float_as_uint(lo);
+}
+__device__ __forceinline__ float f2_lo(unsigned long long v) { return __uint_as_float(static_cast<uint32_t>(v)); }
+__device__ __forceinline__ float f2_hi(unsigned long long v) { return __uint_as_float(static_cast<uint32_t>(v >> 32)); }
+__device__ __forceinline__ unsigned long long f2_add(unsigned long long a, unsigned long long b) {
+    unsigned long long d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ unsigned long long f2_sub(unsigned long long a, unsigned long long b) {
+    unsigned long long d;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ unsigned long long f2_mul(unsigned long long a, unsigned long long b) {
+    unsigned long long d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ unsigned long long f2_fma(unsigned long long a, unsigned long long b, unsigned long long c) {
+    unsigned long long d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+// the two bf16 values of a 32-bit word
+__device__ __forceinline__ unsigned long long f2_bf16x2(uint32_t w) {
+    return f2_pack(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u));
+}
+
+// ------------------------------------------------------------------------------------------
+// The stage-2 input rows for bf16 with d <= 8192: one item per normalised vector, not per row. The
+// M rows (two tokens: M^2) of a depth share their hidden state, so its part of x is computed once
+// per depth and stored to all of them (at most kHRows per item); every embedding is an item of its
+// own. Hidden-state items need no other kernel's output but the right to overwrite X, so they do
+// all but their stores before the dependency wait.
+// An item is a CTA of eight warps. (Items of one or two warps save the block barrier but hold so
+// much in registers that too few warps are in flight: 1928 rows of d = 5120 took 38 us with one CTA
+// per row, 73 with a warp per item.)
+// x is the correctly rounded bf16 value of the definition (an element off by one bf16 ulp would
+// perturb every gate/up output and flip many later roundings), computed in fp32 only (GB300's fp64
+// is too slow even for the few scalar steps of a row):
 //  - mean(h^2): every square of a bf16 value is exact in fp32; the sums, and their warp and block
 //    reductions, are compensated (TwoSum pairs);
 //  - 1 / sqrt(mean + eps) as hi + lo: hi = rsqrtf, then one Newton step in double-float
@@ -1246,140 +1285,145 @@ __device__ __forceinline__ __nv_bfloat16 bf16_round_sum(float r, float t) {
 //  - h * w is exact in fp32 (two 8-bit significands); (h w) * hi is rounded once and its
 //    rounding error recovered with an FMA, so (h w) / sqrt(mean + eps) is known as r + t to
 //    about 2^-45 relative, which decides the bf16 rounding (bf16_round_sum).
-template <int NE>
-__global__ void __launch_bounds__(256) gather_norm_bf16x8_kernel(
-    const uint4* __restrict__ hidden, const uint4* __restrict__ embed, const uint4* __restrict__ norm_h,
-    const uint4* __restrict__ norm_e, const int32_t* __restrict__ root_tok, const int32_t* __restrict__ top_ids,
-    int gamma, int M, int K1, int R, int d, int V, float eps, uint4* __restrict__ X, uint4* __restrict__ hres,
-    int* status) {
-    pdl_trigger();
-    constexpr int kMaxPerThread = 4;          // d <= 256 * 8 * 4 = 8192
-    constexpr int NS = 1 + NE;                // parts of x: the hidden state, then NE embeddings
-    __shared__ float red[NS][2][8];
-    __shared__ float scale[2 * NS];           // hi, lo of 1 / sqrt(mean + eps) of every part
-    const int row = blockIdx.x;
-    const int hid = stage2_row_hidden(row, R, gamma, M, NE == 2);
+// ------------------------------------------------------------------------------------------
+constexpr int kHRows = 8;       // rows that one hidden-state item stores to (16: up to 3% slower, one row each: 2%)
+struct GatherArgs {
+    const uint4 *hidden, *embed, *norm_h, *norm_e;
+    const int32_t *root_tok, *top_ids;
+    int gamma, M, K1, R, d, V, two_prev;
+    float eps;
+    uint4 *X, *hres;
+    int* status;
+    int h_chunks;     // items per hidden state
+    int n_h;          // hidden-state items, the first ones
+};
 
-    const int dv = d / 8;
-    // the hidden state and the norm weights are step inputs (no kernel writes them): read before
-    // waiting for the previous kernel, which produces the candidate tokens
-    const uint4* h = hidden + static_cast<size_t>(hid) * dv;
-    uint4 v[NS][kMaxPerThread], wh[kMaxPerThread], we[kMaxPerThread];
+template <int NV>      // 16-byte units per thread: ceil(d / 2048)
+__global__ void __launch_bounds__(256) gather_norm_bf16_kernel(GatherArgs a) {
+    pdl_trigger();
+    __shared__ float red[8][2];
+    const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+    const int item = blockIdx.x;
+    const bool is_h = item < a.n_h;
+    const int dv = a.d / 8, NS = a.two_prev ? 3 : 2;
+    // norm weights are step inputs: requested before the dependency wait
+    const uint4* wt = is_h ? a.norm_h : a.norm_e;
+    uint4 wv[NV];
 #pragma unroll
-    for (int i = 0; i < kMaxPerThread; ++i) {
-        const int c = threadIdx.x + i * 256;
-        if (c < dv) {
-            v[0][i] = h[c];
-            wh[i] = norm_h[c];
-            we[i] = norm_e[c];
+    for (int j = 0; j < NV; ++j) {
+        const int c = t + j * 256;
+        wv[j] = c < dv ? wt[c] : make_uint4(0u, 0u, 0u, 0u);
+    }
+    // the rows that the item stores to: r0 .. r0 + n - 1 (an embedding: one row, part `part`)
+    int r0 = 0, n = 1, part = 0;
+    const uint4* src = a.hidden;
+    if (is_h) {
+        const int q = item / a.h_chunks, c = item - q * a.h_chunks, sq = q / a.gamma, i = q - sq * a.gamma;
+        const int per = i == 0 ? 1 : a.two_prev && i > 1 ? a.M * a.M : a.M;          // rows of depth i + 1
+        const int at = i == 0 ? 0 : !a.two_prev ? 1 + (i - 1) * a.M : i == 1 ? 1 : 1 + a.M + (i - 2) * a.M * a.M;
+        r0 = sq * a.R + at + c * kHRows;
+        n = min(kHRows, per - c * kHRows);    // (at most 0: nothing to store)
+        src += static_cast<size_t>(sq * a.gamma + i) * dv;
+    } else {
+        pdl_wait();
+        const int q = item - a.n_h;
+        r0 = a.two_prev ? q >> 1 : q;
+        part = a.two_prev ? 1 + (q & 1) : 1;
+        int tok[2] = {0, 0};
+        stage2_row_tokens(r0, a.R, a.gamma, a.M, a.K1, a.two_prev != 0, a.root_tok, a.top_ids, tok);
+        int token = tok[part - 1];
+        if (token < 0 || token >= a.V) {
+            if (t == 0) set_status(a.status, TF_DEV_BAD_TOKEN);
+            token = 0;
+        }
+        src = a.embed + static_cast<size_t>(token) * dv;
+    }
+    uint4 v[NV];
+#pragma unroll
+    for (int j = 0; j < NV; ++j) {
+        const int c = t + j * 256;
+        v[j] = n > 0 && c < dv ? src[c] : make_uint4(0u, 0u, 0u, 0u);
+    }
+    // sums of squares, two packed running sums
+    unsigned long long s2 = 0ull, c2 = 0ull;
+#pragma unroll
+    for (int j = 0; j < NV; ++j) {
+        const uint32_t w[4] = {v[j].x, v[j].y, v[j].z, v[j].w};
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const unsigned long long h = f2_bf16x2(w[k]), x = f2_mul(h, h);
+            const unsigned long long u = f2_add(s2, x), z = f2_sub(u, s2);
+            c2 = f2_add(c2, f2_add(f2_sub(s2, f2_sub(u, z)), f2_sub(x, z)));
+            s2 = u;
         }
     }
-    pdl_wait();
-    // the approximator GEMMs' tail-split counters (after the status word) start each call at zero
-    if (blockIdx.x == 0 && status)
-        for (int i = threadIdx.x; i < kTailSems; i += blockDim.x) status[1 + i] = 0;
-    int tok[2] = {0, 0};
-    stage2_row_tokens(row, R, gamma, M, K1, NE == 2, root_tok, top_ids, tok);
+    float S = f2_lo(s2), C = f2_lo(c2);
+    two_sum_acc(S, C, f2_hi(s2));
+    C += f2_hi(c2);
 #pragma unroll
-    for (int j = 0; j < NE; ++j) {
-        if (tok[j] < 0 || tok[j] >= V) {
-            if (threadIdx.x == 0) set_status(status, TF_DEV_BAD_TOKEN);
-            tok[j] = 0;
-        }
-        const uint4* e = embed + static_cast<size_t>(tok[j]) * dv;
-#pragma unroll
-        for (int i = 0; i < kMaxPerThread; ++i) {
-            const int c = threadIdx.x + i * 256;
-            if (c < dv) v[1 + j][i] = e[c];
-        }
+    for (int o = 16; o > 0; o >>= 1) {
+        const float so = __shfl_down_sync(0xffffffffu, S, o), co = __shfl_down_sync(0xffffffffu, C, o);
+        two_sum_acc(S, C, so);
+        C += co;
     }
-    // sums of squares: every square of a bf16 value is exact in fp32; the running sums are
-    // compensated (TwoSum), and the (sum, compensation) pairs are combined the same way
-    float sum[NS], comp[NS];
-#pragma unroll
-    for (int j = 0; j < NS; ++j) sum[j] = comp[j] = 0.0f;
-#pragma unroll
-    for (int i = 0; i < kMaxPerThread; ++i) {
-        const int c = threadIdx.x + i * 256;
-        if (c < dv) {
-#pragma unroll
-            for (int j = 0; j < NS; ++j) {
-                const __nv_bfloat16* b = reinterpret_cast<const __nv_bfloat16*>(&v[j][i]);
-#pragma unroll
-                for (int k = 0; k < 8; ++k) {
-                    const float a = __bfloat162float(b[k]);
-                    two_sum_acc(sum[j], comp[j], a * a);
-                }
-            }
-        }
+    if (lane == 0) {
+        red[warp][0] = S;
+        red[warp][1] = C;
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-        for (int j = 0; j < NS; ++j) {
-            const float s2 = __shfl_xor_sync(0xffffffffu, sum[j], o);
-            const float c2 = __shfl_xor_sync(0xffffffffu, comp[j], o);
-            two_sum_acc(sum[j], comp[j], s2);
-            comp[j] += c2;
-        }
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (lane == 0)
-#pragma unroll
-        for (int j = 0; j < NS; ++j) {
-            red[j][0][warp] = sum[j];
-            red[j][1][warp] = comp[j];
-        }
     __syncthreads();
-    if (threadIdx.x < NS) {
-        const int j = threadIdx.x;
-        float S = 0.0f, C = 0.0f;
-        for (int w = 0; w < 8; ++w) {
-            two_sum_acc(S, C, red[j][0][w]);
-            C += red[j][1][w];
-        }
-        // m = (S + C) / d + eps as a double-float (mh, ml); d is scaled exactly when it is a
-        // power of two, otherwise the quotient's rounding error is recovered by an FMA
-        const float fd = static_cast<float>(d);
+    S = C = 0.0f;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) {
+        two_sum_acc(S, C, red[w][0]);
+        C += red[w][1];
+    }
+    // m = (S + C) / d + eps as a double-float (mh, ml); d is scaled exactly when it is a power of
+    // two, otherwise the quotient's rounding error is recovered by an FMA
+    float hi, lo;
+    {
+        const float fd = static_cast<float>(a.d);
         const float q = S / fd;
         const float qerr = fmaf(-q, fd, S) / fd + C / fd;
-        float mh = q + eps;
-        float ml = (q - (mh - (mh - q))) + (eps - (mh - q)) + qerr;   // TwoSum(q, eps) plus the rest
-        const float t = mh + ml;
-        ml = ml - (t - mh);
-        mh = t;
+        float mh = q + a.eps;
+        float ml = (q - (mh - (mh - q))) + (a.eps - (mh - q)) + qerr;   // TwoSum(q, eps) plus the rest
+        const float u = mh + ml;
+        ml = ml - (u - mh);
+        mh = u;
         // y = 1 / sqrt(m): y0 = rsqrtf(mh), then one Newton step in double-float arithmetic,
         // y = y0 + y0 (1 - m y0^2) / 2, with y0^2 and m y0^2 formed by exact FMA products
         const float y0 = rsqrtf(mh);
         const float p = y0 * y0, pl = fmaf(y0, y0, -p);          // y0^2 = p + pl exactly
-        const float u = mh * p, ul = fmaf(mh, p, -u);              // mh p = u + ul exactly
-        const float r = ((1.0f - u) - ul) - (mh * pl + ml * p);    // 1 - m y0^2, ~2^-23
-        const float hi = y0, lo = 0.5f * y0 * r;
-        scale[2 * j] = hi;
-        scale[2 * j + 1] = lo;
+        const float w = mh * p, wl = fmaf(mh, p, -w);              // mh p = w + wl exactly
+        const float r = ((1.0f - w) - wl) - (mh * pl + ml * p);    // 1 - m y0^2, ~2^-23
+        hi = y0;
+        lo = 0.5f * y0 * r;
     }
-    __syncthreads();
-    uint4* xr = X + static_cast<size_t>(row) * NS * dv;
+    if (is_h) pdl_wait();
+    // the approximator GEMMs' tail-split counters (after the status word) start each call at zero
+    if (item == 0 && a.status)
+        for (int i = t; i < kTailSems; i += 256) a.status[1 + i] = 0;
+    uint4* out = a.X + static_cast<size_t>(r0) * NS * dv + static_cast<size_t>(part) * dv;
+    uint4* res = a.two_prev && is_h ? a.hres + static_cast<size_t>(r0) * dv : nullptr;
+    const unsigned long long hi2 = f2_pack(hi, hi), lo2 = f2_pack(lo, lo);
 #pragma unroll
-    for (int i = 0; i < kMaxPerThread; ++i) {
-        const int c = threadIdx.x + i * 256;
-        if (c < dv) {
+    for (int j = 0; j < NV; ++j) {
+        const int c = t + j * 256;
+        if (c >= dv) break;
+        const uint32_t xb[4] = {v[j].x, v[j].y, v[j].z, v[j].w}, wb[4] = {wv[j].x, wv[j].y, wv[j].z, wv[j].w};
+        uint32_t o[4];
 #pragma unroll
-            for (int j = 0; j < NS; ++j) {
-                const float is = scale[2 * j], is_lo = scale[2 * j + 1];
-                const __nv_bfloat16* b = reinterpret_cast<const __nv_bfloat16*>(&v[j][i]);
-                const __nv_bfloat16* wb = reinterpret_cast<const __nv_bfloat16*>(j == 0 ? &wh[i] : &we[i]);
-                uint4 o;
-                __nv_bfloat16* ob = reinterpret_cast<__nv_bfloat16*>(&o);
-#pragma unroll
-                for (int k = 0; k < 8; ++k) {
-                    const float pv = __bfloat162float(b[k]) * __bfloat162float(wb[k]);
-                    const float rv = pv * is;
-                    ob[k] = bf16_round_sum(rv, fmaf(pv, is_lo, fmaf(pv, is, -rv)));
-                }
-                xr[j * dv + c] = o;
-            }
-            if (NE == 2) hres[static_cast<size_t>(row) * dv + c] = v[0][i];
+        for (int k = 0; k < 4; ++k) {
+            const unsigned long long pv = f2_mul(f2_bf16x2(xb[k]), f2_bf16x2(wb[k]));
+            const unsigned long long rv = f2_mul(pv, hi2);
+            const float r0v = f2_lo(rv), r1v = f2_hi(rv);
+            const unsigned long long tv = f2_fma(pv, lo2, f2_fma(pv, hi2, f2_pack(-r0v, -r1v)));
+            const __nv_bfloat16 b0 = bf16_round_sum(r0v, f2_lo(tv)), b1 = bf16_round_sum(r1v, f2_hi(tv));
+            o[k] = static_cast<uint32_t>(__bfloat16_as_ushort(b1)) << 16 | __bfloat16_as_ushort(b0);
         }
+        const uint4 ov = make_uint4(o[0], o[1], o[2], o[3]);
+        for (int r = 0; r < n; ++r) out[static_cast<size_t>(r) * NS * dv + c] = ov;
+        if (res)
+            for (int r = 0; r < n; ++r) res[static_cast<size_t>(r) * dv + c] = v[j];
     }
 }
 
@@ -1391,11 +1435,34 @@ cudaError_t launch_gather_norm(const Ctx& ctx, int dtype, const void* hidden, co
     if (two_prev && !hres) return cudaErrorInvalidValue;
     cudaError_t e;
     if (dtype == TF_BF16 && d % 8 == 0 && d <= 8192) {
-        auto kern = two_prev ? gather_norm_bf16x8_kernel<2> : gather_norm_bf16x8_kernel<1>;
-        e = launch_pdl(kern, dim3(rows), dim3(256), 0, ctx.stream, static_cast<const uint4*>(hidden),
-                       static_cast<const uint4*>(embed), static_cast<const uint4*>(norm_h),
-                       static_cast<const uint4*>(norm_e), root_tok, top_ids, gamma, M, K1, R, d, V, eps,
-                       static_cast<uint4*>(X), static_cast<uint4*>(hres), ctx.status);
+        GatherArgs a{};
+        a.hidden = static_cast<const uint4*>(hidden);
+        a.embed = static_cast<const uint4*>(embed);
+        a.norm_h = static_cast<const uint4*>(norm_h);
+        a.norm_e = static_cast<const uint4*>(norm_e);
+        a.root_tok = root_tok;
+        a.top_ids = top_ids;
+        a.gamma = gamma;
+        a.M = M;
+        a.K1 = K1;
+        a.R = R;
+        a.d = d;
+        a.V = V;
+        a.two_prev = two_prev;
+        a.eps = eps;
+        a.X = static_cast<uint4*>(X);
+        a.hres = static_cast<uint4*>(hres);
+        a.status = ctx.status;
+        a.h_chunks = ((two_prev && gamma > 2 ? M * M : M) + kHRows - 1) / kHRows;
+        const long long n_h = static_cast<long long>(b) * gamma * a.h_chunks;
+        const long long n_items = n_h + static_cast<long long>(rows) * (two_prev ? 2 : 1);
+        if (n_items > 0x7fffffffll) return cudaErrorInvalidConfiguration;
+        a.n_h = static_cast<int>(n_h);
+        auto kern = d <= 2048   ? gather_norm_bf16_kernel<1>
+                    : d <= 4096 ? gather_norm_bf16_kernel<2>
+                    : d <= 6144 ? gather_norm_bf16_kernel<3>
+                                : gather_norm_bf16_kernel<4>;
+        e = launch_pdl(kern, dim3(static_cast<unsigned>(n_items)), dim3(256), 0, ctx.stream, a);
     } else if (dtype == TF_BF16) {
         using B16 = __nv_bfloat16;
         auto kern = two_prev ? gather_norm_kernel<B16, 2> : gather_norm_kernel<B16, 1>;
