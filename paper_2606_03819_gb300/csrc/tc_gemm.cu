@@ -69,6 +69,8 @@ struct EpiParams {
     // the epilogue.
     int n_full, tail_split;
     int* sem;
+    // kernels with a width chosen at launch: columns per N tile (a multiple of 8) and ring stages
+    int bn, stages;
 };
 
 // Work unit u -> (N tile, M-tile group, K split); consecutive units share the N tile and K split
@@ -86,18 +88,22 @@ __device__ __forceinline__ Unit decode_unit(int u, int n_mgroups, int k_splits) 
 }
 
 // PAIR: a CTA of a cta_group::2 pair, which stages half of the weight tile (BN / 2 rows).
-template <int MT, int NB, int BN, int STAGES, bool PAIR = false>
+// VAR: tiles of up to BN columns and up to STAGES stages, as many as fit the ring.
+template <int MT, int NB, int BN, int STAGES, bool PAIR = false, bool VAR = false>
 struct TileCfg {
     static constexpr int kABytes = kBM * kBK * 2;
     static constexpr int kBBytes = BN * kBK * 2;                    // the whole weight tile of a stage
     static constexpr int kBBytesCta = PAIR ? kBBytes / 2 : kBBytes;  // the part this CTA stages
     static constexpr int kStageBytes = MT * kABytes + NB * kBBytesCta;
+    static constexpr int kRingBytes = VAR ? 208 * 1024 : STAGES * kStageBytes;
     static constexpr int kBarrierBytes = 256;
-    static constexpr int kSmemBytes = STAGES * kStageBytes + kBarrierBytes + 1024;
+    static constexpr int kSmemBytes = kRingBytes + kBarrierBytes + 1024;
     static_assert(NB * BN <= 256, "one accumulator slot is 256 TMEM columns");
     static_assert(BN % 64 == 0 && BN >= 64 && BN <= 256, "N tile (two epilogue warps split it in 32-column steps)");
     static_assert(kStageBytes % 1024 == 0, "stages must stay 1024-byte aligned for 128B swizzle");
 };
+
+constexpr int kVarMaxStages = 8;   // ring stages of the kernels whose tile width is chosen at launch
 
 __device__ __forceinline__ float silu_f(float g) { return g / (1.0f + __expf(-g)); }
 
@@ -157,7 +163,8 @@ __device__ __forceinline__ ChunkNode chunk_tree(const uint32_t (&r)[32], int v0,
     }
 }
 
-template <int EPI, int MT, int NB, int BN, int STAGES, int CL>
+// VAR: the tile is ep.bn <= BN columns wide and the ring has ep.stages <= STAGES stages.
+template <int EPI, int MT, int NB, int BN, int STAGES, int CL, bool VAR>
 __global__ void __launch_bounds__(kThreads, 1)
 tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ CUtensorMap tmap_w0,
                const __grid_constant__ CUtensorMap tmap_w1, int n_rows, int K, int n_ntiles,
@@ -167,14 +174,17 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant
     // cluster), whose accumulators are summed through distributed shared memory.
     constexpr bool kSplitK = EPI == EPI_CGATEUP || EPI == EPI_CDOWN;
     constexpr bool kPair = CL > 1 && !kSplitK;
-    using C = TileCfg<MT, NB, BN, STAGES, kPair>;
-    static_assert(CL == 1 || kSplitK || (CL == 2 && NB == 1 && MT == 1), "a CTA pair shares one weight operand");
+    using C = TileCfg<MT, NB, BN, STAGES, kPair, VAR>;
+    static_assert(CL == 1 || kSplitK || (CL == 2 && MT == 1), "a CTA of a pair holds one M-tile");
     static_assert(!kSplitK || (CL == 4 && MT == 2 && BN == 128), "cluster split-K: 4 K-ranges of a 256 x 128 tile");
+    static_assert(!VAR || (CL == 1 && EPI != EPI_LMHEAD), "variable width: single CTAs of the approximator");
     pdl_trigger();
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
-    uint64_t* full = reinterpret_cast<uint64_t*>(smem + STAGES * C::kStageBytes);
+    const int bn = VAR ? ep.bn : BN, stages = VAR ? ep.stages : STAGES;
+    const int stage_bytes = VAR ? MT * C::kABytes + NB * bn * kBK * 2 : C::kStageBytes;
+    uint64_t* full = reinterpret_cast<uint64_t*>(smem + C::kRingBytes);
     uint64_t* empty = full + STAGES;
     uint64_t* tfull = empty + STAGES;
     uint64_t* tempty = tfull + 2;
@@ -202,7 +212,8 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant
     };
     // Work items: the units, except that with a tail split each unit of the last round becomes
     // tail_split items over consecutive K-chunks of its range ([kb0, kb1) in K-steps).
-    constexpr bool kTail = CL == 1 && (EPI == EPI_GATEUP || EPI == EPI_DOWN);
+    constexpr bool kTail = !VAR && (EPI == EPI_GATEUP || EPI == EPI_DOWN);
+    constexpr int kUnitTiles = kPair ? 2 : MT;   // M-tiles of a unit
     const int n_split = kTail ? ep.tail_split : 0;
     const int n_items = n_split ? ep.n_full + (n_units - ep.n_full) * n_split : n_units;
     struct Item {
@@ -285,7 +296,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant
             const uint64_t pol_w = w_stream_once ? ptx::policy_evict_first() : ptx::policy_evict_last();
             // Pair: both CTAs' copies of a stage complete on the even CTA's full barrier, which
             // the even CTA alone arms with the bytes of both halves.
-            constexpr uint32_t kTxBytes = (kPair ? 2 : 1) * C::kStageBytes;
+            const uint32_t tx_bytes = (kPair ? 2 : 1) * stage_bytes;
             auto load_x = [&](uint8_t* sp, uint64_t* bar, int j, int kb, int mt) {
                 if constexpr (kPair)
                     ptx::tma_load_2d_pair(sp + j * C::kABytes, &tmap_x, in_leader(bar), kb * kBK, mt * kBM, pol_x);
@@ -293,15 +304,19 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant
                     ptx::tma_load_2d(sp + j * C::kABytes, &tmap_x, bar, kb * kBK, mt * kBM, pol_x);
             };
             // Weight tiles of one stage; in a pair each CTA stages its half of the rows
-            // (tmap_w0's box is BN / 2 rows high).
+            // (one weight matrix: tmap_w0's box is BN / 2 rows high; two: BN, one matrix per CTA).
             auto load_w = [&](uint8_t* sp, uint64_t* bar, int kb, int nt) {
-                if constexpr (kPair) {
+                if constexpr (kPair && NB == 2) {
+                    // the pair's N operand is the gate tile followed by the up tile: one each
+                    ptx::tma_load_2d_pair(sp + MT * C::kABytes, crank ? &tmap_w1 : &tmap_w0, in_leader(bar), kb * kBK,
+                                          nt * BN, pol_w);
+                } else if constexpr (kPair) {
                     ptx::tma_load_2d_pair(sp + MT * C::kABytes, &tmap_w0, in_leader(bar), kb * kBK,
                                           nt * BN + crank * (BN / 2), pol_w);
                 } else {
-                    ptx::tma_load_2d(sp + MT * C::kABytes, &tmap_w0, bar, kb * kBK, nt * BN, pol_w);
+                    ptx::tma_load_2d(sp + MT * C::kABytes, &tmap_w0, bar, kb * kBK, nt * bn, pol_w);
                     if (NB == 2)
-                        ptx::tma_load_2d(sp + MT * C::kABytes + C::kBBytes, &tmap_w1, bar, kb * kBK, nt * BN, pol_w);
+                        ptx::tma_load_2d(sp + MT * C::kABytes + bn * kBK * 2, &tmap_w1, bar, kb * kBK, nt * bn, pol_w);
                 }
             };
             // The weights are no kernel's output: the first unit's first weight tiles are
@@ -309,10 +324,10 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant
             int pre = 0;
             if (cid < n_items) {
                 const Item f = item_of(cid);
-                pre = f.kb1 - f.kb0 < STAGES ? f.kb1 - f.kb0 : STAGES;
+                pre = f.kb1 - f.kb0 < stages ? f.kb1 - f.kb0 : stages;
                 for (int i = 0; i < pre; ++i) {
-                    if (leader) ptx::mbar_arrive_expect_tx(&full[i], kTxBytes);
-                    load_w(smem + i * C::kStageBytes, &full[i], f.kb0 + i, f.w.nt);
+                    if (leader) ptx::mbar_arrive_expect_tx(&full[i], tx_bytes);
+                    load_w(smem + i * stage_bytes, &full[i], f.kb0 + i, f.w.nt);
                 }
             }
             pdl_wait();
@@ -330,15 +345,15 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant
                         ok = false;
                         break;
                     }
-                    uint8_t* sp = smem + stage * C::kStageBytes;
+                    uint8_t* sp = smem + stage * stage_bytes;
                     const bool w_done = it < pre;     // weight tiles already requested above
-                    if (!w_done && leader) ptx::mbar_arrive_expect_tx(&full[stage], kTxBytes);
+                    if (!w_done && leader) ptx::mbar_arrive_expect_tx(&full[stage], tx_bytes);
 #pragma unroll
                     for (int j = 0; j < MT; ++j) load_x(sp, &full[stage], j, kb, mt0 + j);
                     if (!w_done) load_w(sp, &full[stage], kb, nt);
                     issued_mask |= 1u << stage;
                     last_parity[stage] = phase;
-                    if (++stage == STAGES) {
+                    if (++stage == stages) {
                         stage = 0;
                         phase ^= 1u;
                     }
@@ -368,7 +383,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant
         if (lane == 0 && leader) {
             // the NB weight tiles of a stage are adjacent in shared memory with the same swizzle, so
             // one MMA of N = NB * BN covers them: A is read from shared memory once per k-step
-            constexpr uint32_t kIdesc = ptx::idesc_bf16_f32(kPair ? 2 * kBM : kBM, NB * BN);
+            const uint32_t idesc = ptx::idesc_bf16_f32(kPair ? 2 * kBM : kBM, NB * bn);
             int stage = 0;
             uint32_t phase = 0;
             uint32_t use[2] = {0u, 0u};
@@ -391,7 +406,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant
                         break;
                     }
                     ptx::tc_fence_after();
-                    const uint32_t a0 = ptx::smem_u32(smem + stage * C::kStageBytes);
+                    const uint32_t a0 = ptx::smem_u32(smem + stage * stage_bytes);
                     const uint32_t b0 = a0 + MT * C::kABytes;
 #pragma unroll
                     for (int kk = 0; kk < kBK / 16; ++kk) {
@@ -401,9 +416,9 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant
                             const uint64_t ad = ptx::sw128_kmajor_desc(a0 + j * C::kABytes + kk * 32);
                             const uint32_t acc = (kb | kk) != 0 ? 1u : 0u;
                             if constexpr (kPair)
-                                ptx::mma_bf16_pair(tmem_base + 256u * (g0 + j), ad, bd, kIdesc, acc);
+                                ptx::mma_bf16_pair(tmem_base + 256u * (g0 + j), ad, bd, idesc, acc);
                             else
-                                ptx::mma_bf16(tmem_base + 256u * (g0 + j), ad, bd, kIdesc, acc);
+                                ptx::mma_bf16(tmem_base + 256u * (g0 + j), ad, bd, idesc, acc);
                         }
                     }
                     // frees the stage (in both CTAs of a pair) once these MMAs finish
@@ -413,7 +428,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant
                     } else {
                         ptx::mma_commit(&empty[stage]);
                     }
-                    if (++stage == STAGES) {
+                    if (++stage == stages) {
                         stage = 0;
                         phase ^= 1u;
                     }
@@ -477,12 +492,12 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant
             if (kTail && itm.chunk >= 0) {
                 // ---- a K-chunk of a tail unit: its partial sums to `partial`; the group whose
                 // chunk completes the unit's count adds all chunks in chunk order
-                const int j = MT == 2 ? g : 0;                 // M-tile of the unit in this slot
+                const int j = kPair ? crank : MT == 2 ? g : 0; // M-tile of the unit in this slot
                 const int r = q * 32 + lane;                   // row within the M-tile
                 constexpr int kUnitF4 = kBM * NB * BN / 4;     // float4s of one (chunk, M-tile)
                 float4* part = reinterpret_cast<float4*>(ep.partial);
                 auto at = [&](int ch, int col) {               // float4 of columns col..col+3, row r
-                    return (static_cast<size_t>((itm.tail * n_split + ch) * MT + j) * kUnitF4) +
+                    return (static_cast<size_t>((itm.tail * n_split + ch) * kUnitTiles + j) * kUnitF4) +
                            static_cast<size_t>(col >> 2) * kBM + r;
                 };
 #pragma unroll 1
@@ -503,7 +518,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant
                 ptx::named_barrier_sync(1 + g, 32 * kEpiWarps / 2);
                 if (e % (kEpiWarps / 2) == 0 && lane == 0) {
                     __threadfence();
-                    const int done = atomicAdd(ep.sem + itm.tail * MT + j, 1);
+                    const int done = atomicAdd(ep.sem + itm.tail * kUnitTiles + j, 1);
                     last_chunk[g] = done == n_split - 1 ? 1 : 0;
                 }
                 ptx::named_barrier_sync(1 + g, 32 * kEpiWarps / 2);
@@ -550,7 +565,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant
                     }
                     // the count starts from zero for the next call
                     ptx::named_barrier_sync(1 + g, 32 * kEpiWarps / 2);
-                    if (e % (kEpiWarps / 2) == 0 && lane == 0) ep.sem[itm.tail * MT + j] = 0;
+                    if (e % (kEpiWarps / 2) == 0 && lane == 0) ep.sem[itm.tail * kUnitTiles + j] = 0;
                 }
             } else if constexpr (kSplitK) {
                 // the accumulators are summed across the cluster below, once every CTA has them
@@ -609,6 +624,56 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant
                     }
                     if (row < n_rows)
                         P.halves[P.half_at(nt, half, row)] = make_float4(hm, hsum, hbv, __int_as_float(hbid));
+                }
+                release_slot(g);
+            } else if constexpr (VAR) {
+                // Columns in steps of 8, alternating between the two warps of a row quarter; a last
+                // tile may run past the matrix (its weight rows there are zero, its columns dropped).
+                const int n_tot = EPI == EPI_PARTIAL ? ep.n_total : ep.ld_out;
+                const int cols = n_tot - nt * bn < bn ? n_tot - nt * bn : bn;
+                int hid_row = 0;
+                if (EPI == EPI_DOWN && row < n_rows) {
+                    const int sq = row / ep.R, rr = row - sq * ep.R;
+                    hid_row = sq * ep.gamma + stage2_hidden_index(rr, ep.M);
+                }
+#pragma unroll 1
+                for (int c = 8 * half; c < cols; c += 16) {
+                    uint32_t ra[NB][8];
+#pragma unroll
+                    for (int nb = 0; nb < NB; ++nb) ptx::tmem_ld_8cols(tb + nb * bn + c, ra[nb]);
+                    const size_t col = static_cast<size_t>(nt) * bn + c;
+                    if (row >= n_rows) {
+                    } else if constexpr (EPI == EPI_PARTIAL) {
+                        float4* split = reinterpret_cast<float4*>(ep.partial + static_cast<size_t>(w.kx) * ep.n_cols * n_rows);
+#pragma unroll
+                        for (int nb = 0; nb < NB; ++nb) {
+                            float4* dst = split + (nb * static_cast<size_t>(ep.n_total) + col) / 4 * n_rows + row;
+#pragma unroll
+                            for (int j = 0; j < 2; ++j)
+                                dst[static_cast<size_t>(j) * n_rows] =
+                                    make_float4(__uint_as_float(ra[nb][4 * j]), __uint_as_float(ra[nb][4 * j + 1]),
+                                                __uint_as_float(ra[nb][4 * j + 2]), __uint_as_float(ra[nb][4 * j + 3]));
+                        }
+                    } else {
+                        uint32_t o[4];
+                        if constexpr (EPI == EPI_GATEUP) {
+#pragma unroll
+                            for (int t = 0; t < 4; ++t)
+                                o[t] = pack_bf16x2(silu_f(__uint_as_float(ra[0][2 * t])) * __uint_as_float(ra[NB - 1][2 * t]),
+                                                   silu_f(__uint_as_float(ra[0][2 * t + 1])) * __uint_as_float(ra[NB - 1][2 * t + 1]));
+                        } else {
+                            const uint4 hv = *reinterpret_cast<const uint4*>(ep.hidden + static_cast<size_t>(hid_row) * ep.ld_out + col);
+                            const uint32_t hw[4] = {hv.x, hv.y, hv.z, hv.w};
+#pragma unroll
+                            for (int t = 0; t < 4; ++t) {
+                                const __nv_bfloat162 h2 = *reinterpret_cast<const __nv_bfloat162*>(&hw[t]);
+                                o[t] = pack_bf16x2(__bfloat162float(h2.x) + __uint_as_float(ra[0][2 * t]),
+                                                   __bfloat162float(h2.y) + __uint_as_float(ra[0][2 * t + 1]));
+                            }
+                        }
+                        *reinterpret_cast<uint4*>(ep.out + static_cast<size_t>(row) * ep.ld_out + col) = make_uint4(o[0], o[1], o[2], o[3]);
+                    }
+                    __syncwarp();   // converged again for the next TMEM load
                 }
                 release_slot(g);
             } else if constexpr (EPI == EPI_PARTIAL) {
@@ -872,7 +937,7 @@ cudaError_t run_gemm(const Ctx& ctx, const CUtensorMap& tx, const CUtensorMap& t
                      int n_rows, int K, int n_ntiles, int n_mgroups, const EpiParams& ep_in, int k_splits = 1,
                      size_t partial_bytes = 0) {
     using C = TileCfg<MT, NB, BN, STAGES, (CL == 2 && EPI != EPI_CGATEUP && EPI != EPI_CDOWN)>;
-    auto kern = tc_gemm_kernel<EPI, MT, NB, BN, STAGES, CL>;
+    auto kern = tc_gemm_kernel<EPI, MT, NB, BN, STAGES, CL, false>;
     EpiParams ep = ep_in;
     ep.wait_ns = wait_limit_ns();
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes);
@@ -884,18 +949,23 @@ cudaError_t run_gemm(const Ctx& ctx, const CUtensorMap& tx, const CUtensorMap& t
         // that all clusters are resident at once (splitk_clusters_fit)
         e = launch_pdl_cluster(kern, dim3(CL * n_ntiles * n_mgroups), dim3(kThreads), C::kSmemBytes, ctx.stream, CL,
                                tx, tw0, tw1, n_rows, K, n_ntiles, n_mgroups, CL, stream_once, ep, ctx.status);
-    } else if constexpr (CL == 1) {
+    } else {
         int n_items = n_units;
         if constexpr (EPI == EPI_GATEUP || EPI == EPI_DOWN) {
             // Tail split: when the units overflow the SMs by a last round that would leave most of
             // them idle, each unit of that round runs as up to kMaxTailSplit K-chunks on the idle
-            // SMs, summed by the chunk that finishes last (fp32 partial sums in the workspace).
-            const int tail = n_units % ctx.num_sms;
-            int split = tail > 0 ? ctx.num_sms / tail : 0;
+            // SMs, summed by the chunk that finishes last (fp32 partial sums in the workspace). A
+            // pair's unit of 256 columns counts for two SMs, one of 128 + 128 for one (two rounds
+            // of pairs take the time of one round of single CTAs), so that the chunks of an output
+            // do not depend on whether pairs run it.
+            constexpr int kTiles = CL == 1 ? MT : 2;
+            const int slots = CL == 2 && NB == 1 ? ctx.num_sms / 2 : ctx.num_sms;
+            const int tail = n_units % slots;
+            int split = tail > 0 ? slots / tail : 0;
             split = split < kMaxTailSplit ? split : kMaxTailSplit;
             split = split < K / kBK ? split : K / kBK;
-            const size_t need = static_cast<size_t>(tail) * split * MT * kBM * NB * BN * sizeof(float);
-            if (k_splits == 1 && n_units > ctx.num_sms && split >= 2 && ctx.status && tail * MT <= kTailSems &&
+            const size_t need = static_cast<size_t>(tail) * split * kTiles * kBM * NB * BN * sizeof(float);
+            if (k_splits == 1 && n_units > slots && split >= 2 && ctx.status && tail * kTiles <= kTailSems &&
                 ep.partial && need <= partial_bytes) {
                 ep.n_full = n_units - tail;
                 ep.tail_split = split;
@@ -903,14 +973,16 @@ cudaError_t run_gemm(const Ctx& ctx, const CUtensorMap& tx, const CUtensorMap& t
                 n_items = ep.n_full + tail * split;
             }
         }
-        const int grid = n_items < ctx.num_sms ? n_items : ctx.num_sms;
-        e = launch_pdl(kern, dim3(grid), dim3(kThreads), C::kSmemBytes, ctx.stream, tx, tw0, tw1, n_rows, K,
-                       n_ntiles, n_mgroups, k_splits, stream_once, ep, ctx.status);
-    } else {
-        static const int max_cl = resident_clusters(kern, C::kSmemBytes, CL, ctx.num_sms);
-        const int n_cl = n_units < max_cl ? n_units : max_cl;
-        e = launch_pdl_cluster(kern, dim3(CL * n_cl), dim3(kThreads), C::kSmemBytes, ctx.stream, CL, tx, tw0, tw1,
-                               n_rows, K, n_ntiles, n_mgroups, k_splits, stream_once, ep, ctx.status);
+        if constexpr (CL == 1) {
+            const int grid = n_items < ctx.num_sms ? n_items : ctx.num_sms;
+            e = launch_pdl(kern, dim3(grid), dim3(kThreads), C::kSmemBytes, ctx.stream, tx, tw0, tw1, n_rows, K,
+                           n_ntiles, n_mgroups, k_splits, stream_once, ep, ctx.status);
+        } else {
+            static const int max_cl = resident_clusters(kern, C::kSmemBytes, CL, ctx.num_sms);
+            const int n_cl = n_items < max_cl ? n_items : max_cl;
+            e = launch_pdl_cluster(kern, dim3(CL * n_cl), dim3(kThreads), C::kSmemBytes, ctx.stream, CL, tx, tw0, tw1,
+                                   n_rows, K, n_ntiles, n_mgroups, k_splits, stream_once, ep, ctx.status);
+        }
     }
     return e != cudaSuccess ? e : cudaGetLastError();
 }
@@ -930,7 +1002,7 @@ namespace {
 template <int EPI, int MT, int NB, int BN, int STAGES, int CL>
 bool splitk_clusters_fit(const Ctx& ctx, int n_tiles) {
     using C = TileCfg<MT, NB, BN, STAGES>;
-    auto kern = tc_gemm_kernel<EPI, MT, NB, BN, STAGES, CL>;
+    auto kern = tc_gemm_kernel<EPI, MT, NB, BN, STAGES, CL, false>;
     static const int max_cl = [&] {
         if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes) != cudaSuccess) {
             (void)cudaGetLastError();
@@ -991,11 +1063,60 @@ int choose_k_splits(int base_units, int nk, int num_sms) {
     return ks < 1 ? 1 : ks;
 }
 
-// h' = h + In W^T with In [n_rows, K] (tmap_in, boxes of kBK x kBM) and W [d, K] (tmap_w, boxes of
-// kBK x BN, BN = 128 when d % 128 == 0, else 64): the SwiGLU down projection (K = I, In = A) and
-// the linear approximator (K = 2d, In = x). The residual row of stage-2 row r is the hidden state
-// of its depth; the epilogue adds it in fp32 and rounds once to bf16.
-static cudaError_t run_residual_gemm(const Ctx& ctx, const CUtensorMap& ta, const CUtensorMap& td, int K, const void* hidden,
+// Where the fixed-width kernels of Eq. 1 take over from single CTAs of chosen width (GB300, 152 SMs):
+// clusters of four from 96 CTAs (I = d = 3584, 241 rows: Eq. 1 54.0 against 58.6 us; at 64 CTAs, d =
+// 2048, 38.1 against 35.2), pairs from 40 (d = 4096, 723 rows, 48 pairs: 111 against 114 us; d = 2560,
+// 241 rows, 40 pairs: 84.5 against 85.8; d = 2048, 32 pairs: 37.0 against 35.3).
+constexpr int kMinClusterCtas = 96;
+constexpr int kMinPairs = 40;
+
+// A GEMM of single CTAs whose tile width is chosen for the SM count: [n_rows, K] x [N, K]^T (NB
+// matrices side by side), in k_splits K-ranges. A round of units costs about what an SM loads per
+// K-step (its weight tile, and X, mostly from L2, at half weight), so the width in [32, 128] that
+// makes the cheapest whole rounds is taken: 12288 columns of one M-tile run as 140 tiles of 88 on 152
+// SMs instead of 96 of 128 (121 rows, gate/up and down: 114 -> 102 us), 1024 columns in 4 K-ranges as
+// 128 units of 32 instead of 32 of 128. The width does not change any output's sum.
+template <int EPI, int MT, int NB>
+cudaError_t run_gemm_var(const Ctx& ctx, const CUtensorMap& tx, const void* w0, const void* w1, int N, int n_rows, int K,
+                         int n_mgroups, int k_splits, const EpiParams& ep_in) {
+    using C = TileCfg<MT, NB, 128, kVarMaxStages, false, true>;
+    auto kern = tc_gemm_kernel<EPI, MT, NB, 128, kVarMaxStages, 1, true>;
+    int bn = 128;
+    double best = 0.0;
+    // N of an MMA with M = 128 is a multiple of 16; boxes of whole 8-row swizzle groups
+    constexpr int kStep = NB == 1 ? 16 : 8;
+    for (int w = 128; w >= 32; w -= kStep) {
+        const long long units = static_cast<long long>((N + w - 1) / w) * n_mgroups * k_splits;
+        const long long rounds = (units + ctx.num_sms - 1) / ctx.num_sms;
+        const double cost = static_cast<double>(rounds) * (MT * 8.0 + NB * w / 8.0 + 2.0);
+        if (w == 128 || cost < best) {
+            best = cost;
+            bn = w;
+        }
+    }
+    CUtensorMap t0, t1;
+    cudaError_t e = make_tmap(&t0, w0, K, N, kBK, bn);
+    if (e == cudaSuccess) e = make_tmap(&t1, NB == 2 ? w1 : w0, K, N, kBK, bn);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes);
+    if (e != cudaSuccess) return e;
+    EpiParams ep = ep_in;
+    ep.wait_ns = wait_limit_ns();
+    ep.bn = bn;
+    const int stages = C::kRingBytes / (MT * C::kABytes + NB * bn * kBK * 2);
+    ep.stages = stages < kVarMaxStages ? stages : kVarMaxStages;
+    const int n_ntiles = (N + bn - 1) / bn;
+    const long long n_units = static_cast<long long>(n_ntiles) * n_mgroups * k_splits;
+    const int grid = static_cast<int>(n_units < ctx.num_sms ? n_units : ctx.num_sms);
+    e = launch_pdl(kern, dim3(grid), dim3(kThreads), C::kSmemBytes, ctx.stream, tx, t0, t1, n_rows, K, n_ntiles, n_mgroups,
+                   k_splits, n_mgroups == 1 ? 1 : 0, ep, ctx.status);
+    return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+// h' = h + In W^T with In [n_rows, K] (tmap_in, boxes of kBK x kBM) and W [d, K]: the SwiGLU down
+// projection (K = I, In = A) and the linear approximator (K = 2d, In = x). The residual row of
+// stage-2 row r is the hidden state of its depth; the epilogue adds it in fp32 and rounds once to
+// bf16.
+static cudaError_t run_residual_gemm(const Ctx& ctx, const CUtensorMap& ta, const void* W, int K, const void* hidden,
                               int n_rows, int d, int R, int M, int gamma, void* h_prime, float* partial,
                               size_t partial_bytes) {
     constexpr int BN = 128;
@@ -1003,6 +1124,9 @@ static cudaError_t run_residual_gemm(const Ctx& ctx, const CUtensorMap& ta, cons
     const int n_mg = m_tiles == 1 ? 1 : (m_tiles + 1) / 2;
     const int bn_d = d % BN == 0 ? BN : 64;
     const int ks2 = choose_k_splits((d / bn_d) * n_mg, K / kBK, ctx.num_sms);
+    CUtensorMap td;
+    cudaError_t e = make_tmap(&td, W, K, d, kBK, bn_d);
+    if (e != cudaSuccess) return e;
     EpiParams ed{};
     ed.out = static_cast<__nv_bfloat16*>(h_prime);
     ed.ld_out = d;
@@ -1013,22 +1137,24 @@ static cudaError_t run_residual_gemm(const Ctx& ctx, const CUtensorMap& ta, cons
     ed.partial = partial;
     ed.n_cols = d;
     ed.n_total = d;
-    if (ks2 == 1) {
-        if (bn_d == BN)
-            return m_tiles == 1 ? run_gemm<EPI_DOWN, 1, 1, BN, 6>(ctx, ta, td, td, n_rows, K, d / BN, 1, ed, 1, partial_bytes)
-                                : run_gemm<EPI_DOWN, 2, 1, BN, 4>(ctx, ta, td, td, n_rows, K, d / BN, n_mg, ed, 1, partial_bytes);
-        return m_tiles == 1 ? run_gemm<EPI_DOWN, 1, 1, 64, 8>(ctx, ta, td, td, n_rows, K, d / 64, 1, ed, 1, partial_bytes)
-                            : run_gemm<EPI_DOWN, 2, 1, 64, 5>(ctx, ta, td, td, n_rows, K, d / 64, n_mg, ed, 1, partial_bytes);
-    }
-    if (m_tiles == 2 && bn_d == BN && ks2 == 4 && splitk_clusters_fit<EPI_CDOWN, 2, 1, BN, 4, 4>(ctx, d / BN))
+    // Two M-tiles with K split four ways: clusters of four that exchange their partial sums. Two or
+    // more M-tiles otherwise: CTA pairs on 256-column tiles, which stage a third less per SM and overlap
+    // their epilogue with the next unit (1928 rows, K = 8192, d = 4096: 131 -> 108 us with the gather;
+    // gate/up gains nothing from pairs: single CTAs already run N = 256 MMAs there). Both only where
+    // their units fill the SMs.
+    if (m_tiles == 2 && bn_d == BN && ks2 == 4 && d / BN * 4 >= kMinClusterCtas && splitk_clusters_fit<EPI_CDOWN, 2, 1, BN, 4, 4>(ctx, d / BN))
         return run_gemm<EPI_CDOWN, 2, 1, BN, 4, 4>(ctx, ta, td, td, n_rows, K, d / BN, 1, ed, 4);
-    cudaError_t e;
-    if (bn_d == BN)
-        e = m_tiles == 1 ? run_gemm<EPI_PARTIAL, 1, 1, BN, 6>(ctx, ta, td, td, n_rows, K, d / BN, 1, ed, ks2)
-                         : run_gemm<EPI_PARTIAL, 2, 1, BN, 4>(ctx, ta, td, td, n_rows, K, d / BN, n_mg, ed, ks2);
+    const bool pair = m_tiles > 1 && d % 256 == 0 && d / 256 * n_mg * ks2 >= kMinPairs;
+    if (ks2 == 1) {
+        if (pair) return run_gemm<EPI_DOWN, 1, 1, 256, 7, 2>(ctx, ta, td, td, n_rows, K, d / 256, n_mg, ed, 1, partial_bytes);
+        return m_tiles == 1 ? run_gemm_var<EPI_DOWN, 1, 1>(ctx, ta, W, nullptr, d, n_rows, K, 1, 1, ed)
+                            : run_gemm_var<EPI_DOWN, 2, 1>(ctx, ta, W, nullptr, d, n_rows, K, n_mg, 1, ed);
+    }
+    if (pair)
+        e = run_gemm<EPI_PARTIAL, 1, 1, 256, 7, 2>(ctx, ta, td, td, n_rows, K, d / 256, n_mg, ed, ks2);
     else
-        e = m_tiles == 1 ? run_gemm<EPI_PARTIAL, 1, 1, 64, 8>(ctx, ta, td, td, n_rows, K, d / 64, 1, ed, ks2)
-                         : run_gemm<EPI_PARTIAL, 2, 1, 64, 5>(ctx, ta, td, td, n_rows, K, d / 64, n_mg, ed, ks2);
+        e = m_tiles == 1 ? run_gemm_var<EPI_PARTIAL, 1, 1>(ctx, ta, W, nullptr, d, n_rows, K, 1, ks2, ed)
+                         : run_gemm_var<EPI_PARTIAL, 2, 1>(ctx, ta, W, nullptr, d, n_rows, K, n_mg, ks2, ed);
     if (e != cudaSuccess) return e;
     return launch_down_reduce(ctx, partial, ks2, n_rows, d, static_cast<const __nv_bfloat16*>(hidden), R, M, gamma,
                               static_cast<__nv_bfloat16*>(h_prime));
@@ -1042,13 +1168,11 @@ cudaError_t launch_swiglu_tc(const Ctx& ctx, const void* X, int k_in, const void
     const int m_tiles = (n_rows + kBM - 1) / kBM;
     const int n_mg = m_tiles == 1 ? 1 : (m_tiles + 1) / 2;
     const int bn_gu = I % BN == 0 ? BN : 64;
-    const int bn_d = d % BN == 0 ? BN : 64;
-    CUtensorMap tx, tg, tu, ta, td;
+    CUtensorMap tx, tg, tu, ta;
     cudaError_t e = make_tmap(&tx, X, k_in, n_rows, kBK, kBM);
     if (e == cudaSuccess) e = make_tmap(&tg, w_gate, k_in, I, kBK, bn_gu);
     if (e == cudaSuccess) e = make_tmap(&tu, w_up, k_in, I, kBK, bn_gu);
     if (e == cudaSuccess) e = make_tmap(&ta, A, I, n_rows, kBK, kBM);
-    if (e == cudaSuccess) e = make_tmap(&td, w_down, I, d, kBK, bn_d);
     if (e != cudaSuccess) return e;
 
     // ---- gate/up: A = SiLU(X Wg^T) * (X Wu^T)
@@ -1059,43 +1183,32 @@ cudaError_t launch_swiglu_tc(const Ctx& ctx, const void* X, int k_in, const void
     ep.partial = partial;
     ep.n_cols = 2 * I;
     ep.n_total = I;
-    if (ks1 == 1) {
-        if (bn_gu == BN)
-            e = m_tiles == 1 ? run_gemm<EPI_GATEUP, 1, 2, BN, 4>(ctx, tx, tg, tu, n_rows, k_in, I / BN, 1, ep, 1, partial_bytes)
-                             : run_gemm<EPI_GATEUP, 2, 2, BN, 3>(ctx, tx, tg, tu, n_rows, k_in, I / BN, n_mg, ep, 1, partial_bytes);
-        else
-            e = m_tiles == 1 ? run_gemm<EPI_GATEUP, 1, 2, 64, 6>(ctx, tx, tg, tu, n_rows, k_in, I / 64, 1, ep, 1, partial_bytes)
-                             : run_gemm<EPI_GATEUP, 2, 2, 64, 4>(ctx, tx, tg, tu, n_rows, k_in, I / 64, n_mg, ep, 1, partial_bytes);
-        if (e != cudaSuccess) return e;
-    } else if (m_tiles == 2 && bn_gu == BN && ks1 == 4 &&
-               splitk_clusters_fit<EPI_CGATEUP, 2, 2, BN, 3, 4>(ctx, I / BN)) {
+    if (m_tiles == 2 && bn_gu == BN && ks1 == 4 && I / BN * 4 >= kMinClusterCtas &&
+        splitk_clusters_fit<EPI_CGATEUP, 2, 2, BN, 3, 4>(ctx, I / BN)) {
         e = run_gemm<EPI_CGATEUP, 2, 2, BN, 3, 4>(ctx, tx, tg, tu, n_rows, k_in, I / BN, 1, ep, 4);
-        if (e != cudaSuccess) return e;
+    } else if (m_tiles > 1 && bn_gu == BN && ks1 == 1 && I / BN * n_mg > ctx.num_sms) {
+        e = run_gemm<EPI_GATEUP, 2, 2, BN, 3>(ctx, tx, tg, tu, n_rows, k_in, I / BN, n_mg, ep, 1, partial_bytes);
+    } else if (ks1 == 1) {
+        e = m_tiles == 1 ? run_gemm_var<EPI_GATEUP, 1, 2>(ctx, tx, w_gate, w_up, I, n_rows, k_in, 1, 1, ep)
+                         : run_gemm_var<EPI_GATEUP, 2, 2>(ctx, tx, w_gate, w_up, I, n_rows, k_in, n_mg, 1, ep);
     } else {
-        if (bn_gu == BN)
-            e = m_tiles == 1 ? run_gemm<EPI_PARTIAL, 1, 2, BN, 4>(ctx, tx, tg, tu, n_rows, k_in, I / BN, 1, ep, ks1)
-                             : run_gemm<EPI_PARTIAL, 2, 2, BN, 3>(ctx, tx, tg, tu, n_rows, k_in, I / BN, n_mg, ep, ks1);
-        else
-            e = m_tiles == 1 ? run_gemm<EPI_PARTIAL, 1, 2, 64, 6>(ctx, tx, tg, tu, n_rows, k_in, I / 64, 1, ep, ks1)
-                             : run_gemm<EPI_PARTIAL, 2, 2, 64, 4>(ctx, tx, tg, tu, n_rows, k_in, I / 64, n_mg, ep, ks1);
-        if (e != cudaSuccess) return e;
-        e = launch_swiglu_reduce(ctx, partial, ks1, n_rows, I, static_cast<__nv_bfloat16*>(A));
-        if (e != cudaSuccess) return e;
+        e = m_tiles == 1 ? run_gemm_var<EPI_PARTIAL, 1, 2>(ctx, tx, w_gate, w_up, I, n_rows, k_in, 1, ks1, ep)
+                         : run_gemm_var<EPI_PARTIAL, 2, 2>(ctx, tx, w_gate, w_up, I, n_rows, k_in, n_mg, ks1, ep);
+        if (e == cudaSuccess) e = launch_swiglu_reduce(ctx, partial, ks1, n_rows, I, static_cast<__nv_bfloat16*>(A));
     }
+    if (e != cudaSuccess) return e;
 
     // ---- down + residual: h' = h + A Wd^T
-    return run_residual_gemm(ctx, ta, td, I, hidden, n_rows, d, R, M, gamma, h_prime, partial, partial_bytes);
+    return run_residual_gemm(ctx, ta, w_down, I, hidden, n_rows, d, R, M, gamma, h_prime, partial, partial_bytes);
 }
 
 cudaError_t launch_linear_tc(const Ctx& ctx, const void* X, const void* w_lin, const void* hidden, int n_rows, int d,
                              int R, int M, int gamma, void* h_prime, float* partial, size_t partial_bytes) {
     if (n_rows <= 0) return cudaSuccess;
-    const int bn = d % 128 == 0 ? 128 : 64;
-    CUtensorMap tx, tw;
-    cudaError_t e = make_tmap(&tx, X, 2 * d, n_rows, kBK, kBM);
-    if (e == cudaSuccess) e = make_tmap(&tw, w_lin, 2 * d, d, kBK, bn);
+    CUtensorMap tx;
+    const cudaError_t e = make_tmap(&tx, X, 2 * d, n_rows, kBK, kBM);
     if (e != cudaSuccess) return e;
-    return run_residual_gemm(ctx, tx, tw, 2 * d, hidden, n_rows, d, R, M, gamma, h_prime, partial, partial_bytes);
+    return run_residual_gemm(ctx, tx, w_lin, 2 * d, hidden, n_rows, d, R, M, gamma, h_prime, partial, partial_bytes);
 }
 
 }  // namespace tf
