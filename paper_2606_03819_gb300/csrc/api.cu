@@ -28,7 +28,6 @@ namespace {
 using namespace tf;
 
 constexpr size_t kAlign = 256;
-constexpr size_t kMaxMergeSmem = 220 * 1024;
 
 size_t up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 

@@ -18,6 +18,7 @@ constexpr int kMaxM = 64;           // largest M (the builder tests membership w
 constexpr int kMaxB = 1023;         // largest draft budget
 constexpr int kMaxGamma = 64;
 constexpr int kMergeExpandChunks = 64;     // chunks a merge may recompute exactly
+constexpr size_t kMaxMergeSmem = 220 * 1024;   // dynamic shared memory of a merge CTA
 constexpr int kMaxKSplits = 4;        // split-K factor of the approximator GEMMs (workspace sized for it)
 // Counters of the approximator GEMMs' tail split (K-chunks of the units of a last, partial round),
 // kept in the workspace right after the status word and zeroed by the gather of every call.

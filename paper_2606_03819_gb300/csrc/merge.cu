@@ -2,17 +2,21 @@
 // log-softmax + top-k of every stage-2 row).
 //
 // One CTA per row. The CTA
-//   1. combines the row's half-block (max, sum of exp) pairs into its log-sum-exp and forms one
-//      key (value desc, id asc) per half block from the half's best entry;
-//   2. finds theta0, the k-th largest half-block key. Exactly the k halves at or above it can
-//      hold members of the top k (every key elsewhere is below its half's best, hence below
-//      theta0). Their chunks' two largest entries at or above theta0 are the candidates; the
-//      k-th largest candidate key comes from a radix select over 64-bit keys;
-//   3. certifies the result: a chunk whose third-largest value reaches the k-th candidate may
-//      hide further members of the top k. Those chunks' 32 logits are recomputed exactly from
-//      lm_head and x (in rounds of at most 64 chunks), replace the chunk's two candidates, and
-//      the selection is redone;
-//   4. writes the k winners sorted, as (id, logit - LSE).
+//   1. combines the row's half-block (max, sum of exp) pairs into its log-sum-exp;
+//   2. keeps the halves whose best entry can be among the k best: a histogram of the halves' best
+//      values over 256 equal-width buckets gives the bucket of the k-th, and the halves in it or
+//      above are kept (k and a few: every other half's best, hence all of its entries, is below k
+//      other values). Their chunks' two largest entries in those buckets are the candidates;
+//   3. certifies: a kept chunk whose third-largest value reaches the k-th candidate may hide
+//      further members of the top k. Those chunks' 32 logits are recomputed exactly from lm_head
+//      and x (in rounds of at most 64 chunks), replace the chunk's two candidates, and the
+//      selection is redone;
+//   4. writes the k winners sorted, as (id, logit - LSE): the candidates' ranks, by counting.
+// What bounds it is the chain of loads and block barriers, eight in the usual case (an exact k-th
+// half and an exact k-th candidate by two further selections took 21): on GB300, k = 32, 3872 rows
+// 143 -> 90 us, 512 rows 21 -> 12.5; k = 64, 1928 rows 81 -> 60, 241 rows 13.7 -> 10.8. The selections
+// remain for rows with equal or non-finite values, crowded buckets, fewer halves than k, more
+// halves than registers hold, or more candidates than are worth counting.
 // The result is the exact top-k of the full vocabulary whatever the input; a recompute needs
 // three members of the top k in one 32-column chunk (about one row in 500 on random data).
 #include <math.h>
@@ -22,6 +26,9 @@
 namespace tf {
 namespace {
 
+constexpr int kRegHalves = 8;     // half summaries a thread can hold in registers (V <= 262144)
+constexpr int kRankCands = 512;   // candidates that are ranked by counting
+constexpr int kKeepSlack = 64;    // room for halves beyond the k-th in its bucket
 constexpr int kThreads = 256;   // 512 or more: two CTAs no longer fit an SM, so 241 rows take two waves
 
 __device__ __forceinline__ void lse_combine(float& m, float& s, float m2, float s2) {
@@ -103,7 +110,7 @@ __device__ unsigned long long block_kth_largest(const unsigned long long* keys, 
 // Shared state of block_kth_largest_fast.
 constexpr int kBuckets = 256;
 constexpr int kCollectCap = 256;
-struct SelectSmem {
+struct alignas(16) SelectSmem {
     int hist[kBuckets];
     unsigned long long coll[kCollectCap];
     float wmax[kThreads / 32], wmin[kThreads / 32];
@@ -272,20 +279,20 @@ __device__ __forceinline__ float dot_row(const float* w, const float* xs, int d,
     return acc;
 }
 
-// Shared-memory layout of one merge CTA (dynamic part), for a top-k of k.
+// Shared-memory layout of one merge CTA (dynamic part), for a top-k of k and room for kc >= k halves.
 struct MergeSmem {
     unsigned long long* hkey;   // [n_halves] best key of every half block (0 = empty)
-    unsigned long long* cand;   // [2 * 4k + kMergeExpandChunks * kChunk]
+    unsigned long long* cand;   // [2 * 4kc + kMergeExpandChunks * kChunk]
     unsigned long long* cand2;  // the same size: the compacted set of the next round
     unsigned long long* sel;    // [k] the winners
-    float* c3;                  // [4k] third value of each kept chunk (bound on the rest)
-    int* cbase;                 // [4k] first vocabulary id of each kept chunk
-    int* chalf;                 // [k] the halves at or above theta0
-    uint8_t* expanded;          // [4k] chunk recomputed
+    float* c3;                  // [4kc] third value of each kept chunk (bound on the rest)
+    int* cbase;                 // [4kc] first vocabulary id of each kept chunk
+    int* chalf;                 // [kc] the halves kept
+    uint8_t* expanded;          // [4kc] chunk recomputed
     float* xs;                  // [d] x of the row in fp32, staged only for a recompute
 };
-__host__ __device__ inline size_t merge_layout(int n_tiles, int d, int k, uint8_t* base, MergeSmem* m) {
-    const size_t detail = static_cast<size_t>(k) * (kChunks / 2);   // chunks of the k halves kept
+__host__ __device__ inline size_t merge_layout(int n_tiles, int d, int k, int kc, uint8_t* base, MergeSmem* m) {
+    const size_t detail = static_cast<size_t>(kc) * (kChunks / 2);  // chunks of the halves kept
     size_t off = 0;
     auto take = [&](size_t bytes) {
         uint8_t* p = base ? base + off : nullptr;
@@ -298,7 +305,7 @@ __host__ __device__ inline size_t merge_layout(int n_tiles, int d, int k, uint8_
     uint8_t* se = take(static_cast<size_t>(k) * 8);
     uint8_t* c3 = take(detail * 4);
     uint8_t* cb = take(detail * 4);
-    uint8_t* ch = take(static_cast<size_t>(k) * 4);
+    uint8_t* ch = take(static_cast<size_t>(kc) * 4);
     uint8_t* ex = take(detail);
     uint8_t* xs = take(static_cast<size_t>(d) * 4);
     if (m) {
@@ -316,8 +323,8 @@ __host__ __device__ inline size_t merge_layout(int n_tiles, int d, int k, uint8_
 }
 
 template <typename T>
-__global__ void __launch_bounds__(kThreads) lmhead_merge_kernel(Partials partials, int n_rows, int n_tiles, int V,
-                                                                int d, int k, float inv_temp,
+__global__ void __launch_bounds__(kThreads, 2) lmhead_merge_kernel(Partials partials, int n_rows, int n_tiles, int V,
+                                                                int d, int k, int kc, float inv_temp,
                                                                 const T* __restrict__ lm_head,
                                                                 const T* __restrict__ x, int32_t* __restrict__ out_ids,
                                                                 float* __restrict__ out_logp, int* status) {
@@ -325,11 +332,13 @@ __global__ void __launch_bounds__(kThreads) lmhead_merge_kernel(Partials partial
     pdl_wait();
     extern __shared__ __align__(16) uint8_t dsm[];
     MergeSmem S;
-    merge_layout(n_tiles, d, k, dsm, &S);
-    const int n_detail = k * (kChunks / 2);
+    merge_layout(n_tiles, d, k, kc, dsm, &S);
+    const int n_detail = kc * (kChunks / 2);
     __shared__ int hist[256];
     __shared__ SelectSmem SB;
     __shared__ float red_m[kThreads / 32], red_s[kThreads / 32];
+    __shared__ uint32_t wkmax[kThreads / 32], wkmin[kThreads / 32];
+    __shared__ int wcnt[kThreads / 32];
     __shared__ int sel_info[3], n_flag, flag_list[kMergeExpandChunks], n_cand, n_next, n_sel, n_valid, n_chalf;
     __shared__ unsigned long long found;
     __shared__ float zbuf[kMergeExpandChunks * kChunk];
@@ -344,96 +353,258 @@ __global__ void __launch_bounds__(kThreads) lmhead_merge_kernel(Partials partial
         n_chalf = 0;
     }
 
-    // 1. half-block summaries (strided by n_rows, eight loads in flight per thread): the row's
-    //    log-sum-exp and one key per half
-    float m = -INFINITY, s = 0.0f;
-    int my_valid = 0;
-    {
-        const float4* src = partials.halves + row;
-        const size_t stride = static_cast<size_t>(partials.n_rows);
-        for (int base = tid; base < nh; base += 8 * kThreads) {
-            float4 v[8];
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                const int i = base + j * kThreads;
-                if (i < nh) v[j] = src[static_cast<size_t>(i) * stride];
-            }
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                const int i = base + j * kThreads;
-                if (i >= nh) break;
-                const int id = __float_as_int(v[j].w);
-                unsigned long long key = 0ull;
-                if (id >= 0) {
-                    lse_combine(m, s, v[j].x, v[j].y);
-                    key = cand_key(v[j].z, id);
-                    ++my_valid;
-                }
-                S.hkey[i] = key;
-            }
-        }
-    }
     for (int i = tid; i < n_detail; i += kThreads) S.expanded[i] = 0;
+    const float4* half_of = partials.halves + row;   // half i at half_of[i * n_rows]
+    const size_t half_stride = static_cast<size_t>(partials.n_rows);
+    int nch = 0;                 // halves kept
+    bool kept = false;
+    // The usual case (up to kRegHalves halves per thread, finite values): the summaries stay in
+    // registers, one histogram of the halves' best values gives the bucket of the k-th, and every
+    // half in that bucket or above is kept (a few more than k: unless they exceed the room for them,
+    // the exact rank inside the bucket is not needed).
+    if (nh <= kRegHalves * kThreads) {
+        float4 v[kRegHalves];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const float m2 = __shfl_xor_sync(0xffffffffu, m, o);
-        const float s2 = __shfl_xor_sync(0xffffffffu, s, o);
-        lse_combine(m, s, m2, s2);
-    }
-    if (lane == 0) {
-        red_m[warp] = m;
-        red_s[warp] = s;
-    }
-    __syncthreads();
-    atomicAdd(&n_valid, my_valid);
-    __syncthreads();
-    if (warp == 0) {
-        float M = lane < kThreads / 32 ? red_m[lane] : -INFINITY;
-        float Ssum = lane < kThreads / 32 ? red_s[lane] : 0.0f;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const float m2 = __shfl_xor_sync(0xffffffffu, M, o);
-            const float s2 = __shfl_xor_sync(0xffffffffu, Ssum, o);
-            lse_combine(M, Ssum, m2, s2);
+        for (int j = 0; j < kRegHalves; ++j) {
+            const int i = tid + j * kThreads;
+            v[j] = i < nh ? half_of[static_cast<size_t>(i) * half_stride] : make_float4(0.0f, 0.0f, 0.0f, __int_as_float(-1));
         }
+        uint32_t kmax = 0u, kmin = 0xffffffffu;
+        int cnt = 0;
+#pragma unroll
+        for (int j = 0; j < kRegHalves; ++j)
+            if (__float_as_int(v[j].w) >= 0) {
+                const uint32_t key = float_key(v[j].z);
+                kmax = max(kmax, key);
+                kmin = min(kmin, key);
+                ++cnt;
+            }
+        kmax = __reduce_max_sync(0xffffffffu, kmax);
+        kmin = __reduce_min_sync(0xffffffffu, kmin);
+        cnt = __reduce_add_sync(0xffffffffu, cnt);
         if (lane == 0) {
-            const float lse = M + logf(Ssum);
-            lse_s = lse;
-            if (!isfinite(lse)) set_status(status, TF_DEV_NONFINITE);
+            wkmax[warp] = kmax;
+            wkmin[warp] = kmin;
+            wcnt[warp] = cnt;
         }
+        SB.hist[tid] = 0;
+        __syncthreads();
+        cnt = 0;
+#pragma unroll
+        for (int w = 0; w < kThreads / 32; ++w) {
+            kmax = max(kmax, wkmax[w]);
+            kmin = min(kmin, wkmin[w]);
+            cnt += wcnt[w];
+        }
+        const float M = key_float(kmax), lo = key_float(kmin), range = M - lo;
+        if (cnt >= k && range > 0.0f && isfinite(range) && isfinite(M)) {     // (uniform)
+            const float scale = static_cast<float>(kBuckets) / range;
+            auto bucket_of = [&](float x) {
+                const int b = static_cast<int>((x - lo) * scale);
+                return b < 0 ? 0 : b >= kBuckets ? kBuckets - 1 : b;
+            };
+            float s = 0.0f;
+#pragma unroll
+            for (int j = 0; j < kRegHalves; ++j)
+                if (__float_as_int(v[j].w) >= 0) {
+                    atomicAdd(&SB.hist[bucket_of(v[j].z)], 1);
+                    s += v[j].y * __expf(v[j].x - M);
+                }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+            if (lane == 0) red_s[warp] = s;
+            __syncthreads();
+            if (warp == 0) {
+                // lane l holds buckets 8l .. 8l + 7; inclusive suffix sums over lanes
+                const int4 h0 = reinterpret_cast<const int4*>(SB.hist)[2 * lane], h1 = reinterpret_cast<const int4*>(SB.hist)[2 * lane + 1];
+                const int local[8] = {h0.x, h0.y, h0.z, h0.w, h1.x, h1.y, h1.z, h1.w};
+                int incl = 0;
+#pragma unroll
+                for (int b = 0; b < 8; ++b) incl += local[b];
+                const int sum = incl;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int u = __shfl_down_sync(0xffffffffu, incl, o);
+                    if (lane + o < 32) incl += u;
+                }
+                const int excl = incl - sum;
+                if (excl < k && k <= incl) {
+                    int c = excl, bk = 7;
+#pragma unroll
+                    for (int b = 7; b >= 0; --b)
+                        if (c < k) {
+                            c += local[b];
+                            bk = b;
+                        }
+                    SB.bucket = lane * 8 + bk;
+                    SB.count = c;                        // halves in that bucket or above
+                }
+            } else if (tid == 32) {
+                float t = 0.0f;
+                for (int w = 0; w < kThreads / 32; ++w) t += red_s[w];
+                const float lse = M + logf(t);
+                lse_s = lse;
+                if (!isfinite(lse)) set_status(status, TF_DEV_NONFINITE);
+            }
+            __syncthreads();
+            const int bk = SB.bucket;
+            nch = SB.count;
+            kept = nch <= kc;                            // (uniform)
+            if (kept) {
+#pragma unroll
+                for (int j = 0; j < kRegHalves; ++j)
+                    if (__float_as_int(v[j].w) >= 0 && bucket_of(v[j].z) >= bk) S.chalf[atomicAdd(&n_chalf, 1)] = tid + j * kThreads;
+                __syncthreads();
+                // their chunks: the two largest entries in those buckets become candidates
+                for (int i = tid; i < nch * (kChunks / 2); i += kThreads) {
+                    const int h = S.chalf[i >> 2];
+                    const int tile = h >> 1, chunk = (h & 1) * (kChunks / 2) + (i & 3);
+                    const float4 q = partials.chunks[partials.chunk_at(tile, chunk, row)];
+                    const int v0 = tile * kBlockV + chunk * kChunk;
+                    const int ids = __float_as_int(q.w);
+                    S.cbase[i] = v0;
+                    S.c3[i] = q.z;
+                    if (q.x > -INFINITY && bucket_of(q.x) >= bk) S.cand[atomicAdd(&n_cand, 1)] = cand_key(q.x, v0 + (ids & 255));
+                    if (q.y > -INFINITY && bucket_of(q.y) >= bk) S.cand[atomicAdd(&n_cand, 1)] = cand_key(q.y, v0 + ((ids >> 8) & 255));
+                }
+                __syncthreads();
+                // Few candidates: each one's rank by counting, which sorts the winners as well. Done
+                // unless a kept chunk's third value reaches the k-th.
+                const int nc = n_cand;
+                if (nc >= k && nc <= kRankCands) {
+                    unsigned long long mine[kRankCands / kThreads];
+                    int rank[kRankCands / kThreads];
+#pragma unroll
+                    for (int j = 0; j < kRankCands / kThreads; ++j) {
+                        const int i = tid + j * kThreads;
+                        mine[j] = i < nc ? S.cand[i] : 0ull;
+                        rank[j] = 0;
+                    }
+                    if (nc <= kThreads) {
+                        if (tid < nc) {
+#pragma unroll 8
+                            for (int i = 0; i < nc; ++i) rank[0] += S.cand[i] > mine[0] ? 1 : 0;
+                        }
+                    } else {
+#pragma unroll 4
+                        for (int i = 0; i < nc; ++i) {
+                            const unsigned long long key = S.cand[i];
+#pragma unroll
+                            for (int j = 0; j < kRankCands / kThreads; ++j) rank[j] += key > mine[j] ? 1 : 0;
+                        }
+                    }
+#pragma unroll
+                    for (int j = 0; j < kRankCands / kThreads; ++j)
+                        if (mine[j] != 0ull && rank[j] == k - 1) found = mine[j];
+                    __syncthreads();
+                    const float tval = key_value(found);
+                    bool hide = false;
+                    for (int i = tid; i < nch * (kChunks / 2); i += kThreads) hide = hide || S.c3[i] >= tval;
+                    if (!__syncthreads_or(hide ? 1 : 0)) {
+                        const float lse = lse_s;
+#pragma unroll
+                        for (int j = 0; j < kRankCands / kThreads; ++j)
+                            if (mine[j] != 0ull && rank[j] < k) {
+                                out_ids[static_cast<size_t>(row) * k + rank[j]] = key_id(mine[j]);
+                                out_logp[static_cast<size_t>(row) * k + rank[j]] = key_value(mine[j]) - lse;
+                            }
+                        return;
+                    }
+                }
+            }
+        }
+        if (!kept) __syncthreads();                      // the shared words above are reused below
     }
 
-    // 2. theta0 and the halves at or above it (at most k: the keys are distinct)
-    const unsigned long long theta0 =
-        n_valid >= k ? block_kth_largest_fast(S.hkey, nh, k, SB, hist, sel_info, &found) : 0ull;
-    for (int i = tid; i < nh; i += kThreads) {
-        const unsigned long long key = S.hkey[i];
-        if (key != 0ull && key >= theta0) {
-            const int slot = atomicAdd(&n_chalf, 1);
-            if (slot < k) S.chalf[slot] = i;
+    if (!kept) {
+        // 1. half-block summaries (strided by n_rows, eight loads in flight per thread): the row's
+        //    log-sum-exp and one key per half
+        float m = -INFINITY, s = 0.0f;
+        int my_valid = 0;
+        {
+            for (int base = tid; base < nh; base += 8 * kThreads) {
+                float4 v[8];
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    const int i = base + j * kThreads;
+                    if (i < nh) v[j] = half_of[static_cast<size_t>(i) * half_stride];
+                }
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    const int i = base + j * kThreads;
+                    if (i >= nh) break;
+                    const int id = __float_as_int(v[j].w);
+                    unsigned long long key = 0ull;
+                    if (id >= 0) {
+                        lse_combine(m, s, v[j].x, v[j].y);
+                        key = cand_key(v[j].z, id);
+                        ++my_valid;
+                    }
+                    S.hkey[i] = key;
+                }
+            }
         }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const float m2 = __shfl_xor_sync(0xffffffffu, m, o);
+            const float s2 = __shfl_xor_sync(0xffffffffu, s, o);
+            lse_combine(m, s, m2, s2);
+        }
+        if (lane == 0) {
+            red_m[warp] = m;
+            red_s[warp] = s;
+        }
+        __syncthreads();
+        atomicAdd(&n_valid, my_valid);
+        __syncthreads();
+        if (warp == 0) {
+            float M = lane < kThreads / 32 ? red_m[lane] : -INFINITY;
+            float Ssum = lane < kThreads / 32 ? red_s[lane] : 0.0f;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                const float m2 = __shfl_xor_sync(0xffffffffu, M, o);
+                const float s2 = __shfl_xor_sync(0xffffffffu, Ssum, o);
+                lse_combine(M, Ssum, m2, s2);
+            }
+            if (lane == 0) {
+                const float lse = M + logf(Ssum);
+                lse_s = lse;
+                if (!isfinite(lse)) set_status(status, TF_DEV_NONFINITE);
+            }
+        }
+
+        // 2. theta0 and the halves at or above it (at most k: the keys are distinct)
+        const unsigned long long theta0 =
+            n_valid >= k ? block_kth_largest_fast(S.hkey, nh, k, SB, hist, sel_info, &found) : 0ull;
+        for (int i = tid; i < nh; i += kThreads) {
+            const unsigned long long key = S.hkey[i];
+            if (key != 0ull && key >= theta0) {
+                const int slot = atomicAdd(&n_chalf, 1);
+                if (slot < k) S.chalf[slot] = i;
+            }
+        }
+        __syncthreads();
+        nch = min(n_chalf, k);
+        // their chunks: the two largest entries at or above theta0 become candidates
+        for (int i = tid; i < nch * (kChunks / 2); i += kThreads) {
+            const int h = S.chalf[i >> 2];
+            const int tile = h >> 1, chunk = (h & 1) * (kChunks / 2) + (i & 3);
+            const float4 q = partials.chunks[partials.chunk_at(tile, chunk, row)];
+            const int v0 = tile * kBlockV + chunk * kChunk;
+            const int ids = __float_as_int(q.w);
+            S.cbase[i] = v0;
+            S.c3[i] = q.z;
+            if (q.x > -INFINITY) {
+                const unsigned long long key = cand_key(q.x, v0 + (ids & 255));
+                if (key >= theta0) S.cand[atomicAdd(&n_cand, 1)] = key;
+            }
+            if (q.y > -INFINITY) {
+                const unsigned long long key = cand_key(q.y, v0 + ((ids >> 8) & 255));
+                if (key >= theta0) S.cand[atomicAdd(&n_cand, 1)] = key;
+            }
+        }
+        __syncthreads();
     }
-    __syncthreads();
-    const int nch = min(n_chalf, k);
-    // their chunks: the two largest entries at or above theta0 become candidates
-    for (int i = tid; i < nch * (kChunks / 2); i += kThreads) {
-        const int h = S.chalf[i >> 2];
-        const int tile = h >> 1, chunk = (h & 1) * (kChunks / 2) + (i & 3);
-        const float4 q = partials.chunks[partials.chunk_at(tile, chunk, row)];
-        const int v0 = tile * kBlockV + chunk * kChunk;
-        const int ids = __float_as_int(q.w);
-        S.cbase[i] = v0;
-        S.c3[i] = q.z;
-        if (q.x > -INFINITY) {
-            const unsigned long long key = cand_key(q.x, v0 + (ids & 255));
-            if (key >= theta0) S.cand[atomicAdd(&n_cand, 1)] = key;
-        }
-        if (q.y > -INFINITY) {
-            const unsigned long long key = cand_key(q.y, v0 + ((ids >> 8) & 255));
-            if (key >= theta0) S.cand[atomicAdd(&n_cand, 1)] = key;
-        }
-    }
-    __syncthreads();
 
     // 3. select; a kept chunk whose third value reaches the k-th candidate may hide members of
     //    the top k, so its 32 logits are recomputed exactly and the selection is redone. Chunks
@@ -538,19 +709,21 @@ __global__ void __launch_bounds__(kThreads) lmhead_merge_kernel(Partials partial
 
 }  // namespace
 
-size_t merge_smem_bytes(int n_tiles, int d, int k) { return merge_layout(n_tiles, d, k, nullptr, nullptr); }
+size_t merge_smem_bytes(int n_tiles, int d, int k) { return merge_layout(n_tiles, d, k, k, nullptr, nullptr); }
 
 cudaError_t launch_lmhead_merge(const Ctx& ctx, int dtype, Partials partials, int n_rows, int V, int d, int k,
                                 float inv_temp, const void* lm_head, const void* x, int32_t* out_ids,
                                 float* out_logp) {
     if (n_rows <= 0) return cudaSuccess;
     const int n_tiles = (V + kBlockV - 1) / kBlockV;
-    const size_t smem = merge_smem_bytes(n_tiles, d, k);
+    // room for kKeepSlack halves more than k where shared memory has it
+    const int kc = merge_layout(n_tiles, d, k, k + kKeepSlack, nullptr, nullptr) <= kMaxMergeSmem ? k + kKeepSlack : k;
+    const size_t smem = merge_layout(n_tiles, d, k, kc, nullptr, nullptr);
     if (dtype == TF_BF16) {
         auto kern = lmhead_merge_kernel<__nv_bfloat16>;
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
         if (e != cudaSuccess) return e;
-        e = launch_pdl(kern, dim3(n_rows), dim3(kThreads), smem, ctx.stream, partials, n_rows, n_tiles, V, d, k,
+        e = launch_pdl(kern, dim3(n_rows), dim3(kThreads), smem, ctx.stream, partials, n_rows, n_tiles, V, d, k, kc,
                        inv_temp, static_cast<const __nv_bfloat16*>(lm_head), static_cast<const __nv_bfloat16*>(x),
                        out_ids, out_logp, ctx.status);
         if (e != cudaSuccess) return e;
@@ -558,7 +731,7 @@ cudaError_t launch_lmhead_merge(const Ctx& ctx, int dtype, Partials partials, in
         auto kern = lmhead_merge_kernel<float>;
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
         if (e != cudaSuccess) return e;
-        e = launch_pdl(kern, dim3(n_rows), dim3(kThreads), smem, ctx.stream, partials, n_rows, n_tiles, V, d, k,
+        e = launch_pdl(kern, dim3(n_rows), dim3(kThreads), smem, ctx.stream, partials, n_rows, n_tiles, V, d, k, kc,
                        inv_temp, static_cast<const float*>(lm_head), static_cast<const float*>(x), out_ids, out_logp,
                        ctx.status);
         if (e != cudaSuccess) return e;

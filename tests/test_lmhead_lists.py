@@ -1,0 +1,61 @@
+"""The LM head's lists (tf_lmhead_partials, tf_lmhead_merge) against a full fp64 log-softmax, on rows
+that take each way through the merge: a few halves in the k-th's bucket, a bucket too crowded to keep
+(one logit far above all others), equal logits throughout (ids in order), fewer half blocks than k,
+more halves than fit in registers, and k from 1 to 512."""
+import numpy as np
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+CASES = [
+    # V, d, k, dtype, rows
+    (20000, 128, 64, "bf16", "plain"),
+    (20000, 128, 1, "bf16", "plain"),
+    (20000, 64, 512, "bf16", "plain"),
+    (20000, 128, 64, "f32", "plain"),
+    (9001, 64, 32, "bf16", "outlier"),       # every other half in the lowest bucket
+    (9001, 64, 32, "f32", "outlier"),
+    (5000, 64, 40, "bf16", "equal"),
+    (1500, 64, 64, "bf16", "plain"),         # 12 half blocks
+    (270001, 64, 48, "bf16", "plain"),       # 2110 half blocks
+]
+
+
+@pytest.mark.parametrize("V,d,k,dtype,rows", CASES)
+def test_lists_equal_a_full_sort(V, d, k, dtype, rows):
+    from paper_2606_03819_gb300 import Dims
+    from paper_2606_03819_gb300 import binding as B
+    dt = torch.bfloat16 if dtype == "bf16" else torch.float32
+    g = torch.Generator().manual_seed(V + k)
+    n = 21
+    W = torch.randn(V, d, generator=g)
+    x = torch.randn(n, d, generator=g) * 3.0 / d ** 0.5
+    if rows == "outlier":
+        W[V // 2] = 200.0 * torch.sign(x.sum(0))
+        x = x.abs() * torch.sign(W[V // 2])
+    elif rows == "equal":
+        x.zero_()
+    W, x = W.to(dt).cuda(), x.to(dt).cuda()
+    dims = Dims(1, d, V, 64, n, 1, k, 8, dtype=dtype, mode="marginal")
+    ws = B.alloc_workspace(dims)
+    ids = torch.empty(n, k, dtype=torch.int32, device="cuda")
+    logp = torch.empty(n, k, device="cuda")
+    B.tf_status_reset(ws)
+    B.tf_lmhead_partials(dims, W, x, n, ws)
+    B.tf_lmhead_merge(dims, W, x, n, k, ids, logp, ws)
+    assert B.tf_status_read(ws) & ~B.TF_DEV_RECOMPUTED == 0
+    z = x.double() @ W.double().t()
+    lp = torch.log_softmax(z, 1)
+    ids, logp = ids.cpu().numpy(), logp.double().cpu().numpy()
+    if rows == "equal":
+        np.testing.assert_array_equal(ids, np.arange(k)[None].repeat(n, 0))
+        np.testing.assert_allclose(logp, -np.log(V), atol=1e-5)
+        return
+    # fp32 sums of d products of size up to |z|: far below 1e-3 (relative 1e-5 for the outlier's 1e3)
+    tol = 1e-3 * max(1.0, float(z.abs().max()) / 100)
+    want = lp.topk(k, dim=1).values.cpu().numpy()
+    np.testing.assert_allclose(logp, want, atol=tol)
+    np.testing.assert_allclose(lp.cpu().numpy()[np.arange(n)[:, None], ids], logp, atol=tol)
+    for r in range(n):
+        assert len(set(ids[r].tolist())) == k
