@@ -123,7 +123,8 @@ Layout layout(const Dims& D) {
     if (D.dtype == TF_BF16) {
         const size_t partial = static_cast<size_t>(kMaxKSplits) * rows2 *
                                (2 * static_cast<size_t>(D.I) > static_cast<size_t>(D.d) ? 2 * D.I : D.d) * 4;
-        const size_t xg = std::max(splitk_exchange_bytes(D.I, 2), splitk_exchange_bytes(D.d, 1));
+        const int r = static_cast<int>(rows2);
+        const size_t xg = std::max(splitk_exchange_bytes(D.I, 2, r), splitk_exchange_bytes(D.d, 1, r));
         L.kpart_bytes = rows2 > 0 ? std::max(partial, xg) : 0;
         L.kpart = take(L.kpart_bytes);
     } else {

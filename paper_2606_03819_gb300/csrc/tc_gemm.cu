@@ -170,14 +170,15 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant
                const __grid_constant__ CUtensorMap tmap_w1, int n_rows, int K, int n_ntiles,
                int n_mgroups, int k_splits, int w_stream_once, EpiParams ep, int* status) {
     // Two kinds of cluster: kPair, a CTA pair on two M-tiles sharing each weight tile through
-    // cta_group::2 MMAs; kSplitK, CL CTAs on the CL K-ranges of one output tile (one tile per
+    // cta_group::2 MMAs; kSplitK, up to CL CTAs on the K-ranges of one output tile (one tile per
     // cluster), whose accumulators are summed through distributed shared memory.
     constexpr bool kSplitK = EPI == EPI_CGATEUP || EPI == EPI_CDOWN;
     constexpr bool kPair = CL > 1 && !kSplitK;
     using C = TileCfg<MT, NB, BN, STAGES, kPair, VAR>;
     static_assert(CL == 1 || kSplitK || (CL == 2 && MT == 1), "a CTA of a pair holds one M-tile");
-    static_assert(!kSplitK || (CL == 4 && MT == 2 && BN == 128), "cluster split-K: 4 K-ranges of a 256 x 128 tile");
-    static_assert(!VAR || (CL == 1 && EPI != EPI_LMHEAD), "variable width: single CTAs of the approximator");
+    static_assert(!kSplitK || (CL == 4 && kMaxKSplits == 4 && (VAR || (MT == 2 && BN == 128))), "cluster split-K");
+    constexpr bool kShare = kSplitK && VAR && MT == 1;   // both epilogue groups work on one accumulator
+    static_assert(!VAR || (!kPair && EPI != EPI_LMHEAD), "variable width: single CTAs and K-splitting clusters");
     pdl_trigger();
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>(
@@ -475,8 +476,8 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant
             }
         };
         for (int u = cid; u < n_items; u += ncl, ++kl) {
-            if (MT == 1 && (kl & 1) != g) continue;
-            if (!ptx::mbar_wait(&tfull[g], use & 1u, abort_flag, wait_ns)) {
+            if (MT == 1 && !kShare && (kl & 1) != g) continue;
+            if (!ptx::mbar_wait(&tfull[kShare ? 0 : g], use & 1u, abort_flag, wait_ns)) {
                 *abort_flag = 1;
                 set_status(status, TF_DEV_TIMEOUT);
                 break;
@@ -486,8 +487,8 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant
             const Item itm = item_of(u);
             const Unit w = itm.w;
             const int nt = w.nt;
-            const int row = ((w.mg * m_cl + m_rank) * MT + (MT == 2 ? g : 0)) * kBM + q * 32 + lane;
-            const uint32_t tb = tmem_base + 256u * g + (static_cast<uint32_t>(q * 32) << 16);
+            [[maybe_unused]] const int row = ((w.mg * m_cl + m_rank) * MT + (MT == 2 ? g : 0)) * kBM + q * 32 + lane;
+            [[maybe_unused]] const uint32_t tb = tmem_base + 256u * g + (static_cast<uint32_t>(q * 32) << 16);
 
             if (kTail && itm.chunk >= 0) {
                 // ---- a K-chunk of a tail unit: its partial sums to `partial`; the group whose
@@ -753,8 +754,8 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant
         }
     }
 
-    if constexpr (kSplitK) {
-        // ------------------------------------------------------------------ split-K sum
+    if constexpr (kSplitK && !VAR) {
+        // ------------------------------------------------------------------ split-K sum, 128 columns
         // The tile's output columns are owned in CL blocks of BN / CL: CTA o adds the CL partial
         // sums of block o in K-range order (the order of the split-K reduction kernels) and
         // applies the epilogue. Every CTA writes the blocks it does not own to the exchange area
@@ -857,6 +858,123 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant
         }
     }
 
+    if constexpr (kSplitK && VAR) {
+        // ------------------------------------------------------------------ split-K sum, any width
+        // The same with up to CL K-ranges, one or two M-tiles and columns owned in steps of 8; the
+        // exchange area is laid out [cluster][sender][16-byte unit][row].
+        const bool has_unit = cid < n_units;
+        const int e = warp - 2;
+        const int g = e / (kEpiWarps / 2), q = warp & 3, half = (e % (kEpiWarps / 2)) / 4;
+        // a warp's M-tile and its share of the column steps: two warps per row quarter and M-tile
+        // with two M-tiles, four with one
+        constexpr int kColWarps = kShare ? 4 : 2;
+        const int mt = kShare ? 0 : g, cw = kShare ? 2 * g + half : half;
+        const int r = mt * kBM + q * 32 + lane;          // tile row: TMEM slot mt, lane q * 32 + lane
+        const uint32_t tb = tmem_base + 256u * mt + (static_cast<uint32_t>(q * 32) << 16);
+        const int ks = k_splits, n8 = bn / 8;
+        const int o0 = n8 * crank / ks, o1 = n8 * (crank + 1) / ks;    // this CTA's column steps
+        float4* xchg = reinterpret_cast<float4*>(ep.partial);
+        auto at = [&](int sender, int nb, int c8, int f) {              // float4 f of step c8
+            return (static_cast<size_t>(cid * ks + sender) * (NB * n8 * 2) + (nb * n8 + c8) * 2 + f) * (MT * kBM) + r;
+        };
+        // (the epilogue warps waited for this CTA's accumulators in the loop above; warps whose rows are
+        // all padding have nothing to exchange)
+        const bool rows_on = warp >= 2 && has_unit && unit_of(cid).mg * MT * kBM + r - lane < n_rows;
+        if (rows_on) {
+            // four column steps per TMEM wait: the steps of the other owners, in order
+            const int others = n8 - (o1 - o0);
+#pragma unroll 1
+            for (int i = cw; i < others; i += 4 * kColWarps) {
+                int c8[4];
+#pragma unroll
+                for (int t = 0; t < 4; ++t) {
+                    const int j = i + t * kColWarps;
+                    c8[t] = j < others ? (j < o0 ? j : j + o1 - o0) : -1;
+                }
+#pragma unroll
+                for (int nb = 0; nb < NB; ++nb) {
+                    uint32_t ra[32];
+                    ptx::tmem_ld_8cols_nowait<0>(tb + nb * bn + 8 * c8[0], ra);
+                    ptx::tmem_ld_8cols_nowait<8>(tb + nb * bn + 8 * (c8[1] < 0 ? c8[0] : c8[1]), ra);
+                    ptx::tmem_ld_8cols_nowait<16>(tb + nb * bn + 8 * (c8[2] < 0 ? c8[0] : c8[2]), ra);
+                    ptx::tmem_ld_8cols_nowait<24>(tb + nb * bn + 8 * (c8[3] < 0 ? c8[0] : c8[3]), ra);
+                    ptx::tmem_wait_ld_regs(ra);
+#pragma unroll
+                    for (int t = 0; t < 4; ++t)
+                        if (c8[t] >= 0) {
+                            float4* dst = xchg + at(crank, nb, c8[t], 0);
+#pragma unroll
+                            for (int f = 0; f < 2; ++f)
+                                dst[f * (MT * kBM)] = make_float4(__uint_as_float(ra[8 * t + 4 * f]), __uint_as_float(ra[8 * t + 4 * f + 1]),
+                                                                  __uint_as_float(ra[8 * t + 4 * f + 2]), __uint_as_float(ra[8 * t + 4 * f + 3]));
+                        }
+                }
+            }
+        }
+        __syncwarp();
+        ptx::tc_fence_before();
+        ptx::cluster_sync();   // every column step is in the exchange area
+        ptx::tc_fence_after();
+        if (rows_on) {
+            const Unit w = unit_of(cid);
+            const int row = w.mg * MT * kBM + r;
+            int hid_row = 0;
+            if (EPI == EPI_CDOWN && row < n_rows) {
+                const int sq = row / ep.R, rr = row - sq * ep.R;
+                hid_row = sq * ep.gamma + stage2_hidden_index(rr, ep.M);
+            }
+            // the first step of this warp at or after o0
+#pragma unroll 1
+            for (int c8 = o0 + (cw + kColWarps - o0 % kColWarps) % kColWarps; c8 < o1; c8 += kColWarps) {
+                const int col = w.nt * bn + 8 * c8;
+                float4 in[CL][NB][2];
+#pragma unroll
+                for (int kx = 0; kx < CL; ++kx)
+#pragma unroll
+                    for (int nb = 0; nb < NB; ++nb)
+#pragma unroll
+                        for (int f = 0; f < 2; ++f)
+                            in[kx][nb][f] = kx < ks && kx != crank ? xchg[at(kx, nb, c8, f)] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                float acc[NB][8];
+#pragma unroll
+                for (int nb = 0; nb < NB; ++nb) {
+                    uint32_t ra[8];
+                    ptx::tmem_ld_8cols(tb + nb * bn + 8 * c8, ra);
+#pragma unroll
+                    for (int kx = 0; kx < CL; ++kx) {
+                        if (kx >= ks) break;
+                        const float4 p0 = in[kx][nb][0], p1 = in[kx][nb][1];
+                        const float v[8] = {p0.x, p0.y, p0.z, p0.w, p1.x, p1.y, p1.z, p1.w};
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) {
+                            const float t = kx == crank ? __uint_as_float(ra[j]) : v[j];
+                            acc[nb][j] = kx == 0 ? t : acc[nb][j] + t;
+                        }
+                    }
+                }
+                if (row < n_rows && col < ep.ld_out) {
+                    uint32_t o[4];
+                    if constexpr (EPI == EPI_CGATEUP) {
+#pragma unroll
+                        for (int t = 0; t < 4; ++t)
+                            o[t] = pack_bf16x2(silu_f(acc[0][2 * t]) * acc[NB - 1][2 * t],
+                                               silu_f(acc[0][2 * t + 1]) * acc[NB - 1][2 * t + 1]);
+                    } else {
+                        const uint4 hv = *reinterpret_cast<const uint4*>(ep.hidden + static_cast<size_t>(hid_row) * ep.ld_out + col);
+                        const uint32_t hw[4] = {hv.x, hv.y, hv.z, hv.w};
+#pragma unroll
+                        for (int t = 0; t < 4; ++t) {
+                            const __nv_bfloat162 h2 = *reinterpret_cast<const __nv_bfloat162*>(&hw[t]);
+                            o[t] = pack_bf16x2(__bfloat162float(h2.x) + acc[0][2 * t], __bfloat162float(h2.y) + acc[0][2 * t + 1]);
+                        }
+                    }
+                    *reinterpret_cast<uint4*>(ep.out + static_cast<size_t>(row) * ep.ld_out + col) = make_uint4(o[0], o[1], o[2], o[3]);
+                }
+                __syncwarp();   // converged again for the next TMEM load
+            }
+        }
+    }
+
     // the producer and MMA lanes rejoin their warps first: the CTA-wide barrier below must wait
     // for every thread, not only for each warp's first arrivals
     __syncwarp();
@@ -908,7 +1026,7 @@ cudaError_t make_tmap(CUtensorMap* map, const void* base, uint64_t inner, uint64
     return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
-// Clusters of CL CTAs that can be resident at once for this kernel (at most num_sms / CL).
+// Clusters of cl CTAs that can be resident at once for this kernel (at most num_sms / cl).
 template <typename K>
 int resident_clusters(K kern, int smem, int cl, int num_sms) {
     int cap = num_sms / cl;
@@ -936,7 +1054,8 @@ template <int EPI, int MT, int NB, int BN, int STAGES, int CL = 1>
 cudaError_t run_gemm(const Ctx& ctx, const CUtensorMap& tx, const CUtensorMap& tw0, const CUtensorMap& tw1,
                      int n_rows, int K, int n_ntiles, int n_mgroups, const EpiParams& ep_in, int k_splits = 1,
                      size_t partial_bytes = 0) {
-    using C = TileCfg<MT, NB, BN, STAGES, (CL == 2 && EPI != EPI_CGATEUP && EPI != EPI_CDOWN)>;
+    constexpr bool kSplitK = EPI == EPI_CGATEUP || EPI == EPI_CDOWN;
+    using C = TileCfg<MT, NB, BN, STAGES, CL == 2 && !kSplitK>;
     auto kern = tc_gemm_kernel<EPI, MT, NB, BN, STAGES, CL, false>;
     EpiParams ep = ep_in;
     ep.wait_ns = wait_limit_ns();
@@ -944,92 +1063,56 @@ cudaError_t run_gemm(const Ctx& ctx, const CUtensorMap& tx, const CUtensorMap& t
     if (e != cudaSuccess) return e;
     const int n_units = n_ntiles * n_mgroups * k_splits;
     const int stream_once = n_mgroups == 1 ? 1 : 0;
-    if constexpr (EPI == EPI_CGATEUP || EPI == EPI_CDOWN) {
-        // one output tile per cluster, its K-ranges on the cluster's CTAs; the caller has checked
-        // that all clusters are resident at once (splitk_clusters_fit)
+    if constexpr (kSplitK) {   // one output tile per cluster, its K-ranges on the cluster's CTAs
         e = launch_pdl_cluster(kern, dim3(CL * n_ntiles * n_mgroups), dim3(kThreads), C::kSmemBytes, ctx.stream, CL,
                                tx, tw0, tw1, n_rows, K, n_ntiles, n_mgroups, CL, stream_once, ep, ctx.status);
+        return e != cudaSuccess ? e : cudaGetLastError();
+    }
+    int n_items = n_units;
+    if constexpr (EPI == EPI_GATEUP || EPI == EPI_DOWN) {
+        // Tail split: when the units overflow the SMs by a last round that would leave most of
+        // them idle, each unit of that round runs as up to kMaxTailSplit K-chunks on the idle
+        // SMs, summed by the chunk that finishes last (fp32 partial sums in the workspace). A
+        // pair's unit of 256 columns counts for two SMs, one of 128 + 128 for one (two rounds
+        // of pairs take the time of one round of single CTAs), so that the chunks of an output
+        // do not depend on whether pairs run it.
+        constexpr int kTiles = CL == 1 ? MT : 2;
+        const int slots = CL == 2 && NB == 1 ? ctx.num_sms / 2 : ctx.num_sms;
+        const int tail = n_units % slots;
+        int split = tail > 0 ? slots / tail : 0;
+        split = split < kMaxTailSplit ? split : kMaxTailSplit;
+        split = split < K / kBK ? split : K / kBK;
+        const size_t need = static_cast<size_t>(tail) * split * kTiles * kBM * NB * BN * sizeof(float);
+        if (k_splits == 1 && n_units > slots && split >= 2 && ctx.status && tail * kTiles <= kTailSems &&
+            ep.partial && need <= partial_bytes) {
+            ep.n_full = n_units - tail;
+            ep.tail_split = split;
+            ep.sem = ctx.status + 1;
+            n_items = ep.n_full + tail * split;
+        }
+    }
+    if constexpr (CL == 1) {
+        const int grid = n_items < ctx.num_sms ? n_items : ctx.num_sms;
+        e = launch_pdl(kern, dim3(grid), dim3(kThreads), C::kSmemBytes, ctx.stream, tx, tw0, tw1, n_rows, K,
+                       n_ntiles, n_mgroups, k_splits, stream_once, ep, ctx.status);
     } else {
-        int n_items = n_units;
-        if constexpr (EPI == EPI_GATEUP || EPI == EPI_DOWN) {
-            // Tail split: when the units overflow the SMs by a last round that would leave most of
-            // them idle, each unit of that round runs as up to kMaxTailSplit K-chunks on the idle
-            // SMs, summed by the chunk that finishes last (fp32 partial sums in the workspace). A
-            // pair's unit of 256 columns counts for two SMs, one of 128 + 128 for one (two rounds
-            // of pairs take the time of one round of single CTAs), so that the chunks of an output
-            // do not depend on whether pairs run it.
-            constexpr int kTiles = CL == 1 ? MT : 2;
-            const int slots = CL == 2 && NB == 1 ? ctx.num_sms / 2 : ctx.num_sms;
-            const int tail = n_units % slots;
-            int split = tail > 0 ? slots / tail : 0;
-            split = split < kMaxTailSplit ? split : kMaxTailSplit;
-            split = split < K / kBK ? split : K / kBK;
-            const size_t need = static_cast<size_t>(tail) * split * kTiles * kBM * NB * BN * sizeof(float);
-            if (k_splits == 1 && n_units > slots && split >= 2 && ctx.status && tail * kTiles <= kTailSems &&
-                ep.partial && need <= partial_bytes) {
-                ep.n_full = n_units - tail;
-                ep.tail_split = split;
-                ep.sem = ctx.status + 1;
-                n_items = ep.n_full + tail * split;
-            }
-        }
-        if constexpr (CL == 1) {
-            const int grid = n_items < ctx.num_sms ? n_items : ctx.num_sms;
-            e = launch_pdl(kern, dim3(grid), dim3(kThreads), C::kSmemBytes, ctx.stream, tx, tw0, tw1, n_rows, K,
-                           n_ntiles, n_mgroups, k_splits, stream_once, ep, ctx.status);
-        } else {
-            static const int max_cl = resident_clusters(kern, C::kSmemBytes, CL, ctx.num_sms);
-            const int n_cl = n_items < max_cl ? n_items : max_cl;
-            e = launch_pdl_cluster(kern, dim3(CL * n_cl), dim3(kThreads), C::kSmemBytes, ctx.stream, CL, tx, tw0, tw1,
-                                   n_rows, K, n_ntiles, n_mgroups, k_splits, stream_once, ep, ctx.status);
-        }
+        static const int max_cl = resident_clusters(kern, C::kSmemBytes, CL, ctx.num_sms);
+        const int n_cl = n_items < max_cl ? n_items : max_cl;
+        e = launch_pdl_cluster(kern, dim3(CL * n_cl), dim3(kThreads), C::kSmemBytes, ctx.stream, CL, tx, tw0, tw1,
+                               n_rows, K, n_ntiles, n_mgroups, k_splits, stream_once, ep, ctx.status);
     }
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 }  // namespace
 
-// Bytes of the split-K exchange area of the cluster path: per output tile (cluster) of 128
-// columns, CL = 4 owners receive 3 blocks of 2 M-tiles x 128 rows x NB x 32 fp32 columns.
-size_t splitk_exchange_bytes(int n_out_cols, int nb) {
-    return static_cast<size_t>(n_out_cols / 128) * 4 * 3 * (2 * 128) * nb * 32 * 4;
+// Bytes of the split-K exchange area of a cluster GEMM over n_rows <= 256 rows with n_out_cols output
+// columns of nb adjacent matrices: the partial sums of every K-range, whole M-tiles and whole tiles of
+// up to 128 columns.
+size_t splitk_exchange_bytes(int n_out_cols, int nb, int n_rows) {
+    if (n_rows > 2 * kBM) return 0;
+    return static_cast<size_t>(kMaxKSplits) * (n_out_cols + 128) * nb * (n_rows <= kBM ? kBM : 2 * kBM) * sizeof(float);
 }
-
-namespace {
-
-// Whether n_tiles clusters of the split-K kernel can all be resident at once (each cluster then
-// runs its one tile; a second wave would serialise them).
-template <int EPI, int MT, int NB, int BN, int STAGES, int CL>
-bool splitk_clusters_fit(const Ctx& ctx, int n_tiles) {
-    using C = TileCfg<MT, NB, BN, STAGES>;
-    auto kern = tc_gemm_kernel<EPI, MT, NB, BN, STAGES, CL, false>;
-    static const int max_cl = [&] {
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes) != cudaSuccess) {
-            (void)cudaGetLastError();
-            return 0;
-        }
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(CL * (ctx.num_sms / CL));
-        cfg.blockDim = dim3(kThreads);
-        cfg.dynamicSmemBytes = C::kSmemBytes;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = CL;
-        attr[0].val.clusterDim.y = 1;
-        attr[0].val.clusterDim.z = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-        int n = 0;
-        if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess) {
-            (void)cudaGetLastError();
-            return 0;
-        }
-        return n;
-    }();
-    return n_tiles <= max_cl;
-}
-
-}  // namespace
 
 cudaError_t launch_lmhead_tc(const Ctx& ctx, const void* lm_head, const void* x, int n_rows, int d, int V,
                              float inv_temp, Partials partials, bool reset_status) {
@@ -1063,12 +1146,11 @@ int choose_k_splits(int base_units, int nk, int num_sms) {
     return ks < 1 ? 1 : ks;
 }
 
-// Where the fixed-width kernels of Eq. 1 take over from single CTAs of chosen width (GB300, 152 SMs):
-// clusters of four from 96 CTAs (I = d = 3584, 241 rows: Eq. 1 54.0 against 58.6 us; at 64 CTAs, d =
-// 2048, 38.1 against 35.2), pairs from 40 (d = 4096, 723 rows, 48 pairs: 111 against 114 us; d = 2560,
-// 241 rows, 40 pairs: 84.5 against 85.8; d = 2048, 32 pairs: 37.0 against 35.3).
-constexpr int kMinClusterCtas = 96;
+// Units from which CTA pairs take over from single CTAs of chosen width in the down projection (GB300,
+// 152 SMs): d = 4096, 723 rows, 48 pairs: Eq. 1 111 against 114 us; d = 2560, 241 rows, 40 pairs: 84.5
+// against 85.8; d = 2048, 32 pairs: 37.0 against 35.3.
 constexpr int kMinPairs = 40;
+constexpr int kMinClusterCtas = 96;
 
 // A GEMM of single CTAs whose tile width is chosen for the SM count: [n_rows, K] x [N, K]^T (NB
 // matrices side by side), in k_splits K-ranges. A round of units costs about what an SM loads per
@@ -1112,6 +1194,58 @@ cudaError_t run_gemm_var(const Ctx& ctx, const CUtensorMap& tx, const void* w0, 
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
+// The same for one or two M-tiles whose K is split: k_splits CTAs form a cluster on one output tile and
+// exchange their partial sums, so no reduction kernel follows. All clusters must be resident at once
+// (one tile each), which bounds their number; the tile width follows from it. *done stays false, and
+// nothing runs, where N is too wide for that.
+template <int EPI, int MT, int NB>
+cudaError_t run_gemm_cluster(const Ctx& ctx, const CUtensorMap& tx, const void* w0, const void* w1, int N, int n_rows, int K,
+                             int k_splits, const EpiParams& ep_in, size_t partial_bytes, bool* done) {
+    using C = TileCfg<MT, NB, 128, kVarMaxStages, false, true>;
+    auto kern = tc_gemm_kernel<EPI, MT, NB, 128, kVarMaxStages, kMaxKSplits, true>;
+    constexpr int kStep = NB == 1 ? 16 : 8;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes);
+    if (e != cudaSuccess) return e;
+    static const struct Fit {
+        int n[kMaxKSplits + 1];
+    } fit = [&] {
+        Fit f{};
+        for (int c = 2; c <= kMaxKSplits; ++c) f.n[c] = resident_clusters(kern, C::kSmemBytes, c, ctx.num_sms);
+        return f;
+    }();
+    const int max_cl = fit.n[k_splits];
+    int bn = 32;
+    while (bn < 128 && (N + bn - 1) / bn > max_cl) bn += kStep;
+    const int n_ntiles = (N + bn - 1) / bn;
+    const size_t need = static_cast<size_t>(n_ntiles) * k_splits * NB * bn * MT * kBM * sizeof(float);
+    if (n_ntiles > max_cl || !ep_in.partial || need > partial_bytes) return cudaSuccess;
+    CUtensorMap t0, t1;
+    if constexpr (MT == 2) {
+        // Four ranges of two M-tiles in whole tiles of 128 columns that fill the SMs: the kernel with
+        // that width fixed, whose exchange keeps more loads in flight (d = I = 4096, 241 rows: Eq. 1
+        // 59.6 against 63.0 us; d = 2048 would leave half of the SMs idle, 36.8 against 33.2).
+        if (k_splits == 4 && N % 128 == 0 && N / 128 * 4 >= kMinClusterCtas && N / 128 <= max_cl) {
+            e = make_tmap(&t0, w0, K, N, kBK, 128);
+            if (e == cudaSuccess) e = make_tmap(&t1, NB == 2 ? w1 : w0, K, N, kBK, 128);
+            if (e != cudaSuccess) return e;
+            *done = true;
+            return run_gemm<EPI, MT, NB, 128, NB == 2 ? 3 : 4, 4>(ctx, tx, t0, t1, n_rows, K, N / 128, 1, ep_in, 4);
+        }
+    }
+    e = make_tmap(&t0, w0, K, N, kBK, bn);
+    if (e == cudaSuccess) e = make_tmap(&t1, NB == 2 ? w1 : w0, K, N, kBK, bn);
+    if (e != cudaSuccess) return e;
+    EpiParams ep = ep_in;
+    ep.wait_ns = wait_limit_ns();
+    ep.bn = bn;
+    const int stages = C::kRingBytes / (MT * C::kABytes + NB * bn * kBK * 2);
+    ep.stages = stages < kVarMaxStages ? stages : kVarMaxStages;
+    *done = true;
+    e = launch_pdl_cluster(kern, dim3(k_splits * n_ntiles), dim3(kThreads), C::kSmemBytes, ctx.stream, k_splits, tx, t0, t1,
+                           n_rows, K, n_ntiles, 1, k_splits, 1, ep, ctx.status);
+    return e != cudaSuccess ? e : cudaGetLastError();
+}
+
 // h' = h + In W^T with In [n_rows, K] (tmap_in, boxes of kBK x kBM) and W [d, K]: the SwiGLU down
 // projection (K = I, In = A) and the linear approximator (K = 2d, In = x). The residual row of
 // stage-2 row r is the hidden state of its depth; the epilogue adds it in fp32 and rounds once to
@@ -1137,13 +1271,16 @@ static cudaError_t run_residual_gemm(const Ctx& ctx, const CUtensorMap& ta, cons
     ed.partial = partial;
     ed.n_cols = d;
     ed.n_total = d;
-    // Two M-tiles with K split four ways: clusters of four that exchange their partial sums. Two or
-    // more M-tiles otherwise: CTA pairs on 256-column tiles, which stage a third less per SM and overlap
-    // their epilogue with the next unit (1928 rows, K = 8192, d = 4096: 131 -> 108 us with the gather;
-    // gate/up gains nothing from pairs: single CTAs already run N = 256 MMAs there). Both only where
-    // their units fill the SMs.
-    if (m_tiles == 2 && bn_d == BN && ks2 == 4 && d / BN * 4 >= kMinClusterCtas && splitk_clusters_fit<EPI_CDOWN, 2, 1, BN, 4, 4>(ctx, d / BN))
-        return run_gemm<EPI_CDOWN, 2, 1, BN, 4, 4>(ctx, ta, td, td, n_rows, K, d / BN, 1, ed, 4);
+    // One or two M-tiles with K split: clusters that exchange their partial sums. Two or more M-tiles
+    // otherwise: CTA pairs on 256-column tiles, which stage a third less per SM and overlap their
+    // epilogue with the next unit (1928 rows, K = 8192, d = 4096: 131 -> 108 us with the gather; gate/up
+    // gains nothing from pairs: single CTAs already run N = 256 MMAs there), where their units fill
+    // the SMs.
+    bool done = false;
+    if (ks2 > 1 && m_tiles <= 2)
+        e = m_tiles == 1 ? run_gemm_cluster<EPI_CDOWN, 1, 1>(ctx, ta, W, nullptr, d, n_rows, K, ks2, ed, partial_bytes, &done)
+                         : run_gemm_cluster<EPI_CDOWN, 2, 1>(ctx, ta, W, nullptr, d, n_rows, K, ks2, ed, partial_bytes, &done);
+    if (done || e != cudaSuccess) return e;
     const bool pair = m_tiles > 1 && d % 256 == 0 && d / 256 * n_mg * ks2 >= kMinPairs;
     if (ks2 == 1) {
         if (pair) return run_gemm<EPI_DOWN, 1, 1, 256, 7, 2>(ctx, ta, td, td, n_rows, K, d / 256, n_mg, ed, 1, partial_bytes);
@@ -1183,9 +1320,11 @@ cudaError_t launch_swiglu_tc(const Ctx& ctx, const void* X, int k_in, const void
     ep.partial = partial;
     ep.n_cols = 2 * I;
     ep.n_total = I;
-    if (m_tiles == 2 && bn_gu == BN && ks1 == 4 && I / BN * 4 >= kMinClusterCtas &&
-        splitk_clusters_fit<EPI_CGATEUP, 2, 2, BN, 3, 4>(ctx, I / BN)) {
-        e = run_gemm<EPI_CGATEUP, 2, 2, BN, 3, 4>(ctx, tx, tg, tu, n_rows, k_in, I / BN, 1, ep, 4);
+    bool done = false;
+    if (ks1 > 1 && m_tiles <= 2)
+        e = m_tiles == 1 ? run_gemm_cluster<EPI_CGATEUP, 1, 2>(ctx, tx, w_gate, w_up, I, n_rows, k_in, ks1, ep, partial_bytes, &done)
+                         : run_gemm_cluster<EPI_CGATEUP, 2, 2>(ctx, tx, w_gate, w_up, I, n_rows, k_in, ks1, ep, partial_bytes, &done);
+    if (done || e != cudaSuccess) {
     } else if (m_tiles > 1 && bn_gu == BN && ks1 == 1 && I / BN * n_mg > ctx.num_sms) {
         e = run_gemm<EPI_GATEUP, 2, 2, BN, 3>(ctx, tx, tg, tu, n_rows, k_in, I / BN, n_mg, ep, 1, partial_bytes);
     } else if (ks1 == 1) {

@@ -267,6 +267,17 @@ __device__ __forceinline__ float4 ld_cluster_f4(uint32_t addr) {
     return v;
 }
 
+// Load 8 consecutive 32-bit TMEM columns of the warp's 32 lanes into r[OFF ..]; the registers are
+// valid only after tmem_wait_ld_regs(r).
+template <int OFF>
+__device__ __forceinline__ void tmem_ld_8cols_nowait(uint32_t taddr, uint32_t (&r)[32]) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=r"(r[OFF]), "=r"(r[OFF + 1]), "=r"(r[OFF + 2]), "=r"(r[OFF + 3]), "=r"(r[OFF + 4]), "=r"(r[OFF + 5]),
+          "=r"(r[OFF + 6]), "=r"(r[OFF + 7])
+        : "r"(taddr)
+        : "memory");
+}
 // Load 8 or 16 consecutive 32-bit TMEM columns of the warp's 32 lanes and wait for the load.
 __device__ __forceinline__ void tmem_ld_8cols(uint32_t taddr, uint32_t (&r)[8]) {
     asm volatile(
