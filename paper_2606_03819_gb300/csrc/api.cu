@@ -118,14 +118,14 @@ Layout layout(const Dims& D) {
     L.A = take(rows2 * D.I * D.esize);
     L.hp = take(rows2 * D.d * D.esize);
     L.hres = take(D.two_prev ? rows2 * D.d * D.esize : 0);   // residual row of each stage-2 row
-    // split-K partial sums of the bf16 approximator GEMMs: [k_splits][max(2I, d) / 4][rows][4] fp32,
-    // or the exchange area of their cluster path, whichever is larger
+    // split-K partial sums of the bf16 approximator GEMMs: [k_splits][max(2I, d) / 4][rows][4] fp32, or
+    // the same of whole M-tile pairs (one M-tile alone) and N tiles where clusters exchange them (few
+    // rows: a K split over many rows would need more units than there are SMs)
     if (D.dtype == TF_BF16) {
-        const size_t partial = static_cast<size_t>(kMaxKSplits) * rows2 *
-                               (2 * static_cast<size_t>(D.I) > static_cast<size_t>(D.d) ? 2 * D.I : D.d) * 4;
-        const int r = static_cast<int>(rows2);
-        const size_t xg = std::max(splitk_exchange_bytes(D.I, 2, r), splitk_exchange_bytes(D.d, 1, r));
-        L.kpart_bytes = rows2 > 0 ? std::max(partial, xg) : 0;
+        const size_t cols = 2 * static_cast<size_t>(D.I) > static_cast<size_t>(D.d) ? 2 * D.I : D.d;
+        const bool few = rows2 <= 2048;
+        const size_t whole = rows2 <= 128 ? 128 : (rows2 + 255) / 256 * 256;
+        L.kpart_bytes = rows2 > 0 ? static_cast<size_t>(kMaxKSplits) * (few ? whole * (cols + 256) : rows2 * cols) * 4 : 0;
         L.kpart = take(L.kpart_bytes);
     } else {
         L.kpart_bytes = 0;

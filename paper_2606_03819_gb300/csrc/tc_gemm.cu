@@ -1106,14 +1106,6 @@ cudaError_t run_gemm(const Ctx& ctx, const CUtensorMap& tx, const CUtensorMap& t
 
 }  // namespace
 
-// Bytes of the split-K exchange area of a cluster GEMM over n_rows <= 256 rows with n_out_cols output
-// columns of nb adjacent matrices: the partial sums of every K-range, whole M-tiles and whole tiles of
-// up to 128 columns.
-size_t splitk_exchange_bytes(int n_out_cols, int nb, int n_rows) {
-    if (n_rows > 2 * kBM) return 0;
-    return static_cast<size_t>(kMaxKSplits) * (n_out_cols + 128) * nb * (n_rows <= kBM ? kBM : 2 * kBM) * sizeof(float);
-}
-
 cudaError_t launch_lmhead_tc(const Ctx& ctx, const void* lm_head, const void* x, int n_rows, int d, int V,
                              float inv_temp, Partials partials, bool reset_status) {
     if (n_rows <= 0) return cudaSuccess;
@@ -1194,13 +1186,13 @@ cudaError_t run_gemm_var(const Ctx& ctx, const CUtensorMap& tx, const void* w0, 
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
-// The same for one or two M-tiles whose K is split: k_splits CTAs form a cluster on one output tile and
-// exchange their partial sums, so no reduction kernel follows. All clusters must be resident at once
-// (one tile each), which bounds their number; the tile width follows from it. *done stays false, and
-// nothing runs, where N is too wide for that.
+// The same where K is split: k_splits CTAs form a cluster on one output tile and exchange their partial
+// sums, so no reduction kernel follows. All clusters must be resident at once (one tile each), which
+// bounds their number; the tile width follows from it. *done stays false, and nothing runs, where there
+// are too many tiles for that.
 template <int EPI, int MT, int NB>
 cudaError_t run_gemm_cluster(const Ctx& ctx, const CUtensorMap& tx, const void* w0, const void* w1, int N, int n_rows, int K,
-                             int k_splits, const EpiParams& ep_in, size_t partial_bytes, bool* done) {
+                             int n_mgroups, int k_splits, const EpiParams& ep_in, size_t partial_bytes, bool* done) {
     using C = TileCfg<MT, NB, 128, kVarMaxStages, false, true>;
     auto kern = tc_gemm_kernel<EPI, MT, NB, 128, kVarMaxStages, kMaxKSplits, true>;
     constexpr int kStep = NB == 1 ? 16 : 8;
@@ -1215,16 +1207,17 @@ cudaError_t run_gemm_cluster(const Ctx& ctx, const CUtensorMap& tx, const void* 
     }();
     const int max_cl = fit.n[k_splits];
     int bn = 32;
-    while (bn < 128 && (N + bn - 1) / bn > max_cl) bn += kStep;
+    while (bn < 128 && static_cast<long long>((N + bn - 1) / bn) * n_mgroups > max_cl) bn += kStep;
     const int n_ntiles = (N + bn - 1) / bn;
-    const size_t need = static_cast<size_t>(n_ntiles) * k_splits * NB * bn * MT * kBM * sizeof(float);
-    if (n_ntiles > max_cl || !ep_in.partial || need > partial_bytes) return cudaSuccess;
+    const long long n_cl = static_cast<long long>(n_ntiles) * n_mgroups;
+    const size_t need = static_cast<size_t>(n_cl) * k_splits * NB * bn * MT * kBM * sizeof(float);
+    if (n_cl > max_cl || !ep_in.partial || need > partial_bytes) return cudaSuccess;
     CUtensorMap t0, t1;
     if constexpr (MT == 2) {
         // Four ranges of two M-tiles in whole tiles of 128 columns that fill the SMs: the kernel with
         // that width fixed, whose exchange keeps more loads in flight (d = I = 4096, 241 rows: Eq. 1
         // 59.6 against 63.0 us; d = 2048 would leave half of the SMs idle, 36.8 against 33.2).
-        if (k_splits == 4 && N % 128 == 0 && N / 128 * 4 >= kMinClusterCtas && N / 128 <= max_cl) {
+        if (n_mgroups == 1 && k_splits == 4 && N % 128 == 0 && N / 128 * 4 >= kMinClusterCtas && N / 128 <= max_cl) {
             e = make_tmap(&t0, w0, K, N, kBK, 128);
             if (e == cudaSuccess) e = make_tmap(&t1, NB == 2 ? w1 : w0, K, N, kBK, 128);
             if (e != cudaSuccess) return e;
@@ -1241,8 +1234,9 @@ cudaError_t run_gemm_cluster(const Ctx& ctx, const CUtensorMap& tx, const void* 
     const int stages = C::kRingBytes / (MT * C::kABytes + NB * bn * kBK * 2);
     ep.stages = stages < kVarMaxStages ? stages : kVarMaxStages;
     *done = true;
-    e = launch_pdl_cluster(kern, dim3(k_splits * n_ntiles), dim3(kThreads), C::kSmemBytes, ctx.stream, k_splits, tx, t0, t1,
-                           n_rows, K, n_ntiles, 1, k_splits, 1, ep, ctx.status);
+    e = launch_pdl_cluster(kern, dim3(static_cast<unsigned>(k_splits * n_cl)), dim3(kThreads), C::kSmemBytes, ctx.stream,
+                           k_splits, tx, t0, t1, n_rows, K, n_ntiles, n_mgroups, k_splits, n_mgroups == 1 ? 1 : 0, ep,
+                           ctx.status);
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
@@ -1271,15 +1265,15 @@ static cudaError_t run_residual_gemm(const Ctx& ctx, const CUtensorMap& ta, cons
     ed.partial = partial;
     ed.n_cols = d;
     ed.n_total = d;
-    // One or two M-tiles with K split: clusters that exchange their partial sums. Two or more M-tiles
+    // K split: clusters that exchange their partial sums. Two or more M-tiles
     // otherwise: CTA pairs on 256-column tiles, which stage a third less per SM and overlap their
     // epilogue with the next unit (1928 rows, K = 8192, d = 4096: 131 -> 108 us with the gather; gate/up
     // gains nothing from pairs: single CTAs already run N = 256 MMAs there), where their units fill
     // the SMs.
     bool done = false;
-    if (ks2 > 1 && m_tiles <= 2)
-        e = m_tiles == 1 ? run_gemm_cluster<EPI_CDOWN, 1, 1>(ctx, ta, W, nullptr, d, n_rows, K, ks2, ed, partial_bytes, &done)
-                         : run_gemm_cluster<EPI_CDOWN, 2, 1>(ctx, ta, W, nullptr, d, n_rows, K, ks2, ed, partial_bytes, &done);
+    if (ks2 > 1)
+        e = m_tiles == 1 ? run_gemm_cluster<EPI_CDOWN, 1, 1>(ctx, ta, W, nullptr, d, n_rows, K, 1, ks2, ed, partial_bytes, &done)
+                         : run_gemm_cluster<EPI_CDOWN, 2, 1>(ctx, ta, W, nullptr, d, n_rows, K, n_mg, ks2, ed, partial_bytes, &done);
     if (done || e != cudaSuccess) return e;
     const bool pair = m_tiles > 1 && d % 256 == 0 && d / 256 * n_mg * ks2 >= kMinPairs;
     if (ks2 == 1) {
@@ -1321,9 +1315,9 @@ cudaError_t launch_swiglu_tc(const Ctx& ctx, const void* X, int k_in, const void
     ep.n_cols = 2 * I;
     ep.n_total = I;
     bool done = false;
-    if (ks1 > 1 && m_tiles <= 2)
-        e = m_tiles == 1 ? run_gemm_cluster<EPI_CGATEUP, 1, 2>(ctx, tx, w_gate, w_up, I, n_rows, k_in, ks1, ep, partial_bytes, &done)
-                         : run_gemm_cluster<EPI_CGATEUP, 2, 2>(ctx, tx, w_gate, w_up, I, n_rows, k_in, ks1, ep, partial_bytes, &done);
+    if (ks1 > 1)
+        e = m_tiles == 1 ? run_gemm_cluster<EPI_CGATEUP, 1, 2>(ctx, tx, w_gate, w_up, I, n_rows, k_in, 1, ks1, ep, partial_bytes, &done)
+                         : run_gemm_cluster<EPI_CGATEUP, 2, 2>(ctx, tx, w_gate, w_up, I, n_rows, k_in, n_mg, ks1, ep, partial_bytes, &done);
     if (done || e != cudaSuccess) {
     } else if (m_tiles > 1 && bn_gu == BN && ks1 == 1 && I / BN * n_mg > ctx.num_sms) {
         e = run_gemm<EPI_GATEUP, 2, 2, BN, 3>(ctx, tx, tg, tu, n_rows, k_in, I / BN, n_mg, ep, 1, partial_bytes);
