@@ -11,6 +11,7 @@ from __future__ import annotations
 import ctypes
 import os
 from dataclasses import dataclass
+from functools import cached_property
 from typing import Optional
 
 import torch
@@ -137,6 +138,14 @@ class Dims:
     def torch_dtype(self):
         return torch.bfloat16 if self.dtype == "bf16" else torch.float32
 
+    @cached_property
+    def ref(self):
+        """ctypes reference to the C struct of these (immutable) dimensions, built once."""
+        return ctypes.byref(self.c())
+
+    def __getstate__(self):
+        return {k: v for k, v in self.__dict__.items() if k != "ref"}   # copies and pickles make their own
+
     def c(self) -> TfDims:
         return TfDims(self.batch, self.d, self.V, self.I, self.gamma, self.M, self.K2, self.B,
                       self.temperature, self.rms_eps, TF_BF16 if self.dtype == "bf16" else TF_F32,
@@ -156,16 +165,25 @@ def _ptr(t: Optional[torch.Tensor]):
         return None
     if not t.is_contiguous():
         raise ValueError("tensors passed to the TreeFlash ABI must be contiguous")
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
+
+
+# The handle of the current stream alone: a Stream object costs more than the rest of a call's
+# marshalling (and the small calls are bound by the host).
+_current_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
 
 
 def _stream(stream=None):
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return ctypes.c_void_p(s.cuda_stream)
+    if stream is not None:
+        return stream.cuda_stream
+    if _current_raw_stream is None:
+        return torch.cuda.current_stream().cuda_stream
+    return _current_raw_stream(torch.cuda.current_device())
 
 
 def weights_struct(w: dict) -> TfWeights:
-    return TfWeights(*[w[k].data_ptr() if w.get(k) is not None else None for k in WEIGHT_KEYS])
+    get = w.get
+    return TfWeights(*[None if (t := get(k)) is None else t.data_ptr() for k in WEIGHT_KEYS])
 
 
 def tf_version() -> int:
@@ -185,7 +203,7 @@ def tf_set_wait_limit_ns(ns: int) -> None:
 
 def tf_workspace_size(dims: Dims) -> int:
     n = ctypes.c_size_t(0)
-    _check("tf_workspace_size", load_library().tf_workspace_size(ctypes.byref(dims.c()), ctypes.byref(n)))
+    _check("tf_workspace_size", load_library().tf_workspace_size(dims.ref, ctypes.byref(n)))
     return n.value
 
 
@@ -211,35 +229,35 @@ def tf_status_read(ws: torch.Tensor, stream=None, raise_on_error: bool = False) 
 
 def tf_stage1_marginals(dims: Dims, w: dict, hidden, top_ids, top_logp, ws, stream=None):
     _check("tf_stage1_marginals", load_library().tf_stage1_marginals(
-        ctypes.byref(dims.c()), ctypes.byref(weights_struct(w)), _ptr(hidden), _ptr(top_ids),
+        dims.ref, ctypes.byref(weights_struct(w)), _ptr(hidden), _ptr(top_ids),
         _ptr(top_logp), _ptr(ws), ws.numel(), _stream(stream)))
 
 
 def tf_stage2_ar_approx(dims: Dims, w: dict, hidden, root_tok, top_ids, child_ids, child_logp, ws,
                         stream=None):
     _check("tf_stage2_ar_approx", load_library().tf_stage2_ar_approx(
-        ctypes.byref(dims.c()), ctypes.byref(weights_struct(w)), _ptr(hidden), _ptr(root_tok),
+        dims.ref, ctypes.byref(weights_struct(w)), _ptr(hidden), _ptr(root_tok),
         _ptr(top_ids), _ptr(child_ids), _ptr(child_logp), _ptr(ws), ws.numel(), _stream(stream)))
 
 
 def tf_build_tree(dims: Dims, root_tok, top_ids, top_logp, child_ids, child_logp, node_tok, node_parent,
                   node_depth, node_score, dev_status, stream=None):
     _check("tf_build_tree", load_library().tf_build_tree(
-        ctypes.byref(dims.c()), _ptr(root_tok), _ptr(top_ids), _ptr(top_logp), _ptr(child_ids),
+        dims.ref, _ptr(root_tok), _ptr(top_ids), _ptr(top_logp), _ptr(child_ids),
         _ptr(child_logp), _ptr(node_tok), _ptr(node_parent), _ptr(node_depth), _ptr(node_score),
         _ptr(dev_status), _stream(stream)))
 
 
 def tf_tree_mask(dims: Dims, node_parent, node_depth, root_pos, mask, pos_ids, stream=None):
     _check("tf_tree_mask", load_library().tf_tree_mask(
-        ctypes.byref(dims.c()), _ptr(node_parent), _ptr(node_depth), _ptr(root_pos), _ptr(mask),
+        dims.ref, _ptr(node_parent), _ptr(node_depth), _ptr(root_pos), _ptr(mask),
         _ptr(pos_ids), _stream(stream)))
 
 
 def tf_build_tree_mask(dims: Dims, root_tok, root_pos, top_ids, top_logp, child_ids, child_logp, node_tok,
                        node_parent, node_depth, node_score, mask, pos_ids, dev_status, stream=None):
     _check("tf_build_tree_mask", load_library().tf_build_tree_mask(
-        ctypes.byref(dims.c()), _ptr(root_tok), _ptr(root_pos), _ptr(top_ids), _ptr(top_logp), _ptr(child_ids),
+        dims.ref, _ptr(root_tok), _ptr(root_pos), _ptr(top_ids), _ptr(top_logp), _ptr(child_ids),
         _ptr(child_logp), _ptr(node_tok), _ptr(node_parent), _ptr(node_depth), _ptr(node_score), _ptr(mask),
         _ptr(pos_ids), _ptr(dev_status), _stream(stream)))
 
@@ -248,7 +266,7 @@ def tf_draft_tree_host(dims: Dims, w: dict, hidden, root_tok, root_pos, node_tok
                        node_score, mask, pos_ids, dev_status, ws, stream=None):
     """Host tensors in and out (pinned memory recommended); weights and workspace on the device."""
     st = load_library().tf_draft_tree_host(
-        ctypes.byref(dims.c()), ctypes.byref(weights_struct(w)), _ptr(hidden), _ptr(root_tok),
+        dims.ref, ctypes.byref(weights_struct(w)), _ptr(hidden), _ptr(root_tok),
         _ptr(root_pos), _ptr(node_tok), _ptr(node_parent), _ptr(node_depth), _ptr(node_score), _ptr(mask),
         _ptr(pos_ids), _ptr(dev_status), _ptr(ws), ws.numel(), _stream(stream))
     if st not in (TF_OK, TF_ERR_DEVICE_STATUS):
@@ -259,24 +277,24 @@ def tf_draft_tree_host(dims: Dims, w: dict, hidden, root_tok, root_pos, node_tok
 def tf_accept_walk(dims: Dims, node_tok, node_parent, verifier_tok, accept_len, accept_path, next_tok,
                    stream=None):
     _check("tf_accept_walk", load_library().tf_accept_walk(
-        ctypes.byref(dims.c()), _ptr(node_tok), _ptr(node_parent), _ptr(verifier_tok), _ptr(accept_len),
+        dims.ref, _ptr(node_tok), _ptr(node_parent), _ptr(verifier_tok), _ptr(accept_len),
         _ptr(accept_path), _ptr(next_tok), _stream(stream)))
 
 
 def tf_lmhead_partials(dims: Dims, lm_head, x, n_rows: int, ws, stream=None):
     _check("tf_lmhead_partials", load_library().tf_lmhead_partials(
-        ctypes.byref(dims.c()), _ptr(lm_head), _ptr(x), n_rows, _ptr(ws), ws.numel(), _stream(stream)))
+        dims.ref, _ptr(lm_head), _ptr(x), n_rows, _ptr(ws), ws.numel(), _stream(stream)))
 
 
 def tf_lmhead_merge(dims: Dims, lm_head, x, n_rows: int, k: int, out_ids, out_logp, ws, stream=None):
     _check("tf_lmhead_merge", load_library().tf_lmhead_merge(
-        ctypes.byref(dims.c()), _ptr(lm_head), _ptr(x), n_rows, k, _ptr(out_ids), _ptr(out_logp), _ptr(ws),
+        dims.ref, _ptr(lm_head), _ptr(x), n_rows, k, _ptr(out_ids), _ptr(out_logp), _ptr(ws),
         ws.numel(), _stream(stream)))
 
 
 def tf_ar_approx(dims: Dims, w: dict, hidden, root_tok, top_ids, h_prime, ws, stream=None):
     _check("tf_ar_approx", load_library().tf_ar_approx(
-        ctypes.byref(dims.c()), ctypes.byref(weights_struct(w)), _ptr(hidden), _ptr(root_tok), _ptr(top_ids),
+        dims.ref, ctypes.byref(weights_struct(w)), _ptr(hidden), _ptr(root_tok), _ptr(top_ids),
         _ptr(h_prime), _ptr(ws), ws.numel(), _stream(stream)))
 
 
@@ -284,7 +302,7 @@ def tf_workspace_h_prime(dims: Dims, ws) -> torch.Tensor:
     """h' [b, R, d] as a tensor view of the workspace (no copy)."""
     p = ctypes.c_void_p()
     _check("tf_workspace_h_prime", load_library().tf_workspace_h_prime(
-        ctypes.byref(dims.c()), _ptr(ws), ws.numel(), ctypes.byref(p)))
+        dims.ref, _ptr(ws), ws.numel(), ctypes.byref(p)))
     off = p.value - ws.data_ptr()
     esize = 2 if dims.dtype == "bf16" else 4
     n = dims.batch * dims.R * dims.d * esize
@@ -300,7 +318,7 @@ def tf_workspace_view(dims: Dims, ws, view: int, n_rows: Optional[int] = None) -
     float32 [n_tiles, 2 or 8, n_rows, 4]."""
     p, n = ctypes.c_void_p(), ctypes.c_size_t()
     _check("tf_workspace_view", load_library().tf_workspace_view(
-        ctypes.byref(dims.c()), _ptr(ws), ws.numel(), view, ctypes.byref(p), ctypes.byref(n)))
+        dims.ref, _ptr(ws), ws.numel(), view, ctypes.byref(p), ctypes.byref(n)))
     off = p.value - ws.data_ptr()
     if view in (TF_VIEW_HALVES, TF_VIEW_CHUNKS):
         n_tiles = (dims.V + 255) // 256
@@ -319,5 +337,5 @@ def tf_stage1_marginals_static(dims: Dims, w: dict, hidden, top_ids, top_logp, d
     scratch array instead. dev_status is a 1-element int32 device tensor that receives the call's
     TF_DEV_* flags. Calls that overlap on the GPU share that array and race."""
     _check("tf_stage1_marginals_static", load_library().tf_stage1_marginals_static(
-        ctypes.byref(dims.c()), ctypes.byref(weights_struct(w)), _ptr(hidden), _ptr(top_ids),
+        dims.ref, ctypes.byref(weights_struct(w)), _ptr(hidden), _ptr(top_ids),
         _ptr(top_logp), _ptr(dev_status), _stream(stream)))
