@@ -243,40 +243,61 @@ __device__ unsigned long long block_kth_largest_fast(const unsigned long long* k
     return r;
 }
 
-// <w, x> for one weight row (d elements) and x in shared memory (fp32), by one warp: lanes take
-// 8-element slices; all of a lane's 16-byte loads are issued before the multiply-adds.
-__device__ __forceinline__ float dot_row(const __nv_bfloat16* w, const float* xs, int d, int lane) {
-    float acc = 0.0f;
-    if ((d & 255) == 0 && (reinterpret_cast<uintptr_t>(w) & 15) == 0) {
-        const uint4* w4 = reinterpret_cast<const uint4*>(w);
+// <w_c, x> for four weight rows of d elements (row c at w + c * d), by one warp: lanes take 8-element
+// slices, four slices of all rows in flight; every sum in the order of its slices. acc[c] on every lane.
+__device__ __forceinline__ void dot_rows4(const __nv_bfloat16* const (&w)[4], const __nv_bfloat16* x, int d, int lane,
+                                          float (&acc)[4]) {
+#pragma unroll
+    for (int c = 0; c < 4; ++c) acc[c] = 0.0f;
+    if ((d & 255) == 0 && ((reinterpret_cast<uintptr_t>(w[0]) | reinterpret_cast<uintptr_t>(x)) & 15) == 0) {
+        const uint4* x4 = reinterpret_cast<const uint4*>(x);
         const int n = d / 256;                       // 16-byte slices per lane
-        for (int base = 0; base < n; base += 8) {
-            uint4 buf[8];
+        for (int base = 0; base < n; base += 4) {
+            uint4 xb[4], wb[4][4];
 #pragma unroll
-            for (int i = 0; i < 8; ++i)
-                if (base + i < n) buf[i] = w4[(base + i) * 32 + lane];
+            for (int i = 0; i < 4; ++i)
+                if (base + i < n) {
+                    xb[i] = x4[(base + i) * 32 + lane];
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
+                    for (int c = 0; c < 4; ++c) wb[c][i] = reinterpret_cast<const uint4*>(w[c])[(base + i) * 32 + lane];
+                }
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
                 if (base + i >= n) break;
-                const __nv_bfloat16* b = reinterpret_cast<const __nv_bfloat16*>(&buf[i]);
-                const float* xv = xs + ((base + i) * 32 + lane) * 8;
+                const __nv_bfloat16* xv = reinterpret_cast<const __nv_bfloat16*>(&xb[i]);
 #pragma unroll
-                for (int j = 0; j < 8; ++j) acc = fmaf(__bfloat162float(b[j]), xv[j], acc);
+                for (int c = 0; c < 4; ++c) {
+                    const __nv_bfloat16* b = reinterpret_cast<const __nv_bfloat16*>(&wb[c][i]);
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) acc[c] = fmaf(__bfloat162float(b[j]), __bfloat162float(xv[j]), acc[c]);
+                }
             }
         }
     } else {
-        for (int k = lane; k < d; k += 32) acc = fmaf(__bfloat162float(w[k]), xs[k], acc);
+        for (int k = lane; k < d; k += 32) {
+            const float xk = __bfloat162float(x[k]);
+#pragma unroll
+            for (int c = 0; c < 4; ++c) acc[c] = fmaf(__bfloat162float(w[c][k]), xk, acc[c]);
+        }
     }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    return acc;
-}
-__device__ __forceinline__ float dot_row(const float* w, const float* xs, int d, int lane) {
-    float acc = 0.0f;
-    for (int k = lane; k < d; k += 32) acc = fmaf(w[k], xs[k], acc);
+    for (int o = 16; o > 0; o >>= 1)
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    return acc;
+        for (int c = 0; c < 4; ++c) acc[c] += __shfl_xor_sync(0xffffffffu, acc[c], o);
+}
+__device__ __forceinline__ void dot_rows4(const float* const (&w)[4], const float* x, int d, int lane, float (&acc)[4]) {
+#pragma unroll
+    for (int c = 0; c < 4; ++c) acc[c] = 0.0f;
+#pragma unroll 4
+    for (int k = lane; k < d; k += 32) {
+        const float xk = x[k];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) acc[c] = fmaf(w[c][k], xk, acc[c]);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) acc[c] += __shfl_xor_sync(0xffffffffu, acc[c], o);
 }
 
 // Shared-memory layout of one merge CTA (dynamic part), for a top-k of k and room for kc >= k halves.
@@ -289,9 +310,8 @@ struct MergeSmem {
     int* cbase;                 // [4kc] first vocabulary id of each kept chunk
     int* chalf;                 // [kc] the halves kept
     uint8_t* expanded;          // [4kc] chunk recomputed
-    float* xs;                  // [d] x of the row in fp32, staged only for a recompute
 };
-__host__ __device__ inline size_t merge_layout(int n_tiles, int d, int k, int kc, uint8_t* base, MergeSmem* m) {
+__host__ __device__ inline size_t merge_layout(int n_tiles, int k, int kc, uint8_t* base, MergeSmem* m) {
     const size_t detail = static_cast<size_t>(kc) * (kChunks / 2);  // chunks of the halves kept
     size_t off = 0;
     auto take = [&](size_t bytes) {
@@ -307,7 +327,6 @@ __host__ __device__ inline size_t merge_layout(int n_tiles, int d, int k, int kc
     uint8_t* cb = take(detail * 4);
     uint8_t* ch = take(static_cast<size_t>(kc) * 4);
     uint8_t* ex = take(detail);
-    uint8_t* xs = take(static_cast<size_t>(d) * 4);
     if (m) {
         m->hkey = reinterpret_cast<unsigned long long*>(hk);
         m->cand = reinterpret_cast<unsigned long long*>(cd);
@@ -317,7 +336,6 @@ __host__ __device__ inline size_t merge_layout(int n_tiles, int d, int k, int kc
         m->cbase = reinterpret_cast<int*>(cb);
         m->chalf = reinterpret_cast<int*>(ch);
         m->expanded = ex;
-        m->xs = reinterpret_cast<float*>(xs);
     }
     return off;
 }
@@ -332,7 +350,7 @@ __global__ void __launch_bounds__(kThreads, 2) lmhead_merge_kernel(Partials part
     pdl_wait();
     extern __shared__ __align__(16) uint8_t dsm[];
     MergeSmem S;
-    merge_layout(n_tiles, d, k, kc, dsm, &S);
+    merge_layout(n_tiles, k, kc, dsm, &S);
     const int n_detail = kc * (kChunks / 2);
     __shared__ int hist[256];
     __shared__ SelectSmem SB;
@@ -468,49 +486,6 @@ __global__ void __launch_bounds__(kThreads, 2) lmhead_merge_kernel(Partials part
                     if (q.y > -INFINITY && bucket_of(q.y) >= bk) S.cand[atomicAdd(&n_cand, 1)] = cand_key(q.y, v0 + ((ids >> 8) & 255));
                 }
                 __syncthreads();
-                // Few candidates: each one's rank by counting, which sorts the winners as well. Done
-                // unless a kept chunk's third value reaches the k-th.
-                const int nc = n_cand;
-                if (nc >= k && nc <= kRankCands) {
-                    unsigned long long mine[kRankCands / kThreads];
-                    int rank[kRankCands / kThreads];
-#pragma unroll
-                    for (int j = 0; j < kRankCands / kThreads; ++j) {
-                        const int i = tid + j * kThreads;
-                        mine[j] = i < nc ? S.cand[i] : 0ull;
-                        rank[j] = 0;
-                    }
-                    if (nc <= kThreads) {
-                        if (tid < nc) {
-#pragma unroll 8
-                            for (int i = 0; i < nc; ++i) rank[0] += S.cand[i] > mine[0] ? 1 : 0;
-                        }
-                    } else {
-#pragma unroll 4
-                        for (int i = 0; i < nc; ++i) {
-                            const unsigned long long key = S.cand[i];
-#pragma unroll
-                            for (int j = 0; j < kRankCands / kThreads; ++j) rank[j] += key > mine[j] ? 1 : 0;
-                        }
-                    }
-#pragma unroll
-                    for (int j = 0; j < kRankCands / kThreads; ++j)
-                        if (mine[j] != 0ull && rank[j] == k - 1) found = mine[j];
-                    __syncthreads();
-                    const float tval = key_value(found);
-                    bool hide = false;
-                    for (int i = tid; i < nch * (kChunks / 2); i += kThreads) hide = hide || S.c3[i] >= tval;
-                    if (!__syncthreads_or(hide ? 1 : 0)) {
-                        const float lse = lse_s;
-#pragma unroll
-                        for (int j = 0; j < kRankCands / kThreads; ++j)
-                            if (mine[j] != 0ull && rank[j] < k) {
-                                out_ids[static_cast<size_t>(row) * k + rank[j]] = key_id(mine[j]);
-                                out_logp[static_cast<size_t>(row) * k + rank[j]] = key_value(mine[j]) - lse;
-                            }
-                        return;
-                    }
-                }
             }
         }
         if (!kept) __syncthreads();                      // the shared words above are reused below
@@ -611,17 +586,46 @@ __global__ void __launch_bounds__(kThreads, 2) lmhead_merge_kernel(Partials part
     //    are recomputed in rounds of at most kMergeExpandChunks; after each round only keys at or
     //    above the k-th candidate survive (the candidates are logits of the row, so every member
     //    of the true top k is at or above it, and it only rises), which bounds the set by
-    //    k + kMergeExpandChunks * kChunk whatever the input.
-    bool x_staged = false;
+    //    k + kMergeExpandChunks * kChunk whatever the input. Few candidates (the usual case) are
+    //    ranked by counting, which sorts the winners as well.
     unsigned long long theta = 0;
     unsigned long long* cand = S.cand;
     unsigned long long* spare = S.cand2;
     for (;;) {
         const int nc = n_cand;
-        theta = nc >= k ? block_kth_largest_fast(cand, nc, k, SB, hist, sel_info, &found) : 0ull;
-        const float tval = key_value(theta);
+        const bool few = nc >= k && nc <= kRankCands;
+        unsigned long long mine[kRankCands / kThreads];
+        int rank[kRankCands / kThreads];
+        if (few) {
+#pragma unroll
+            for (int j = 0; j < kRankCands / kThreads; ++j) {
+                const int i = tid + j * kThreads;
+                mine[j] = i < nc ? cand[i] : 0ull;
+                rank[j] = 0;
+            }
+            if (nc <= kThreads) {
+                if (tid < nc) {
+#pragma unroll 8
+                    for (int i = 0; i < nc; ++i) rank[0] += cand[i] > mine[0] ? 1 : 0;
+                }
+            } else {
+#pragma unroll 4
+                for (int i = 0; i < nc; ++i) {
+                    const unsigned long long key = cand[i];
+#pragma unroll
+                    for (int j = 0; j < kRankCands / kThreads; ++j) rank[j] += key > mine[j] ? 1 : 0;
+                }
+            }
+#pragma unroll
+            for (int j = 0; j < kRankCands / kThreads; ++j)
+                if (mine[j] != 0ull && rank[j] == k - 1) found = mine[j];
+        } else {
+            theta = nc >= k ? block_kth_largest_fast(cand, nc, k, SB, hist, sel_info, &found) : 0ull;
+        }
         if (tid == 0) n_flag = 0;
         __syncthreads();
+        if (few) theta = found;
+        const float tval = key_value(theta);
         for (int i = tid; i < nch * (kChunks / 2); i += kThreads) {
             if (S.expanded[i] || !(S.c3[i] > -INFINITY)) continue;
             if (nc < k || S.c3[i] >= tval) {
@@ -631,23 +635,33 @@ __global__ void __launch_bounds__(kThreads, 2) lmhead_merge_kernel(Partials part
         }
         __syncthreads();
         const int nf = min(n_flag, kMergeExpandChunks);   // the rest wait for the next round
-        if (nf == 0) break;
+        if (nf == 0) {
+            if (!few) break;
+            const float lse = lse_s;
+#pragma unroll
+            for (int j = 0; j < kRankCands / kThreads; ++j)
+                if (mine[j] != 0ull && rank[j] < k) {
+                    out_ids[static_cast<size_t>(row) * k + rank[j]] = key_id(mine[j]);
+                    out_logp[static_cast<size_t>(row) * k + rank[j]] = key_value(mine[j]) - lse;
+                }
+            return;
+        }
         if (tid == 0) {
             set_status(status, TF_DEV_RECOMPUTED);
             n_next = 0;
         }
-        // exact logits of this round's chunks: x staged once in shared memory, then one warp per
-        // column with all of its 16-byte weight loads issued before the multiply-adds
-        if (!x_staged) {
-            for (int i = tid; i < d; i += kThreads) S.xs[i] = to_f32(x[static_cast<size_t>(row) * d + i]);
-            x_staged = true;
-        }
-        __syncthreads();
-        for (int q = warp; q < nf * kChunk; q += kThreads / 32) {
-            const int f = q / kChunk, cc = q - f * kChunk;
-            const int v = S.cbase[flag_list[f]] + cc;
-            const float acc = v < V ? dot_row(lm_head + static_cast<size_t>(v) * d, S.xs, d, lane) : 0.0f;
-            if (lane == 0) zbuf[q] = v < V ? acc * inv_temp : -INFINITY;
+        // exact logits of this round's chunks, four columns per warp
+        for (int q = 4 * warp; q < nf * kChunk; q += 4 * (kThreads / 32)) {
+            const int v = S.cbase[flag_list[q / kChunk]] + q % kChunk;
+            const T* w[4];
+#pragma unroll
+            for (int c = 0; c < 4; ++c) w[c] = lm_head + static_cast<size_t>(min(v + c, V - 1)) * d;
+            float acc[4];
+            dot_rows4(w, x + static_cast<size_t>(row) * d, d, lane, acc);
+            if (lane < 4) {
+                const float z = lane == 0 ? acc[0] : lane == 1 ? acc[1] : lane == 2 ? acc[2] : acc[3];
+                zbuf[q + lane] = v + lane < V ? z * inv_temp : -INFINITY;
+            }
         }
         __syncthreads();
         // the next set: surviving keys not from this round's chunks, then their exact logits
@@ -709,7 +723,10 @@ __global__ void __launch_bounds__(kThreads, 2) lmhead_merge_kernel(Partials part
 
 }  // namespace
 
-size_t merge_smem_bytes(int n_tiles, int d, int k) { return merge_layout(n_tiles, d, k, k, nullptr, nullptr); }
+// What the dims check counts per merge CTA; with a row of x in fp32, which bounds d.
+size_t merge_smem_bytes(int n_tiles, int d, int k) {
+    return merge_layout(n_tiles, k, k, nullptr, nullptr) + (static_cast<size_t>(d) * 4 + 15) / 16 * 16;
+}
 
 cudaError_t launch_lmhead_merge(const Ctx& ctx, int dtype, Partials partials, int n_rows, int V, int d, int k,
                                 float inv_temp, const void* lm_head, const void* x, int32_t* out_ids,
@@ -717,8 +734,8 @@ cudaError_t launch_lmhead_merge(const Ctx& ctx, int dtype, Partials partials, in
     if (n_rows <= 0) return cudaSuccess;
     const int n_tiles = (V + kBlockV - 1) / kBlockV;
     // room for kKeepSlack halves more than k where shared memory has it
-    const int kc = merge_layout(n_tiles, d, k, k + kKeepSlack, nullptr, nullptr) <= kMaxMergeSmem ? k + kKeepSlack : k;
-    const size_t smem = merge_layout(n_tiles, d, k, kc, nullptr, nullptr);
+    const int kc = merge_layout(n_tiles, k, k + kKeepSlack, nullptr, nullptr) <= kMaxMergeSmem ? k + kKeepSlack : k;
+    const size_t smem = merge_layout(n_tiles, k, kc, nullptr, nullptr);
     if (dtype == TF_BF16) {
         auto kern = lmhead_merge_kernel<__nv_bfloat16>;
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
