@@ -264,6 +264,8 @@ __device__ __forceinline__ void write_nodes(const TreeArgs& a, int s, const Tree
 // underfull tree, or behind a broken link) get an empty row and column and pos -1.
 // par, dep: the tree's n parents and depths (shared memory); anc: (r1 - r0) x W words of shared
 // scratch; mask_s [n][n] and pos_s [n]: this sequence's outputs.
+// WORDS: four-byte stores; single bytes are quicker for the few rows of a small tree.
+template <bool WORDS>
 __device__ __forceinline__ void mask_rows(int n, const int* par, const int* dep, int root_pos, int r0, int r1,
                                           uint32_t* anc, uint8_t* mask_s, int32_t* pos_s) {
     const int W = (n + 31) / 32;
@@ -291,9 +293,16 @@ __device__ __forceinline__ void mask_rows(int n, const int* par, const int* dep,
     // single bytes before the first and after the last.
     const int total = (r1 - r0) * n;
     uint8_t* out = mask_s + static_cast<size_t>(r0) * n;
+    auto entry = [&](int i, int j) { return (anc[i * W + (j >> 5)] >> (j & 31)) & 1u; };
+    if constexpr (!WORDS) {
+        for (int at = threadIdx.x; at < total; at += blockDim.x) {
+            const int i = at / n;
+            out[at] = static_cast<uint8_t>(entry(i, at - i * n));
+        }
+        return;
+    }
     const int head = min(total, static_cast<int>(-reinterpret_cast<intptr_t>(out) & 3));
     const int words = (total - head) / 4;
-    auto entry = [&](int i, int j) { return (anc[i * W + (j >> 5)] >> (j & 31)) & 1u; };
     for (int w = threadIdx.x; w < words; w += blockDim.x) {
         const int at = head + 4 * w;
         int i = at / n, j = at - i * n;
@@ -323,7 +332,7 @@ __device__ __forceinline__ void mask_rows(int n, const int* par, const int* dep,
 __device__ __forceinline__ void fused_mask(const TreeArgs& a, int s, const TreeSmem& t) {
     if (!a.mask) return;
     const int n = a.B + 1;
-    mask_rows(n, t.o_par, t.o_dep, a.root_pos[s], 0, n, t.anc, a.mask + static_cast<size_t>(s) * n * n,
+    mask_rows<true>(n, t.o_par, t.o_dep, a.root_pos[s], 0, n, t.anc, a.mask + static_cast<size_t>(s) * n * n,
               a.pos_ids + static_cast<size_t>(s) * n);
 }
 
@@ -455,8 +464,7 @@ __device__ void build_tree_queue(const TreeArgs& a, int s, const TreeSmem& t, co
 }
 
 // ------------------------------------------------------------------------------------------
-// Builder with a sorted queue, for the one-token rule and the marginal modes with B <= 64 and
-// every reachable list entry staged. The same pops, tie rules and results as
+// Builder with a sorted queue, for B <= 64 (used up to 48) with every reachable list entry staged. The same pops, tie rules and results as
 // build_tree_queue. After t pops only the B - t best live entries can still be popped (each
 // needs every better entry popped first), and at most t + 1 entries are live (a pop replaces its
 // entry by the next sibling and adds at most the node's first child), so at most
@@ -473,7 +481,7 @@ constexpr int kFastThreads = 512;
 // lists (token and log-probability of every entry).
 __host__ __device__ inline size_t fast_tree_smem(int B, int gamma, int M, int rows, int sw, bool with_mask) {
     const size_t n = static_cast<size_t>(B) + 1;
-    size_t bytes = n * 16 + static_cast<size_t>(gamma) * M * 4;
+    size_t bytes = n * 20 + static_cast<size_t>(gamma) * M * 4;
     bytes = (bytes + 15) & ~static_cast<size_t>(15);
     if (with_mask) bytes += (tree_mask_words(static_cast<int>(n)) * 4 + 15) & ~static_cast<size_t>(15);
     return bytes + static_cast<size_t>(rows) * sw * 8 + 16;
@@ -483,6 +491,7 @@ __device__ __forceinline__ bool key_gt(uint32_t ahi, uint32_t alo, uint32_t bhi,
     return ahi > bhi || (ahi == bhi && alo > blo);
 }
 
+template <bool TWO>   // the two-previous-token rule
 __global__ void __launch_bounds__(kFastThreads) build_tree_fast_kernel(TreeArgs a, int sw) {
     pdl_trigger();
     pdl_wait();
@@ -499,7 +508,8 @@ __global__ void __launch_bounds__(kFastThreads) build_tree_fast_kernel(TreeArgs 
     int* o_par = o_tok + n_out;
     int* o_dep = o_par + n_out;
     float* o_score = reinterpret_cast<float*>(o_dep + n_out);
-    int* topm = reinterpret_cast<int*>(o_score + n_out);
+    int* o_m = reinterpret_cast<int*>(o_score + n_out);   // candidate index (two-token rule)
+    int* topm = o_m + n_out;
     size_t off = (static_cast<size_t>(reinterpret_cast<uint8_t*>(topm + a.gamma * a.M) - smem_raw) + 15) & ~static_cast<size_t>(15);
     uint32_t* anc = reinterpret_cast<uint32_t*>(smem_raw + off);
     if (a.mask) off += (tree_mask_words(n_out) * 4 + 15) & ~static_cast<size_t>(15);
@@ -552,7 +562,7 @@ __global__ void __launch_bounds__(kFastThreads) build_tree_fast_kernel(TreeArgs 
         const int lane = tid;
         const int list_len = a.K2 < sw ? a.K2 : sw;   // staged ranks; a pop never reaches rank sw
         int flags = 0;
-        const int root = a.root_tok[s];
+        const int root = a.root_tok[TWO ? 2 * s : s];
         if (root < 0 || root >= a.V) flags |= TF_DEV_BAD_TOKEN;
         uint32_t khi = 0u, klo = 0u;
         int rr = 0;
@@ -600,7 +610,10 @@ __global__ void __launch_bounds__(kFastThreads) build_tree_fast_kernel(TreeArgs 
                 const unsigned b1 = __ballot_sync(kFull, lane + 32 < a.M && c1 == tok);
                 m = b0 ? m : b1 ? 32 + __ffs(b1) - 1 : -1;
             }
-            const int crow = dep >= a.gamma ? -1 : !mary ? dep : m < 0 ? -1 : ar ? 1 + (dep - 1) * a.M + m : dep;
+            int crow = dep >= a.gamma ? -1 : !mary ? dep : m < 0 ? -1 : ar ? 1 + (dep - 1) * a.M + m : dep;
+            // two-token rule: the row of (this node's candidate, its parent's); the parent was expanded,
+            // so it has one
+            if (TWO && crow >= 0 && dep >= 2) crow = 1 + a.M + (dep - 2) * a.M * a.M + m * a.M + o_m[par];
             const bool sib_ok = rank + 1 < list_len;
             const float slp = l_lp[sib_ok ? idx + 1 : idx];
             const bool ch_ok = crow >= 0 && node + 1 < n_out;   // nothing is popped after the last node
@@ -612,6 +625,7 @@ __global__ void __launch_bounds__(kFastThreads) build_tree_fast_kernel(TreeArgs 
                 o_par[node] = par;
                 o_dep[node] = dep;
                 o_score[node] = sc;
+                if (TWO) o_m[node] = m;
             }
             // its successors, A before B in queue order (0 = none): the next sibling shares the
             // head's depth and parent (the low word of its key), the child is one level deeper
@@ -653,14 +667,14 @@ __global__ void __launch_bounds__(kFastThreads) build_tree_fast_kernel(TreeArgs 
         a.node_score[o] = o_score[i];
     }
     if (a.mask)
-        mask_rows(n_out, o_par, o_dep, a.root_pos[s], 0, n_out, anc, a.mask + static_cast<size_t>(s) * n_out * n_out,
+        mask_rows<false>(n_out, o_par, o_dep, a.root_pos[s], 0, n_out, anc, a.mask + static_cast<size_t>(s) * n_out * n_out,
                   a.pos_ids + static_cast<size_t>(s) * n_out);
 }
 
 // ------------------------------------------------------------------------------------------
 // Builder by levels, for large budgets. A pop sequence is a chain: with the queue in shared memory
-// 512 pops took 343 us on GB300, about 0.65 us each on one warp (46 us this way; 64 pops of the
-// two-token rule 44 us with the queue in registers, 25 us this way). But the B popped nodes are simply
+// 512 pops took 343 us on GB300, about 0.65 us each on one warp (41 us this way; 64 pops of the
+// two-token rule 44 us with the queue in registers, 18.5 us this way). But the B popped nodes are simply
 // the B first of all nodes in the order (score, smaller depth, earlier parent, earlier list entry),
 // as long as no node outscores its parent or its list predecessor (log-probabilities <= 0, lists
 // sorted): then the first B nodes contain every ancestor and predecessor of each of them. So the
@@ -678,23 +692,29 @@ constexpr int kLvWarps = kLvThreads / 32;
 constexpr int kLvCap = 4096;       // nodes held at once
 constexpr int kLvBins = 2 * kLvThreads;
 constexpr int kLvSort = 2048;      // nodes that can be sorted
+constexpr int kLvCount = 256;      // up to this many by counting
 constexpr int kLvTies = 32;        // ties resolved in place, and the longest run of equal nodes
 
+// Nodes to expand: the node (kNoNode: dropped), the next 32-entry chunk of its child list, the list.
+struct ActList {
+    int* row;
+    uint16_t* node;
+    uint8_t* chunk;
+};
 struct LevelSmem {
+    unsigned long long* key;   // [kLvSort]
     float* score;          // [kLvCap]; node 0 is the root
     int* tok;
+    int* hist;             // [kLvBins]
     uint16_t *par, *rank;
     uint16_t* place;       // new index in a compaction; 1 + place in the order at the end
-    uint16_t* act[2];      // parents still to expand (kNoNode: dropped) and the next list chunk of each
-    uint8_t* chunk[2];
     uint8_t* dep;
-    int8_t* m;             // candidate index of an expandable node (two-token rule), else -1
-    unsigned long long* key;   // [kLvSort]
-    int* hist;             // [kLvBins]
+    int8_t* m;             // candidate index of an expandable node (two-token rule)
+    ActList act[3];        // [kLvCap] each: this pass, the lists that go on, the next level
     int* topm;             // [gamma * M]
 };
 constexpr uint16_t kNoNode = 0xffff;
-constexpr size_t kLvFixedBytes = kLvCap * (4 + 4 + 2 + 2 + 2 + 4 + 2 + 1 + 1) + kLvSort * 8 + kLvBins * 4;
+constexpr size_t kLvFixedBytes = kLvCap * (4 + 4 + 2 + 2 + 2 + 1 + 1 + 3 * 7) + kLvSort * 8 + kLvBins * 4;
 __host__ __device__ inline size_t level_smem_bytes(int B, int gamma, int M, bool with_mask) {
     const size_t mine = kLvFixedBytes + static_cast<size_t>(gamma) * M * 4;
     const size_t queue = tree_smem_fixed(B, gamma, M, with_mask);
@@ -711,11 +731,12 @@ __device__ __forceinline__ LevelSmem level_smem(uint8_t* p) {
     t.score = reinterpret_cast<float*>(take(kLvCap * 4));
     t.tok = reinterpret_cast<int*>(take(kLvCap * 4));
     t.hist = reinterpret_cast<int*>(take(kLvBins * 4));
+    for (ActList& l : t.act) l.row = reinterpret_cast<int*>(take(kLvCap * 4));
     t.par = reinterpret_cast<uint16_t*>(take(kLvCap * 2));
     t.rank = reinterpret_cast<uint16_t*>(take(kLvCap * 2));
     t.place = reinterpret_cast<uint16_t*>(take(kLvCap * 2));
-    for (int i = 0; i < 2; ++i) t.act[i] = reinterpret_cast<uint16_t*>(take(kLvCap * 2));
-    for (int i = 0; i < 2; ++i) t.chunk[i] = take(kLvCap);
+    for (ActList& l : t.act) l.node = reinterpret_cast<uint16_t*>(take(kLvCap * 2));
+    for (ActList& l : t.act) l.chunk = take(kLvCap);
     t.dep = take(kLvCap);
     t.m = reinterpret_cast<int8_t*>(take(kLvCap));
     t.topm = reinterpret_cast<int*>(p);
@@ -734,7 +755,10 @@ __global__ void __launch_bounds__(kLvThreads) build_tree_level_kernel(TreeArgs a
     pdl_wait();
     extern __shared__ __align__(16) uint8_t smem_raw[];
     __shared__ float theta_s, wmin[kLvWarps];
-    __shared__ int wsum[kLvWarps], count_s, bad_s, n_act_s, n_ties_s, ties[kLvTies], flags_s;
+    // n_cont_s, n_next_s: lists that go on after a pass, nodes that the next level expands; a pass
+    // (level) uses one of three counters and zeroes the next one, whose last readers are a pass
+    // (level) behind
+    __shared__ int wsum[kLvWarps], count_s, bad_s, n_cont_s[3], n_next_s[3], n_keys_s, n_ties_s, ties[kLvTies], flags_s;
     constexpr unsigned kFull = 0xffffffffu;
     const LevelSmem t = level_smem(smem_raw);
     const int s = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -751,8 +775,10 @@ __global__ void __launch_bounds__(kLvThreads) build_tree_level_kernel(TreeArgs a
         t.par[0] = t.rank[0] = 0;
         t.dep[0] = 0;
         t.m[0] = -1;
-        t.act[0][0] = 0;
-        t.chunk[0][0] = 0;
+        t.act[0].node[0] = 0;
+        t.act[0].chunk[0] = 0;
+        t.act[0].row[0] = 0;
+        n_cont_s[0] = n_next_s[1] = 0;
         count_s = 1;
         bad_s = 0;
         flags_s = root < 0 || root >= a.V ? TF_DEV_BAD_TOKEN : 0;
@@ -803,9 +829,9 @@ __global__ void __launch_bounds__(kLvThreads) build_tree_level_kernel(TreeArgs a
         __syncthreads();
     };
 
-    // Drops the nodes below theta, keeping the others' order; `first` (the first node of the level)
-    // and the parents still to expand move along. Returns the new count.
-    auto compact = [&](int count, int& first, uint16_t* act, int n_act) {
+    // Drops the nodes below theta, keeping the others' order; the nodes still to expand (two lists) move
+    // along. Returns the new count.
+    auto compact = [&](int count, uint16_t* act, int n_act, uint16_t* next, int n_next) {
         constexpr int kPer = kLvCap / kLvThreads;
         const float theta = theta_s;
         float sc[kPer];
@@ -849,13 +875,8 @@ __global__ void __launch_bounds__(kLvThreads) build_tree_level_kernel(TreeArgs a
             base += keep[j] ? 1 : 0;
         }
         __syncthreads();
-        // the level's first kept node: the smallest new index at or after `first`
-        if (tid == 0) {
-            int f = first;
-            while (f < count && t.place[f] == kNoNode) ++f;
-            wsum[0] = f < count ? t.place[f] : total;
-        }
         for (int i = tid; i < n_act; i += kLvThreads) act[i] = act[i] == kNoNode ? kNoNode : t.place[act[i]];
+        for (int i = tid; i < n_next; i += kLvThreads) next[i] = next[i] == kNoNode ? kNoNode : t.place[next[i]];
         uint16_t to[kPer], np[kPer];
 #pragma unroll
         for (int j = 0; j < kPer; ++j)
@@ -864,7 +885,6 @@ __global__ void __launch_bounds__(kLvThreads) build_tree_level_kernel(TreeArgs a
                 np[j] = t.place[pr[j]];                  // a kept node's parent scores no less: kept
             }
         __syncthreads();
-        first = wsum[0];
 #pragma unroll
         for (int j = 0; j < kPer; ++j)
             if (keep[j]) {
@@ -880,20 +900,22 @@ __global__ void __launch_bounds__(kLvThreads) build_tree_level_kernel(TreeArgs a
         return total;
     };
 
-    int cur = 0, n_act = 1, count = 1, seen = 1;         // seen: the count at the last raise_theta
+    int li = 0, lc = 1, ln = 2;                          // act lists: this pass, going on, next level
+    int n_act = 1, count = 1, seen = 1, pass = 0;        // seen: the count at the last raise_theta
     for (int d = 1; d <= a.gamma && n_act > 0; ++d) {
         // the nodes of depth d: children of the n_act expandable nodes of depth d - 1
-        int first = count;
+        int& n_next = n_next_s[d % 3];
+        if (tid == 0) n_next_s[(d + 1) % 3] = 0;
+        const int* cand = t.topm + (d - 1) * a.M;
+        const bool deeper = d < a.gamma;
         int g = 32 / n_act;                              // list chunks taken of each parent per pass
         g = g < 1 ? 1 : g > n_chunks ? n_chunks : g;
         while (n_act > 0) {
-            uint16_t* act = t.act[cur];
-            uint8_t* chunk = t.chunk[cur];
-            uint16_t* nact = t.act[cur ^ 1];
-            uint8_t* nchunk = t.chunk[cur ^ 1];
+            const ActList act = t.act[li], cont = t.act[lc], next = t.act[ln];
             if (kLvCap - count < 32 * kLvWarps) {
+                __syncthreads();                         // (n_next is final for the passes so far)
                 raise_theta(count);
-                count = seen = compact(count, first, act, n_act);
+                count = seen = compact(count, act.node, n_act, next.node, n_next);
             }
             int nb = (kLvCap - count) / (32 * g);        // parents of this pass: all their entries fit
             nb = nb < n_act ? nb : n_act;
@@ -902,26 +924,16 @@ __global__ void __launch_bounds__(kLvThreads) build_tree_level_kernel(TreeArgs a
                 __syncthreads();
                 break;
             }
-            if (tid == 0) n_act_s = 0;
-            __syncthreads();
+            int& n_cont = n_cont_s[pass % 3];
+            if (tid == 0) n_cont_s[(pass + 1) % 3] = 0;
+            ++pass;
             const float theta = theta_s;
             for (int item = warp; item < nb * g; item += kLvWarps) {
-                const int pi = item / g, c = chunk[pi] + (item - pi * g);
-                const int p = act[pi];
+                const int pi = item / g, c = act.chunk[pi] + (item - pi * g);
+                const int p = act.node[pi], row = act.row[pi];
                 if (p == kNoNode || c >= n_chunks) continue;
                 const float ps = t.score[p];
                 if (ps < theta) continue;
-                int row;
-                if (d == 1) {
-                    row = 0;
-                } else if (!ar) {
-                    row = d - 1;
-                } else {
-                    const int m = t.m[p];
-                    row = !a.two_prev ? 1 + (d - 2) * a.M + m
-                          : d == 2    ? 1 + m
-                                      : 1 + a.M + (d - 3) * a.M * a.M + m * a.M + t.m[t.par[p]];
-                }
                 const int rank = c * 32 + lane;
                 const bool in = rank < a.K2;
                 const float lp = in ? lists.lp(row, rank) : 0.0f;
@@ -940,108 +952,146 @@ __global__ void __launch_bounds__(kLvThreads) build_tree_level_kernel(TreeArgs a
                     base = atomicAdd(&count_s, __popc(bal));
                     // every entry so far counts: the list goes on in the next pass
                     if (item - pi * g == g - 1 && bal == kFull && c + 1 < n_chunks) {
-                        const int q = atomicAdd(&n_act_s, 1);
-                        nact[q] = static_cast<uint16_t>(p);
-                        nchunk[q] = static_cast<uint8_t>(c + 1);
+                        const int q = atomicAdd(&n_cont, 1);
+                        cont.node[q] = static_cast<uint16_t>(p);
+                        cont.chunk[q] = static_cast<uint8_t>(c + 1);
+                        cont.row[q] = row;
                     }
                 }
                 base = __shfl_sync(kFull, base, 0);
-                if (take) {
-                    const int i = base + __popc(bal & ((1u << lane) - 1u));
-                    t.score[i] = sc;
-                    t.tok[i] = tok;
-                    t.par[i] = static_cast<uint16_t>(p);
-                    t.rank[i] = static_cast<uint16_t>(rank);
-                    t.dep[i] = static_cast<uint8_t>(d);
-                    t.m[i] = -1;
+                if (!take) continue;
+                const int i = base + __popc(bal & ((1u << lane) - 1u));
+                // expandable? (M-ary rule: the first equal candidate of its depth) and its child list
+                int m = -1, crow = -1;
+                if (deeper) {
+                    if (!mary) {
+                        crow = d;
+                    } else {
+                        for (int j = a.M - 1; j >= 0; --j) m = cand[j] == tok ? j : m;
+                        if (m >= 0)
+                            crow = !ar              ? d
+                                   : !a.two_prev    ? 1 + (d - 1) * a.M + m
+                                   : d == 1         ? 1 + m
+                                                    : 1 + a.M + (d - 2) * a.M * a.M + m * a.M + t.m[p];
+                    }
+                }
+                t.score[i] = sc;
+                t.tok[i] = tok;
+                t.par[i] = static_cast<uint16_t>(p);
+                t.rank[i] = static_cast<uint16_t>(rank);
+                t.dep[i] = static_cast<uint8_t>(d);
+                t.m[i] = static_cast<int8_t>(m);
+                if (crow >= 0) {
+                    const int q = atomicAdd(&n_next, 1);
+                    if (q < kLvCap) {
+                        next.node[q] = static_cast<uint16_t>(i);
+                        next.chunk[q] = 0;
+                        next.row[q] = crow;
+                    } else {
+                        bad_s = 1;                       // (dropped nodes keep their entries)
+                    }
                 }
             }
             __syncthreads();
             count = count_s;
-            const int more = n_act_s, rest = n_act - nb;
-            if (bad_s) break;                            // (uniform: written before the barrier)
-            for (int i = tid; i < rest; i += kLvThreads) {
-                nact[more + i] = act[nb + i];
-                nchunk[more + i] = chunk[nb + i];
+            const int more = n_cont, rest = n_act - nb;
+            const bool bad = bad_s != 0;
+            __syncthreads();                             // everyone has read them before the next pass writes
+            if (bad) break;
+            if (rest > 0) {                              // parents left out of this pass
+                for (int i = tid; i < rest; i += kLvThreads) {
+                    cont.node[more + i] = act.node[nb + i];
+                    cont.chunk[more + i] = act.chunk[nb + i];
+                    cont.row[more + i] = act.row[nb + i];
+                }
+                __syncthreads();
             }
             n_act = more + rest;
-            cur ^= 1;
-            if (count - seen >= (a.B >> 3) || n_act > 0) {
-                __syncthreads();
+            const int old = li;
+            li = lc;
+            lc = old;
+            if (count - seen >= (a.B >> 2) || n_act > 0) {
                 raise_theta(count);
                 seen = count;
             }
-            __syncthreads();
         }
-        __syncthreads();
-        if (bad_s) break;
-        n_act = 0;
-        if (d < a.gamma) {
-            // the expandable nodes of depth d
-            if (tid == 0) n_act_s = 0;
-            __syncthreads();
+        if (n_act > 0) break;                            // (left by one of the breaks above)
+        n_act = n_next;
+        const int old = li;
+        li = ln;
+        ln = old;
+        if (n_act > 2 * kLvWarps) {                      // many: only those that theta leaves
+            const ActList all = t.act[li], few = t.act[lc];
+            int& n_few = n_cont_s[pass % 3];
+            if (tid == 0) n_cont_s[(pass + 1) % 3] = 0;
+            ++pass;
             const float theta = theta_s;
-            const int* cand = t.topm + (d - 1) * a.M;
-            for (int i = first + tid; i < count; i += kLvThreads) {
-                if (t.score[i] < theta) continue;
-                if (mary) {
-                    const int tok = t.tok[i];
-                    int m = -1;
-                    for (int j = 0; j < a.M; ++j)
-                        if (cand[j] == tok) {
-                            m = j;
-                            break;
-                        }
-                    if (m < 0) continue;
-                    t.m[i] = static_cast<int8_t>(m);
-                }
-                const int q = atomicAdd(&n_act_s, 1);
-                t.act[cur][q] = static_cast<uint16_t>(i);
-                t.chunk[cur][q] = 0;
+            for (int i = tid; i < n_act; i += kLvThreads) {
+                const uint16_t p = all.node[i];
+                if (p == kNoNode || t.score[p] < theta) continue;
+                const int q = atomicAdd(&n_few, 1);
+                few.node[q] = p;
+                few.chunk[q] = 0;
+                few.row[q] = all.row[i];
             }
             __syncthreads();
-            n_act = n_act_s;
+            n_act = n_few;
+            __syncthreads();
+            const int o = li;
+            li = lc;
+            lc = o;
         }
     }
+    __syncthreads();
 
     // ---- the order of the survivors
     int n = 0;
     if (!bad_s) {
+        if (tid == 0) n_keys_s = n_ties_s = 0;
         raise_theta(count);
-        __syncthreads();
-        if (tid == 0) {
-            n_act_s = 0;
-            n_ties_s = 0;
-        }
         __syncthreads();
         const float theta = theta_s;
         for (int i = 1 + tid; i < count; i += kLvThreads)
             if (t.score[i] >= theta) {
-                const int q = atomicAdd(&n_act_s, 1);
+                const int q = atomicAdd(&n_keys_s, 1);
                 if (q < kLvSort) t.key[q] = level_key(t.score[i], t.dep[i], t.rank[i], i);
             }
         __syncthreads();
-        n = n_act_s;
+        n = n_keys_s;
         if (n > kLvSort) {
             if (tid == 0) bad_s = 1;
         } else {
-            int N = 64;
-            while (N < n) N <<= 1;
-            for (int i = n + tid; i < N; i += kLvThreads) t.key[i] = 0ull;
-            // bitonic sort, largest key first
-            for (int size = 2; size <= N; size <<= 1)
-                for (int step = size >> 1; step > 0; step >>= 1) {
-                    __syncthreads();
-                    for (int q = tid; q < N / 2; q += kLvThreads) {
-                        const int i = 2 * q - (q & (step - 1)), j = i + step;
-                        const unsigned long long x = t.key[i], y = t.key[j];
-                        if ((x < y) == ((i & size) == 0)) {
-                            t.key[i] = y;
-                            t.key[j] = x;
+            if (n <= kLvCount) {
+                // few: each key's place by counting the larger ones
+                unsigned long long x = 0ull;
+                int r = 0;
+                if (tid < n) {
+                    x = t.key[tid];
+#pragma unroll 8
+                    for (int i = 0; i < n; ++i) r += t.key[i] > x ? 1 : 0;
+                }
+                __syncthreads();
+                if (tid < n) t.key[r] = x;
+                __syncthreads();
+            } else {
+                // bitonic sort, largest key first
+                int N = kLvCount;
+                while (N < n) N <<= 1;
+                for (int i = n + tid; i < N; i += kLvThreads) t.key[i] = 0ull;
+                for (int size = 2; size <= N; size <<= 1)
+                    for (int step = size >> 1; step > 0; step >>= 1) {
+                        __syncthreads();
+                        for (int q = tid; q < N / 2; q += kLvThreads) {
+                            const int i = 2 * q - (q & (step - 1)), j = i + step;
+                            const unsigned long long x = t.key[i], y = t.key[j];
+                            if ((x < y) == ((i & size) == 0)) {
+                                t.key[i] = y;
+                                t.key[j] = x;
+                            }
                         }
                     }
-                }
-            __syncthreads();
+                __syncthreads();
+            }
             for (int i = tid; i < n; i += kLvThreads) {
                 const unsigned long long x = t.key[i];
                 const int xi = static_cast<int>(x & 0xfff);
@@ -1129,7 +1179,7 @@ __global__ void __launch_bounds__(kLvThreads) build_tree_level_kernel(TreeArgs a
     __syncthreads();
     if (tid == 0) a.dev_status[s] = sequence_status(a, flags_s);
     if (a.mask)
-        mask_rows(n_out, t.hist, t.hist + kFusedMaskMaxNodes, a.root_pos[s], 0, n_out, reinterpret_cast<uint32_t*>(t.key),
+        mask_rows<true>(n_out, t.hist, t.hist + kFusedMaskMaxNodes, a.root_pos[s], 0, n_out, reinterpret_cast<uint32_t*>(t.key),
                   a.mask + static_cast<size_t>(s) * n_out * n_out, a.pos_ids + o0);
 }
 
@@ -1159,7 +1209,7 @@ __global__ void __launch_bounds__(256) tree_mask_kernel(int n, const int32_t* __
         dep[i] = D[i];
     }
     __syncthreads();
-    mask_rows(n, par, dep, root_pos[s], r0, r1, anc, mask + static_cast<size_t>(s) * n * n,
+    mask_rows<true>(n, par, dep, root_pos[s], r0, r1, anc, mask + static_cast<size_t>(s) * n * n,
               pos_ids + static_cast<size_t>(s) * n);
 }
 
@@ -1492,16 +1542,17 @@ cudaError_t launch_build_tree(const Ctx& ctx, int b, int gamma, int M, int K1, i
     const int rows_l = mode == TF_MODE_AR ? R : gamma;
     const int stride = mode == TF_MODE_AR ? K2 : K1;
     const int sw = stride < B + 1 ? stride : B + 1;   // list entries that a tree can reach
-    // The sorted-queue builder for the one-token rule and the marginal modes with B <= 64 and every
-    // reachable entry in shared memory: its cost is the pops (0.25 us each), the builder by levels
-    // pays 1 to 1.5 us per level and pass whatever the budget. Measured on GB300 (16 depths, one
-    // sequence): B = 32 13.8 against 16.7 us, B = 64 21.4 against 23.0.
+    // The sorted-queue builder for small budgets with every reachable entry in shared memory: its cost is
+    // the pops (0.25 us each, more with the two-token rule); the builder by levels pays about a
+    // microsecond per level whatever the budget. Measured on GB300 (16 depths, one sequence): B = 32
+    // 12.0 against 13.1 us, B = 48 16.7 against 16.5, B = 64 21.3 against 17.3; two-token rule (12
+    // depths) B = 32 13.2 against 14.3, B = 64 22.8 against 17.1.
     const size_t fsm = fast_tree_smem(B, gamma, M, rows_l, sw, mask != nullptr);
-    if (!a.two_prev && B <= 64 && fsm <= kTreeSmemLimit) {
-        cudaError_t e = cudaFuncSetAttribute(build_tree_fast_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             static_cast<int>(fsm));
+    if (B <= (a.two_prev ? 32 : 48) && fsm <= kTreeSmemLimit) {
+        auto kern = a.two_prev ? build_tree_fast_kernel<true> : build_tree_fast_kernel<false>;
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(fsm));
         if (e != cudaSuccess) return e;
-        e = launch_pdl(build_tree_fast_kernel, dim3(b), dim3(kFastThreads), fsm, ctx.stream, a, sw);
+        e = launch_pdl(kern, dim3(b), dim3(kFastThreads), fsm, ctx.stream, a, sw);
         return e != cudaSuccess ? e : cudaGetLastError();
     }
     const size_t lsm = level_smem_bytes(B, gamma, M, mask != nullptr);

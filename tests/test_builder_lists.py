@@ -2,9 +2,9 @@
 bit for bit (tokens, parents, depths, scores, status). Log-probabilities are multiples of 1/8 (or
 1/4096) in [-6, 0], so every path score is exact in fp32 and fp64 alike and equal scores are frequent
 (or a few per tree: the tie rules decide many pops, or some); a random share of every list's tokens are stage-1 candidates of the
-list's depth, so the M-ary rule expands often and the trees grow deep and wide. Budgets up to 64
-run the sorted-queue builder, larger ones and the two-token rule the builder by levels, which hands
-trees with many ties to the queue in shared memory."""
+list's depth, so the M-ary rule expands often and the trees grow deep and wide. Budgets up to 48
+(two-token rule: 32) run the sorted-queue builder, larger ones the builder by levels, which hands trees
+with many ties to the queue in shared memory."""
 import numpy as np
 import pytest
 import torch
@@ -112,7 +112,8 @@ O_UNDERFULL = 2   # TF_DEV_UNDERFULL
 
 LEVEL_CASES = [
     # mode, batch, gamma, M, K2, B, V, two-token rule
-    ("ar", 3, 16, 16, 65, 65, 3000, False),       # the smallest budget of the builder by levels
+    ("ar", 3, 16, 16, 48, 48, 3000, False),       # the largest budget of the sorted queue
+    ("ar", 3, 16, 16, 49, 49, 3000, False),       # the smallest of the builder by levels
     ("ar", 2, 16, 16, 512, 512, 5000, False),     # exact lists, sixteen chunks per list
     ("ar", 2, 4, 64, 500, 1023, 5000, False),     # the largest budget, wide branching: nodes dropped as theta rises
     ("ar", 2, 16, 5, 33, 300, 2000, False),       # a list of one chunk and one entry; K2 < B
@@ -120,7 +121,8 @@ LEVEL_CASES = [
     ("ar", 2, 1, 4, 100, 100, 500, False),        # one level
     ("marginal", 2, 6, 4, 256, 256, 1000, False),  # every node expands
     ("marginal_mary", 2, 12, 20, 130, 127, 2000, False),
-    ("ar", 2, 8, 4, 40, 40, 1000, True),          # two-token rule: small, register-sized and large budgets
+    ("ar", 2, 8, 4, 32, 32, 1000, True),          # two-token rule: the sorted queue, and by levels
+    ("ar", 2, 8, 4, 40, 40, 1000, True),
     ("ar", 2, 6, 5, 100, 100, 1000, True),
     ("ar", 1, 5, 6, 200, 300, 1000, True),
 ]
