@@ -1010,7 +1010,7 @@ __global__ void __launch_bounds__(kLvThreads) build_tree_level_kernel(TreeArgs a
             const int old = li;
             li = lc;
             lc = old;
-            if (count - seen >= (a.B >> 2) || n_act > 0) {
+            if (count - seen >= (a.B >> 1) || n_act > 0) {
                 raise_theta(count);
                 seen = count;
             }
