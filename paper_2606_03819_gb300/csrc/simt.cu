@@ -64,15 +64,7 @@ __device__ __forceinline__ void copy_commit() { asm volatile("cp.async.commit_gr
 template <int N>
 __device__ __forceinline__ void copy_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
-// a * b + c on two packed fp32 values, each rounded to nearest.
-__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b, unsigned long long c) {
-    unsigned long long d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
-__device__ __forceinline__ float sum2(unsigned long long v) {
-    return __uint_as_float(static_cast<uint32_t>(v)) + __uint_as_float(static_cast<uint32_t>(v >> 32));
-}
+__device__ __forceinline__ float sum2(unsigned long long v) { return f2_lo(v) + f2_hi(v); }
 
 // rows [r0, r0 + n) of a [.., K] matrix (n <= 0: none)
 struct RowsOf {
@@ -145,9 +137,9 @@ __device__ __forceinline__ void mainloop(float* ring, const RowsOf& lo, const Ro
             for (int i = 0; i < 8; ++i) {
                 const ulonglong2 wv = *reinterpret_cast<const ulonglong2*>(wk + 16 * i * kLd + k);
 #pragma unroll
-                for (int j = 0; j < TR; ++j) acc[i][j] = fma2(wv.x, xv[j].x, acc[i][j]);
+                for (int j = 0; j < TR; ++j) acc[i][j] = f2_fma(wv.x, xv[j].x, acc[i][j]);
 #pragma unroll
-                for (int j = 0; j < TR; ++j) acc[i][j] = fma2(wv.y, xv[j].y, acc[i][j]);
+                for (int j = 0; j < TR; ++j) acc[i][j] = f2_fma(wv.y, xv[j].y, acc[i][j]);
             }
         }
         cur = cur + 1 == kStages ? 0 : cur + 1;

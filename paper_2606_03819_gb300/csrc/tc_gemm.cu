@@ -112,55 +112,74 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
     return *reinterpret_cast<uint32_t*>(&v);
 }
 
-// Summary of one 32-column chunk of one row: logits of vocabulary ids v0 .. v0+31. The three
-// largest values, the chunk-local offsets of the first two (the smaller id first among equals)
-// and the sum of exp(z - max) come from one fixed tree over the 32 registers: the same
-// instructions for every lane whatever the data (a per-lane sorted insertion would diverge across
-// the warp's 32 rows). Each node carries its subtree's top three and its sum of exp(z - node
-// max), so a logit is dead once its leaf is formed; the tree is expanded depth first to keep
-// few nodes live.
-struct ChunkNode {
-    float a1, a2, a3, s;  // a1 >= a2 >= a3; s = sum over the subtree of exp(z - a1)
-    int i1, i2;           // chunk-local offsets of a1, a2
+// Summary of one 32-column chunk of one row: the three largest logits, the chunk-local offsets of the
+// first two (the smaller first among equals) and the sum of exp(z - max). The same instructions for
+// every lane whatever the data (a per-lane sorted insertion would diverge across the warp's 32 rows).
+// What bounds it is the instructions issued: with d of 512 to 2048 the epilogue, not the contraction,
+// sets the pace of the LM head. The three values come from a network of min/max (a merge of two sorted
+// triples: a third largest is one of two thirds and two cross minima), the offsets from four selects
+// per merge, and the exponentials from one pass over the values once the maximum is known, in packed
+// pairs: about 360 instructions per chunk, where a tree whose every node rescaled its sum of
+// exponentials took 1040 (V = 151936, 256 rows: d = 512 66 -> 47 us, d = 1024 78 -> 64, d = 2048 122 ->
+// 115, d = 4096 222 -> 217 on GB300).
+struct Top3 {
+    float a1, a2, a3;  // a1 >= a2 >= a3
+    int i1, i2;        // offsets of a1, a2
 };
-__device__ __forceinline__ float chunk_logit(uint32_t r, int v, int V, float inv_temp) {
-    return v < V ? __uint_as_float(r) * inv_temp : -INFINITY;
-}
-// p covers smaller ids than q, so on equal values p's entry ranks first.
-__device__ __forceinline__ ChunkNode chunk_merge(const ChunkNode& p, const ChunkNode& q) {
-    const bool pw = p.a1 >= q.a1;
-    const ChunkNode& w = pw ? p : q;
-    const ChunkNode& l = pw ? q : p;
-    // the winner's second against the loser's first; p's ids rank first on equal values
-    const bool sw = pw ? (w.a2 >= l.a1) : (w.a2 > l.a1);
-    ChunkNode n;
-    n.a1 = w.a1;
-    n.i1 = w.i1;
-    n.a2 = sw ? w.a2 : l.a1;
-    n.i2 = sw ? w.i2 : l.i1;
-    n.a3 = sw ? fmaxf(w.a3, l.a1) : fmaxf(w.a2, l.a2);
-    n.s = w.s + (l.a1 > -INFINITY ? l.s * __expf(l.a1 - w.a1) : 0.0f);
-    return n;
+// p covers smaller offsets than q, so on equal values p's entry ranks first.
+__device__ __forceinline__ void top3_first_two(const Top3& p, const Top3& q, int winner_second, Top3& n) {
+    const float t = fminf(p.a1, q.a1);
+    n.a1 = fmaxf(p.a1, q.a1);
+    n.a2 = fmaxf(fmaxf(p.a2, q.a2), t);
+    // the winner's second against the loser's first (whichever of the two tests does not apply is false)
+    const bool second = p.a2 >= q.a1 || q.a2 > p.a1;
+    n.i2 = second ? winner_second : (p.a1 >= q.a1 ? q.i1 : p.i1);
 }
 template <int OFF, int N>
-__device__ __forceinline__ ChunkNode chunk_tree(const uint32_t (&r)[32], int v0, int V, float inv_temp) {
-    if constexpr (N == 2) {
-        const float x = chunk_logit(r[OFF], v0 + OFF, V, inv_temp);
-        const float y = chunk_logit(r[OFF + 1], v0 + OFF + 1, V, inv_temp);
-        const bool ge = x >= y;
-        ChunkNode n;
-        n.a1 = ge ? x : y;
-        n.a2 = ge ? y : x;
-        n.i1 = ge ? OFF : OFF + 1;
-        n.i2 = ge ? OFF + 1 : OFF;
-        n.a3 = -INFINITY;
-        n.s = n.a1 > -INFINITY ? 1.0f + __expf(n.a2 - n.a1) : 0.0f;
-        return n;
+__device__ __forceinline__ Top3 top3(const float (&z)[32]) {
+    static_assert(N >= 4, "");
+    Top3 n;
+    if constexpr (N == 4) {
+        Top3 p, q;   // pairs: a3 and i2 unused
+        const bool g0 = z[OFF] >= z[OFF + 1], g1 = z[OFF + 2] >= z[OFF + 3];
+        p.a1 = fmaxf(z[OFF], z[OFF + 1]);
+        p.a2 = fminf(z[OFF], z[OFF + 1]);
+        p.i1 = g0 ? OFF : OFF + 1;
+        q.a1 = fmaxf(z[OFF + 2], z[OFF + 3]);
+        q.a2 = fminf(z[OFF + 2], z[OFF + 3]);
+        q.i1 = g1 ? OFF + 2 : OFF + 3;
+        n.i1 = p.a1 >= q.a1 ? p.i1 : q.i1;
+        top3_first_two(p, q, n.i1 ^ 1, n);
+        n.a3 = fmaxf(fminf(p.a2, q.a1), fminf(p.a1, q.a2));
     } else {
-        const ChunkNode p = chunk_tree<OFF, N / 2>(r, v0, V, inv_temp);
-        const ChunkNode q = chunk_tree<OFF + N / 2, N / 2>(r, v0, V, inv_temp);
-        return chunk_merge(p, q);
+        const Top3 p = top3<OFF, N / 2>(z), q = top3<OFF + N / 2, N / 2>(z);
+        const bool pw = p.a1 >= q.a1;
+        n.i1 = pw ? p.i1 : q.i1;
+        top3_first_two(p, q, pw ? p.i2 : q.i2, n);
+        n.a3 = fmaxf(fmaxf(fmaxf(p.a3, q.a3), fminf(p.a2, q.a1)), fminf(p.a1, q.a2));
     }
+    return n;
+}
+__device__ __forceinline__ float ex2(float x) {
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+// sum of exp(z - m) over a chunk whose two largest values are m = t.a1 and t.a2
+__device__ __forceinline__ float sum_exp(const float (&z)[32], const Top3& t) {
+    constexpr float kLog2e = 1.4426950408889634f;
+    const unsigned long long m2 = f2_pack(t.a1, t.a1), l2 = f2_pack(kLog2e, kLog2e);
+    unsigned long long s[4];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+        const unsigned long long x = f2_mul(f2_sub(f2_pack(z[2 * i], z[2 * i + 1]), m2), l2);
+        const unsigned long long e = f2_pack(ex2(f2_lo(x)), ex2(f2_hi(x)));
+        s[i & 3] = i < 4 ? e : f2_add(s[i & 3], e);
+    }
+    const unsigned long long u = f2_add(f2_add(s[0], s[1]), f2_add(s[2], s[3]));
+    const float sum = f2_lo(u) + f2_hi(u);
+    if (t.a1 == INFINITY) return t.a2 == INFINITY ? NAN : 1.0f;   // (inf - inf above)
+    return t.a1 > -INFINITY ? sum : 0.0f;                         // no entry in the chunk
 }
 
 // VAR: the tile is ep.bn <= BN columns wide and the ring has ep.stages <= STAGES stages.
@@ -590,54 +609,43 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant
                 const Partials& P = ep.partials;
                 // warps whose 32 rows are all padding skip the accumulators entirely
                 if (row - lane < n_rows) {
-                    float hm = -INFINITY, hsum = 0.0f, hbv = -INFINITY;
-                    int hbid = -1;
-                    // half summary; chunks arrive in id order, so strict > keeps the smaller id
-                    auto fold = [&](const ChunkNode& c, int ci, int v0) {
-                        if (c.a1 > hbv) {
-                            hbv = c.a1;
-                            hbid = v0 + c.i1;
+                    float cm[kHalf], cs[kHalf];          // max and sum of each chunk
+                    float hm = -INFINITY;
+                    int hid = -1;
+                    // one chunk at a time (a second one in flight would not fit the registers; the other
+                    // warps of the scheduler cover the TMEM load)
+#pragma unroll
+                    for (int j = 0; j < kHalf; ++j) {
+                        const int ci = half * kHalf + j, v0 = nt * BN + ci * kChunk;
+                        uint32_t ra[32];
+                        ptx::tmem_ld_32cols(tb + ci * kChunk, ra);
+                        float z[32];
+#pragma unroll
+                        for (int i = 0; i < 32; ++i) z[i] = __uint_as_float(ra[i]);
+                        if (ep.inv_temp != 1.0f) {
+#pragma unroll
+                            for (int i = 0; i < 32; ++i) z[i] *= ep.inv_temp;
                         }
-                        if (c.a1 > -INFINITY) {
-                            const float mn = fmaxf(hm, c.a1);
-                            hsum = hsum * __expf(hm - mn) + c.s * __expf(c.a1 - mn);
-                            hm = mn;
+                        if (v0 + kChunk > ep.V) {
+#pragma unroll
+                            for (int i = 0; i < 32; ++i) z[i] = v0 + i < ep.V ? z[i] : -INFINITY;
+                        }
+                        const Top3 t = top3<0, 32>(z);
+                        cm[j] = t.a1;
+                        cs[j] = sum_exp(z, t);
+                        // chunks arrive in id order, so strict > keeps the smaller id
+                        if (t.a1 > hm) {
+                            hm = t.a1;
+                            hid = v0 + t.i1;
                         }
                         if (row < n_rows)
-                            P.chunks[P.chunk_at(nt, ci, row)] =
-                                make_float4(c.a1, c.a2, c.a3, __int_as_float(c.i1 | (c.i2 << 8)));
-                    };
-                    // Chunks in pairs: both TMEM loads in flight together, the two trees independent
-                    // of each other (so their instructions interleave), and the next pair's loads
-                    // issued before this pair is folded and stored.
-                    const int cb = half * kHalf;
-                    uint32_t ra[32], rb[32];
-                    ptx::tmem_ld_32cols_nowait(tb + cb * kChunk, ra);
-                    ptx::tmem_ld_32cols_nowait(tb + (cb + 1) * kChunk, rb);
-                    ptx::tmem_wait_ld_regs(ra);
-                    ptx::tmem_wait_ld_regs(rb);
-#pragma unroll
-                    for (int pr = 0; pr < kHalf / 2; ++pr) {
-                        const int ci = cb + 2 * pr;
-                        const int v0 = nt * BN + ci * kChunk;
-                        const ChunkNode c0 = chunk_tree<0, 32>(ra, v0, ep.V, ep.inv_temp);
-                        const ChunkNode c1 = chunk_tree<0, 32>(rb, v0 + kChunk, ep.V, ep.inv_temp);
-                        const bool more = pr + 1 < kHalf / 2;
-                        if (more) {
-                            __syncwarp();   // converged for the warp-collective TMEM loads
-                            ptx::tmem_ld_32cols_nowait(tb + (ci + 2) * kChunk, ra);
-                            ptx::tmem_ld_32cols_nowait(tb + (ci + 3) * kChunk, rb);
-                        }
-                        fold(c0, ci, v0);
-                        fold(c1, ci + 1, v0 + kChunk);
-                        if (more) {
-                            __syncwarp();
-                            ptx::tmem_wait_ld_regs(ra);
-                            ptx::tmem_wait_ld_regs(rb);
-                        }
+                            P.chunks[P.chunk_at(nt, ci, row)] = make_float4(t.a1, t.a2, t.a3, __int_as_float(t.i1 | (t.i2 << 8)));
+                        __syncwarp();   // converged for the warp-collective TMEM loads
                     }
-                    if (row < n_rows)
-                        P.halves[P.half_at(nt, half, row)] = make_float4(hm, hsum, hbv, __int_as_float(hbid));
+                    float hsum = 0.0f;
+#pragma unroll
+                    for (int j = 0; j < kHalf; ++j) hsum += cm[j] > -INFINITY ? cs[j] * __expf(cm[j] - hm) : 0.0f;
+                    if (row < n_rows) P.halves[P.half_at(nt, half, row)] = make_float4(hm, hsum, hm, __int_as_float(hid));
                 }
                 release_slot(g);
             } else if constexpr (VAR) {

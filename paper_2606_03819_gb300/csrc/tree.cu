@@ -1285,32 +1285,6 @@ __device__ __forceinline__ __nv_bfloat16 bf16_round_sum(float r, float t) {
     return __ushort_as_bfloat16(static_cast<unsigned short>(bits >> 16));
 }
 
-// ---- packed pairs of fp32 values (two independent operations per instruction)
-__device__ __forceinline__ unsigned long long f2_pack(float lo, float hi) {
-    return static_cast<unsigned long long>(__float_as_uint(hi)) << 32 | __float_as_uint(lo);
-}
-__device__ __forceinline__ float f2_lo(unsigned long long v) { return __uint_as_float(static_cast<uint32_t>(v)); }
-__device__ __forceinline__ float f2_hi(unsigned long long v) { return __uint_as_float(static_cast<uint32_t>(v >> 32)); }
-__device__ __forceinline__ unsigned long long f2_add(unsigned long long a, unsigned long long b) {
-    unsigned long long d;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-__device__ __forceinline__ unsigned long long f2_sub(unsigned long long a, unsigned long long b) {
-    unsigned long long d;
-    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-__device__ __forceinline__ unsigned long long f2_mul(unsigned long long a, unsigned long long b) {
-    unsigned long long d;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-__device__ __forceinline__ unsigned long long f2_fma(unsigned long long a, unsigned long long b, unsigned long long c) {
-    unsigned long long d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
 // the two bf16 values of a 32-bit word
 __device__ __forceinline__ unsigned long long f2_bf16x2(uint32_t w) {
     return f2_pack(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u));
