@@ -71,6 +71,10 @@ struct EpiParams {
     int* sem;
     // kernels with a width chosen at launch: columns per N tile (a multiple of 8) and ring stages
     int bn, stages;
+    // LMHEAD with single CTAs and at most 64 (32) rows: 2 (4) copies of the rows, one per half (quarter)
+    // of the TMEM lanes, so that all epilogue warps share the chunks of a block; otherwise 1. x_rows:
+    // rows that a copy of X brings in (tmap_x's box)
+    int copies, x_rows;
 };
 
 // Work unit u -> (N tile, M-tile group, K split); consecutive units share the N tile and K split
@@ -196,6 +200,9 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant
     using C = TileCfg<MT, NB, BN, STAGES, kPair, VAR>;
     static_assert(CL == 1 || kSplitK || (CL == 2 && MT == 1), "a CTA of a pair holds one M-tile");
     static_assert(!kSplitK || (CL == 4 && kMaxKSplits == 4 && (VAR || (MT == 2 && BN == 128))), "cluster split-K");
+    constexpr bool kCopies = EPI == EPI_LMHEAD && CL == 1;
+    // copies: half summaries of the copies' chunks, [group][half][parity of the unit][copy][row]
+    __shared__ float4 copy_sums[kCopies ? 2 * 2 * 2 * kBM : 1];
     constexpr bool kShare = kSplitK && VAR && MT == 1;   // both epilogue groups work on one accumulator
     static_assert(!VAR || (!kPair && EPI != EPI_LMHEAD), "variable width: single CTAs and K-splitting clusters");
     pdl_trigger();
@@ -316,12 +323,14 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant
             const uint64_t pol_w = w_stream_once ? ptx::policy_evict_first() : ptx::policy_evict_last();
             // Pair: both CTAs' copies of a stage complete on the even CTA's full barrier, which
             // the even CTA alone arms with the bytes of both halves.
-            const uint32_t tx_bytes = (kPair ? 2 : 1) * stage_bytes;
+            const int copies = kCopies ? ep.copies : 1;
+            const uint32_t tx_bytes = kCopies ? copies * ep.x_rows * kBK * 2 + C::kBBytes : (kPair ? 2 : 1) * stage_bytes;
             auto load_x = [&](uint8_t* sp, uint64_t* bar, int j, int kb, int mt) {
                 if constexpr (kPair)
                     ptx::tma_load_2d_pair(sp + j * C::kABytes, &tmap_x, in_leader(bar), kb * kBK, mt * kBM, pol_x);
                 else
-                    ptx::tma_load_2d(sp + j * C::kABytes, &tmap_x, bar, kb * kBK, mt * kBM, pol_x);
+                    for (int c = 0; c < copies; ++c)
+                        ptx::tma_load_2d(sp + j * C::kABytes + c * (C::kABytes / copies), &tmap_x, bar, kb * kBK, mt * kBM, pol_x);
             };
             // Weight tiles of one stage; in a pair each CTA stages its half of the rows
             // (one weight matrix: tmap_w0's box is BN / 2 rows high; two: BN, one matrix per CTA).
@@ -604,19 +613,30 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant
                 // the accumulators are summed across the cluster below, once every CTA has them
             } else if constexpr (EPI == EPI_LMHEAD) {
                 static_assert(BN == kBlockV, "one LM-head N tile is one vocabulary block");
-                // this warp's half of the block: chunks [half * 4, half * 4 + 4)
+                // this warp's chunks: a half of the block, or with copies of the rows its copy's part
                 constexpr int kHalf = kChunks / 2;
                 const Partials& P = ep.partials;
-                // warps whose 32 rows are all padding skip the accumulators entirely
-                if (row - lane < n_rows) {
-                    float cm[kHalf], cs[kHalf];          // max and sum of each chunk
-                    float hm = -INFINITY;
-                    int hid = -1;
+                const int copies = kCopies ? ep.copies : 1;
+                const int per = kHalf / copies;          // chunks of this warp
+                const int copy = q * copies / 4;         // (4 / copies row quarters per copy)
+                const int crow = kCopies ? row - copy * (kBM / copies) : row;
+                // warps whose 32 rows are all padding skip the accumulators entirely (with copies there
+                // are none)
+                const bool on = crow - lane < n_rows;
+                float cm[kHalf], cs[kHalf];              // max and sum of each chunk
+                float hm = -INFINITY;
+                int hid = -1;
+                if (on) {
                     // one chunk at a time (a second one in flight would not fit the registers; the other
                     // warps of the scheduler cover the TMEM load)
 #pragma unroll
                     for (int j = 0; j < kHalf; ++j) {
-                        const int ci = half * kHalf + j, v0 = nt * BN + ci * kChunk;
+                        if (kCopies && j >= per) {
+                            cm[j] = -INFINITY;
+                            cs[j] = 0.0f;
+                            continue;
+                        }
+                        const int ci = half * kHalf + copy * per + j, v0 = nt * BN + ci * kChunk;
                         uint32_t ra[32];
                         ptx::tmem_ld_32cols(tb + ci * kChunk, ra);
                         float z[32];
@@ -638,16 +658,36 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant
                             hm = t.a1;
                             hid = v0 + t.i1;
                         }
-                        if (row < n_rows)
-                            P.chunks[P.chunk_at(nt, ci, row)] = make_float4(t.a1, t.a2, t.a3, __int_as_float(t.i1 | (t.i2 << 8)));
+                        if (crow < n_rows)
+                            P.chunks[P.chunk_at(nt, ci, crow)] = make_float4(t.a1, t.a2, t.a3, __int_as_float(t.i1 | (t.i2 << 8)));
                         __syncwarp();   // converged for the warp-collective TMEM loads
                     }
+                }
+                release_slot(g);
+                if (on) {
                     float hsum = 0.0f;
 #pragma unroll
                     for (int j = 0; j < kHalf; ++j) hsum += cm[j] > -INFINITY ? cs[j] * __expf(cm[j] - hm) : 0.0f;
-                    if (row < n_rows) P.halves[P.half_at(nt, half, row)] = make_float4(hm, hsum, hm, __int_as_float(hid));
+                    if (!kCopies || copies == 1) {
+                        if (crow < n_rows) P.halves[P.half_at(nt, half, crow)] = make_float4(hm, hsum, hm, __int_as_float(hid));
+                    } else {
+                        // the half's copies meet in shared memory; the first one folds them in chunk order.
+                        // (A buffer is written again two units later, after a barrier that its readers pass.)
+                        float4* sums = copy_sums + ((g * 2 + half) * 2 + (use & 1u)) * kBM;
+                        sums[copy * (kBM / copies) + crow] = make_float4(hm, hsum, 0.0f, __int_as_float(hid));
+                        ptx::named_barrier_sync(1 + g * 2 + half, 128);
+                        if (copy == 0 && crow < n_rows) {
+                            for (int c = 1; c < copies; ++c) {
+                                const float4 o = sums[c * (kBM / copies) + crow];
+                                if (o.x > hm) hid = __float_as_int(o.w);
+                                const float m = fmaxf(hm, o.x);
+                                if (m > -INFINITY) hsum = hsum * __expf(hm - m) + o.y * __expf(o.x - m);
+                                hm = m;
+                            }
+                            P.halves[P.half_at(nt, half, crow)] = make_float4(hm, hsum, hm, __int_as_float(hid));
+                        }
+                    }
                 }
-                release_slot(g);
             } else if constexpr (VAR) {
                 // Columns in steps of 8, alternating between the two warps of a row quarter; a last
                 // tile may run past the matrix (its weight rows there are zero, its columns dropped).
@@ -1138,7 +1178,14 @@ cudaError_t launch_lmhead_tc(const Ctx& ctx, const void* lm_head, const void* x,
     // per CTA and stage leaves room for seven stages.
     const int cl = m_tiles == 1 ? 1 : 2;
     CUtensorMap tx, tw;
-    cudaError_t e = make_tmap(&tx, x, d, n_rows, kBK, kBM);
+    // Few rows would leave all epilogue work to the warps of one TMEM lane quarter, which share one
+    // scheduler (the TMA producer's): copies of the rows in the other quarters spread it over all sixteen
+    // warps (V = 151936, 16 rows: d = 512 34 -> 28 us, d = 1024 63 -> 50, d = 2048 118 -> 99, d = 4096 the
+    // same on GB300).
+    const int copies = n_rows <= 32 ? 4 : n_rows <= 64 ? 2 : 1;
+    // (whole 8-row swizzle groups; the accumulator rows beyond them are never read)
+    const int x_rows = m_tiles > 1 ? kBM : (n_rows + 7) / 8 * 8;
+    cudaError_t e = make_tmap(&tx, x, d, n_rows, kBK, x_rows);
     if (e == cudaSuccess) e = make_tmap(&tw, lm_head, d, V, kBK, kBlockV / cl);
     if (e != cudaSuccess) return e;
     EpiParams ep{};
@@ -1146,6 +1193,8 @@ cudaError_t launch_lmhead_tc(const Ctx& ctx, const void* lm_head, const void* x,
     ep.V = V;
     ep.inv_temp = inv_temp;
     ep.reset_status = reset_status ? 1 : 0;
+    ep.copies = copies;
+    ep.x_rows = x_rows;
     if (m_tiles == 1) return run_gemm<EPI_LMHEAD, 1, 1, kBlockV, 4>(ctx, tx, tw, tw, n_rows, d, n_tiles, 1, ep);
     return run_gemm<EPI_LMHEAD, 1, 1, kBlockV, 7, 2>(ctx, tx, tw, tw, n_rows, d, n_tiles, (m_tiles + 1) / 2, ep);
 }

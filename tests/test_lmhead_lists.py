@@ -20,15 +20,21 @@ CASES = [
     (1500, 64, 64, "bf16", "plain"),         # 12 half blocks
     (270001, 64, 48, "bf16", "plain"),       # 2110 half blocks
 ]
+# numbers of rows at which the tensor-core epilogue changes: four copies of the rows, two, one, CTA pairs
+ROWS = [1, 32, 33, 64, 65, 128, 129]
+
+
+@pytest.mark.parametrize("n", ROWS)
+def test_lists_at_every_row_split(n):
+    test_lists_equal_a_full_sort(9001, 64, 32, "bf16", "plain", n)
 
 
 @pytest.mark.parametrize("V,d,k,dtype,rows", CASES)
-def test_lists_equal_a_full_sort(V, d, k, dtype, rows):
+def test_lists_equal_a_full_sort(V, d, k, dtype, rows, n=21):
     from paper_2606_03819_gb300 import Dims
     from paper_2606_03819_gb300 import binding as B
     dt = torch.bfloat16 if dtype == "bf16" else torch.float32
     g = torch.Generator().manual_seed(V + k)
-    n = 21
     W = torch.randn(V, d, generator=g)
     x = torch.randn(n, d, generator=g) * 3.0 / d ** 0.5
     if rows == "outlier":
@@ -37,7 +43,7 @@ def test_lists_equal_a_full_sort(V, d, k, dtype, rows):
     elif rows == "equal":
         x.zero_()
     W, x = W.to(dt).cuda(), x.to(dt).cuda()
-    dims = Dims(1, d, V, 64, n, 1, k, 8, dtype=dtype, mode="marginal")
+    dims = Dims(n, d, V, 64, 1, 1, k, 8, dtype=dtype, mode="marginal")
     ws = B.alloc_workspace(dims)
     ids = torch.empty(n, k, dtype=torch.int32, device="cuda")
     logp = torch.empty(n, k, device="cuda")
