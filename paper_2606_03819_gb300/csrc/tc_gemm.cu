@@ -72,9 +72,8 @@ struct EpiParams {
     // kernels with a width chosen at launch: columns per N tile (a multiple of 8) and ring stages
     int bn, stages;
     // LMHEAD with single CTAs and at most 64 (32) rows: 2 (4) copies of the rows, one per half (quarter)
-    // of the TMEM lanes, so that all epilogue warps share the chunks of a block; otherwise 1. x_rows:
-    // rows that a copy of X brings in (tmap_x's box)
-    int copies, x_rows;
+    // of the TMEM lanes, so that all epilogue warps share the chunks of a block; otherwise 1
+    int copies;
 };
 
 // Work unit u -> (N tile, M-tile group, K split); consecutive units share the N tile and K split
@@ -107,6 +106,7 @@ struct TileCfg {
     static_assert(kStageBytes % 1024 == 0, "stages must stay 1024-byte aligned for 128B swizzle");
 };
 
+constexpr int kShortRows = 64;     // rows of a last M-tile that is loaded through a shorter box
 constexpr int kVarMaxStages = 8;   // ring stages of the kernels whose tile width is chosen at launch
 
 __device__ __forceinline__ float silu_f(float g) { return g / (1.0f + __expf(-g)); }
@@ -189,8 +189,8 @@ __device__ __forceinline__ float sum_exp(const float (&z)[32], const Top3& t) {
 // VAR: the tile is ep.bn <= BN columns wide and the ring has ep.stages <= STAGES stages.
 template <int EPI, int MT, int NB, int BN, int STAGES, int CL, bool VAR>
 __global__ void __launch_bounds__(kThreads, 1)
-tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ CUtensorMap tmap_w0,
-               const __grid_constant__ CUtensorMap tmap_w1, int n_rows, int K, int n_ntiles,
+tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ CUtensorMap tmap_xl,
+               const __grid_constant__ CUtensorMap tmap_w0, const __grid_constant__ CUtensorMap tmap_w1, int n_rows, int K, int n_ntiles,
                int n_mgroups, int k_splits, int w_stream_once, EpiParams ep, int* status) {
     // Two kinds of cluster: kPair, a CTA pair on two M-tiles sharing each weight tile through
     // cta_group::2 MMAs; kSplitK, up to CL CTAs on the K-ranges of one output tile (one tile per
@@ -316,21 +316,45 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant
     if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer
         if (lane == 0) {
-            ptx::prefetch_tmap(&tmap_x);
+            const int rem = n_rows % kBM, x_last = (rem + 7) / 8 * 8;
+            const int m_all = (n_rows + kBM - 1) / kBM, m_short = !kPair && rem > 0 && rem <= kShortRows ? m_all - 1 : -1;
+            const CUtensorMap* only = m_short == 0 ? &tmap_xl : &tmap_x;
+            ptx::prefetch_tmap(only);
             ptx::prefetch_tmap(&tmap_w0);
             if (NB == 2) ptx::prefetch_tmap(&tmap_w1);
             const uint64_t pol_x = ptx::policy_evict_last();
             const uint64_t pol_w = w_stream_once ? ptx::policy_evict_first() : ptx::policy_evict_last();
             // Pair: both CTAs' copies of a stage complete on the even CTA's full barrier, which
             // the even CTA alone arms with the bytes of both halves.
+            // X rows: M-tiles through tmap_x; a last one of at most kShortRows rows through tmap_xl, whose box
+            // ends with the rows (in whole 8-row swizzle groups: a box mostly outside the tensor is slow
+            // to fill); an M-tile past the rows not at all. Pairs always take whole boxes: their MMAs
+            // cover the padding, and zeros there cost less power than what the stage held before (320
+            // rows of the LM head 383 against 440 us under the board's power cap).
             const int copies = kCopies ? ep.copies : 1;
-            const uint32_t tx_bytes = kCopies ? copies * ep.x_rows * kBK * 2 + C::kBBytes : (kPair ? 2 : 1) * stage_bytes;
             auto load_x = [&](uint8_t* sp, uint64_t* bar, int j, int kb, int mt) {
-                if constexpr (kPair)
-                    ptx::tma_load_2d_pair(sp + j * C::kABytes, &tmap_x, in_leader(bar), kb * kBK, mt * kBM, pol_x);
-                else
+                uint8_t* dst = sp + j * C::kABytes;
+                if constexpr (kPair) {
+                    ptx::tma_load_2d_pair(dst, &tmap_x, in_leader(bar), kb * kBK, mt * kBM, pol_x);
+                } else if (MT == 1 && !kCopies) {        // one M-tile in all
+                    ptx::tma_load_2d(dst, only, bar, kb * kBK, 0, pol_x);
+                } else if (mt != m_short) {
+                    if (mt < m_all) ptx::tma_load_2d(dst, &tmap_x, bar, kb * kBK, mt * kBM, pol_x);
+                } else {
                     for (int c = 0; c < copies; ++c)
-                        ptx::tma_load_2d(sp + j * C::kABytes + c * (C::kABytes / copies), &tmap_x, bar, kb * kBK, mt * kBM, pol_x);
+                        ptx::tma_load_2d(dst + (kCopies ? c * (C::kABytes / copies) : 0), &tmap_xl, bar, kb * kBK, mt * kBM, pol_x);
+                }
+            };
+            // Bytes that land on a stage's full barrier. Pair: both CTAs' copies of a stage complete on the
+            // even CTA's barrier, which the even CTA alone arms.
+            auto stage_tx = [&](const Unit& w) {
+                if constexpr (kPair) return static_cast<uint32_t>(2 * C::kStageBytes);
+                uint32_t n = NB * bn * kBK * 2;
+                for (int j = 0; j < MT; ++j) {
+                    const int mt = w.mg * MT + j;
+                    n += mt == m_short ? copies * x_last * kBK * 2 : mt < m_all ? C::kABytes : 0;
+                }
+                return n;
             };
             // Weight tiles of one stage; in a pair each CTA stages its half of the rows
             // (one weight matrix: tmap_w0's box is BN / 2 rows high; two: BN, one matrix per CTA).
@@ -353,9 +377,10 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant
             int pre = 0;
             if (cid < n_items) {
                 const Item f = item_of(cid);
+                const uint32_t tx = stage_tx(f.w);
                 pre = f.kb1 - f.kb0 < stages ? f.kb1 - f.kb0 : stages;
                 for (int i = 0; i < pre; ++i) {
-                    if (leader) ptx::mbar_arrive_expect_tx(&full[i], tx_bytes);
+                    if (leader) ptx::mbar_arrive_expect_tx(&full[i], tx);
                     load_w(smem + i * stage_bytes, &full[i], f.kb0 + i, f.w.nt);
                 }
             }
@@ -369,6 +394,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant
             for (int u = cid; u < n_items && ok; u += ncl) {
                 const Item itm = item_of(u);
                 const int nt = itm.w.nt, mt0 = (itm.w.mg * m_cl + m_rank) * MT;
+                const uint32_t tx = stage_tx(itm.w);
                 for (int kb = itm.kb0; kb < itm.kb1; ++kb, ++it) {
                     if (!ptx::mbar_wait(&empty[stage], phase ^ 1u, abort_flag, wait_ns)) {
                         ok = false;
@@ -376,7 +402,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant
                     }
                     uint8_t* sp = smem + stage * stage_bytes;
                     const bool w_done = it < pre;     // weight tiles already requested above
-                    if (!w_done && leader) ptx::mbar_arrive_expect_tx(&full[stage], tx_bytes);
+                    if (!w_done && leader) ptx::mbar_arrive_expect_tx(&full[stage], tx);
 #pragma unroll
                     for (int j = 0; j < MT; ++j) load_x(sp, &full[stage], j, kb, mt0 + j);
                     if (!w_done) load_w(sp, &full[stage], kb, nt);
@@ -422,6 +448,8 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant
                 const int g0 = (MT == 2) ? 0 : (kl & 1);
                 const Item itm = item_of(u);
                 const int nk_u = itm.kb1 - itm.kb0;
+                // M-tiles past the rows are left out
+                const int mts = MT == 1 ? 1 : min(MT, (n_rows + kBM - 1) / kBM - itm.w.mg * MT);
                 for (int j = 0; j < MT && ok; ++j)
                     ok = kPair ? ptx::mbar_wait_cluster(&tempty[g0 + j], (use[g0 + j] & 1u) ^ 1u, abort_flag, wait_ns)
                                : ptx::mbar_wait(&tempty[g0 + j], (use[g0 + j] & 1u) ^ 1u, abort_flag, wait_ns);
@@ -446,7 +474,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant
                             const uint32_t acc = (kb | kk) != 0 ? 1u : 0u;
                             if constexpr (kPair)
                                 ptx::mma_bf16_pair(tmem_base + 256u * (g0 + j), ad, bd, idesc, acc);
-                            else
+                            else if (MT == 1 || j == 0 || j < mts)
                                 ptx::mma_bf16(tmem_base + 256u * (g0 + j), ad, bd, idesc, acc);
                         }
                     }
@@ -623,19 +651,13 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant
                 // warps whose 32 rows are all padding skip the accumulators entirely (with copies there
                 // are none)
                 const bool on = crow - lane < n_rows;
-                float cm[kHalf], cs[kHalf];              // max and sum of each chunk
-                float hm = -INFINITY;
+                float hm = -INFINITY, hsum = 0.0f;       // max of the chunks so far, sum of exp(z - hm)
                 int hid = -1;
                 if (on) {
                     // one chunk at a time (a second one in flight would not fit the registers; the other
                     // warps of the scheduler cover the TMEM load)
-#pragma unroll
-                    for (int j = 0; j < kHalf; ++j) {
-                        if (kCopies && j >= per) {
-                            cm[j] = -INFINITY;
-                            cs[j] = 0.0f;
-                            continue;
-                        }
+#pragma unroll 1
+                    for (int j = 0; j < per; ++j) {
                         const int ci = half * kHalf + copy * per + j, v0 = nt * BN + ci * kChunk;
                         uint32_t ra[32];
                         ptx::tmem_ld_32cols(tb + ci * kChunk, ra);
@@ -651,13 +673,12 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant
                             for (int i = 0; i < 32; ++i) z[i] = v0 + i < ep.V ? z[i] : -INFINITY;
                         }
                         const Top3 t = top3<0, 32>(z);
-                        cm[j] = t.a1;
-                        cs[j] = sum_exp(z, t);
+                        const float cs = sum_exp(z, t);
                         // chunks arrive in id order, so strict > keeps the smaller id
-                        if (t.a1 > hm) {
-                            hm = t.a1;
-                            hid = v0 + t.i1;
-                        }
+                        if (t.a1 > hm) hid = v0 + t.i1;
+                        const float m = fmaxf(hm, t.a1);
+                        if (t.a1 > -INFINITY) hsum = hsum * __expf(hm - m) + cs * __expf(t.a1 - m);
+                        hm = m;
                         if (crow < n_rows)
                             P.chunks[P.chunk_at(nt, ci, crow)] = make_float4(t.a1, t.a2, t.a3, __int_as_float(t.i1 | (t.i2 << 8)));
                         __syncwarp();   // converged for the warp-collective TMEM loads
@@ -665,9 +686,6 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant
                 }
                 release_slot(g);
                 if (on) {
-                    float hsum = 0.0f;
-#pragma unroll
-                    for (int j = 0; j < kHalf; ++j) hsum += cm[j] > -INFINITY ? cs[j] * __expf(cm[j] - hm) : 0.0f;
                     if (!kCopies || copies == 1) {
                         if (crow < n_rows) P.halves[P.half_at(nt, half, crow)] = make_float4(hm, hsum, hm, __int_as_float(hid));
                     } else {
@@ -1087,6 +1105,17 @@ cudaError_t make_tmap(CUtensorMap* map, const void* base, uint64_t inner, uint64
     return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
+// The maps of a kernel's X operand [n_rows, K]: whole M-tiles, and the rows of the last one.
+struct XMaps {
+    CUtensorMap whole, last;
+};
+cudaError_t make_xmaps(XMaps* m, const void* x, int K, int n_rows) {
+    const int rem = n_rows % kBM;
+    cudaError_t e = make_tmap(&m->whole, x, K, n_rows, kBK, kBM);
+    if (e == cudaSuccess) e = make_tmap(&m->last, x, K, n_rows, kBK, rem ? (rem + 7) / 8 * 8 : kBM);
+    return e;
+}
+
 // Clusters of cl CTAs that can be resident at once for this kernel (at most num_sms / cl).
 template <typename K>
 int resident_clusters(K kern, int smem, int cl, int num_sms) {
@@ -1112,7 +1141,7 @@ int resident_clusters(K kern, int smem, int cl, int num_sms) {
 }
 
 template <int EPI, int MT, int NB, int BN, int STAGES, int CL = 1>
-cudaError_t run_gemm(const Ctx& ctx, const CUtensorMap& tx, const CUtensorMap& tw0, const CUtensorMap& tw1,
+cudaError_t run_gemm(const Ctx& ctx, const XMaps& tx, const CUtensorMap& tw0, const CUtensorMap& tw1,
                      int n_rows, int K, int n_ntiles, int n_mgroups, const EpiParams& ep_in, int k_splits = 1,
                      size_t partial_bytes = 0) {
     constexpr bool kSplitK = EPI == EPI_CGATEUP || EPI == EPI_CDOWN;
@@ -1126,7 +1155,7 @@ cudaError_t run_gemm(const Ctx& ctx, const CUtensorMap& tx, const CUtensorMap& t
     const int stream_once = n_mgroups == 1 ? 1 : 0;
     if constexpr (kSplitK) {   // one output tile per cluster, its K-ranges on the cluster's CTAs
         e = launch_pdl_cluster(kern, dim3(CL * n_ntiles * n_mgroups), dim3(kThreads), C::kSmemBytes, ctx.stream, CL,
-                               tx, tw0, tw1, n_rows, K, n_ntiles, n_mgroups, CL, stream_once, ep, ctx.status);
+                               tx.whole, tx.last, tw0, tw1, n_rows, K, n_ntiles, n_mgroups, CL, stream_once, ep, ctx.status);
         return e != cudaSuccess ? e : cudaGetLastError();
     }
     int n_items = n_units;
@@ -1154,12 +1183,12 @@ cudaError_t run_gemm(const Ctx& ctx, const CUtensorMap& tx, const CUtensorMap& t
     }
     if constexpr (CL == 1) {
         const int grid = n_items < ctx.num_sms ? n_items : ctx.num_sms;
-        e = launch_pdl(kern, dim3(grid), dim3(kThreads), C::kSmemBytes, ctx.stream, tx, tw0, tw1, n_rows, K,
+        e = launch_pdl(kern, dim3(grid), dim3(kThreads), C::kSmemBytes, ctx.stream, tx.whole, tx.last, tw0, tw1, n_rows, K,
                        n_ntiles, n_mgroups, k_splits, stream_once, ep, ctx.status);
     } else {
         static const int max_cl = resident_clusters(kern, C::kSmemBytes, CL, ctx.num_sms);
         const int n_cl = n_items < max_cl ? n_items : max_cl;
-        e = launch_pdl_cluster(kern, dim3(CL * n_cl), dim3(kThreads), C::kSmemBytes, ctx.stream, CL, tx, tw0, tw1,
+        e = launch_pdl_cluster(kern, dim3(CL * n_cl), dim3(kThreads), C::kSmemBytes, ctx.stream, CL, tx.whole, tx.last, tw0, tw1,
                                n_rows, K, n_ntiles, n_mgroups, k_splits, stream_once, ep, ctx.status);
     }
     return e != cudaSuccess ? e : cudaGetLastError();
@@ -1177,15 +1206,14 @@ cudaError_t launch_lmhead_tc(const Ctx& ctx, const void* lm_head, const void* x,
     // CTA keeps one TMEM slot per unit and overlaps its epilogue with the next unit's MMAs; 32 KB
     // per CTA and stage leaves room for seven stages.
     const int cl = m_tiles == 1 ? 1 : 2;
-    CUtensorMap tx, tw;
+    XMaps tx;
+    CUtensorMap tw;
     // Few rows would leave all epilogue work to the warps of one TMEM lane quarter, which share one
     // scheduler (the TMA producer's): copies of the rows in the other quarters spread it over all sixteen
     // warps (V = 151936, 16 rows: d = 512 34 -> 28 us, d = 1024 63 -> 50, d = 2048 118 -> 99, d = 4096 the
     // same on GB300).
     const int copies = n_rows <= 32 ? 4 : n_rows <= 64 ? 2 : 1;
-    // (whole 8-row swizzle groups; the accumulator rows beyond them are never read)
-    const int x_rows = m_tiles > 1 ? kBM : (n_rows + 7) / 8 * 8;
-    cudaError_t e = make_tmap(&tx, x, d, n_rows, kBK, x_rows);
+    cudaError_t e = make_xmaps(&tx, x, d, n_rows);
     if (e == cudaSuccess) e = make_tmap(&tw, lm_head, d, V, kBK, kBlockV / cl);
     if (e != cudaSuccess) return e;
     EpiParams ep{};
@@ -1194,7 +1222,6 @@ cudaError_t launch_lmhead_tc(const Ctx& ctx, const void* lm_head, const void* x,
     ep.inv_temp = inv_temp;
     ep.reset_status = reset_status ? 1 : 0;
     ep.copies = copies;
-    ep.x_rows = x_rows;
     if (m_tiles == 1) return run_gemm<EPI_LMHEAD, 1, 1, kBlockV, 4>(ctx, tx, tw, tw, n_rows, d, n_tiles, 1, ep);
     return run_gemm<EPI_LMHEAD, 1, 1, kBlockV, 7, 2>(ctx, tx, tw, tw, n_rows, d, n_tiles, (m_tiles + 1) / 2, ep);
 }
@@ -1221,7 +1248,7 @@ constexpr int kMinClusterCtas = 96;
 // SMs instead of 96 of 128 (121 rows, gate/up and down: 114 -> 102 us), 1024 columns in 4 K-ranges as
 // 128 units of 32 instead of 32 of 128. The width does not change any output's sum.
 template <int EPI, int MT, int NB>
-cudaError_t run_gemm_var(const Ctx& ctx, const CUtensorMap& tx, const void* w0, const void* w1, int N, int n_rows, int K,
+cudaError_t run_gemm_var(const Ctx& ctx, const XMaps& tx, const void* w0, const void* w1, int N, int n_rows, int K,
                          int n_mgroups, int k_splits, const EpiParams& ep_in) {
     using C = TileCfg<MT, NB, 128, kVarMaxStages, false, true>;
     auto kern = tc_gemm_kernel<EPI, MT, NB, 128, kVarMaxStages, 1, true>;
@@ -1251,7 +1278,7 @@ cudaError_t run_gemm_var(const Ctx& ctx, const CUtensorMap& tx, const void* w0, 
     const int n_ntiles = (N + bn - 1) / bn;
     const long long n_units = static_cast<long long>(n_ntiles) * n_mgroups * k_splits;
     const int grid = static_cast<int>(n_units < ctx.num_sms ? n_units : ctx.num_sms);
-    e = launch_pdl(kern, dim3(grid), dim3(kThreads), C::kSmemBytes, ctx.stream, tx, t0, t1, n_rows, K, n_ntiles, n_mgroups,
+    e = launch_pdl(kern, dim3(grid), dim3(kThreads), C::kSmemBytes, ctx.stream, tx.whole, tx.last, t0, t1, n_rows, K, n_ntiles, n_mgroups,
                    k_splits, n_mgroups == 1 ? 1 : 0, ep, ctx.status);
     return e != cudaSuccess ? e : cudaGetLastError();
 }
@@ -1261,7 +1288,7 @@ cudaError_t run_gemm_var(const Ctx& ctx, const CUtensorMap& tx, const void* w0, 
 // bounds their number; the tile width follows from it. *done stays false, and nothing runs, where there
 // are too many tiles for that.
 template <int EPI, int MT, int NB>
-cudaError_t run_gemm_cluster(const Ctx& ctx, const CUtensorMap& tx, const void* w0, const void* w1, int N, int n_rows, int K,
+cudaError_t run_gemm_cluster(const Ctx& ctx, const XMaps& tx, const void* w0, const void* w1, int N, int n_rows, int K,
                              int n_mgroups, int k_splits, const EpiParams& ep_in, size_t partial_bytes, bool* done) {
     using C = TileCfg<MT, NB, 128, kVarMaxStages, false, true>;
     auto kern = tc_gemm_kernel<EPI, MT, NB, 128, kVarMaxStages, kMaxKSplits, true>;
@@ -1305,7 +1332,7 @@ cudaError_t run_gemm_cluster(const Ctx& ctx, const CUtensorMap& tx, const void* 
     ep.stages = stages < kVarMaxStages ? stages : kVarMaxStages;
     *done = true;
     e = launch_pdl_cluster(kern, dim3(static_cast<unsigned>(k_splits * n_cl)), dim3(kThreads), C::kSmemBytes, ctx.stream,
-                           k_splits, tx, t0, t1, n_rows, K, n_ntiles, n_mgroups, k_splits, n_mgroups == 1 ? 1 : 0, ep,
+                           k_splits, tx.whole, tx.last, t0, t1, n_rows, K, n_ntiles, n_mgroups, k_splits, n_mgroups == 1 ? 1 : 0, ep,
                            ctx.status);
     return e != cudaSuccess ? e : cudaGetLastError();
 }
@@ -1314,7 +1341,7 @@ cudaError_t run_gemm_cluster(const Ctx& ctx, const CUtensorMap& tx, const void* 
 // projection (K = I, In = A) and the linear approximator (K = 2d, In = x). The residual row of
 // stage-2 row r is the hidden state of its depth; the epilogue adds it in fp32 and rounds once to
 // bf16.
-static cudaError_t run_residual_gemm(const Ctx& ctx, const CUtensorMap& ta, const void* W, int K, const void* hidden,
+static cudaError_t run_residual_gemm(const Ctx& ctx, const XMaps& ta, const void* W, int K, const void* hidden,
                               int n_rows, int d, int R, int M, int gamma, void* h_prime, float* partial,
                               size_t partial_bytes) {
     constexpr int BN = 128;
@@ -1369,11 +1396,12 @@ cudaError_t launch_swiglu_tc(const Ctx& ctx, const void* X, int k_in, const void
     const int m_tiles = (n_rows + kBM - 1) / kBM;
     const int n_mg = m_tiles == 1 ? 1 : (m_tiles + 1) / 2;
     const int bn_gu = I % BN == 0 ? BN : 64;
-    CUtensorMap tx, tg, tu, ta;
-    cudaError_t e = make_tmap(&tx, X, k_in, n_rows, kBK, kBM);
+    XMaps tx, ta;
+    CUtensorMap tg, tu;
+    cudaError_t e = make_xmaps(&tx, X, k_in, n_rows);
     if (e == cudaSuccess) e = make_tmap(&tg, w_gate, k_in, I, kBK, bn_gu);
     if (e == cudaSuccess) e = make_tmap(&tu, w_up, k_in, I, kBK, bn_gu);
-    if (e == cudaSuccess) e = make_tmap(&ta, A, I, n_rows, kBK, kBM);
+    if (e == cudaSuccess) e = make_xmaps(&ta, A, I, n_rows);
     if (e != cudaSuccess) return e;
 
     // ---- gate/up: A = SiLU(X Wg^T) * (X Wu^T)
@@ -1408,8 +1436,8 @@ cudaError_t launch_swiglu_tc(const Ctx& ctx, const void* X, int k_in, const void
 cudaError_t launch_linear_tc(const Ctx& ctx, const void* X, const void* w_lin, const void* hidden, int n_rows, int d,
                              int R, int M, int gamma, void* h_prime, float* partial, size_t partial_bytes) {
     if (n_rows <= 0) return cudaSuccess;
-    CUtensorMap tx;
-    const cudaError_t e = make_tmap(&tx, X, 2 * d, n_rows, kBK, kBM);
+    XMaps tx;
+    const cudaError_t e = make_xmaps(&tx, X, 2 * d, n_rows);
     if (e != cudaSuccess) return e;
     return run_residual_gemm(ctx, tx, w_lin, 2 * d, hidden, n_rows, d, R, M, gamma, h_prime, partial, partial_bytes);
 }
