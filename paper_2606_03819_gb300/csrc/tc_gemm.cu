@@ -1204,8 +1204,14 @@ cudaError_t launch_lmhead_tc(const Ctx& ctx, const void* lm_head, const void* x,
     // More than one M-tile: CTA pairs (clusters of two), one M-tile each, share every weight tile
     // through cta_group::2 MMAs (each stages half of its rows), so W_lm is read once while each
     // CTA keeps one TMEM slot per unit and overlaps its epilogue with the next unit's MMAs; 32 KB
-    // per CTA and stage leaves room for seven stages.
-    const int cl = m_tiles == 1 ? 1 : 2;
+    // per CTA and stage leaves room for seven stages. Three and five M-tiles run on single CTAs, which
+    // read each weight tile once per M-tile from L2 but leave out the missing half of the last pair
+    // (V = 151936, d = 4096: 320 rows 390 -> 345 us, 600 rows 575 -> 552; d = 1024: 115 -> 92, 174 -> 150;
+    // seven M-tiles gain nothing), and so do small d, where the epilogue sets the pace and single CTAs
+    // hand over their accumulators sooner (d = 512: 250 rows 46 -> 41 us, 1020 rows 147 -> 139; d = 1024:
+    // 64 -> 71, so pairs from there on).
+    const bool single = m_tiles == 1 || m_tiles == 3 || m_tiles == 5 || d <= 512;
+    const int cl = single ? 1 : 2;
     XMaps tx;
     CUtensorMap tw;
     // Few rows would leave all epilogue work to the warps of one TMEM lane quarter, which share one
@@ -1222,7 +1228,7 @@ cudaError_t launch_lmhead_tc(const Ctx& ctx, const void* lm_head, const void* x,
     ep.inv_temp = inv_temp;
     ep.reset_status = reset_status ? 1 : 0;
     ep.copies = copies;
-    if (m_tiles == 1) return run_gemm<EPI_LMHEAD, 1, 1, kBlockV, 4>(ctx, tx, tw, tw, n_rows, d, n_tiles, 1, ep);
+    if (single) return run_gemm<EPI_LMHEAD, 1, 1, kBlockV, 4>(ctx, tx, tw, tw, n_rows, d, n_tiles, m_tiles, ep);
     return run_gemm<EPI_LMHEAD, 1, 1, kBlockV, 7, 2>(ctx, tx, tw, tw, n_rows, d, n_tiles, (m_tiles + 1) / 2, ep);
 }
 

@@ -20,13 +20,15 @@ CASES = [
     (1500, 64, 64, "bf16", "plain"),         # 12 half blocks
     (270001, 64, 48, "bf16", "plain"),       # 2110 half blocks
 ]
-# numbers of rows at which the tensor-core epilogue changes: four copies of the rows, two, one, CTA pairs
-ROWS = [1, 32, 33, 64, 65, 128, 129]
+# numbers of rows at which the tensor-core kernel changes: four copies of the rows, two, one; then
+# with d > 512 CTA pairs, single CTAs over three (and five) M-tiles, pairs again
+ROWS = [(1, 64), (32, 64), (33, 64), (64, 64), (65, 64), (128, 64), (129, 64), (129, 576), (256, 576), (257, 576),
+        (385, 576), (513, 576), (641, 576)]
 
 
-@pytest.mark.parametrize("n", ROWS)
-def test_lists_at_every_row_split(n):
-    test_lists_equal_a_full_sort(9001, 64, 32, "bf16", "plain", n)
+@pytest.mark.parametrize("n,d", ROWS)
+def test_lists_at_every_row_split(n, d):
+    test_lists_equal_a_full_sort(9001, d, 32, "bf16", "plain", n)
 
 
 @pytest.mark.parametrize("V,d,k,dtype,rows", CASES)
