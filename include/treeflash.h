@@ -240,12 +240,13 @@ tf_status tf_build_tree_mask(const tf_dims* dims, const int32_t* root_tok, const
  * address, the kernels read root_tok and root_pos and write every output in host memory
  * directly; other buffers go through the workspace and copies. On a created stream (not the
  * legacy default stream) with page-locked buffers, the first call with a given set of arguments
- * (dims, weight, buffer and workspace pointers, device, wait limit) captures the step as a CUDA
- * graph and later calls replay it: the buffers' contents may change between calls, their
- * addresses may not without a new capture. The library keeps the last 8 such graphs (the CUDA
- * driver instantiates them; the library itself allocates no memory); a capture that fails leaves
- * the step on plain launches. The call must not itself be made inside a stream capture (it
- * synchronises).
+ * (dims, weight, buffer and workspace pointers, device, wait limit) captures the step's kernels as a
+ * CUDA graph and later calls replay it after the copy of hidden: the buffers' contents may change
+ * between calls, their addresses may not without a new capture. (Buffers freed in between whose
+ * addresses new ones have taken are fine: the graph holds kernels alone.) The library keeps the last
+ * 8 such graphs (the CUDA driver instantiates them; the library itself allocates no memory); a
+ * capture that fails leaves the step on plain launches. The call must not itself be made inside a
+ * stream capture (it synchronises).
  * Host inputs: hidden [b, gamma, d] dtype, root_tok [b] ([b, 2] with TF_APPROX_SWIGLU_2PREV),
  * root_pos [b]. Host outputs:
  * node_tok, node_parent, node_depth [b, B+1] int32, node_score [b, B+1] float,

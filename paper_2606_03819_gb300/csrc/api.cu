@@ -311,11 +311,18 @@ Mapped map_host_buffers(const HostStep& h) {
     return m;
 }
 
-// Enqueues the whole host-buffer step on the stream, without synchronising: the hidden states to
-// the workspace, stage 1, stage 2, the tree and its mask (dev_status with the workspace status
-// word folded in by the builder, so no separate read is needed). With page-locked buffers that
+// Enqueues the host-buffer step on the stream, without synchronising: the hidden states to the
+// workspace (copy_hidden), then stage 1, stage 2, the tree and its mask (dev_status with the workspace
+// status word folded in by the builder, so no separate read is needed). With page-locked buffers that
 // the device can address (m.ok) the kernels read root_tok / root_pos and write the outputs in
 // host memory directly; otherwise those go through the workspace and copies.
+tf_status copy_hidden(const Prepared& p, const HostStep& h) {
+    const Dims& D = p.D;
+    return cuda_status(cudaMemcpyAsync(at<void>(h.ws, p.L.h_hidden), h.hidden,
+                                       static_cast<size_t>(D.b) * D.gamma * D.d * D.esize, cudaMemcpyHostToDevice,
+                                       p.ctx.stream));
+}
+
 tf_status enqueue_host_step(const Prepared& p, const HostStep& h, const Mapped& m) {
     const Dims& D = p.D;
     const Layout& L = p.L;
@@ -323,9 +330,7 @@ tf_status enqueue_host_step(const Prepared& p, const HostStep& h, const Mapped& 
     cudaStream_t st = ctx.stream;
     void* ws = h.ws;
     const size_t nn = static_cast<size_t>(D.b) * (D.B + 1);
-    void* d_hidden = at<void>(ws, L.h_hidden);
-    TF_TRY(cuda_status(cudaMemcpyAsync(d_hidden, h.hidden, static_cast<size_t>(D.b) * D.gamma * D.d * D.esize,
-                                       cudaMemcpyHostToDevice, st)));
+    void* d_hidden = at<void>(ws, L.h_hidden);   // (filled by copy_hidden)
     const int32_t* d_root = m.root_tok;
     const int32_t* d_pos = m.root_pos;
     if (!m.ok) {
@@ -369,14 +374,16 @@ tf_status enqueue_host_step(const Prepared& p, const HostStep& h, const Mapped& 
     return cuda_status(cudaMemcpyAsync(h.dev_status, o_stat, D.b * 4, cudaMemcpyDeviceToHost, st));
 }
 
-// The host-buffer step as a CUDA graph, captured on the first call with a given set of arguments
-// and replayed afterwards: one graph launch in place of three copies, eight to nine kernel launches
-// and seven copies, and the next step's first kernel no longer waits for the host to issue it.
+// The kernels of the host-buffer step as a CUDA graph, captured on the first call with a given set of
+// arguments and replayed afterwards: one graph launch in place of eight to nine kernel launches.
 // Only for a created stream (the legacy default stream cannot be captured) and page-locked host
-// buffers (copies from pageable memory cannot be captured); otherwise, or when the capture or the
-// instantiation fails, the step runs as plain launches. The key holds everything the captured
-// kernels and copies read at capture time: dims, weight, buffer and workspace pointers, the device
-// and the wait limit of the tensor-core kernels. At most kMaxHostGraphs are kept (oldest evicted).
+// buffers that the device can address, so that no copy belongs to the graph: a copy node binds the
+// allocations that it was captured with, and a caller may free its buffers and get the same addresses
+// for new ones, whereas a kernel node holds nothing but its arguments. The hidden states are copied
+// before the graph. Otherwise, or when the capture or the instantiation fails, the step runs as plain
+// launches. The key holds everything the captured kernels read at capture time: dims, weight, buffer
+// and workspace pointers, the device and the wait limit of the tensor-core kernels. At most
+// kMaxHostGraphs are kept (oldest evicted).
 struct HostGraph {
     std::vector<uint64_t> key;
     cudaGraphExec_t exec;       // nullptr: this step could not be captured, run it as plain launches
@@ -392,6 +399,19 @@ uint32_t float_bits(float f) {
     return u;
 }
 
+// Whether a captured graph consists of kernel nodes alone.
+bool only_kernels(cudaGraph_t graph) {
+    size_t n = 0;
+    if (cudaGraphGetNodes(graph, nullptr, &n) != cudaSuccess) return false;
+    std::vector<cudaGraphNode_t> nodes(n);
+    if (n == 0 || cudaGraphGetNodes(graph, nodes.data(), &n) != cudaSuccess) return false;
+    for (cudaGraphNode_t node : nodes) {
+        cudaGraphNodeType type;
+        if (cudaGraphNodeGetType(node, &type) != cudaSuccess || type != cudaGraphNodeTypeKernel) return false;
+    }
+    return true;
+}
+
 bool page_locked(const void* ptr) {
     cudaPointerAttributes a;
     if (cudaPointerGetAttributes(&a, ptr) != cudaSuccess) {
@@ -404,6 +424,7 @@ bool page_locked(const void* ptr) {
 tf_status launch_host_graph(const Prepared& p, const HostStep& h, const Mapped& m, bool* replayed) {
     *replayed = false;
     cudaStream_t st = p.ctx.stream;
+    if (!m.ok) return TF_OK;
     if (st == nullptr || st == cudaStreamLegacy || st == cudaStreamPerThread) return TF_OK;
     cudaStreamCaptureStatus cs;
     if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) {
@@ -446,7 +467,7 @@ tf_status launch_host_graph(const Prepared& p, const HostStep& h, const Mapped& 
         cudaGraph_t graph = nullptr;
         const cudaError_t ce = cudaStreamEndCapture(st, &graph);
         cudaGraphExec_t exec = nullptr;
-        if (es == TF_OK && ce == cudaSuccess && graph &&
+        if (es == TF_OK && ce == cudaSuccess && graph && only_kernels(graph) &&
             cudaGraphInstantiate(&exec, graph, 0) != cudaSuccess)
             exec = nullptr;
         if (graph) cudaGraphDestroy(graph);
@@ -460,6 +481,7 @@ tf_status launch_host_graph(const Prepared& p, const HostStep& h, const Mapped& 
         hit = &g_host_graphs.back();
     }
     if (!hit->exec) return TF_OK;
+    TF_TRY(copy_hidden(p, h));
     if (cudaGraphLaunch(hit->exec, st) != cudaSuccess) return TF_ERR_CUDA;
     tf::g_kernel_launches.fetch_add(hit->kernels, std::memory_order_relaxed);
     *replayed = true;
@@ -696,7 +718,10 @@ tf_status tf_draft_tree_host(const tf_dims* dims, const tf_weights* w, const voi
     const Mapped m = map_host_buffers(h);
     bool replayed = false;
     TF_TRY(launch_host_graph(p, h, m, &replayed));
-    if (!replayed) TF_TRY(enqueue_host_step(p, h, m));
+    if (!replayed) {
+        TF_TRY(copy_hidden(p, h));
+        TF_TRY(enqueue_host_step(p, h, m));
+    }
     if (cudaStreamSynchronize(st) != cudaSuccess) return TF_ERR_CUDA;
     // every dev_status entry carries the workspace word in bits 16 and up (folded by the builder)
     const int32_t flags = dev_status[0] >> 16;

@@ -66,3 +66,28 @@ def test_replayed_step_equals_the_device_path(name, over):
         expect = Bn.TF_ERR_DEVICE_STATUS if ref["flags"] & ~16 else Bn.TF_OK
         assert st == expect, (call, st, ref["flags"])
     assert launches[1] == launches[2] == launches[0] > 0
+
+
+def test_replay_after_the_buffers_were_freed_and_allocated_again():
+    # the caching allocator hands a new workspace and weights the addresses of freed ones, so a call
+    # finds the graph captured on those: the step must read and write the new allocations
+    from paper_2606_03819_gb300 import Dims, alloc_workspace
+    from paper_2606_03819_gb300 import binding as Bn
+    cfg = synth.get_config("tiny_peaked", dtype="bf16", batch=3, V=2000)
+    dims = Dims.from_config(cfg)
+    stream = torch.cuda.Stream()
+    h = {k: torch.empty_like(v).pin_memory() for k, v in synth.make_inputs(cfg).items() if k in ("hidden", "root_tok", "root_pos")}
+    out = _host_buffers(cfg)
+    for call in range(4):
+        base = synth.make_inputs(cfg, seed=50 + call)
+        for k in h:
+            h[k].copy_(base[k])
+        d = parity.device_inputs(base)
+        ws = alloc_workspace(dims)
+        assert _call(Bn, dims, d, h, out, ws, stream) == Bn.TF_OK
+        ref = parity.run_gpu(cfg, d)
+        for k in ("node_tok", "node_parent", "node_depth", "mask", "pos_ids"):
+            np.testing.assert_array_equal(out[k].numpy(), ref[k], err_msg=f"call {call}: {k}")
+        del d, ws, ref
+        torch.cuda.synchronize()
+        torch.cuda.empty_cache()
