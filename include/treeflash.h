@@ -194,7 +194,7 @@ tf_status tf_stage2_ar_approx(const tf_dims* dims, const tf_weights* w, const vo
                               int32_t* child_ids, float* child_logp,
                               void* ws, size_t ws_bytes, tf_stream_t stream);
 
-/* Algorithm 1 Part 2 (OPT-Tree selection, Sec. 3): one warp per sequence grows the tree by
+/* Algorithm 1 Part 2 (OPT-Tree selection, Sec. 3): each sequence's tree grows by
  * popping the candidate of highest cumulative log-probability B times. The root's children
  * are row 0 of child_ids (TF_MODE_AR) or depth 1 of top_ids (marginal modes). A popped node
  * at depth i < gamma whose token is x^(m)_{t+i} (m < M) makes row 1 + (i-1) M + m available

@@ -208,7 +208,8 @@ cudaError_t launch_swiglu_tc(const Ctx&, const void* X, int k_in, const void* w_
                              const void* w_up, const void* w_down, const void* hidden, int n_rows,
                              int d, int I, int R, int M, int gamma, void* A, void* h_prime,
                              float* partial, size_t partial_bytes);
-// split-K reductions of the approximator GEMMs (partial sums in fp32, [k_splits][N / 4][rows][4])
+// split-K reductions of the approximator GEMMs that no cluster takes (partial sums in fp32,
+// [k_splits][N / 4][rows][4])
 cudaError_t launch_swiglu_reduce(const Ctx&, const float* partial, int k_splits, int n_rows, int I,
                                  __nv_bfloat16* A);
 cudaError_t launch_down_reduce(const Ctx&, const float* partial, int k_splits, int n_rows, int d,

@@ -4,7 +4,7 @@
 //
 // X rows sit in the 128 TMEM lanes (M = 128 per tile), weight rows in the MMA N dimension, so
 // every epilogue thread owns one activation row and walks its logits / outputs serially.
-// Three fused epilogues:
+// Fused epilogues:
 //   LMHEAD  the LM-head pass of Algorithm 1 (stage 1 and stage 2): for each (row, block of 256
 //           vocabulary entries) it keeps per half block the max, the sum of exp(z - max) and the
 //           best (z, id), and per 32-wide chunk the three largest z with the ids of the first
@@ -12,6 +12,8 @@
 //   GATEUP  SwiGLU of Eq. 1, first half: A = SiLU(X W_gate^T) * (X W_up^T), bf16 out.
 //   DOWN    SwiGLU of Eq. 1, second half plus the residual: h' = h + A W_down^T, bf16 out; the
 //           same epilogue serves the linear approximator of the ablations, h' = h + x W_lin^T.
+//   CGATEUP, CDOWN  the same two results where K is split over the CTAs of a cluster.
+//   PARTIAL fp32 sums of a K-range, for the reduction kernels, where no cluster can take the split.
 //
 // Warp roles (576 threads, one CTA per SM, persistent over work units):
 //   warp 0      TMA producer: one elected lane streams X and W tiles into a ring of stages.
@@ -21,8 +23,8 @@
 //               the two warps of a group on the same lanes split the columns in halves.
 // A work unit is (N tile, group of MT M-tiles). With MT = 2 both slots hold one unit (M-tile j
 // in slot j); with MT = 1 consecutive units alternate slots so the epilogue of one overlaps the
-// MMAs of the next. With clusters of CL = 2 CTAs (the LM head over more than 128 rows) the two
-// CTAs are a tcgen05 CTA pair: units are dealt to clusters, CTA r of a cluster stages M-tile r of
+// MMAs of the next. With clusters of CL = 2 CTAs (most LM heads over more than 128 rows, the down
+// projection of many rows) the two CTAs are a tcgen05 CTA pair: units are dealt to clusters, CTA r of a cluster stages M-tile r of
 // the unit's pair of M-tiles and weight rows [128 r, 128 r + 128) of the unit's 256-row weight
 // tile, and the even CTA issues one cta_group::2 MMA (M = 256, N = 256) per K slice that reads
 // both CTAs' shared memory and writes each CTA's 128 rows into its own TMEM. W is read once, each
@@ -45,7 +47,7 @@ constexpr int kThreads = 64 + 32 * kEpiWarps;
 constexpr uint64_t kWaitLimitNs = 2000000000ull;
 
 // EPI_CGATEUP / EPI_CDOWN: the GATEUP / DOWN results from split-K over the CTAs of a cluster, the
-// partial sums added in shared memory across the cluster instead of through global memory.
+// partial sums exchanged through an area of the workspace that stays in L2.
 enum { EPI_LMHEAD = 0, EPI_GATEUP = 1, EPI_DOWN = 2, EPI_PARTIAL = 3, EPI_CGATEUP = 4, EPI_CDOWN = 5 };
 
 struct EpiParams {
@@ -62,7 +64,7 @@ struct EpiParams {
     int reset_status;            // LMHEAD: zero *status first (the first kernel of a stage-1 call)
     unsigned long long wait_ns;  // limit of every wait for progress (0: kWaitLimitNs); the waits
                                  // that drain in-flight copies and MMAs always take kWaitLimitNs
-    // GATEUP / DOWN with one CTA per SM: units n_full.. (the last, partial round) run as
+    // GATEUP / DOWN of fixed width, single CTAs or pairs: units n_full.. (the last, partial round) run as
     // tail_split K-chunks each (0: none). A chunk writes its fp32 partial sums to `partial`, laid
     // out [tail unit][chunk][M-tile][col / 4][128 rows][4]; the chunk that finishes last (counted
     // in sem[tail unit * MT + M-tile], zero between calls) adds them in chunk order and applies
@@ -123,8 +125,8 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
 // sets the pace of the LM head. The three values come from a network of min/max (a merge of two sorted
 // triples: a third largest is one of two thirds and two cross minima), the offsets from four selects
 // per merge, and the exponentials from one pass over the values once the maximum is known, in packed
-// pairs: about 360 instructions per chunk, where a tree whose every node rescaled its sum of
-// exponentials took 1040 (V = 151936, 256 rows: d = 512 66 -> 47 us, d = 1024 78 -> 64, d = 2048 122 ->
+// pairs. A warp issues 508 instructions per chunk of its 32 rows (loads, tests and stores included),
+// where a tree whose every node rescaled its sum of exponentials took 1040 (V = 151936, 256 rows: d = 512 66 -> 47 us, d = 1024 78 -> 64, d = 2048 122 ->
 // 115, d = 4096 222 -> 217 on GB300).
 struct Top3 {
     float a1, a2, a3;  // a1 >= a2 >= a3
@@ -194,7 +196,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant
                int n_mgroups, int k_splits, int w_stream_once, EpiParams ep, int* status) {
     // Two kinds of cluster: kPair, a CTA pair on two M-tiles sharing each weight tile through
     // cta_group::2 MMAs; kSplitK, up to CL CTAs on the K-ranges of one output tile (one tile per
-    // cluster), whose accumulators are summed through distributed shared memory.
+    // cluster), whose accumulators are summed through an exchange area in L2.
     constexpr bool kSplitK = EPI == EPI_CGATEUP || EPI == EPI_CDOWN;
     constexpr bool kPair = CL > 1 && !kSplitK;
     using C = TileCfg<MT, NB, BN, STAGES, kPair, VAR>;

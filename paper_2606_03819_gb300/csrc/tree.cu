@@ -115,7 +115,7 @@ __global__ void __launch_bounds__(256) gather_norm_kernel(const T* __restrict__ 
 }
 
 // ------------------------------------------------------------------------------------------
-// OPT-Tree selection (Algorithm 1 Part 2), one warp per sequence. The queue holds one entry per
+// OPT-Tree selection (Algorithm 1 Part 2) by a queue, one warp per sequence. It holds one entry per
 // open child list: (path score, depth, parent node) packed into one 64-bit key, plus the list
 // row, the rank in the list, the parent's score and the token. Popping rank k of a list
 // replaces the entry by rank k+1 of the same list (its next sibling), and an expandable popped
