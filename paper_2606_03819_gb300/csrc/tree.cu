@@ -225,7 +225,7 @@ struct TreeSmem {
     int *o_tok, *o_par, *o_dep;
     float* o_score;
     int* topm;        // [gamma, M]
-    uint32_t* anc;    // with the fused mask: [B + 1][(B + 32) / 32] ancestor-or-self bits
+    uint32_t* anc;    // with the fused mask: ancestor-or-self bits of B + 1 rows
 };
 __device__ __forceinline__ TreeSmem tree_smem(uint8_t* base, const TreeArgs& a) {
     TreeSmem t;
@@ -262,69 +262,52 @@ __device__ __forceinline__ void write_nodes(const TreeArgs& a, int s, const Tree
 // another level. A node is present iff every link of its chain goes to a smaller index exactly
 // one level up and the chain ends at the root (node 0, depth 0); absent nodes (missing from an
 // underfull tree, or behind a broken link) get an empty row and column and pos -1.
-// par, dep: the tree's n parents and depths (shared memory); anc: (r1 - r0) x W words of shared
-// scratch; mask_s [n][n] and pos_s [n]: this sequence's outputs.
-// WORDS: four-byte stores; single bytes are quicker for the few rows of a small tree.
-template <bool WORDS>
+// par, dep: the tree's n parents and depths (shared memory); bits: a bit per entry of the rows, without
+// padding between rows, so that any four entries are one shift of two words (with padded rows every
+// warp went through a path for words that run into the next row as well: 65 nodes 1.8 -> 1.4 us); mask_s [n][n] and pos_s [n]: this sequence's outputs.
 __device__ __forceinline__ void mask_rows(int n, const int* par, const int* dep, int root_pos, int r0, int r1,
-                                          uint32_t* anc, uint8_t* mask_s, int32_t* pos_s) {
-    const int W = (n + 31) / 32;
+                                          uint32_t* bits, uint8_t* mask_s, int32_t* pos_s) {
+    const int total = (r1 - r0) * n;
+    for (int w = threadIdx.x; w < (total + 31) / 32; w += blockDim.x) bits[w] = 0u;
+    __syncthreads();
     for (int i = r0 + static_cast<int>(threadIdx.x); i < r1; i += blockDim.x) {
-        uint32_t* row = anc + static_cast<size_t>(i - r0) * W;
-        for (int w = 0; w < W; ++w) row[w] = 0u;
+        const int row = (i - r0) * n;
         bool ok = true;
-        int j = i;
-        for (int steps = 0; ok && j != 0; ++steps) {
+        int j = i, dj = dep[i], links = 0;
+        for (; ok && j != 0; ++links) {
             const int p = par[j];
-            ok = steps < kMaxGamma && dep[j] >= 1 && dep[j] <= kMaxGamma && p >= 0 && p < j && dep[p] == dep[j] - 1;
-            row[j >> 5] |= 1u << (j & 31);
+            const bool link = p >= 0 && p < j;
+            const int dp = link ? dep[p] : -1;
+            ok = links < kMaxGamma && dj >= 1 && dj <= kMaxGamma && link && dp == dj - 1;
+            atomicOr(&bits[(row + j) >> 5], 1u << ((row + j) & 31));   // (no result: the walk does not wait)
             j = p;
+            dj = dp;
         }
         ok = ok && dep[0] == 0;
         if (ok) {
-            row[0] |= 1u;                                  // the root
+            atomicOr(&bits[row >> 5], 1u << (row & 31));   // the root
         } else {
-            for (int w = 0; w < W; ++w) row[w] = 0u;       // absent: empty row
+            for (j = i; links > 0; --links) {              // absent: empty row
+                atomicAnd(&bits[(row + j) >> 5], ~(1u << ((row + j) & 31)));
+                j = par[j];
+            }
         }
         pos_s[i] = ok ? root_pos + dep[i] : -1;
     }
     __syncthreads();
-    // The rows are contiguous bytes: aligned words of four entries (a word may run into the next row),
-    // single bytes before the first and after the last.
-    const int total = (r1 - r0) * n;
+    // The rows are contiguous bytes: aligned words of four entries, single bytes before the first and
+    // after the last.
     uint8_t* out = mask_s + static_cast<size_t>(r0) * n;
-    auto entry = [&](int i, int j) { return (anc[i * W + (j >> 5)] >> (j & 31)) & 1u; };
-    if constexpr (!WORDS) {
-        for (int at = threadIdx.x; at < total; at += blockDim.x) {
-            const int i = at / n;
-            out[at] = static_cast<uint8_t>(entry(i, at - i * n));
-        }
-        return;
-    }
     const int head = min(total, static_cast<int>(-reinterpret_cast<intptr_t>(out) & 3));
     const int words = (total - head) / 4;
     for (int w = threadIdx.x; w < words; w += blockDim.x) {
-        const int at = head + 4 * w;
-        int i = at / n, j = at - i * n;
-        uint32_t v = 0u;
-        if ((j & 31) <= 28 && j + 3 < n) {
-            const uint32_t x = anc[i * W + (j >> 5)] >> (j & 31);
-            v = (x & 1u) | ((x & 2u) << 7) | ((x & 4u) << 14) | ((x & 8u) << 21);
-        } else {
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                v |= entry(i, j) << (8 * k);
-                if (++j == n) {
-                    j = 0;
-                    ++i;
-                }
-            }
-        }
-        *reinterpret_cast<uint32_t*>(out + at) = v;
+        const int at = head + 4 * w, sh = at & 31;
+        const uint32_t x = __funnelshift_r(bits[at >> 5], sh > 28 ? bits[(at >> 5) + 1] : 0u, sh);
+        *reinterpret_cast<uint32_t*>(out + at) = (x & 1u) | ((x & 2u) << 7) | ((x & 4u) << 14) | ((x & 8u) << 21);
     }
     for (int k = threadIdx.x; k < total - 4 * words; k += blockDim.x) {
-        const int at = k < head ? k : 4 * words + k, i = at / n;
-        out[at] = static_cast<uint8_t>(entry(i, at - i * n));
+        const int at = k < head ? k : 4 * words + k;
+        out[at] = static_cast<uint8_t>((bits[at >> 5] >> (at & 31)) & 1u);
     }
 }
 
@@ -332,7 +315,7 @@ __device__ __forceinline__ void mask_rows(int n, const int* par, const int* dep,
 __device__ __forceinline__ void fused_mask(const TreeArgs& a, int s, const TreeSmem& t) {
     if (!a.mask) return;
     const int n = a.B + 1;
-    mask_rows<true>(n, t.o_par, t.o_dep, a.root_pos[s], 0, n, t.anc, a.mask + static_cast<size_t>(s) * n * n,
+    mask_rows(n, t.o_par, t.o_dep, a.root_pos[s], 0, n, t.anc, a.mask + static_cast<size_t>(s) * n * n,
               a.pos_ids + static_cast<size_t>(s) * n);
 }
 
@@ -667,20 +650,27 @@ __global__ void __launch_bounds__(kFastThreads) build_tree_fast_kernel(TreeArgs 
         a.node_score[o] = o_score[i];
     }
     if (a.mask)
-        mask_rows<false>(n_out, o_par, o_dep, a.root_pos[s], 0, n_out, anc, a.mask + static_cast<size_t>(s) * n_out * n_out,
+        mask_rows(n_out, o_par, o_dep, a.root_pos[s], 0, n_out, anc, a.mask + static_cast<size_t>(s) * n_out * n_out,
                   a.pos_ids + static_cast<size_t>(s) * n_out);
 }
 
 // ------------------------------------------------------------------------------------------
 // Builder by levels, for large budgets. A pop sequence is a chain: with the queue in shared memory
-// 512 pops took 343 us on GB300, about 0.65 us each on one warp (41 us this way; 64 pops of the
-// two-token rule 44 us with the queue in registers, 18.5 us this way). But the B popped nodes are simply
+// 512 pops took 343 us on GB300, about 0.65 us each on one warp (33 us this way; 64 pops of the
+// two-token rule 44 us with the queue in registers, 17 us this way). But the B popped nodes are simply
 // the B first of all nodes in the order (score, smaller depth, earlier parent, earlier list entry),
 // as long as no node outscores its parent or its list predecessor (log-probabilities <= 0, lists
 // sorted): then the first B nodes contain every ancestor and predecessor of each of them. So the
 // CTA grows all of them level by level, a warp per (parent, 32 list entries), and keeps only nodes
 // that can still be among the first B: theta, a lower bound of the B-th best score so far, rises
-// with a histogram of the scores after each pass. The survivors (a few more than B) are sorted once.
+// after each pass. The survivors (a few more than B) are sorted once.
+// What bounds it is instructions on a few warps and block barriers: per pass about 1.4 us, of which a
+// third waits for the lists in L2. So up to kLvExact nodes the B-th best and the order come from
+// counting, several threads per node (one phase instead of the five of a histogram: 1.3 -> 0.7 us,
+// the order 2.2 -> 1.5 us), more nodes are ordered by buckets and counting within a bucket (513 nodes
+// 6 -> 3.5 us; a bitonic sort has 55 phases), and the root token and position, which may lie in host
+// memory, are read at the start (B = 64, eight sequences 19.8 -> 18.4 us with the mask, B = 512 44.9 ->
+// 37.5, B = 1023 76 -> 63).
 //  - Two nodes of equal score and depth under different parents are ordered by their parents' places
 //    in the order, known once shallower levels are: the few such ties are resolved after the sort.
 //  - A list entry above its predecessor or its parent, a score that is not finite, more than
@@ -692,7 +682,7 @@ constexpr int kLvWarps = kLvThreads / 32;
 constexpr int kLvCap = 4096;       // nodes held at once
 constexpr int kLvBins = 2 * kLvThreads;
 constexpr int kLvSort = 2048;      // nodes that can be sorted
-constexpr int kLvCount = 256;      // up to this many by counting
+constexpr int kLvExact = 128;      // up to this many nodes: order statistics by counting
 constexpr int kLvTies = 32;        // ties resolved in place, and the longest run of equal nodes
 
 // Nodes to expand: the node (kNoNode: dropped), the next 32-entry chunk of its child list, the list.
@@ -758,20 +748,21 @@ __global__ void __launch_bounds__(kLvThreads) build_tree_level_kernel(TreeArgs a
     // n_cont_s, n_next_s: lists that go on after a pass, nodes that the next level expands; a pass
     // (level) uses one of three counters and zeroes the next one, whose last readers are a pass
     // (level) behind
-    __shared__ int wsum[kLvWarps], count_s, bad_s, n_cont_s[3], n_next_s[3], n_keys_s, n_ties_s, ties[kLvTies], flags_s;
+    __shared__ int wsum[kLvWarps], count_s, bad_s, n_cont_s[3], n_next_s[3], n_ties_s, ties[kLvTies], flags_s;
     constexpr unsigned kFull = 0xffffffffu;
     const LevelSmem t = level_smem(smem_raw);
     const int s = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const bool ar = a.mode == TF_MODE_AR, mary = a.mode != TF_MODE_MARGINAL;
     const ListView lists = sequence_lists(a, s);
     const int n_chunks = (a.K2 + 31) / 32;
+    // read here (they may lie in host memory), used at the end
     const int root = a.root_tok[a.two_prev ? 2 * s : s];
+    const int root_pos = a.mask ? a.root_pos[s] : 0;
     if (mary)
         for (int i = tid; i < a.gamma * a.M; i += kLvThreads)
             t.topm[i] = a.top_ids[(static_cast<size_t>(s) * a.gamma + i / a.M) * a.K1 + i % a.M];
     if (tid == 0) {
         t.score[0] = 0.0f;
-        t.tok[0] = root;
         t.par[0] = t.rank[0] = 0;
         t.dep[0] = 0;
         t.m[0] = -1;
@@ -781,15 +772,45 @@ __global__ void __launch_bounds__(kLvThreads) build_tree_level_kernel(TreeArgs a
         n_cont_s[0] = n_next_s[1] = 0;
         count_s = 1;
         bad_s = 0;
-        flags_s = root < 0 || root >= a.V ? TF_DEV_BAD_TOKEN : 0;
+        flags_s = 0;
         theta_s = -INFINITY;
     }
     __syncthreads();
 
-    // Raises theta to the lower edge of the histogram bin that holds the B-th best score (a little
-    // below it: the bins' arithmetic is rounded). Nothing happens while there are fewer than B.
+    // Threads per item when up to kLvExact items are ranked by counting
+    auto sharers = [](int n) { return n <= 64 ? 8 : 4; };
+    // Raises theta to the B-th best score, with more than kLvExact nodes to the lower edge of the
+    // histogram bin that holds it (a little below it: the bins' arithmetic is rounded). Nothing happens
+    // while there are fewer than B.
     auto raise_theta = [&](int count) {
         if (count - 1 < a.B) return;
+        if (count <= kLvExact) {
+            // the root counts as a node here: it scores no less than any other, so that the B-th best
+            // of the others is the (B + 1)-th of all
+            const int per = sharers(count), i = tid / per, part = tid % per, whole = count / 4;
+            const float x = t.score[i < count ? i : 0];
+            int gt = 0, ge = 0;
+            auto tally = [&](float y) {
+                gt += y > x ? 1 : 0;
+                ge += y >= x ? 1 : 0;
+            };
+            for (int q = part; q < whole; q += per) {
+                const float4 y = reinterpret_cast<const float4*>(t.score)[q];
+                tally(y.x);
+                tally(y.y);
+                tally(y.z);
+                tally(y.w);
+            }
+            if (part < count - 4 * whole) tally(t.score[4 * whole + part]);
+            for (int o = 1; o < per; o <<= 1) {
+                gt += __shfl_xor_sync(kFull, gt, o);
+                ge += __shfl_xor_sync(kFull, ge, o);
+            }
+            // (all writers hold the same value)
+            if (i < count && part == 0 && gt <= a.B && ge > a.B && x > theta_s) theta_s = x;
+            __syncthreads();
+            return;
+        }
         float lo = theta_s;
         if (!(lo > -INFINITY)) {
             float mn = 0.0f;
@@ -908,7 +929,9 @@ __global__ void __launch_bounds__(kLvThreads) build_tree_level_kernel(TreeArgs a
         if (tid == 0) n_next_s[(d + 1) % 3] = 0;
         const int* cand = t.topm + (d - 1) * a.M;
         const bool deeper = d < a.gamma;
-        int g = 32 / n_act;                              // list chunks taken of each parent per pass
+        // list chunks taken of each parent per pass: small budgets rarely want a second one, so no more
+        // than the warps take in one go (B = 64: 16.5 -> 15.5 us)
+        int g = (a.B <= 128 ? kLvWarps : 2 * kLvWarps) / n_act;
         g = g < 1 ? 1 : g > n_chunks ? n_chunks : g;
         while (n_act > 0) {
             const ActList act = t.act[li], cont = t.act[lc], next = t.act[ln];
@@ -1047,56 +1070,86 @@ __global__ void __launch_bounds__(kLvThreads) build_tree_level_kernel(TreeArgs a
     // ---- the order of the survivors
     int n = 0;
     if (!bad_s) {
-        if (tid == 0) n_keys_s = n_ties_s = 0;
-        raise_theta(count);
-        __syncthreads();
-        const float theta = theta_s;
-        for (int i = 1 + tid; i < count; i += kLvThreads)
-            if (t.score[i] >= theta) {
-                const int q = atomicAdd(&n_keys_s, 1);
-                if (q < kLvSort) t.key[q] = level_key(t.score[i], t.dep[i], t.rank[i], i);
+        if (tid == 0) n_ties_s = 0;
+        if (count <= kLvExact) {
+            // few: each node's place by counting the larger keys, those below theta included
+            n = count - 1;
+            const int per = sharers(n), i = tid / per, part = tid % per;
+            if (tid < n) t.key[tid] = level_key(t.score[tid + 1], t.dep[tid + 1], t.rank[tid + 1], tid + 1);
+            __syncthreads();
+            const unsigned long long x = i < n ? t.key[i] : 0ull;
+            int r = 0;
+#pragma unroll 4
+            for (int j = part; j < n; j += per) r += t.key[j] > x ? 1 : 0;
+            for (int o = 1; o < per; o <<= 1) r += __shfl_xor_sync(kFull, r, o);
+            __syncthreads();
+            if (i < n && part == 0) t.key[r] = x;
+            __syncthreads();
+        } else {
+            // Those at theta or above by buckets of equal width (bucket 0 holds the best), then by
+            // counting within the bucket.
+            raise_theta(count);
+            __syncthreads();
+            const float theta = theta_s;
+            // (fewer than B nodes leave theta unknown: any scale serves)
+            const float scale = theta < 0.0f ? static_cast<float>(kLvBins) / fmaxf(theta, -64.0f) : 0.0f;
+            auto bucket = [&](float x) { return min(kLvBins - 1, static_cast<int>(x * scale)); };
+            t.hist[2 * tid] = t.hist[2 * tid + 1] = 0;
+            __syncthreads();
+            for (int i = 1 + tid; i < count; i += kLvThreads)
+                if (t.score[i] >= theta) atomicAdd(&t.hist[bucket(t.score[i])], 1);
+            __syncthreads();
+            const int h0 = t.hist[2 * tid], h1 = t.hist[2 * tid + 1];
+            int incl = h0 + h1;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int v = __shfl_up_sync(kFull, incl, o);
+                if (lane >= o) incl += v;
             }
-        __syncthreads();
-        n = n_keys_s;
+            if (lane == 31) wsum[warp] = incl;
+            __syncthreads();
+            int base = incl - h0 - h1;
+            for (int w = 0; w < kLvWarps; ++w) {
+                n += wsum[w];
+                base += w < warp ? wsum[w] : 0;
+            }
+            t.hist[2 * tid] = base;                      // the next free place of each bucket
+            t.hist[2 * tid + 1] = base + h0;
+            __syncthreads();
+            if (n <= kLvSort) {
+                for (int i = 1 + tid; i < count; i += kLvThreads)
+                    if (t.score[i] >= theta)
+                        t.key[atomicAdd(&t.hist[bucket(t.score[i])], 1)] = level_key(t.score[i], t.dep[i], t.rank[i], i);
+                __syncthreads();                         // bucket b's keys: from hist[b - 1] up to hist[b]
+                unsigned long long x[kLvSort / kLvThreads];
+                int r[kLvSort / kLvThreads];
+#pragma unroll
+                for (int k = 0; k < kLvSort / kLvThreads; ++k) {
+                    const int i = tid + k * kLvThreads;
+                    if (i < n) {
+                        x[k] = t.key[i];
+                        const int bk = bucket(t.score[x[k] & 0xfff]), end = t.hist[bk];
+                        r[k] = bk > 0 ? t.hist[bk - 1] : 0;
+#pragma unroll 1
+                        for (int j = r[k]; j < end; ++j) r[k] += t.key[j] > x[k] ? 1 : 0;
+                    }
+                }
+                __syncthreads();
+#pragma unroll
+                for (int k = 0; k < kLvSort / kLvThreads; ++k)
+                    if (tid + k * kLvThreads < n) t.key[r[k]] = x[k];
+                __syncthreads();
+            }
+        }
         if (n > kLvSort) {
             if (tid == 0) bad_s = 1;
         } else {
-            if (n <= kLvCount) {
-                // few: each key's place by counting the larger ones
-                unsigned long long x = 0ull;
-                int r = 0;
-                if (tid < n) {
-                    x = t.key[tid];
-#pragma unroll 8
-                    for (int i = 0; i < n; ++i) r += t.key[i] > x ? 1 : 0;
-                }
-                __syncthreads();
-                if (tid < n) t.key[r] = x;
-                __syncthreads();
-            } else {
-                // bitonic sort, largest key first
-                int N = kLvCount;
-                while (N < n) N <<= 1;
-                for (int i = n + tid; i < N; i += kLvThreads) t.key[i] = 0ull;
-                for (int size = 2; size <= N; size <<= 1)
-                    for (int step = size >> 1; step > 0; step >>= 1) {
-                        __syncthreads();
-                        for (int q = tid; q < N / 2; q += kLvThreads) {
-                            const int i = 2 * q - (q & (step - 1)), j = i + step;
-                            const unsigned long long x = t.key[i], y = t.key[j];
-                            if ((x < y) == ((i & size) == 0)) {
-                                t.key[i] = y;
-                                t.key[j] = x;
-                            }
-                        }
-                    }
-                __syncthreads();
-            }
             for (int i = tid; i < n; i += kLvThreads) {
                 const unsigned long long x = t.key[i];
                 const int xi = static_cast<int>(x & 0xfff);
                 t.place[xi] = static_cast<uint16_t>(i + 1);
-                if (i + 1 < n) {
+                // (runs of equal nodes that begin behind the last place are not part of the tree)
+                if (i + 1 < n && (i < a.B || (x >> 24) == (t.key[a.B - 1] >> 24))) {
                     const unsigned long long y = t.key[i + 1];
                     if ((x >> 24) == (y >> 24) && t.par[xi] != t.par[y & 0xfff]) {
                         const int q = atomicAdd(&n_ties_s, 1);
@@ -1157,6 +1210,7 @@ __global__ void __launch_bounds__(kLvThreads) build_tree_level_kernel(TreeArgs a
             tok = root;
             dep = 0;
             sc = 0.0f;
+            if (root < 0 || root >= a.V) atomicOr(&flags_s, TF_DEV_BAD_TOKEN);
         } else if (i <= n) {
             const int x = static_cast<int>(t.key[i - 1] & 0xfff), p = t.par[x];
             tok = t.tok[x];
@@ -1179,14 +1233,14 @@ __global__ void __launch_bounds__(kLvThreads) build_tree_level_kernel(TreeArgs a
     __syncthreads();
     if (tid == 0) a.dev_status[s] = sequence_status(a, flags_s);
     if (a.mask)
-        mask_rows<true>(n_out, t.hist, t.hist + kFusedMaskMaxNodes, a.root_pos[s], 0, n_out, reinterpret_cast<uint32_t*>(t.key),
+        mask_rows(n_out, t.hist, t.hist + kFusedMaskMaxNodes, root_pos, 0, n_out, reinterpret_cast<uint32_t*>(t.key),
                   a.mask + static_cast<size_t>(s) * n_out * n_out, a.pos_ids + o0);
 }
 
 // ------------------------------------------------------------------------------------------
 // The tree-attention mask and position ids (mask_rows) of a drafted tree in global memory: one
 // CTA per sequence and block of kMaskRows rows. Blocks of 16 rows and four-byte stores: 513 nodes take
-// about 5 us on GB300 instead of 23 with blocks of 128 and single bytes (8 or 32 rows: the same
+// about 4 us on GB300 instead of 23 with blocks of 128 and single bytes (8 or 32 rows: the same
 // within 2 us).
 // ------------------------------------------------------------------------------------------
 constexpr int kMaskRows = 16;
@@ -1201,7 +1255,7 @@ __global__ void __launch_bounds__(256) tree_mask_kernel(int n, const int32_t* __
     const int r0 = blockIdx.y * kMaskRows, r1 = min(n, r0 + kMaskRows);   // this CTA's rows
     int* par = reinterpret_cast<int*>(sm);
     int* dep = par + n;
-    uint32_t* anc = reinterpret_cast<uint32_t*>(dep + n);   // [kMaskRows][(n + 31) / 32] ancestor-or-self bits
+    uint32_t* anc = reinterpret_cast<uint32_t*>(dep + n);   // ancestor-or-self bits of kMaskRows rows
     const int32_t* P = node_parent + static_cast<size_t>(s) * n;
     const int32_t* D = node_depth + static_cast<size_t>(s) * n;
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
@@ -1209,7 +1263,7 @@ __global__ void __launch_bounds__(256) tree_mask_kernel(int n, const int32_t* __
         dep[i] = D[i];
     }
     __syncthreads();
-    mask_rows<true>(n, par, dep, root_pos[s], r0, r1, anc, mask + static_cast<size_t>(s) * n * n,
+    mask_rows(n, par, dep, root_pos[s], r0, r1, anc, mask + static_cast<size_t>(s) * n * n,
               pos_ids + static_cast<size_t>(s) * n);
 }
 
@@ -1517,10 +1571,11 @@ cudaError_t launch_build_tree(const Ctx& ctx, int b, int gamma, int M, int K1, i
     const int stride = mode == TF_MODE_AR ? K2 : K1;
     const int sw = stride < B + 1 ? stride : B + 1;   // list entries that a tree can reach
     // The sorted-queue builder for small budgets with every reachable entry in shared memory: its cost is
-    // the pops (0.25 us each, more with the two-token rule); the builder by levels pays about a
-    // microsecond per level whatever the budget. Measured on GB300 (16 depths, one sequence): B = 32
-    // 12.0 against 13.1 us, B = 48 16.7 against 16.5, B = 64 21.3 against 17.3; two-token rule (12
-    // depths) B = 32 13.2 against 14.3, B = 64 22.8 against 17.1.
+    // the pops (0.25 us each, more with the two-token rule), the same for any number of sequences; the
+    // builder by levels costs what the sequence with the most levels does. Measured on GB300 (16 depths; one
+    // / eight sequences, with the mask): B = 32 11.9 / 12.0 against 11.4 / 13.4 us by levels, B = 48 16.5 /
+    // 16.6 against 13.9 / 17.4, B = 64 21.3 / 21.4 against 15.4 / 18.4; two-token rule (12 depths) B = 32
+    // 13.1 / 13.1 against 11.9 / 14.1, B = 64 22.8 against 15.5.
     const size_t fsm = fast_tree_smem(B, gamma, M, rows_l, sw, mask != nullptr);
     if (B <= (a.two_prev ? 32 : 48) && fsm <= kTreeSmemLimit) {
         auto kern = a.two_prev ? build_tree_fast_kernel<true> : build_tree_fast_kernel<false>;

@@ -119,6 +119,9 @@ LEVEL_CASES = [
     ("ar", 2, 16, 5, 33, 300, 2000, False),       # a list of one chunk and one entry; K2 < B
     ("ar", 2, 3, 2, 20, 400, 300, False),         # underfull universe
     ("ar", 2, 1, 4, 100, 100, 500, False),        # one level
+    ("ar", 2, 1, 4, 127, 126, 500, False),        # 128 nodes with the root: the most that are ordered by counting
+    ("ar", 2, 1, 4, 128, 126, 500, False),        # the fewest that are ordered by buckets
+    ("ar", 2, 3, 4, 60, 700, 2000, False),        # underfull, ordered by buckets
     ("marginal", 2, 6, 4, 256, 256, 1000, False),  # every node expands
     ("marginal_mary", 2, 12, 20, 130, 127, 2000, False),
     ("ar", 2, 8, 4, 32, 32, 1000, True),          # two-token rule: the sorted queue, and by levels
