@@ -1142,6 +1142,20 @@ int resident_clusters(K kern, int smem, int cl, int num_sms) {
     return n < cap ? n : cap;
 }
 
+// Tail split: when the units overflow the SMs by a last round that would leave most of them idle, each
+// unit of that round runs as up to kMaxTailSplit K-chunks on the idle SMs, summed by the chunk that
+// finishes last (fp32 partial sums in the workspace). K-chunks per unit, or 0: no tail split. A pair's
+// unit of 256 columns counts for two SMs (slots), one of 128 + 128 for one.
+int tail_chunks(const Ctx& ctx, int n_units, int slots, int m_tiles, int cols, int K, size_t partial_bytes) {
+    const int tail = n_units % slots;
+    int split = tail > 0 ? slots / tail : 0;
+    split = split < kMaxTailSplit ? split : kMaxTailSplit;
+    split = split < K / kBK ? split : K / kBK;
+    const size_t need = static_cast<size_t>(tail) * split * m_tiles * kBM * cols * sizeof(float);
+    const bool fits = ctx.status && tail * m_tiles <= kTailSems && need <= partial_bytes;
+    return n_units > slots && split >= 2 && fits ? split : 0;
+}
+
 template <int EPI, int MT, int NB, int BN, int STAGES, int CL = 1>
 cudaError_t run_gemm(const Ctx& ctx, const XMaps& tx, const CUtensorMap& tw0, const CUtensorMap& tw1,
                      int n_rows, int K, int n_ntiles, int n_mgroups, const EpiParams& ep_in, int k_splits = 1,
@@ -1162,21 +1176,12 @@ cudaError_t run_gemm(const Ctx& ctx, const XMaps& tx, const CUtensorMap& tw0, co
     }
     int n_items = n_units;
     if constexpr (EPI == EPI_GATEUP || EPI == EPI_DOWN) {
-        // Tail split: when the units overflow the SMs by a last round that would leave most of
-        // them idle, each unit of that round runs as up to kMaxTailSplit K-chunks on the idle
-        // SMs, summed by the chunk that finishes last (fp32 partial sums in the workspace). A
-        // pair's unit of 256 columns counts for two SMs, one of 128 + 128 for one (two rounds
-        // of pairs take the time of one round of single CTAs), so that the chunks of an output
-        // do not depend on whether pairs run it.
         constexpr int kTiles = CL == 1 ? MT : 2;
         const int slots = CL == 2 && NB == 1 ? ctx.num_sms / 2 : ctx.num_sms;
-        const int tail = n_units % slots;
-        int split = tail > 0 ? slots / tail : 0;
-        split = split < kMaxTailSplit ? split : kMaxTailSplit;
-        split = split < K / kBK ? split : K / kBK;
-        const size_t need = static_cast<size_t>(tail) * split * kTiles * kBM * NB * BN * sizeof(float);
-        if (k_splits == 1 && n_units > slots && split >= 2 && ctx.status && tail * kTiles <= kTailSems &&
-            ep.partial && need <= partial_bytes) {
+        const int split = k_splits == 1 && ep.partial
+                              ? tail_chunks(ctx, n_units, slots, kTiles, NB * BN, K, partial_bytes) : 0;
+        if (split) {
+            const int tail = n_units % slots;
             ep.n_full = n_units - tail;
             ep.tail_split = split;
             ep.sem = ctx.status + 1;
@@ -1380,8 +1385,23 @@ static cudaError_t run_residual_gemm(const Ctx& ctx, const XMaps& ta, const void
         e = m_tiles == 1 ? run_gemm_cluster<EPI_CDOWN, 1, 1>(ctx, ta, W, nullptr, d, n_rows, K, 1, ks2, ed, partial_bytes, &done)
                          : run_gemm_cluster<EPI_CDOWN, 2, 1>(ctx, ta, W, nullptr, d, n_rows, K, n_mg, ks2, ed, partial_bytes, &done);
     if (done || e != cudaSuccess) return e;
-    const bool pair = m_tiles > 1 && d % 256 == 0 && d / 256 * n_mg * ks2 >= kMinPairs;
+    // With a tail split pairs take over only where they chunk the same outputs, and widths are not
+    // chosen, so that which outputs are summed in chunks, and so their bits, does not depend on the kernel
+    // that runs: near ties of a tree follow the last bit of h'. Pairs for other tails would save 0.5 % of a
+    // step (32 sequences, 3872 rows, d = 4096: 4132 against 4155 us), widths chosen all the same most where
+    // they replace tiles of 64 (720 rows, d = 3776, I = 11072: 671 against 730 us).
+    const int units = d / bn_d * n_mg;
+    const int tail = ks2 == 1 && tail_chunks(ctx, units, ctx.num_sms, m_tiles == 1 ? 1 : 2, bn_d, K, partial_bytes)
+                         ? units % ctx.num_sms : 0;
+    const bool pair = m_tiles > 1 && d % 256 == 0 && d / 256 * n_mg * ks2 >= kMinPairs && tail % (2 * n_mg) == 0;
     if (ks2 == 1) {
+        if (tail && !pair) {
+            if (bn_d == BN)
+                return m_tiles == 1 ? run_gemm<EPI_DOWN, 1, 1, BN, 6>(ctx, ta, td, td, n_rows, K, d / BN, 1, ed, 1, partial_bytes)
+                                    : run_gemm<EPI_DOWN, 2, 1, BN, 4>(ctx, ta, td, td, n_rows, K, d / BN, n_mg, ed, 1, partial_bytes);
+            return m_tiles == 1 ? run_gemm<EPI_DOWN, 1, 1, 64, 8>(ctx, ta, td, td, n_rows, K, d / 64, 1, ed, 1, partial_bytes)
+                                : run_gemm<EPI_DOWN, 2, 1, 64, 5>(ctx, ta, td, td, n_rows, K, d / 64, n_mg, ed, 1, partial_bytes);
+        }
         if (pair) return run_gemm<EPI_DOWN, 1, 1, 256, 7, 2>(ctx, ta, td, td, n_rows, K, d / 256, n_mg, ed, 1, partial_bytes);
         return m_tiles == 1 ? run_gemm_var<EPI_DOWN, 1, 1>(ctx, ta, W, nullptr, d, n_rows, K, 1, 1, ed)
                             : run_gemm_var<EPI_DOWN, 2, 1>(ctx, ta, W, nullptr, d, n_rows, K, n_mg, 1, ed);
@@ -1424,9 +1444,18 @@ cudaError_t launch_swiglu_tc(const Ctx& ctx, const void* X, int k_in, const void
     if (ks1 > 1)
         e = m_tiles == 1 ? run_gemm_cluster<EPI_CGATEUP, 1, 2>(ctx, tx, w_gate, w_up, I, n_rows, k_in, 1, ks1, ep, partial_bytes, &done)
                          : run_gemm_cluster<EPI_CGATEUP, 2, 2>(ctx, tx, w_gate, w_up, I, n_rows, k_in, n_mg, ks1, ep, partial_bytes, &done);
+    const int units = I / bn_gu * n_mg;
     if (done || e != cudaSuccess) {
+    } else if (ks1 == 1 && tail_chunks(ctx, units, ctx.num_sms, m_tiles == 1 ? 1 : 2, 2 * bn_gu, k_in, partial_bytes)) {
+        // a tail split: fixed widths, as in the down projection
+        if (bn_gu == BN)
+            e = m_tiles == 1 ? run_gemm<EPI_GATEUP, 1, 2, BN, 4>(ctx, tx, tg, tu, n_rows, k_in, I / BN, 1, ep, 1, partial_bytes)
+                             : run_gemm<EPI_GATEUP, 2, 2, BN, 3>(ctx, tx, tg, tu, n_rows, k_in, I / BN, n_mg, ep, 1, partial_bytes);
+        else
+            e = m_tiles == 1 ? run_gemm<EPI_GATEUP, 1, 2, 64, 6>(ctx, tx, tg, tu, n_rows, k_in, I / 64, 1, ep, 1, partial_bytes)
+                             : run_gemm<EPI_GATEUP, 2, 2, 64, 4>(ctx, tx, tg, tu, n_rows, k_in, I / 64, n_mg, ep, 1, partial_bytes);
     } else if (m_tiles > 1 && bn_gu == BN && ks1 == 1 && I / BN * n_mg > ctx.num_sms) {
-        e = run_gemm<EPI_GATEUP, 2, 2, BN, 3>(ctx, tx, tg, tu, n_rows, k_in, I / BN, n_mg, ep, 1, partial_bytes);
+        e = run_gemm<EPI_GATEUP, 2, 2, BN, 3>(ctx, tx, tg, tu, n_rows, k_in, I / BN, n_mg, ep);
     } else if (ks1 == 1) {
         e = m_tiles == 1 ? run_gemm_var<EPI_GATEUP, 1, 2>(ctx, tx, w_gate, w_up, I, n_rows, k_in, 1, 1, ep)
                          : run_gemm_var<EPI_GATEUP, 2, 2>(ctx, tx, w_gate, w_up, I, n_rows, k_in, n_mg, 1, ep);

@@ -160,6 +160,20 @@ def test_bf16_tail_split_of_the_last_round():
         np.testing.assert_array_equal(gpu[k], again[k], err_msg=k)
 
 
+# (batch, d, I): tail splits of other tiles than 128 columns of two M-tiles (13 rows per sequence, 152 SMs)
+TAIL_TILES = [
+    (2, 320, 9920),     # gate/up, one M-tile, 155 tiles of 64 columns
+    (24, 320, 4928),    # gate/up, 3 M-tiles, 77 x 2 units of 64 columns
+    (24, 4928, 192),    # down, the same, and fewer K-steps than chunks
+    (40, 6656, 192),    # down, 52 x 3 units of 128 columns, four of them in chunks: not the ones pairs would chunk
+]
+
+
+@pytest.mark.parametrize("b,d,I", TAIL_TILES)
+def test_bf16_tail_split_of_other_tiles(b, d, I):
+    check(synth.get_config("tiny_peaked", dtype="bf16", batch=b, d=d, I=I, V=2000, wd_std=0.05))
+
+
 @pytest.mark.parametrize("mode", ["marginal", "marginal_mary"])
 def test_bf16_marginal_modes(mode):
     check(synth.get_config("tiny_peaked", dtype="bf16", batch=3, V=2000, mode=mode))
