@@ -1572,12 +1572,15 @@ cudaError_t launch_build_tree(const Ctx& ctx, int b, int gamma, int M, int K1, i
     const int sw = stride < B + 1 ? stride : B + 1;   // list entries that a tree can reach
     // The sorted-queue builder for small budgets with every reachable entry in shared memory: its cost is
     // the pops (0.25 us each, more with the two-token rule), the same for any number of sequences; the
-    // builder by levels costs what the sequence with the most levels does. Measured on GB300 (16 depths; one
-    // / eight sequences, with the mask): B = 32 11.9 / 12.0 against 11.4 / 13.4 us by levels, B = 48 16.5 /
-    // 16.6 against 13.9 / 17.4, B = 64 21.3 / 21.4 against 15.4 / 18.4; two-token rule (12 depths) B = 32
-    // 13.1 / 13.1 against 11.9 / 14.1, B = 64 22.8 against 15.5.
+    // builder by levels costs what the sequence with the most levels does, so the line rises with the
+    // number of sequences. Measured on GB300 (16 depths, with the mask; queue against levels): one sequence
+    // B = 32 11.9, 11.4 us, B = 40 14.3, 13.6, B = 48 16.5, 13.9; four B = 40 14.4, 15.1, B = 48 16.5, 16.2;
+    // eight B = 48 16.6, 17.4, B = 52 18.0, 17.8, B = 64 21.0, 18.4; 32 sequences B = 52 17.9, 19.9, B = 56
+    // 19.0, 20.4, B = 64 21.0, 20.7; two-token rule (12 depths) B = 32 13.1 in both cases against 11.9 for one
+    // sequence and 14.1 for eight, B = 40, eight sequences 15.8, 15.6.
+    const int queue_budget = a.two_prev ? 32 : b <= 2 ? 40 : b < 16 ? 48 : 60;
     const size_t fsm = fast_tree_smem(B, gamma, M, rows_l, sw, mask != nullptr);
-    if (B <= (a.two_prev ? 32 : 48) && fsm <= kTreeSmemLimit) {
+    if (B <= queue_budget && fsm <= kTreeSmemLimit) {
         auto kern = a.two_prev ? build_tree_fast_kernel<true> : build_tree_fast_kernel<false>;
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(fsm));
         if (e != cudaSuccess) return e;

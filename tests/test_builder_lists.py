@@ -2,9 +2,9 @@
 bit for bit (tokens, parents, depths, scores, status). Log-probabilities are multiples of 1/8 (or
 1/4096) in [-6, 0], so every path score is exact in fp32 and fp64 alike and equal scores are frequent
 (or a few per tree: the tie rules decide many pops, or some); a random share of every list's tokens are stage-1 candidates of the
-list's depth, so the M-ary rule expands often and the trees grow deep and wide. Budgets up to 48
-(two-token rule: 32) run the sorted-queue builder, larger ones the builder by levels, which hands trees
-with many ties to the queue in shared memory."""
+list's depth, so the M-ary rule expands often and the trees grow deep and wide. Budgets up to 40
+(from three sequences on 48, from sixteen on 60; two-token rule: 32) run the sorted-queue builder, larger
+ones the builder by levels, which hands trees with many ties to the queue in shared memory."""
 import numpy as np
 import pytest
 import torch
@@ -112,8 +112,12 @@ O_UNDERFULL = 2   # TF_DEV_UNDERFULL
 
 LEVEL_CASES = [
     # mode, batch, gamma, M, K2, B, V, two-token rule
-    ("ar", 3, 16, 16, 48, 48, 3000, False),       # the largest budget of the sorted queue
+    ("ar", 3, 16, 16, 48, 48, 3000, False),       # the largest budget of the sorted queue for 3 to 15 sequences
     ("ar", 3, 16, 16, 49, 49, 3000, False),       # the smallest of the builder by levels
+    ("ar", 2, 12, 8, 40, 40, 2000, False),        # the same for one and two
+    ("ar", 2, 12, 8, 41, 41, 2000, False),
+    ("ar", 16, 6, 4, 60, 60, 400, False),         # and from 16 on
+    ("ar", 16, 6, 4, 61, 61, 400, False),
     ("ar", 2, 16, 16, 512, 512, 5000, False),     # exact lists, sixteen chunks per list
     ("ar", 2, 4, 64, 500, 1023, 5000, False),     # the largest budget, wide branching: nodes dropped as theta rises
     ("ar", 2, 16, 5, 33, 300, 2000, False),       # a list of one chunk and one entry; K2 < B
