@@ -218,7 +218,8 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant
     uint64_t* tfull = empty + STAGES;
     uint64_t* tempty = tfull + 2;
     uint64_t* drain = tempty + 2;
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
+    uint64_t* meet = drain + 1;   // [4]: where epilogue warps wait for one another
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(meet + 4);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
     volatile int* last_chunk = abort_flag + 1;   // [2]: this group's chunk was its unit's last
 
@@ -285,6 +286,8 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant
             ptx::mbar_init(&tempty[g], kPair ? 2 * (kEpiWarps / 2) : 32 * kEpiWarps / 2);
         }
         ptx::mbar_init(drain, 1);
+        // one arrival per warp: the warps of a group (tail split), of a group and column half (copies)
+        for (int i = 0; i < 4; ++i) ptx::mbar_init(&meet[i], EPI == EPI_LMHEAD ? kEpiWarps / 4 : kEpiWarps / 2);
         *abort_flag = 0;
         ptx::fence_barrier_init();
     }
@@ -520,8 +523,24 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant
         const int g = e / (kEpiWarps / 2);          // accumulator slot of this group
         const int q = warp & 3;                     // TMEM lane quarter of this warp
         const int half = (e % (kEpiWarps / 2)) / 4; // which half of the columns this warp takes
-        uint32_t use = 0;
+        uint32_t use = 0, met = 0;
         int kl = 0;
+        // A wait of this warp, with one outcome for its 32 lanes: a lane that gave up alone would be missing
+        // from the warp-collective loads that follow.
+        auto wait_warp = [&](uint64_t* bar, uint32_t parity) {
+            if (__all_sync(0xffffffffu, ptx::mbar_wait(bar, parity, abort_flag, wait_ns))) return true;
+            *abort_flag = 1;
+            set_status(status, TF_DEV_TIMEOUT);
+            return false;
+        };
+        // Meeting i of the epilogue warps that share it, after which each sees what the others wrote. Each warp
+        // decides by itself whether its accumulator came in time, so one that has given up never
+        // arrives here: the others give up in turn, where a hardware barrier would keep them for ever.
+        auto meet_warps = [&](int i) {
+            __syncwarp();
+            if (lane == 0) ptx::mbar_arrive(&meet[i]);
+            return wait_warp(&meet[i], met++ & 1u);
+        };
         // hands the accumulator slot back to the MMA issuer; in a pair one arrival per warp on
         // the even CTA's barrier, after the warp's TMEM loads have completed
         auto release_slot = [&](int slot) {
@@ -535,11 +554,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant
         };
         for (int u = cid; u < n_items; u += ncl, ++kl) {
             if (MT == 1 && !kShare && (kl & 1) != g) continue;
-            if (!ptx::mbar_wait(&tfull[kShare ? 0 : g], use & 1u, abort_flag, wait_ns)) {
-                *abort_flag = 1;
-                set_status(status, TF_DEV_TIMEOUT);
-                break;
-            }
+            if (!wait_warp(&tfull[kShare ? 0 : g], use & 1u)) break;
             ++use;
             ptx::tc_fence_after();
             const Item itm = item_of(u);
@@ -574,13 +589,13 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant
                 }
                 release_slot(g);
                 __threadfence();                                // this thread's partial sums, device-wide
-                ptx::named_barrier_sync(1 + g, 32 * kEpiWarps / 2);
+                if (!meet_warps(g)) break;
                 if (e % (kEpiWarps / 2) == 0 && lane == 0) {
                     __threadfence();
                     const int done = atomicAdd(ep.sem + itm.tail * kUnitTiles + j, 1);
                     last_chunk[g] = done == n_split - 1 ? 1 : 0;
                 }
-                ptx::named_barrier_sync(1 + g, 32 * kEpiWarps / 2);
+                if (!meet_warps(g)) break;
                 if (last_chunk[g]) {
                     __threadfence();                            // every chunk's partial sums
                     // 8 output columns at a time: this warp's half of the tile
@@ -635,8 +650,8 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant
                                 make_uint4(o[0], o[1], o[2], o[3]);
                         }
                     }
-                    // the count starts from zero for the next call
-                    ptx::named_barrier_sync(1 + g, 32 * kEpiWarps / 2);
+                    // the count starts from zero for the next call (nothing reads it before: every chunk has
+                    // been counted)
                     if (e % (kEpiWarps / 2) == 0 && lane == 0) ep.sem[itm.tail * kUnitTiles + j] = 0;
                 }
             } else if constexpr (kSplitK) {
@@ -692,10 +707,10 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant
                         if (crow < n_rows) P.halves[P.half_at(nt, half, crow)] = make_float4(hm, hsum, hm, __int_as_float(hid));
                     } else {
                         // the half's copies meet in shared memory; the first one folds them in chunk order.
-                        // (A buffer is written again two units later, after a barrier that its readers pass.)
+                        // (A buffer is written again two units later, after a meeting that its readers have come to.)
                         float4* sums = copy_sums + ((g * 2 + half) * 2 + (use & 1u)) * kBM;
                         sums[copy * (kBM / copies) + crow] = make_float4(hm, hsum, 0.0f, __int_as_float(hid));
-                        ptx::named_barrier_sync(1 + g * 2 + half, 128);
+                        if (!meet_warps(g * 2 + half)) break;
                         if (copy == 0 && crow < n_rows) {
                             for (int c = 1; c < copies; ++c) {
                                 const float4 o = sums[c * (kBM / copies) + crow];
