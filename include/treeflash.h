@@ -111,7 +111,9 @@ typedef struct {
                              TF_APPROX_LINEAR, I is ignored */
 } tf_dims;
 
-/* Model parameters (device, dims->dtype, row-major, read only, never copied). */
+/* Model parameters (device, dims->dtype, row-major, read only, never copied). The kernels read them, and
+ * nothing else, before the kernel just ahead on the stream has finished, if that kernel lets its
+ * dependents start early (programmatic dependent launch): such a kernel must not write them. */
 typedef struct {
     const void* lm_head;  /* [V, d]  verifier output embedding W_lm */
     const void* embed;    /* [V, d]  verifier input embedding Embd */

@@ -15,7 +15,6 @@ namespace {
 //  x_{t-1}) = root_tok[2 sq], root_tok[2 sq + 1]; rows 1..M depth 2 with (candidate m of depth 1,
 //  x_t); row 1 + M + (i-3) M^2 + m1 M + m2 depth i >= 3 with (candidate m1 of depth i-1,
 //  candidate m2 of depth i-2).
-// The hidden-state index needs no kernel's output, so it is separate from the token reads.
 // ------------------------------------------------------------------------------------------
 __device__ __forceinline__ int stage2_row_hidden(int row, int R, int gamma, int M, bool two_prev) {
     const int sq = row / R, r = row - sq * R;
@@ -1348,8 +1347,8 @@ __device__ __forceinline__ unsigned long long f2_bf16x2(uint32_t w) {
 // The stage-2 input rows for bf16 with d <= 8192: one item per normalised vector, not per row. The
 // M rows (two tokens: M^2) of a depth share their hidden state, so its part of x is computed once
 // per depth and stored to all of them (at most kHRows per item); every embedding is an item of its
-// own. Hidden-state items need no other kernel's output but the right to overwrite X, so they do
-// all but their stores before the dependency wait.
+// own. Only the norm weights are read before the dependency wait: the hidden states may be the output
+// of the kernel just before.
 // An item is a CTA of eight warps. (Items of one or two warps save the block barrier but hold so
 // much in registers that too few warps are in flight: 1928 rows of d = 5120 took 38 us with one CTA
 // per row, 73 with a warp per item.)
@@ -1384,7 +1383,7 @@ __global__ void __launch_bounds__(256) gather_norm_bf16_kernel(GatherArgs a) {
     const int item = blockIdx.x;
     const bool is_h = item < a.n_h;
     const int dv = a.d / 8, NS = a.two_prev ? 3 : 2;
-    // norm weights are step inputs: requested before the dependency wait
+    // the norm weights are no kernel's output: requested before the dependency wait
     const uint4* wt = is_h ? a.norm_h : a.norm_e;
     uint4 wv[NV];
 #pragma unroll
@@ -1392,6 +1391,7 @@ __global__ void __launch_bounds__(256) gather_norm_bf16_kernel(GatherArgs a) {
         const int c = t + j * 256;
         wv[j] = c < dv ? wt[c] : make_uint4(0u, 0u, 0u, 0u);
     }
+    pdl_wait();
     // the rows that the item stores to: r0 .. r0 + n - 1 (an embedding: one row, part `part`)
     int r0 = 0, n = 1, part = 0;
     const uint4* src = a.hidden;
@@ -1403,7 +1403,6 @@ __global__ void __launch_bounds__(256) gather_norm_bf16_kernel(GatherArgs a) {
         n = min(kHRows, per - c * kHRows);    // (at most 0: nothing to store)
         src += static_cast<size_t>(sq * a.gamma + i) * dv;
     } else {
-        pdl_wait();
         const int q = item - a.n_h;
         r0 = a.two_prev ? q >> 1 : q;
         part = a.two_prev ? 1 + (q & 1) : 1;
@@ -1476,7 +1475,6 @@ __global__ void __launch_bounds__(256) gather_norm_bf16_kernel(GatherArgs a) {
         hi = y0;
         lo = 0.5f * y0 * r;
     }
-    if (is_h) pdl_wait();
     // the approximator GEMMs' tail-split counters (after the status word) start each call at zero
     if (item == 0 && a.status)
         for (int i = t; i < kTailSems; i += 256) a.status[1 + i] = 0;
