@@ -302,7 +302,8 @@ __device__ __forceinline__ void dot_rows4(const float* const (&w)[4], const floa
 
 // Shared-memory layout of one merge CTA (dynamic part), for a top-k of k and room for kc >= k halves.
 struct MergeSmem {
-    unsigned long long* hkey;   // [n_halves] best key of every half block (0 = empty)
+    unsigned long long* hkey;   // [n_halves] best key of every half block (0 = empty); once the halves are chosen,
+    float* zbuf;                // in its place, [kMergeExpandChunks * kChunk] recomputed logits
     unsigned long long* cand;   // [2 * 4kc + kMergeExpandChunks * kChunk]
     unsigned long long* cand2;  // the same size: the compacted set of the next round
     unsigned long long* sel;    // [k] the winners
@@ -311,6 +312,12 @@ struct MergeSmem {
     int* chalf;                 // [kc] the halves kept
     uint8_t* expanded;          // [4kc] chunk recomputed
 };
+constexpr size_t kZbufBytes = static_cast<size_t>(kMergeExpandChunks) * kChunk * sizeof(float);
+__host__ __device__ inline size_t merge_key_bytes(int n_tiles) { return static_cast<size_t>(2) * n_tiles * 8; }
+// The static part is 4.7 KB: with the most that the dims check lets through, a CTA stays within the 227 KB
+// of a block.
+constexpr size_t kMergeStaticBytes = 5 * 1024;
+static_assert(kMaxMergeSmem + kMergeStaticBytes <= 227 * 1024, "shared memory of a merge CTA");
 __host__ __device__ inline size_t merge_layout(int n_tiles, int k, int kc, uint8_t* base, MergeSmem* m) {
     const size_t detail = static_cast<size_t>(kc) * (kChunks / 2);  // chunks of the halves kept
     size_t off = 0;
@@ -319,7 +326,7 @@ __host__ __device__ inline size_t merge_layout(int n_tiles, int k, int kc, uint8
         off += (bytes + 15) / 16 * 16;
         return p;
     };
-    uint8_t* hk = take(static_cast<size_t>(2) * n_tiles * 8);
+    uint8_t* hk = take(merge_key_bytes(n_tiles) > kZbufBytes ? merge_key_bytes(n_tiles) : kZbufBytes);
     uint8_t* cd = take((2 * detail + static_cast<size_t>(kMergeExpandChunks) * kChunk) * 8);
     uint8_t* cd2 = take((2 * detail + static_cast<size_t>(kMergeExpandChunks) * kChunk) * 8);
     uint8_t* se = take(static_cast<size_t>(k) * 8);
@@ -329,6 +336,7 @@ __host__ __device__ inline size_t merge_layout(int n_tiles, int k, int kc, uint8
     uint8_t* ex = take(detail);
     if (m) {
         m->hkey = reinterpret_cast<unsigned long long*>(hk);
+        m->zbuf = reinterpret_cast<float*>(hk);
         m->cand = reinterpret_cast<unsigned long long*>(cd);
         m->cand2 = reinterpret_cast<unsigned long long*>(cd2);
         m->sel = reinterpret_cast<unsigned long long*>(se);
@@ -359,7 +367,6 @@ __global__ void __launch_bounds__(kThreads, 2) lmhead_merge_kernel(Partials part
     __shared__ int wcnt[kThreads / 32];
     __shared__ int sel_info[3], n_flag, flag_list[kMergeExpandChunks], n_cand, n_next, n_sel, n_valid, n_chalf;
     __shared__ unsigned long long found;
-    __shared__ float zbuf[kMergeExpandChunks * kChunk];
     __shared__ float lse_s;
 
     const int row = blockIdx.x;
@@ -660,7 +667,7 @@ __global__ void __launch_bounds__(kThreads, 2) lmhead_merge_kernel(Partials part
             dot_rows4(w, x + static_cast<size_t>(row) * d, d, lane, acc);
             if (lane < 4) {
                 const float z = lane == 0 ? acc[0] : lane == 1 ? acc[1] : lane == 2 ? acc[2] : acc[3];
-                zbuf[q + lane] = v + lane < V ? z * inv_temp : -INFINITY;
+                S.zbuf[q + lane] = v + lane < V ? z * inv_temp : -INFINITY;
             }
         }
         __syncthreads();
@@ -680,7 +687,7 @@ __global__ void __launch_bounds__(kThreads, 2) lmhead_merge_kernel(Partials part
             const int f = q / kChunk, cc = q - f * kChunk;
             const int v = S.cbase[flag_list[f]] + cc;
             if (v < V) {
-                const unsigned long long key = cand_key(zbuf[q], v);
+                const unsigned long long key = cand_key(S.zbuf[q], v);
                 if (key >= theta) spare[atomicAdd(&n_next, 1)] = key;
             }
         }
@@ -723,9 +730,11 @@ __global__ void __launch_bounds__(kThreads, 2) lmhead_merge_kernel(Partials part
 
 }  // namespace
 
-// What the dims check counts per merge CTA; with a row of x in fp32, which bounds d.
+// What the dims check counts per merge CTA: the keys alone in their place, and a row of x in fp32, which
+// bounds d. (Where the recomputed logits need more room than the keys, the rest is far below the limit.)
 size_t merge_smem_bytes(int n_tiles, int d, int k) {
-    return merge_layout(n_tiles, k, k, nullptr, nullptr) + (static_cast<size_t>(d) * 4 + 15) / 16 * 16;
+    const size_t keys = merge_key_bytes(n_tiles), more = keys < kZbufBytes ? kZbufBytes - keys : 0;
+    return merge_layout(n_tiles, k, k, nullptr, nullptr) - more + (static_cast<size_t>(d) * 4 + 15) / 16 * 16;
 }
 
 cudaError_t launch_lmhead_merge(const Ctx& ctx, int dtype, Partials partials, int n_rows, int V, int d, int k,

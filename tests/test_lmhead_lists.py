@@ -19,6 +19,8 @@ CASES = [
     (5000, 64, 40, "bf16", "equal"),
     (1500, 64, 64, "bf16", "plain"),         # 12 half blocks
     (270001, 64, 48, "bf16", "plain"),       # 2110 half blocks
+    (2687777, 64, 64, "bf16", "plain"),      # shared memory for k halves, but not for more
+    (2895800, 64, 64, "bf16", "plain"),      # the largest vocabulary of these dims
 ]
 # numbers of rows at which the tensor-core kernel changes: four copies of the rows, two, one; then
 # with d > 512 CTA pairs, single CTAs over three (and five) M-tiles, pairs again
