@@ -590,11 +590,13 @@ __global__ void __launch_bounds__(kThreads, 2) lmhead_merge_kernel(Partials part
 
     // 3. select; a kept chunk whose third value reaches the k-th candidate may hide members of
     //    the top k, so its 32 logits are recomputed exactly and the selection is redone. Chunks
-    //    are recomputed in rounds of at most kMergeExpandChunks; after each round only keys at or
+    //    are recomputed in rounds of at most kMergeExpandChunks; after each round the keys at or
     //    above the k-th candidate survive (the candidates are logits of the row, so every member
-    //    of the true top k is at or above it, and it only rises), which bounds the set by
-    //    k + kMergeExpandChunks * kChunk whatever the input. Few candidates (the usual case) are
-    //    ranked by counting, which sorts the winners as well.
+    //    of the true top k is at or above it), and all logits of the round's chunks join them, which bounds
+    //    the set by k + kMergeExpandChunks * kChunk whatever the input. (All: a recomputed logit is summed in
+    //    another order, so one that was at the k-th candidate may come out a little below it. Without it the
+    //    set could fall below k and be filled up with far smaller ones.) Few candidates (the usual case)
+    //    are ranked by counting, which sorts the winners as well.
     unsigned long long theta = 0;
     unsigned long long* cand = S.cand;
     unsigned long long* spare = S.cand2;
@@ -688,7 +690,7 @@ __global__ void __launch_bounds__(kThreads, 2) lmhead_merge_kernel(Partials part
             const int v = S.cbase[flag_list[f]] + cc;
             if (v < V) {
                 const unsigned long long key = cand_key(S.zbuf[q], v);
-                if (key >= theta) spare[atomicAdd(&n_next, 1)] = key;
+                if (key >= theta || S.zbuf[q] > -INFINITY) spare[atomicAdd(&n_next, 1)] = key;
             }
         }
         for (int f = tid; f < nf; f += kThreads) S.expanded[flag_list[f]] = 1;

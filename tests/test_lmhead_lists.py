@@ -21,6 +21,8 @@ CASES = [
     (270001, 64, 48, "bf16", "plain"),       # 2110 half blocks
     (2687777, 64, 64, "bf16", "plain"),      # shared memory for k halves, but not for more
     (2895800, 64, 64, "bf16", "plain"),      # the largest vocabulary of these dims
+    (20000, 320, 40, "bf16", "twins"),       # 120 equal rows of W above all others, three per chunk
+    (20000, 320, 40, "f32", "twins"),
 ]
 # numbers of rows at which the tensor-core kernel changes: four copies of the rows, two, one; then
 # with d > 512 CTA pairs, single CTAs over three (and five) M-tiles, pairs again
@@ -44,6 +46,12 @@ def test_lists_equal_a_full_sort(V, d, k, dtype, rows, n=21):
     if rows == "outlier":
         W[V // 2] = 200.0 * torch.sign(x.sum(0))
         x = x.abs() * torch.sign(W[V // 2])
+    elif rows == "twins":
+        # their chunks are all recomputed, with the sum in another order: all of them may come out lower than
+        # the k-th candidate was
+        W = -(0.5 + torch.rand(V, d, generator=g))
+        x = x.abs()
+        W[(32 * torch.arange(50, 90)[:, None] + torch.arange(3)).flatten()] = -0.2 * torch.rand(d, generator=g)
     elif rows == "equal":
         x.zero_()
     W, x = W.to(dt).cuda(), x.to(dt).cuda()
