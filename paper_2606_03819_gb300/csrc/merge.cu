@@ -27,9 +27,11 @@ namespace tf {
 namespace {
 
 constexpr int kRegHalves = 8;     // half summaries a thread can hold in registers (V <= 262144)
-constexpr int kRankCands = 512;   // candidates that are ranked by counting
 constexpr int kKeepSlack = 64;    // room for halves beyond the k-th in its bucket
 constexpr int kThreads = 256;   // 512 or more: two CTAs no longer fit an SM, so 241 rows take two waves
+// Candidates that are ranked by counting: one per thread. Two per thread cost more than a selection (V =
+// 151936, d = 1024, 1000 rows, k = 256: 87 against 76 us).
+constexpr int kRankCands = kThreads;
 
 __device__ __forceinline__ void lse_combine(float& m, float& s, float m2, float s2) {
     if (m2 > m) {
@@ -603,31 +605,15 @@ __global__ void __launch_bounds__(kThreads, 2) lmhead_merge_kernel(Partials part
     for (;;) {
         const int nc = n_cand;
         const bool few = nc >= k && nc <= kRankCands;
-        unsigned long long mine[kRankCands / kThreads];
-        int rank[kRankCands / kThreads];
+        unsigned long long mine = 0ull;
+        int rank = 0;
         if (few) {
-#pragma unroll
-            for (int j = 0; j < kRankCands / kThreads; ++j) {
-                const int i = tid + j * kThreads;
-                mine[j] = i < nc ? cand[i] : 0ull;
-                rank[j] = 0;
-            }
-            if (nc <= kThreads) {
-                if (tid < nc) {
+            if (tid < nc) {
+                mine = cand[tid];
 #pragma unroll 8
-                    for (int i = 0; i < nc; ++i) rank[0] += cand[i] > mine[0] ? 1 : 0;
-                }
-            } else {
-#pragma unroll 4
-                for (int i = 0; i < nc; ++i) {
-                    const unsigned long long key = cand[i];
-#pragma unroll
-                    for (int j = 0; j < kRankCands / kThreads; ++j) rank[j] += key > mine[j] ? 1 : 0;
-                }
+                for (int i = 0; i < nc; ++i) rank += cand[i] > mine ? 1 : 0;
+                if (rank == k - 1) found = mine;
             }
-#pragma unroll
-            for (int j = 0; j < kRankCands / kThreads; ++j)
-                if (mine[j] != 0ull && rank[j] == k - 1) found = mine[j];
         } else {
             theta = nc >= k ? block_kth_largest_fast(cand, nc, k, SB, hist, sel_info, &found) : 0ull;
         }
@@ -646,13 +632,10 @@ __global__ void __launch_bounds__(kThreads, 2) lmhead_merge_kernel(Partials part
         const int nf = min(n_flag, kMergeExpandChunks);   // the rest wait for the next round
         if (nf == 0) {
             if (!few) break;
-            const float lse = lse_s;
-#pragma unroll
-            for (int j = 0; j < kRankCands / kThreads; ++j)
-                if (mine[j] != 0ull && rank[j] < k) {
-                    out_ids[static_cast<size_t>(row) * k + rank[j]] = key_id(mine[j]);
-                    out_logp[static_cast<size_t>(row) * k + rank[j]] = key_value(mine[j]) - lse;
-                }
+            if (mine != 0ull && rank < k) {
+                out_ids[static_cast<size_t>(row) * k + rank] = key_id(mine);
+                out_logp[static_cast<size_t>(row) * k + rank] = key_value(mine) - lse_s;
+            }
             return;
         }
         if (tid == 0) {
@@ -744,8 +727,16 @@ cudaError_t launch_lmhead_merge(const Ctx& ctx, int dtype, Partials partials, in
                                 float* out_logp) {
     if (n_rows <= 0) return cudaSuccess;
     const int n_tiles = (V + kBlockV - 1) / kBlockV;
-    // room for kKeepSlack halves more than k where shared memory has it
-    const int kc = merge_layout(n_tiles, k, k + kKeepSlack, nullptr, nullptr) <= kMaxMergeSmem ? k + kKeepSlack : k;
+    // Room for up to kKeepSlack halves more than k, as far as it leaves as many CTAs on an SM (228 KB, 1 KB of
+    // it per CTA for the system) as k alone (V = 151936, d = 1024, 241 rows: k = 320 32 -> 23 us, k = 384 41 ->
+    // 32).
+    auto resident = [&](int c) {
+        const size_t smem = merge_layout(n_tiles, k, c, nullptr, nullptr);
+        return smem > kMaxMergeSmem ? 0 : (228 * 1024) / (smem + kMergeStaticBytes + 1024);
+    };
+    int kc = k + kKeepSlack;
+    while (kc > k && resident(kc) < resident(k)) kc -= 8;
+    if (kc < k) kc = k;
     const size_t smem = merge_layout(n_tiles, k, kc, nullptr, nullptr);
     if (dtype == TF_BF16) {
         auto kern = lmhead_merge_kernel<__nv_bfloat16>;

@@ -14,6 +14,9 @@ CASES = [
     (20000, 128, 1, "bf16", "plain"),
     (20000, 64, 512, "bf16", "plain"),
     (20000, 128, 64, "f32", "plain"),
+    (60000, 128, 200, "bf16", "plain"),      # candidates around 256, up to which they are ranked by counting
+    (60000, 128, 240, "bf16", "plain"),
+    (60000, 128, 320, "bf16", "plain"),
     (9001, 64, 32, "bf16", "outlier"),       # every other half in the lowest bucket
     (9001, 64, 32, "f32", "outlier"),
     (5000, 64, 40, "bf16", "equal"),
