@@ -46,7 +46,7 @@ class TfWeights(ctypes.Structure):
                 ("lm_head", "embed", "norm_h", "norm_e", "w_gate", "w_up", "w_down", "w_lin")]
 
 
-EXPORTS = ("tf_status_string", "tf_version", "tf_kernel_launches", "tf_workspace_size", "tf_status_reset", "tf_status_read",
+EXPORTS = ("tf_status_string", "tf_version", "tf_kernel_launches", "tf_builder_counts", "tf_workspace_size", "tf_status_reset", "tf_status_read",
            "tf_stage1_marginals", "tf_stage2_ar_approx", "tf_build_tree", "tf_tree_mask", "tf_build_tree_mask",
            "tf_draft_tree_host", "tf_lmhead_partials", "tf_lmhead_merge", "tf_ar_approx",
            "tf_workspace_h_prime", "tf_workspace_view", "tf_stage1_marginals_static", "tf_accept_walk",
@@ -71,6 +71,7 @@ def load_library(path: Optional[str] = None) -> ctypes.CDLL:
         "tf_status_string": (ctypes.c_char_p, [ctypes.c_int]),
         "tf_version": (I32, []),
         "tf_kernel_launches": (ctypes.c_uint64, []),
+        "tf_builder_counts": (ctypes.c_int, [ctypes.POINTER(ctypes.c_uint64)]),
         "tf_set_wait_limit_ns": (ctypes.c_int, [ctypes.c_uint64]),
         "tf_workspace_size": (ctypes.c_int, [D, ctypes.POINTER(SZ)]),
         "tf_status_reset": (ctypes.c_int, [P, SZ, P]),
@@ -193,6 +194,14 @@ def tf_version() -> int:
 def tf_kernel_launches() -> int:
     """Kernels launched by the library so far in this process."""
     return int(load_library().tf_kernel_launches())
+
+
+def tf_builder_counts() -> tuple:
+    """(trees that the builder by levels left to the queue, times it dropped nodes to make room), on the
+    current device since the library was loaded. Synchronises the device."""
+    n = (ctypes.c_uint64 * 2)()
+    _check("tf_builder_counts", load_library().tf_builder_counts(n))
+    return n[0], n[1]
 
 
 def tf_set_wait_limit_ns(ns: int) -> None:

@@ -509,6 +509,15 @@ int32_t tf_version(void) { return 100; }
 
 uint64_t tf_kernel_launches(void) { return tf::g_kernel_launches.load(std::memory_order_relaxed); }
 
+tf_status tf_builder_counts(uint64_t counts[2]) {
+    if (!counts) return TF_ERR_INVALID_ARG;
+    unsigned long long n[2];
+    TF_TRY(cuda_status(tf::builder_counts(n)));
+    counts[0] = n[0];
+    counts[1] = n[1];
+    return TF_OK;
+}
+
 tf_status tf_set_wait_limit_ns(uint64_t ns) {
     if (ns > 60ull * 1000000000ull) return TF_ERR_INVALID_ARG;
     tf::g_wait_limit_ns.store(ns, std::memory_order_relaxed);

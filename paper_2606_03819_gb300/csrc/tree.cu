@@ -739,6 +739,9 @@ __device__ __forceinline__ unsigned long long level_key(float score, int dep, in
 }
 static_assert(kLvCap <= 1 << 12 && kMaxK <= 1 << 12 && kMaxGamma <= 127, "fields of level_key");
 
+// What builders by levels have done on this device: trees left to the queue, compactions of their nodes.
+__device__ unsigned long long g_builder_counts[2];
+
 __global__ void __launch_bounds__(kLvThreads) build_tree_level_kernel(TreeArgs a) {
     pdl_trigger();
     pdl_wait();
@@ -938,6 +941,7 @@ __global__ void __launch_bounds__(kLvThreads) build_tree_level_kernel(TreeArgs a
                 __syncthreads();                         // (n_next is final for the passes so far)
                 raise_theta(count);
                 count = seen = compact(count, act.node, n_act, next.node, n_next);
+                if (tid == 0) atomicAdd(&g_builder_counts[1], 1ull);
             }
             int nb = (kLvCap - count) / (32 * g);        // parents of this pass: all their entries fit
             nb = nb < n_act ? nb : n_act;
@@ -1192,6 +1196,7 @@ __global__ void __launch_bounds__(kLvThreads) build_tree_level_kernel(TreeArgs a
     const int n_out = a.B + 1;
     if (bad_s) {
         __syncthreads();
+        if (tid == 0) atomicAdd(&g_builder_counts[0], 1ull);
         const TreeSmem q = tree_smem(smem_raw, a);
         for (int i = tid; i < a.gamma * a.M; i += kLvThreads)
             q.topm[i] = a.top_ids[(static_cast<size_t>(s) * a.gamma + i / a.M) * a.K1 + i % a.M];
@@ -1591,6 +1596,11 @@ cudaError_t launch_build_tree(const Ctx& ctx, int b, int gamma, int M, int K1, i
     if (e != cudaSuccess) return e;
     e = launch_pdl(build_tree_level_kernel, dim3(b), dim3(kLvThreads), lsm, ctx.stream, a);
     return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+cudaError_t builder_counts(unsigned long long out[2]) {
+    const cudaError_t e = cudaDeviceSynchronize();
+    return e != cudaSuccess ? e : cudaMemcpyFromSymbol(out, g_builder_counts, sizeof(g_builder_counts));
 }
 
 cudaError_t launch_tree_mask(const Ctx& ctx, int b, int B, const int32_t* node_parent, const int32_t* node_depth,

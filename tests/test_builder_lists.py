@@ -5,6 +5,8 @@ bit for bit (tokens, parents, depths, scores, status). Log-probabilities are mul
 list's depth, so the M-ary rule expands often and the trees grow deep and wide. Budgets up to 40
 (from three sequences on 48, from sixteen on 60; two-token rule: 32) run the sorted-queue builder, larger
 ones the builder by levels, which hands trees with many ties to the queue in shared memory."""
+import heapq
+
 import numpy as np
 import pytest
 import torch
@@ -135,11 +137,11 @@ LEVEL_CASES = [
 ]
 
 
-@pytest.mark.parametrize("grain", [4096, 64])
+@pytest.mark.parametrize("grain", [65536, 4096, 64])
 @pytest.mark.parametrize("mode,b,gamma,M,K2,B,V,two", LEVEL_CASES)
 def test_large_budgets_equal_the_oracle(mode, b, gamma, M, K2, B, V, two, grain):
-    # grain 4096: a few equal scores under different parents per tree, resolved in place; grain 64:
-    # too many of them, so the queue takes over
+    # grain 65536: hardly an equal score; grain 4096: a few under different parents per tree, resolved in place
+    # (with B = 1023 too many); grain 64: too many of them in the larger trees, so the queue takes over
     from paper_2606_03819_gb300 import Dims
     from paper_2606_03819_gb300 import binding as Bn
     dims = Dims(b, 64, V, 64, gamma, M, K2, B, dtype="f32", mode=mode, approx="swiglu_2prev" if two else "swiglu")
@@ -152,10 +154,16 @@ def test_large_budgets_equal_the_oracle(mode, b, gamma, M, K2, B, V, two, grain)
     stat = torch.full((b,), -7, dtype=torch.int32, device="cuda")
     ar = mode == "ar"
     roots = np.stack([root, root], 1) if two else root
+    before = Bn.tf_builder_counts()
     Bn.tf_build_tree(dims, dev(roots, torch.int32), dev(top_ids, torch.int32), dev(top_lp, torch.float32),
                      dev(child_ids, torch.int32) if ar else None, dev(child_lp, torch.float32) if ar else None,
                      out["tok"], out["par"], out["dep"], out["score"], stat)
-    torch.cuda.synchronize()
+    by_queue, compactions = (x - y for x, y in zip(Bn.tf_builder_counts(), before))
+    if grain != 64 and mode != "marginal":
+        assert by_queue == (b if grain == 4096 and B == 1023 else 0)
+        assert compactions > 0 or B < 1023       # 64 parents, 500 entries each, of which 1023 stay
+    elif B == 512:
+        assert by_queue == b
     for s in range(b):
         s1 = _full_rows(top_ids[s], top_lp[s], V)
         s2 = _full_rows(child_ids[s], child_lp[s], V) if ar else None
@@ -166,3 +174,98 @@ def test_large_budgets_equal_the_oracle(mode, b, gamma, M, K2, B, V, two, grain)
         np.testing.assert_array_equal(out["dep"][s].cpu().numpy(), t.depth)
         np.testing.assert_array_equal(out["score"][s].cpu().numpy().astype(np.float64), t.score)
         assert stat[s].item() == (O_UNDERFULL if t.underfull else 0)
+
+
+def _queue_fp32(mode, gamma, M, K2, B, V, top_ids, ids, lp, root, two):
+    """One sequence's tree by the queue of tf_build_tree in fp32, for lists in any order and of any values."""
+    def key(x):                                   # larger scores first
+        u = int(np.float32(x).view(np.uint32))
+        return -((~u & 0xffffffff) if u & 0x80000000 else u | 0x80000000)
+    lp = lp.astype(np.float32)
+    tok, par, dep, score = [int(root)], [-1], [0], [np.float32(0)]
+    cand = [{int(t): m for m, t in reversed(list(enumerate(top_ids[i, :M])))} for i in range(gamma)]
+    heap = [(key(np.float32(0) + lp[0, 0]), 1, 0, 0, 0)]
+    nonfinite = False
+    while heap and len(tok) <= B:
+        _, d, p, row, rank = heapq.heappop(heap)
+        t, node, sc = int(ids[row, rank]), len(tok), score[p] + lp[row, rank]
+        nonfinite |= not np.isfinite(sc)
+        tok.append(t), par.append(p), dep.append(d), score.append(sc)
+        if rank + 1 < K2:
+            heapq.heappush(heap, (key(score[p] + lp[row, rank + 1]), d, p, row, rank + 1))
+        m = cand[d - 1].get(t, -1)
+        if d < gamma and (mode == "marginal" or m >= 0):
+            crow = d if mode != "ar" else 1 + (d - 1) * M + m if not two else 1 + m if d == 1 else \
+                1 + M + (d - 2) * M * M + m * M + cand[d - 2][tok[p]]
+            heapq.heappush(heap, (key(sc + lp[crow, 0]), d + 1, node, crow, 0))
+    short = B + 1 - len(tok)
+    return (tok + [-1] * short, par + [-1] * short, dep + [-1] * short, score + [-np.inf] * short,
+            (O_UNDERFULL if short else 0) | (O_NONFINITE if nonfinite else 0))
+
+
+O_NONFINITE = 4   # TF_DEV_NONFINITE
+
+ODD_DIMS = [
+    # mode, gamma, M, K2, B, two-token rule
+    ("ar", 16, 8, 64, 64, False),
+    ("ar", 3, 8, 64, 64, False),
+    ("ar", 8, 8, 100, 100, False),
+    ("ar", 6, 8, 300, 300, False),
+    ("marginal", 6, 4, 300, 200, False),
+    ("ar", 6, 4, 64, 64, True),
+]
+# and whether a builder by levels leaves them to the queue
+ODD_LISTS = {"unsorted": True, "above 0": True, "nan": True, "short": True}
+
+
+@pytest.mark.parametrize("kind", ODD_LISTS)
+@pytest.mark.parametrize("mode,gamma,M,K2,B,two", ODD_DIMS)
+def test_lists_that_no_stage_leaves(mode, gamma, M, K2, B, two, kind):
+    rng = np.random.default_rng(B + gamma)
+    b, V = 2, 3000
+    top_ids, top_lp, child_ids, child_lp, root = _make(rng, mode, b, gamma, M, K2, V, 8, two)
+    ids, lp = (child_ids, child_lp) if mode == "ar" else (top_ids[..., :K2], top_lp[..., :K2])
+    lp = -np.sort(rng.exponential(2.0, lp.shape).astype(np.float32), axis=-1)
+    if kind == "unsorted":
+        lp = rng.permuted(lp, axis=-1)
+    elif kind == "above 0":
+        lp[:, 0, 0] = 0.5
+    elif kind == "nan":
+        lp[:, 0, 1] = np.nan
+    elif kind == "short":                         # one entry per list: fewer finite nodes than the budget
+        lp[..., 1:] = -np.inf
+    _check_odd(mode, gamma, M, K2, B, V, two, top_ids, ids, lp, root, ODD_LISTS[kind])
+
+
+@pytest.mark.parametrize("K2,gamma", [(512, 3), (60, 2)], ids=["no_room", "too_many_to_order"])
+def test_ties_of_thousands_of_nodes(K2, gamma):
+    # every list flat, every node expands: a level of ties wider than the nodes held at once, or than those sorted
+    rng = np.random.default_rng(K2)
+    b, V, M, B = 2, 3000, 4, 1023
+    top_ids, _, _, _, root = _make(rng, "marginal", b, gamma, M, K2, V)
+    lp = np.full(top_ids.shape, -0.125, np.float32)
+    _check_odd("marginal", gamma, M, K2, B, V, False, top_ids, top_ids, lp, root, True)
+
+
+def _check_odd(mode, gamma, M, K2, B, V, two, top_ids, ids, lp, root, queue):
+    from paper_2606_03819_gb300 import Dims
+    from paper_2606_03819_gb300 import binding as Bn
+    b, n = root.shape[0], B + 1
+    dims = Dims(b, 64, V, 64, gamma, M, K2, B, dtype="f32", mode=mode, approx="swiglu_2prev" if two else "swiglu")
+    dev = lambda a, t: torch.from_numpy(np.ascontiguousarray(a)).to(device="cuda", dtype=t)  # noqa: E731
+    i32, f32 = torch.int32, torch.float32
+    out = [torch.full((b, n), -7, dtype=t, device="cuda") for t in (i32, i32, i32, f32)]
+    stat = torch.full((b,), -7, dtype=i32, device="cuda")
+    ar = mode == "ar"
+    before = Bn.tf_builder_counts()
+    Bn.tf_build_tree(dims, dev(np.stack([root, root], 1) if two else root, i32), dev(top_ids, i32),
+                     dev(np.zeros(top_ids.shape) if ar else lp, f32), dev(ids, i32) if ar else None,
+                     dev(lp, f32) if ar else None, *out, stat)
+    by_queue = Bn.tf_builder_counts()[0] - before[0]
+    for s in range(b if not np.isnan(lp).any() else 0):   # (NaN has no place in the order: the route alone)
+        want = _queue_fp32(mode, gamma, M, K2, B, V, top_ids[s], ids[s], lp[s], root[s], two)
+        for got, w in zip(out, want):
+            np.testing.assert_array_equal(got[s].cpu().numpy(), np.asarray(w))
+        assert stat[s].item() == want[4]
+    if B > 64:                                    # (up to 64 the sorted queue may have built them)
+        assert by_queue == (b if queue else 0)
