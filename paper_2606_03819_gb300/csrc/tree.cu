@@ -852,9 +852,11 @@ __global__ void __launch_bounds__(kLvThreads) build_tree_level_kernel(TreeArgs a
         __syncthreads();
     };
 
-    // Drops the nodes below theta, keeping the others' order; the nodes still to expand (two lists) move
-    // along. Returns the new count.
-    auto compact = [&](int count, uint16_t* act, int n_act, uint16_t* next, int n_next) {
+    // Drops the nodes below theta, keeping the others' order; the nodes still to expand move along: in `act`
+    // a dropped one leaves a gap, of `next` those kept go to `spare` (n_spare of them, zero before).
+    // Returns the new count.
+    auto compact = [&](int count, const ActList& act, int n_act, const ActList& next, int n_next, const ActList& spare,
+                       int& n_spare) {
         constexpr int kPer = kLvCap / kLvThreads;
         const float theta = theta_s;
         float sc[kPer];
@@ -898,8 +900,16 @@ __global__ void __launch_bounds__(kLvThreads) build_tree_level_kernel(TreeArgs a
             base += keep[j] ? 1 : 0;
         }
         __syncthreads();
-        for (int i = tid; i < n_act; i += kLvThreads) act[i] = act[i] == kNoNode ? kNoNode : t.place[act[i]];
-        for (int i = tid; i < n_next; i += kLvThreads) next[i] = next[i] == kNoNode ? kNoNode : t.place[next[i]];
+        for (int i = tid; i < n_act; i += kLvThreads)
+            act.node[i] = act.node[i] == kNoNode ? kNoNode : t.place[act.node[i]];
+        for (int i = tid; i < n_next; i += kLvThreads) {
+            const uint16_t to = t.place[next.node[i]];
+            if (to == kNoNode) continue;
+            const int q = atomicAdd(&n_spare, 1);
+            spare.node[q] = to;
+            spare.chunk[q] = 0;
+            spare.row[q] = next.row[i];
+        }
         uint16_t to[kPer], np[kPer];
 #pragma unroll
         for (int j = 0; j < kPer; ++j)
@@ -936,13 +946,22 @@ __global__ void __launch_bounds__(kLvThreads) build_tree_level_kernel(TreeArgs a
         int g = (a.B <= 128 ? kLvWarps : 2 * kLvWarps) / n_act;
         g = g < 1 ? 1 : g > n_chunks ? n_chunks : g;
         while (n_act > 0) {
-            const ActList act = t.act[li], cont = t.act[lc], next = t.act[ln];
             if (kLvCap - count < 32 * kLvWarps) {
                 __syncthreads();                         // (n_next is final for the passes so far)
                 raise_theta(count);
-                count = seen = compact(count, act.node, n_act, next.node, n_next);
-                if (tid == 0) atomicAdd(&g_builder_counts[1], 1ull);
+                int& n_spare = n_next_s[(d + 1) % 3];    // (zero, and zero again below)
+                count = seen = compact(count, t.act[li], n_act, t.act[ln], n_next, t.act[lc], n_spare);
+                if (tid == 0) {
+                    n_next = n_spare;
+                    n_spare = 0;
+                    atomicAdd(&g_builder_counts[1], 1ull);
+                }
+                const int old = ln;
+                ln = lc;
+                lc = old;
+                __syncthreads();
             }
+            const ActList act = t.act[li], cont = t.act[lc], next = t.act[ln];
             int nb = (kLvCap - count) / (32 * g);        // parents of this pass: all their entries fit
             nb = nb < n_act ? nb : n_act;
             if (nb < 1) {                                // too many nodes at theta
@@ -1008,14 +1027,10 @@ __global__ void __launch_bounds__(kLvThreads) build_tree_level_kernel(TreeArgs a
                 t.dep[i] = static_cast<uint8_t>(d);
                 t.m[i] = static_cast<int8_t>(m);
                 if (crow >= 0) {
-                    const int q = atomicAdd(&n_next, 1);
-                    if (q < kLvCap) {
-                        next.node[q] = static_cast<uint16_t>(i);
-                        next.chunk[q] = 0;
-                        next.row[q] = crow;
-                    } else {
-                        bad_s = 1;                       // (dropped nodes keep their entries)
-                    }
+                    const int q = atomicAdd(&n_next, 1); // (one entry per node held: it fits)
+                    next.node[q] = static_cast<uint16_t>(i);
+                    next.chunk[q] = 0;
+                    next.row[q] = crow;
                 }
             }
             __syncthreads();
@@ -1054,7 +1069,7 @@ __global__ void __launch_bounds__(kLvThreads) build_tree_level_kernel(TreeArgs a
             const float theta = theta_s;
             for (int i = tid; i < n_act; i += kLvThreads) {
                 const uint16_t p = all.node[i];
-                if (p == kNoNode || t.score[p] < theta) continue;
+                if (t.score[p] < theta) continue;
                 const int q = atomicAdd(&n_few, 1);
                 few.node[q] = p;
                 few.chunk[q] = 0;

@@ -159,7 +159,7 @@ def test_large_budgets_equal_the_oracle(mode, b, gamma, M, K2, B, V, two, grain)
                      dev(child_ids, torch.int32) if ar else None, dev(child_lp, torch.float32) if ar else None,
                      out["tok"], out["par"], out["dep"], out["score"], stat)
     by_queue, compactions = (x - y for x, y in zip(Bn.tf_builder_counts(), before))
-    if grain != 64 and mode != "marginal":
+    if grain != 64:
         assert by_queue == (b if grain == 4096 and B == 1023 else 0)
         assert compactions > 0 or B < 1023       # 64 parents, 500 entries each, of which 1023 stay
     elif B == 512:
