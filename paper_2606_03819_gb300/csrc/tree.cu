@@ -672,9 +672,10 @@ __global__ void __launch_bounds__(kFastThreads) build_tree_fast_kernel(TreeArgs 
 // 37.5, B = 1023 76 -> 63).
 //  - Two nodes of equal score and depth under different parents are ordered by their parents' places
 //    in the order, known once shallower levels are: the few such ties are resolved after the sort.
-//  - A list entry above its predecessor or its parent, a score that is not finite, more than
-//    kLvTies ties near the tree, or more nodes at theta than there is room for send the sequence to
-//    the queue (build_tree_queue) instead: the same results, at the old speed.
+//  - A score of -inf ends its list (as padding of short lists does). A list entry above its predecessor or
+//    its parent, NaN, fewer finite nodes than B where lists ended early, more than kLvTies ties near
+//    the tree, or more nodes at theta than there is room for send the sequence to the queue
+//    (build_tree_queue) instead: the same results, at the queue's speed on top of the levels done by then.
 // ------------------------------------------------------------------------------------------
 constexpr int kLvThreads = 512;
 constexpr int kLvWarps = kLvThreads / 32;
@@ -750,7 +751,7 @@ __global__ void __launch_bounds__(kLvThreads) build_tree_level_kernel(TreeArgs a
     // n_cont_s, n_next_s: lists that go on after a pass, nodes that the next level expands; a pass
     // (level) uses one of three counters and zeroes the next one, whose last readers are a pass
     // (level) behind
-    __shared__ int wsum[kLvWarps], count_s, bad_s, n_cont_s[3], n_next_s[3], n_ties_s, ties[kLvTies], flags_s;
+    __shared__ int wsum[kLvWarps], count_s, bad_s, ended_s, n_cont_s[3], n_next_s[3], n_ties_s, ties[kLvTies], flags_s;
     constexpr unsigned kFull = 0xffffffffu;
     const LevelSmem t = level_smem(smem_raw);
     const int s = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -773,7 +774,7 @@ __global__ void __launch_bounds__(kLvThreads) build_tree_level_kernel(TreeArgs a
         t.act[0].row[0] = 0;
         n_cont_s[0] = n_next_s[1] = 0;
         count_s = 1;
-        bad_s = 0;
+        bad_s = ended_s = 0;
         flags_s = 0;
         theta_s = -INFINITY;
     }
@@ -987,9 +988,10 @@ __global__ void __launch_bounds__(kLvThreads) build_tree_level_kernel(TreeArgs a
                 const float sc = ps + lp;
                 float prev = __shfl_up_sync(kFull, sc, 1);
                 if (lane == 0) prev = ps + before;       // the parent itself above a list's first entry
-                // (also false for NaN)
-                if (in && !(sc <= prev && sc > -INFINITY)) bad_s = 1;
-                const bool take = in && sc >= theta;
+                if (in && !(sc <= prev)) bad_s = 1;      // (also for NaN)
+                const bool finite = sc > -INFINITY;
+                if (in && !finite) ended_s = 1;          // the list ends before its length
+                const bool take = in && finite && sc >= theta;
                 const unsigned bal = __ballot_sync(kFull, take);
                 if (bal == 0u) continue;
                 int base = 0;
@@ -1085,8 +1087,11 @@ __global__ void __launch_bounds__(kLvThreads) build_tree_level_kernel(TreeArgs a
     }
     __syncthreads();
 
-    // ---- the order of the survivors
+    // ---- the order of the survivors. (Entries of -inf come after all others; the tree holds some only
+    // where there are too few others, and then the queue places them.)
     int n = 0;
+    if (tid == 0 && ended_s && count - 1 < a.B) bad_s = 1;
+    __syncthreads();
     if (!bad_s) {
         if (tid == 0) n_ties_s = 0;
         if (count <= kLvExact) {
