@@ -684,6 +684,9 @@ constexpr int kLvBins = 2 * kLvThreads;
 constexpr int kLvSort = 2048;      // nodes that can be sorted
 constexpr int kLvExact = 128;      // up to this many nodes: order statistics by counting
 constexpr int kLvTies = 32;        // ties resolved in place, and the longest run of equal nodes
+// The lowest score that theta's histogram covers: entries far below (lists padded with a type's lowest
+// value) would leave one bin for all others.
+constexpr float kLvFloor = -1024.0f;
 
 // Nodes to expand: the node (kNoNode: dropped), the next 32-entry chunk of its child list, the list.
 struct ActList {
@@ -784,7 +787,7 @@ __global__ void __launch_bounds__(kLvThreads) build_tree_level_kernel(TreeArgs a
     auto sharers = [](int n) { return n <= 64 ? 8 : 4; };
     // Raises theta to the B-th best score, with more than kLvExact nodes to the lower edge of the
     // histogram bin that holds it (a little below it: the bins' arithmetic is rounded). Nothing happens
-    // while there are fewer than B.
+    // while there are fewer than B (with more than kLvExact nodes: fewer than B from kLvFloor up).
     auto raise_theta = [&](int count) {
         if (count - 1 < a.B) return;
         if (count <= kLvExact) {
@@ -815,9 +818,12 @@ __global__ void __launch_bounds__(kLvThreads) build_tree_level_kernel(TreeArgs a
             return;
         }
         float lo = theta_s;
-        if (!(lo > -INFINITY)) {
+        if (lo < kLvFloor) {
             float mn = 0.0f;
-            for (int i = 1 + tid; i < count; i += kLvThreads) mn = fminf(mn, t.score[i]);
+            for (int i = 1 + tid; i < count; i += kLvThreads) {
+                const float x = t.score[i];
+                if (x >= kLvFloor) mn = fminf(mn, x);
+            }
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) mn = fminf(mn, __shfl_xor_sync(kFull, mn, o));
             if (lane == 0) wmin[warp] = mn;
@@ -825,7 +831,7 @@ __global__ void __launch_bounds__(kLvThreads) build_tree_level_kernel(TreeArgs a
             lo = wmin[0];
             for (int w = 1; w < kLvWarps; ++w) lo = fminf(lo, wmin[w]);
         }
-        if (!(lo < 0.0f) || !(lo > -INFINITY)) return;   // (uniform: every thread holds the same lo)
+        if (!(lo < 0.0f)) return;                        // (uniform: every thread holds the same lo)
         t.hist[2 * tid] = t.hist[2 * tid + 1] = 0;
         __syncthreads();
         const float scale = static_cast<float>(kLvBins) / -lo;

@@ -215,7 +215,7 @@ ODD_DIMS = [
     ("ar", 6, 4, 64, 64, True),
 ]
 # and whether a builder by levels leaves them to the queue
-ODD_LISTS = {"unsorted": True, "above 0": True, "nan": True, "padded": False, "short": True}
+ODD_LISTS = {"unsorted": True, "above 0": True, "nan": True, "padded": False, "lowest": False, "short": True}
 
 
 @pytest.mark.parametrize("kind", ODD_LISTS)
@@ -234,6 +234,8 @@ def test_lists_that_no_stage_leaves(mode, gamma, M, K2, B, two, kind):
         lp[:, 0, 1] = np.nan
     elif kind == "padded":                        # the last quarter of every list missing
         lp[..., K2 - K2 // 4:] = -np.inf
+    elif kind == "lowest":
+        lp[..., K2 - K2 // 4:] = np.finfo(np.float32).min
     elif kind == "short":                         # one entry per list: fewer finite nodes than the budget
         lp[..., 1:] = -np.inf
     _check_odd(mode, gamma, M, K2, B, V, two, top_ids, ids, lp, root, ODD_LISTS[kind])
