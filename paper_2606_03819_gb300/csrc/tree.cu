@@ -446,8 +446,8 @@ __device__ void build_tree_queue(const TreeArgs& a, int s, const TreeSmem& t, co
 }
 
 // ------------------------------------------------------------------------------------------
-// Builder with a sorted queue, for B <= 64 (used up to 48) with every reachable list entry staged. The same pops, tie rules and results as
-// build_tree_queue. After t pops only the B - t best live entries can still be popped (each
+// Builder with a sorted queue, for B <= 64 with every reachable list entry staged. The same pops, tie
+// rules and results as build_tree_queue. After t pops only the B - t best live entries can still be popped (each
 // needs every better entry popped first), and at most t + 1 entries are live (a pop replaces its
 // entry by the next sibling and adds at most the node's first child), so at most
 // min(t + 1, B - t) <= 32 entries matter: lane i of one warp holds the i-th best. A pop takes
@@ -459,6 +459,7 @@ __device__ void build_tree_queue(const TreeArgs& a, int s, const TreeSmem& t, co
 // 250 ns on GB300, a chain of about a hundred dependent single-warp instructions.
 // ------------------------------------------------------------------------------------------
 constexpr int kFastThreads = 512;
+constexpr int kSortedQueueMax = 64;
 // Shared-memory bytes of build_tree_fast_kernel: nodes, candidates, mask bits and the staged
 // lists (token and log-probability of every entry).
 __host__ __device__ inline size_t fast_tree_smem(int B, int gamma, int M, int rows, int sw, bool with_mask) {
@@ -654,9 +655,8 @@ __global__ void __launch_bounds__(kFastThreads) build_tree_fast_kernel(TreeArgs 
 }
 
 // ------------------------------------------------------------------------------------------
-// Builder by levels, for large budgets. A pop sequence is a chain: with the queue in shared memory
-// 512 pops took 343 us on GB300, about 0.65 us each on one warp (33 us this way; 64 pops of the
-// two-token rule 44 us with the queue in registers, 17 us this way). But the B popped nodes are simply
+// Builder by levels, for large budgets and for few depths. A pop sequence is a chain: with the queue in shared
+// memory 512 pops took 343 us on GB300, about 0.65 us each on one warp (33 us this way). But the B popped nodes are simply
 // the B first of all nodes in the order (score, smaller depth, earlier parent, earlier list entry),
 // as long as no node outscores its parent or its list predecessor (log-probabilities <= 0, lists
 // sorted): then the first B nodes contain every ancestor and predecessor of each of them. So the
@@ -1599,17 +1599,17 @@ cudaError_t launch_build_tree(const Ctx& ctx, int b, int gamma, int M, int K1, i
     const int rows_l = mode == TF_MODE_AR ? R : gamma;
     const int stride = mode == TF_MODE_AR ? K2 : K1;
     const int sw = stride < B + 1 ? stride : B + 1;   // list entries that a tree can reach
-    // The sorted-queue builder for small budgets with every reachable entry in shared memory: its cost is
-    // the pops (0.25 us each, more with the two-token rule), the same for any number of sequences; the
-    // builder by levels costs what the sequence with the most levels does, so the line rises with the
-    // number of sequences. Measured on GB300 (16 depths, with the mask; queue against levels): one sequence
-    // B = 32 11.9, 11.4 us, B = 40 14.3, 13.6, B = 48 16.5, 13.9; four B = 40 14.4, 15.1, B = 48 16.5, 16.2;
-    // eight B = 48 16.6, 17.4, B = 52 18.0, 17.8, B = 64 21.0, 18.4; 32 sequences B = 52 17.9, 19.9, B = 56
-    // 19.0, 20.4, B = 64 21.0, 20.7; two-token rule (12 depths) B = 32 13.1 in both cases against 11.9 for one
-    // sequence and 14.1 for eight, B = 40, eight sequences 15.8, 15.6.
-    const int queue_budget = a.two_prev ? 32 : b <= 2 ? 40 : b < 16 ? 48 : 60;
+    // The sorted-queue builder for small budgets with every reachable entry in shared memory. Its cost is the
+    // pops, about 3.2 us + 0.26 B, whatever the lists and the number of sequences. The builder by levels
+    // costs what the deepest of the trees does, 1.7 to 3 us per level, which no size tells: gamma at
+    // worst. So up to 64 nodes it takes over where all gamma levels cost no more than the pops. Measured on
+    // GB300 (with the mask; queue against levels for trees of two to five kinds, one and eight sequences): gamma =
+    // 1, B = 16 6.9, 6.5; gamma = 2, B = 32 11.0, 8.5 to 9.1; gamma = 3, B = 48 15.2, 12.4 to 14.3, B = 32
+    // 11.1, 10.9 to 11.7; gamma = 4, B = 64 19.5, 15.7 to 19.6, B = 48 15.4, 13.9 to 17.9; gamma = 16, B = 64
+    // 20.2, 15.9 (4 levels) to 40.5 (16). Two-token rule: gamma = 4, B = 64 21, 13.8 to 16.2; gamma = 12 23, 16 to 35.
+    // Beyond 64 nodes the queue lies in shared memory (0.6 us per pop).
     const size_t fsm = fast_tree_smem(B, gamma, M, rows_l, sw, mask != nullptr);
-    if (B <= queue_budget && fsm <= kTreeSmemLimit) {
+    if (B <= kSortedQueueMax && B < 16 * gamma && fsm <= kTreeSmemLimit) {
         auto kern = a.two_prev ? build_tree_fast_kernel<true> : build_tree_fast_kernel<false>;
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(fsm));
         if (e != cudaSuccess) return e;

@@ -1,10 +1,10 @@
 """Part 2 of Algorithm 1 on hand-made child lists: tf_build_tree against the oracle's lazy queue,
 bit for bit (tokens, parents, depths, scores, status). Log-probabilities are multiples of 1/8 (or
-1/4096) in [-6, 0], so every path score is exact in fp32 and fp64 alike and equal scores are frequent
-(or a few per tree: the tie rules decide many pops, or some); a random share of every list's tokens are stage-1 candidates of the
-list's depth, so the M-ary rule expands often and the trees grow deep and wide. Budgets up to 40
-(from three sequences on 48, from sixteen on 60; two-token rule: 32) run the sorted-queue builder, larger
-ones the builder by levels, which hands trees with many ties to the queue in shared memory."""
+1/64 to 1/65536) in [-6, 0], so every path score is exact in fp32 and fp64 alike and equal scores are
+frequent (or a few per tree: the tie rules decide many pops, or some); a random share of every list's
+tokens are stage-1 candidates of the list's depth, so the M-ary rule expands often and the trees grow deep
+and wide. Budgets up to 64 and below 16 per depth run the sorted-queue builder, others the builder by levels,
+which hands trees with many ties to the queue in shared memory."""
 import heapq
 
 import numpy as np
@@ -114,12 +114,15 @@ O_UNDERFULL = 2   # TF_DEV_UNDERFULL
 
 LEVEL_CASES = [
     # mode, batch, gamma, M, K2, B, V, two-token rule
-    ("ar", 3, 16, 16, 48, 48, 3000, False),       # the largest budget of the sorted queue for 3 to 15 sequences
-    ("ar", 3, 16, 16, 49, 49, 3000, False),       # the smallest of the builder by levels
-    ("ar", 2, 12, 8, 40, 40, 2000, False),        # the same for one and two
-    ("ar", 2, 12, 8, 41, 41, 2000, False),
-    ("ar", 16, 6, 4, 60, 60, 400, False),         # and from 16 on
-    ("ar", 16, 6, 4, 61, 61, 400, False),
+    ("ar", 3, 16, 16, 64, 64, 3000, False),       # the largest budget of the sorted queue with four depths or more
+    ("ar", 3, 16, 16, 65, 65, 3000, False),       # the smallest of the builder by levels
+    ("ar", 16, 4, 8, 63, 63, 400, False),         # four depths: the lines of both rules meet
+    ("ar", 16, 4, 8, 64, 64, 400, False),
+    ("ar", 2, 3, 8, 47, 47, 2000, False),         # three
+    ("ar", 2, 3, 8, 48, 48, 2000, False),
+    ("ar", 2, 1, 8, 15, 15, 500, False),          # and one
+    ("ar", 2, 1, 8, 16, 16, 500, False),
+    ("ar", 2, 40, 16, 50, 50, 3000, False),       # lists that do not fit shared memory
     ("ar", 2, 16, 16, 512, 512, 5000, False),     # exact lists, sixteen chunks per list
     ("ar", 2, 4, 64, 500, 1023, 5000, False),     # the largest budget, wide branching: nodes dropped as theta rises
     ("ar", 2, 16, 5, 33, 300, 2000, False),       # a list of one chunk and one entry; K2 < B
@@ -130,8 +133,10 @@ LEVEL_CASES = [
     ("ar", 2, 3, 4, 60, 700, 2000, False),        # underfull, ordered by buckets
     ("marginal", 2, 6, 4, 256, 256, 1000, False),  # every node expands
     ("marginal_mary", 2, 12, 20, 130, 127, 2000, False),
-    ("ar", 2, 8, 4, 32, 32, 1000, True),          # two-token rule: the sorted queue, and by levels
-    ("ar", 2, 8, 4, 40, 40, 1000, True),
+    ("ar", 2, 8, 4, 64, 64, 1000, True),          # two-token rule: the sorted queue, and by levels
+    ("ar", 2, 8, 4, 65, 65, 1000, True),
+    ("ar", 2, 2, 4, 31, 31, 1000, True),
+    ("ar", 2, 2, 4, 32, 32, 1000, True),
     ("ar", 2, 6, 5, 100, 100, 1000, True),
     ("ar", 1, 5, 6, 200, 300, 1000, True),
 ]
@@ -208,7 +213,7 @@ O_NONFINITE = 4   # TF_DEV_NONFINITE
 ODD_DIMS = [
     # mode, gamma, M, K2, B, two-token rule
     ("ar", 16, 8, 64, 64, False),
-    ("ar", 3, 8, 64, 64, False),
+    ("ar", 4, 8, 64, 64, False),
     ("ar", 8, 8, 100, 100, False),
     ("ar", 6, 8, 300, 300, False),
     ("marginal", 6, 4, 300, 200, False),
@@ -271,5 +276,5 @@ def _check_odd(mode, gamma, M, K2, B, V, two, top_ids, ids, lp, root, queue):
         for got, w in zip(out, want):
             np.testing.assert_array_equal(got[s].cpu().numpy(), np.asarray(w))
         assert stat[s].item() == want[4]
-    if B > 64:                                    # (up to 64 the sorted queue may have built them)
+    if B >= min(65, 16 * gamma):                  # (the sorted queue has built the others)
         assert by_queue == (b if queue else 0)
