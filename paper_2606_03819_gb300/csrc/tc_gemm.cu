@@ -200,7 +200,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant
     constexpr bool kSplitK = EPI == EPI_CGATEUP || EPI == EPI_CDOWN;
     constexpr bool kPair = CL > 1 && !kSplitK;
     using C = TileCfg<MT, NB, BN, STAGES, kPair, VAR>;
-    static_assert(CL == 1 || kSplitK || (CL == 2 && MT == 1), "a CTA of a pair holds one M-tile");
+    static_assert(CL == 1 || kSplitK || (CL == 2 && MT == 1 && NB == 1), "a CTA pair: one M-tile each, one weight matrix");
     static_assert(!kSplitK || (CL == 4 && kMaxKSplits == 4 && (VAR || (MT == 2 && BN == 128))), "cluster split-K");
     constexpr bool kCopies = EPI == EPI_LMHEAD && CL == 1;
     // copies: half summaries of the copies' chunks, [group][half][parity of the unit][copy][row]
@@ -361,14 +361,10 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant
                 }
                 return n;
             };
-            // Weight tiles of one stage; in a pair each CTA stages its half of the rows
-            // (one weight matrix: tmap_w0's box is BN / 2 rows high; two: BN, one matrix per CTA).
+            // Weight tiles of one stage; in a pair each CTA stages its half of the rows (tmap_w0's box is then
+            // BN / 2 rows high).
             auto load_w = [&](uint8_t* sp, uint64_t* bar, int kb, int nt) {
-                if constexpr (kPair && NB == 2) {
-                    // the pair's N operand is the gate tile followed by the up tile: one each
-                    ptx::tma_load_2d_pair(sp + MT * C::kABytes, crank ? &tmap_w1 : &tmap_w0, in_leader(bar), kb * kBK,
-                                          nt * BN, pol_w);
-                } else if constexpr (kPair) {
+                if constexpr (kPair) {
                     ptx::tma_load_2d_pair(sp + MT * C::kABytes, &tmap_w0, in_leader(bar), kb * kBK,
                                           nt * BN + crank * (BN / 2), pol_w);
                 } else {
@@ -1159,8 +1155,8 @@ int resident_clusters(K kern, int smem, int cl, int num_sms) {
 
 // Tail split: when the units overflow the SMs by a last round that would leave most of them idle, each
 // unit of that round runs as up to kMaxTailSplit K-chunks on the idle SMs, summed by the chunk that
-// finishes last (fp32 partial sums in the workspace). K-chunks per unit, or 0: no tail split. A pair's
-// unit of 256 columns counts for two SMs (slots), one of 128 + 128 for one.
+// finishes last (fp32 partial sums in the workspace). K-chunks per unit, or 0: no tail split. slots: the
+// units that run at once, one per SM or pair of SMs.
 int tail_chunks(const Ctx& ctx, int n_units, int slots, int m_tiles, int cols, int K, size_t partial_bytes) {
     const int tail = n_units % slots;
     int split = tail > 0 ? slots / tail : 0;
@@ -1192,7 +1188,7 @@ cudaError_t run_gemm(const Ctx& ctx, const XMaps& tx, const CUtensorMap& tw0, co
     int n_items = n_units;
     if constexpr (EPI == EPI_GATEUP || EPI == EPI_DOWN) {
         constexpr int kTiles = CL == 1 ? MT : 2;
-        const int slots = CL == 2 && NB == 1 ? ctx.num_sms / 2 : ctx.num_sms;
+        const int slots = CL == 2 ? ctx.num_sms / 2 : ctx.num_sms;
         const int split = k_splits == 1 && ep.partial
                               ? tail_chunks(ctx, n_units, slots, kTiles, NB * BN, K, partial_bytes) : 0;
         if (split) {
