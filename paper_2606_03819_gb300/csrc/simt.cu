@@ -328,9 +328,12 @@ cudaError_t run_swiglu(const Ctx& ctx, const float* X, const float* W0, const fl
 
 // Row group of a contraction with n_rows rows: the smallest that holds them all; beyond 64 rows
 // groups of 64, or of 32 where those pad less (the thread tile is the same, W is read twice as
-// often from L2).
-int row_group(int n_rows) {
+// often from L2). Rows that do not start at multiples of 16 bytes (!vec) arrive by copies of four bytes, 80
+// per thread and stage with the 64 threads of a group of 32: groups of 16 up to 32 rows, of 64 from there
+// on (V = 9001, d = 2050: 17 rows 541 -> 117 us, 65 rows 680 -> 252, 200 rows 1240 -> 300).
+int row_group(int n_rows, bool vec) {
     if (n_rows <= 16) return n_rows <= 8 ? 8 : 16;
+    if (!vec) return n_rows <= 32 ? 16 : 64;
     return (n_rows + 31) / 32 % 2 == 0 ? 64 : 32;
 }
 
@@ -341,19 +344,18 @@ cudaError_t swiglu_gemm(const Ctx& ctx, const float* X, const float* W0, const f
     // K-ranges per tile: enough CTAs for three on every SM, at least two stages each. Where even
     // eight ranges per tile leave SMs idle, smaller row groups make more tiles.
     const long long tiles = (N + kOut - 1) / kOut;
-    int rt = row_group(n_rows);
-    while (rt > 16 && tiles * ((n_rows + rt - 1) / rt) * kMaxClusterK < 2ll * ctx.num_sms) rt /= 2;
+    const bool vec = K % 4 == 0;
+    int rt = row_group(n_rows, vec);
+    while (rt > 16 && tiles * ((n_rows + rt - 1) / rt) * kMaxClusterK < 2ll * ctx.num_sms) rt /= vec ? 2 : 4;
     const long long base = tiles * ((n_rows + rt - 1) / rt);
     int ks = 1;
     while (ks < kMaxClusterK && base * ks * 2 <= 3ll * ctx.num_sms && K >= 2 * kKC * ks * 2) ks *= 2;
-    const bool vec = K % 4 == 0;
     auto run = vec ? (rt == 8    ? run_swiglu<GATEUP, 8, true>
                       : rt == 16 ? run_swiglu<GATEUP, 16, true>
                       : rt == 32 ? run_swiglu<GATEUP, 32, true>
                                  : run_swiglu<GATEUP, 64, true>)
                    : (rt == 8    ? run_swiglu<GATEUP, 8, false>
                       : rt == 16 ? run_swiglu<GATEUP, 16, false>
-                      : rt == 32 ? run_swiglu<GATEUP, 32, false>
                                  : run_swiglu<GATEUP, 64, false>);
     return run(ctx, X, W0, W1, n_rows, K, N, out, hidden, R, M, gamma, ks);
 }
@@ -366,14 +368,13 @@ cudaError_t launch_lmhead_simt(const Ctx& ctx, int dtype, const void* lm_head, c
     if (n_rows <= 0) return cudaSuccess;
     const float* W = static_cast<const float*>(lm_head);
     const float* X = static_cast<const float*>(x);
-    const int rt = row_group(n_rows);
+    const int rt = row_group(n_rows, d % 4 == 0);
     auto run = d % 4 == 0 ? (rt == 8    ? run_lmhead<8, true>
                              : rt == 16 ? run_lmhead<16, true>
                              : rt == 32 ? run_lmhead<32, true>
                                         : run_lmhead<64, true>)
                           : (rt == 8    ? run_lmhead<8, false>
                              : rt == 16 ? run_lmhead<16, false>
-                             : rt == 32 ? run_lmhead<32, false>
                                         : run_lmhead<64, false>);
     const cudaError_t e = run(ctx, W, X, n_rows, d, V, inv_temp, partials, reset_status);
     return e != cudaSuccess ? e : cudaGetLastError();

@@ -38,6 +38,11 @@ def test_lists_at_every_row_split(n, d):
     test_lists_equal_a_full_sort(9001, d, 32, "bf16", "plain", n)
 
 
+@pytest.mark.parametrize("n", [8, 16, 17, 32, 33, 65])
+def test_fp32_lists_of_rows_that_are_no_multiple_of_16_bytes(n):
+    test_lists_equal_a_full_sort(3001, 130, 32, "f32", "plain", n)
+
+
 @pytest.mark.parametrize("V,d,k,dtype,rows", CASES)
 def test_lists_equal_a_full_sort(V, d, k, dtype, rows, n=21):
     from paper_2606_03819_gb300 import Dims
