@@ -73,8 +73,9 @@ struct EpiParams {
     int* sem;
     // kernels with a width chosen at launch: columns per N tile (a multiple of 8) and ring stages
     int bn, stages;
-    // LMHEAD with single CTAs and at most 64 (32) rows: 2 (4) copies of the rows, one per half (quarter)
-    // of the TMEM lanes, so that all epilogue warps share the chunks of a block; otherwise 1
+    // LMHEAD with single CTAs: 2 copies of 33 to 64 rows, 4 of up to 32, one per half (quarter) of the TMEM
+    // lanes, so that all epilogue warps share the chunks of a block (each of them has rows: they wait for
+    // one another); otherwise 1
     int copies;
 };
 
@@ -321,8 +322,9 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant
     if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer
         if (lane == 0) {
+            const bool short_box = EPI == EPI_LMHEAD ? kCopies && ep.copies > 1 : !kPair;
             const int rem = n_rows % kBM, x_last = (rem + 7) / 8 * 8;
-            const int m_all = (n_rows + kBM - 1) / kBM, m_short = !kPair && rem > 0 && rem <= kShortRows ? m_all - 1 : -1;
+            const int m_all = (n_rows + kBM - 1) / kBM, m_short = short_box && rem > 0 && rem <= kShortRows ? m_all - 1 : -1;
             const CUtensorMap* only = m_short == 0 ? &tmap_xl : &tmap_x;
             ptx::prefetch_tmap(only);
             ptx::prefetch_tmap(&tmap_w0);
@@ -333,9 +335,10 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant
             // the even CTA alone arms with the bytes of both halves.
             // X rows: M-tiles through tmap_x; a last one of at most kShortRows rows through tmap_xl, whose box
             // ends with the rows (in whole 8-row swizzle groups: a box mostly outside the tensor is slow
-            // to fill); an M-tile past the rows not at all. Pairs always take whole boxes: their MMAs
-            // cover the padding, and zeros there cost less power than what the stage held before (320
-            // rows of the LM head 383 against 440 us under the board's power cap).
+            // to fill); an M-tile past the rows not at all. Pairs, and the LM head but for copies of the rows,
+            // always take whole boxes: their MMAs cover the padding, and zeros there cost less than what the
+            // stage held before (V = 151936, d = 4096: 320 rows on pairs 383 against 440 us under the board's
+            // power cap, 270 on single CTAs 315 against 325; V = 9001, 16 rows 27 against 30).
             const int copies = kCopies ? ep.copies : 1;
             auto load_x = [&](uint8_t* sp, uint64_t* bar, int j, int kb, int mt) {
                 uint8_t* dst = sp + j * C::kABytes;
@@ -1234,9 +1237,12 @@ cudaError_t launch_lmhead_tc(const Ctx& ctx, const void* lm_head, const void* x,
     CUtensorMap tw;
     // Few rows would leave all epilogue work to the warps of one TMEM lane quarter, which share one
     // scheduler (the TMA producer's): copies of the rows in the other quarters spread it over all sixteen
-    // warps (V = 151936, 16 rows: d = 512 34 -> 28 us, d = 1024 63 -> 50, d = 2048 118 -> 99, d = 4096 the
-    // same on GB300).
-    const int copies = n_rows <= 32 ? 4 : n_rows <= 64 ? 2 : 1;
+    // warps (V = 151936, 16 rows: d = 512 37 -> 28 us, d = 1024 64 -> 49, d = 2048 116 -> 101, d = 3072 174 ->
+    // 144 on GB300). None from d = 4096 on, where the stream of W sets the pace and more copies per stage delay
+    // it (V = 45000 79 against 85 us with copies), nor where a CTA's only block waits for its loads, with
+    // half of the SMs idle (V = 9001: d = 2048 16.5 against 20.6, but d = 512 9.6 against 9.1).
+    const bool copied = d < 4096 && (2 * n_tiles > ctx.num_sms || d <= 512);
+    const int copies = !copied ? 1 : n_rows <= 32 ? 4 : n_rows <= 64 ? 2 : 1;
     cudaError_t e = make_xmaps(&tx, x, d, n_rows);
     if (e == cudaSuccess) e = make_tmap(&tw, lm_head, d, V, kBK, kBlockV / cl);
     if (e != cudaSuccess) return e;

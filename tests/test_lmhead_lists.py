@@ -13,6 +13,8 @@ CASES = [
     (20000, 128, 64, "bf16", "plain"),
     (20000, 128, 1, "bf16", "plain"),
     (20000, 64, 512, "bf16", "plain"),
+    (20000, 576, 32, "bf16", "plain"),       # copies of the rows with d > 512 (79 blocks)
+    (20000, 4096, 32, "bf16", "plain"),      # and none from d = 4096 on
     (20000, 128, 64, "f32", "plain"),
     (60000, 128, 200, "bf16", "plain"),      # candidates around 256, up to which they are ranked by counting
     (60000, 128, 240, "bf16", "plain"),
@@ -28,9 +30,9 @@ CASES = [
     (20000, 320, 40, "f32", "twins"),
 ]
 # numbers of rows at which the tensor-core kernel changes: four copies of the rows, two, one; then
-# with d > 512 CTA pairs, single CTAs over three (and five) M-tiles, pairs again
-ROWS = [(1, 64), (32, 64), (33, 64), (64, 64), (65, 64), (128, 64), (129, 64), (129, 576), (256, 576), (257, 576),
-        (385, 576), (513, 576), (641, 576)]
+# with d > 512 no copies (of 36 vocabulary blocks), CTA pairs, single CTAs over three (and five) M-tiles, pairs again
+ROWS = [(1, 64), (32, 64), (33, 64), (64, 64), (65, 64), (128, 64), (129, 64), (1, 576), (40, 576), (129, 576),
+        (256, 576), (257, 576), (385, 576), (513, 576), (641, 576)]
 
 
 @pytest.mark.parametrize("n,d", ROWS)
