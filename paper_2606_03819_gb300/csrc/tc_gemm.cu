@@ -1313,6 +1313,12 @@ cudaError_t run_gemm_var(const Ctx& ctx, const XMaps& tx, const void* w0, const 
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
+// Clusters of three left unused of those that fit an empty GPU: with as many as fit, one often finds no place
+// beside clusters of the next or the previous kernel, and runs a round of its own (46 clusters, Eq. 1 of 241 rows,
+// d = 1920, I = 5120 57 to 66 us; with two to spare 49, with reduction kernels 50). Clusters of two and four
+// always found one (d = I = 4608, 36 of four: 64 us, 73 with two to spare).
+constexpr int kSpareTriples = 2;
+
 // The same where K is split: k_splits CTAs form a cluster on one output tile and exchange their partial
 // sums, so no reduction kernel follows. All clusters must be resident at once (one tile each), which
 // bounds their number; the tile width follows from it. *done stays false, and nothing runs, where there
@@ -1332,7 +1338,7 @@ cudaError_t run_gemm_cluster(const Ctx& ctx, const XMaps& tx, const void* w0, co
         for (int c = 2; c <= kMaxKSplits; ++c) f.n[c] = resident_clusters(kern, C::kSmemBytes, c, ctx.num_sms);
         return f;
     }();
-    const int max_cl = fit.n[k_splits];
+    const int max_cl = fit.n[k_splits] - (k_splits == 3 ? kSpareTriples : 0);
     int bn = 32;
     while (bn < 128 && static_cast<long long>((N + bn - 1) / bn) * n_mgroups > max_cl) bn += kStep;
     const int n_ntiles = (N + bn - 1) / bn;
