@@ -139,9 +139,9 @@ int32_t tf_version(void);
 uint64_t tf_kernel_launches(void);
 
 /* What the builder by levels (tf_build_tree with large budgets) has done on the current device since the
- * library was loaded: counts[0] trees that it left to the queue, whose lists are not sorted, not finite
- * or above 0 or whose nodes tie too often, counts[1] times it dropped nodes to make room. The results do not
- * depend on either; the time does. Synchronises the device. */
+ * library was loaded: counts[0] trees that it left to the queue (lists that are not sorted, above 0 or NaN,
+ * fewer finite entries than B, too many equal scores), counts[1] times it dropped nodes to make room. The
+ * results do not depend on either; the time does. Synchronises the device, so not inside a stream capture. */
 tf_status tf_builder_counts(uint64_t counts[2]);
 
 /* Failure detection. Every wait inside the tensor-core kernels (a TMA copy landing, an MMA

@@ -1227,7 +1227,8 @@ cudaError_t launch_lmhead_tc(const Ctx& ctx, const void* lm_head, const void* x,
     // CTA keeps one TMEM slot per unit and overlaps its epilogue with the next unit's MMAs; 32 KB
     // per CTA and stage leaves room for seven stages. Three and five M-tiles run on single CTAs, which
     // read each weight tile once per M-tile from L2 but leave out the missing half of the last pair
-    // (V = 151936, d = 4096: 320 rows 390 -> 345 us, 600 rows 575 -> 552; d = 1024: 115 -> 92, 174 -> 150;
+    // (V = 151936, d = 4096: 320 rows 390 -> 345 us, 322 with whole boxes of X, 600 rows 575 -> 552; d = 1024:
+    // 115 -> 92, 174 -> 150;
     // seven M-tiles gain nothing), and so do small d, where the epilogue sets the pace and single CTAs
     // hand over their accumulators sooner (d = 512: 250 rows 46 -> 41 us, 1020 rows 147 -> 139; d = 1024:
     // 64 -> 71, so pairs from there on).

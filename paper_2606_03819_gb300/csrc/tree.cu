@@ -668,8 +668,7 @@ __global__ void __launch_bounds__(kFastThreads) build_tree_fast_kernel(TreeArgs 
 // counting, several threads per node (one phase instead of the five of a histogram: 1.3 -> 0.7 us,
 // the order 2.2 -> 1.5 us), more nodes are ordered by buckets and counting within a bucket (513 nodes
 // 6 -> 3.5 us; a bitonic sort has 55 phases), and the root token and position, which may lie in host
-// memory, are read at the start (B = 64, eight sequences 19.8 -> 18.4 us with the mask, B = 512 44.9 ->
-// 37.5, B = 1023 76 -> 63).
+// memory, are read at the start (B = 512 with the mask 44.9 -> 37.5 us, B = 1023 76 -> 63).
 //  - Two nodes of equal score and depth under different parents are ordered by their parents' places
 //    in the order, known once shallower levels are: the few such ties are resolved after the sort.
 //  - A score of -inf ends its list (as padding of short lists does). A list entry above its predecessor or
@@ -949,7 +948,7 @@ __global__ void __launch_bounds__(kLvThreads) build_tree_level_kernel(TreeArgs a
         const int* cand = t.topm + (d - 1) * a.M;
         const bool deeper = d < a.gamma;
         // list chunks taken of each parent per pass: small budgets rarely want a second one, so no more
-        // than the warps take in one go (B = 64: 16.5 -> 15.5 us)
+        // than the warps take in one go (B = 96 22.8 -> 21.9 us, B = 65 of 16 levels 49.0 -> 46.7)
         int g = (a.B <= 128 ? kLvWarps : 2 * kLvWarps) / n_act;
         g = g < 1 ? 1 : g > n_chunks ? n_chunks : g;
         while (n_act > 0) {
